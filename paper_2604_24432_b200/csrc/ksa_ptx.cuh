@@ -148,6 +148,44 @@ __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 
+// The same for an issuing warp that stays converged: every lane passes the same (warp-uniform) operands, which the
+// compiler then keeps in uniform registers, and only the lane with `leader` != 0 issues.  Issued from inside an
+// `if (lane == 0)` region, every operand of every MMA is moved to a uniform register on its own, and that serial
+// instruction stream, not the tensor pipe, sets the rate.  Descriptors come as the low word (address, leading
+// dimension) and the high word (stride, version, swizzle), which is the same for all tiles of this library.
+__device__ __forceinline__ void mma_ss_warp(uint32_t leader, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 e, %0, 0;\n\tsetp.ne.b32 p, %6, 0;\n\t"
+        "mov.b64 da, {%2, %4};\n\tmov.b64 db, {%3, %4};\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%1], da, db, %5, p;\n\t}"
+        ::"r"(leader), "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void mma_ts_warp(uint32_t leader, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\t.reg .b64 db;\n\t"
+        "setp.ne.b32 e, %0, 0;\n\tsetp.ne.b32 p, %6, 0;\n\t"
+        "mov.b64 db, {%3, %4};\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%1], [%2], db, %5, p;\n\t}"
+        ::"r"(leader), "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void tc_commit_warp(uint32_t leader, uint32_t bar)
+{
+    asm volatile(
+        "{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %0, 0;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%1];\n\t}"
+        ::"r"(leader), "r"(bar) : "memory");
+}
+// One lane of a converged warp (1 there, 0 elsewhere)
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e;
+}
+
 // Instruction descriptor, kind::f16: bf16 A and B, fp32 accumulator, M x N tile.
 // Bit layout: [4,6) D format (1 = f32); [7,10) A format (1 = bf16); [10,13) B format;
 // 15 A major (0 = K-major); 16 B major (1 = MN-major); [17,23) N >> 3; [24,29) M >> 4.
@@ -170,6 +208,11 @@ __device__ __forceinline__ uint64_t make_smem_desc_sw128(uint32_t saddr, uint32_
     d |= (uint64_t)2 << 61;
     return d;
 }
+
+// The two words of that descriptor for mma_*_warp: leading dimension and address in the low one, which may be
+// advanced by (bytes >> 4), the rest in the high one.
+__device__ __forceinline__ constexpr uint32_t smem_desc_hi_sw128(uint32_t sbo_bytes) { return (sbo_bytes >> 4) | (1u << 14) | (2u << 29); }
+__device__ __forceinline__ constexpr uint32_t smem_desc_lo(uint32_t saddr, uint32_t lbo_bytes) { return ((saddr & 0x3FFFFu) >> 4) | ((lbo_bytes >> 4) << 16); }
 
 // ---- tcgen05: TMEM <-> registers, 32 lanes x 32-bit, 32 consecutive columns -----------
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])

@@ -5,23 +5,37 @@
 // tiles Eq. 3 makes visible to it: tiles of the packed summary stream first, then tiles of
 // the packed text stream (the sliding-chunk band up to the diagonal).
 //
-// Warp roles (384 threads = three warpgroups; warps 10-11 idle, they complete the third one):
+// Warp roles (384 threads = three warpgroups):
 //   warps 0-3   softmax of query tile 0 (one row per thread), O rescale, epilogue
 //   warps 4-7   softmax of query tile 1
-//   warp  8     TMA producer: Q tiles, then K and V tiles through a ring of smem stages
-//   warp  9     MMA issuer: S = Q K^T (smem x smem) and O += P V (P from TMEM) via tcgen05.mma
-// TMEM (512 columns): S0 [0,128), S1 [128,256), O0 [256,256+D), O1 [384,384+D); the bf16
-// probabilities P_t overwrite the first 64 columns of S_t.
+//   warp  8     TMA: Q tiles and K tiles (a ring of shared-memory stages)
+//   warp  9     issues S = Q K^T (smem x smem, tcgen05.mma)
+//   warp 10     issues O += P V (P from TMEM)
+//   warp 11     TMA: V tiles (a ring of their own)
+// TMEM (512 columns): one score slot S [0,128) that the two query tiles take in turns, the bf16
+// probabilities P0 [128,192) and P1 [192,256), O0 [256,256+D), O1 [384,384+D).
 //
 // Pipeline per key/value tile j and query tile t:
-//   MMA:     S_t(j) = Q_t K(j)^T                                   -> s_full[t]
-//   softmax: load S_t, mask (only on tiles flagged partial), running max with lazy rescale,
-//            p = 2^(s*scale*log2e - m), row sum, write P_t, rescale O_t if the max moved -> p_full[t]
-//   MMA:     O_t += P_t V(j), then at once S_t(j+1) = Q_t K(j+1)^T -> s_full[t]
-// so that while one query tile is in its softmax the tensor pipe works for the other.
-// tcgen05.mma operations of one thread execute in issue order, which is what lets S_t(j+1)
-// overwrite P_t(j) right after O_t += P_t(j) V(j) was issued, and what makes s_full[t] of
-// tile j imply that O_t += P_t V(j-1) has completed (so the softmax warps may rescale O_t).
+//   warp 9:  once the slot is free (loaded[] of the scores before): S_t(j) = Q_t K(j)^T -> s_full[t]
+//   softmax: load S_t into registers, hand the slot on                                  -> loaded[t]
+//            mask (only on tiles flagged partial), running max with lazy rescale,
+//            p = 2^(s*scale*log2e - m), row sum; wait for O_t += P_t V(j-1), rescale O_t
+//            if the max moved, write P_t                                                -> p_full[t]
+//   warp 10: O_t += P_t V(j)                                                            -> pv_done[t]
+// A score row only has to stand in TMEM between its product and its load: the exponentials (most of a
+// tile's time) work from registers.  So one slot serves both query tiles, and the scores of a query
+// tile's next key tile are formed while its softmax still works on the one before: neither the
+// products nor the two hand-overs stand between one softmax and the next.  (With a slot per query tile
+// and P over it, every tile went through softmax, hand-over, 16 products, hand-over one after the other.)
+// The two products have an issuing warp each, so that neither waits in the other's instruction stream:
+// an issuing warp executes about one instruction in seven cycles beside the softmax warps, so the eight
+// MMAs of a product take it as long to issue as the tensor pipe needs for them, and every barrier check
+// on top left the pipe idle.  One sequence of 32,768 tokens, 32/8 heads, whole call: 1.532 ms with a slot per query
+// tile, 1.477 ms with the shared slot and one issuing thread, 1.466 ms with a converged issuing warp, 1.328 ms with
+// two.  131,072 tokens, 32/4 heads: 18.9 -> 16.6 ms a call (the clock falls from 1,700 to 1,430 MHz under the
+// power limit as the pipes fill), 8,192 tokens: 258 -> 229 us.
+// What bounds it now: the softmax warps.  A key tile and pair of query tiles takes 2,920 cycles, 2,048 of them
+// exponentials on the special-function unit; the issuing warps wait 60 % of the time.
 //
 // Every mbarrier wait is bounded: on timeout the thread records which wait gave up in the
 // status word, raises a CTA-wide abort flag, all roles leave their loops, the producer
@@ -36,61 +50,39 @@ namespace ksa {
 
 using namespace ptx;
 
-// Optional event trace (compile with -DKSA_TRACE): CTAs 0 and 100 record (event id, clock) pairs
-// per role into a device buffer that ksa_debug_read_trace() copies out.  Compiled out by default.
-#ifdef KSA_TRACE
-constexpr int kTraceEvents = 8192;
-constexpr int kTraceRoles = 12;             // 0 MMA issuer, 1-2 softmax row 0 of tile 0/1, 3 producer, 4-11 per-warp arrivals
-__device__ uint2 g_trace[2][kTraceRoles][kTraceEvents];
-__device__ uint32_t g_trace_cnt[2][kTraceRoles];
-__device__ unsigned long long g_cta_span[2][256];   // start / end of every CTA (globaltimer, ns)
-#define KSA_TR(role, id)                                                                           \
-    do {                                                                                           \
-        if (tr_slot >= 0 && tr_n < (uint32_t)kTraceEvents) {                                       \
-            g_trace[tr_slot][role][tr_n] = make_uint2((uint32_t)(id), (uint32_t)clock64());        \
-            g_trace_cnt[tr_slot][role] = ++tr_n;                                                   \
-        }                                                                                          \
-    } while (0)
-#else
-#define KSA_TR(role, id) do { } while (0)
-#endif
-
-constexpr int kThreadsTc = 384;           // three warpgroups; warps 10 and 11 only take part in the register hand-over
+constexpr int kThreadsTc = 384;           // three warpgroups
 constexpr int kRegsSoftmax = 216;         // registers per thread of the softmax warpgroups after the hand-over
-constexpr int kRegsOther = 72;            // ... of the producer / MMA warpgroup
+constexpr int kRegsOther = 72;            // ... of the TMA / MMA warpgroup
 // The CTA's register allocation is fixed at launch (65,536 / 384 threads = 170 -> 168 per thread): the softmax warps
 // can only gain what the third warpgroup gives up; a larger setmaxnreg.inc would wait forever.
 static_assert(8 * kRegsSoftmax + 4 * kRegsOther <= 12 * ((65536 / 384) / 8 * 8), "register hand-over exceeds the CTA's allocation");
-constexpr int kProducerWarp = 8;
-constexpr int kMmaWarp = 9;
+constexpr int kLoadQkWarp = 8, kQkWarp = 9, kPvWarp = 10, kLoadVWarp = 11;
 // log2 units: P stays below 2^12.  A small threshold costs rescales of O: with 1 % of the keys four times larger (the 128k
 // workload) some row of nearly every warp outgrew 2^8 once or twice per work item.  Measured at 128k: 8 -> 1,032,
 // 12 -> 1,047, 20 -> 1,058 TFLOP/s, but the error against the fp64 oracle grows with it (mean |err| 5.6e-4, 5.9e-4,
 // 6.2e-4; at 20 one sampled element of the 64 + 8 layout left the 2e-2 bound), so 12 it is.
 constexpr float kRescaleThreshold = 12.0f;
 
+// barrier slots; then K full, K empty, V full, V empty per stage
+enum : int { BAR_QFULL = 0, BAR_QEMPTY = 2, BAR_SFULL = 4, BAR_LOADED = 6, BAR_PFULL = 8, BAR_PVDONE = 10, BAR_DRAIN = 12, kBarKv = 14 };
+
 template <int D>
 struct TcCfg {
     static constexpr int kTileBytes = 128 * D * 2;
     static constexpr int kHalves = D / 64;                       // 64-column (128-byte) swizzle panels
-    static constexpr int kStages = (D == 128) ? 5 : 10;          // K/V ring depth (tiles)
+    // Ring depths (tiles).  A K stage is taken up early (scores are formed a tile ahead), a V stage as its
+    // probabilities are ready: with five stages beside the two Q tiles (all that fits at D = 128) K gets three.
+    static constexpr int kStagesK = (D == 128) ? 3 : 5, kStagesV = (D == 128) ? 2 : 5;
     static constexpr int kQOff = 0;
-    static constexpr int kRingOff = 2 * kTileBytes;
-    static constexpr int kBarOff = kRingOff + kStages * kTileBytes;
-    static constexpr int kNumBars = 9 + 2 * kStages;
+    static constexpr int kKOff = 2 * kTileBytes;
+    static constexpr int kVOff = kKOff + kStagesK * kTileBytes;
+    static constexpr int kBarOff = kVOff + kStagesV * kTileBytes;
+    static constexpr int kNumBars = kBarKv + 2 * (kStagesK + kStagesV);
     static constexpr int kSmemBytes = kBarOff + 8 * kNumBars + 64 + 1024;   // + slack for 1024-byte alignment
     // MN-major V operand: the two 64-column panels of a D = 128 tile are 16 KB apart,
     // groups of 8 keys are 1 KB apart.
     static constexpr uint32_t kVLbo = 16384;
     static constexpr uint32_t kVSbo = 1024;
-};
-
-// barrier slots
-enum : int { BAR_QFULL = 0, BAR_QEMPTY = 1, BAR_SFULL = 2, BAR_PFULL = 4, BAR_OFULL = 6, BAR_DRAIN = 8, BAR_KV = 9 };
-
-struct TcShared {
-    uint32_t bars;        // smem address of barrier 0
-    uint32_t abort_addr;  // smem address of the abort flag
 };
 
 template <int D>
@@ -101,38 +93,37 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t sQ = smem_base + Cfg::kQOff;
-    const uint32_t sRing = smem_base + Cfg::kRingOff;
+    const uint32_t sK = smem_base + Cfg::kKOff, sV = smem_base + Cfg::kVOff;
     const uint32_t bars = smem_base + Cfg::kBarOff;
     const uint32_t tmem_slot = bars + 8 * Cfg::kNumBars;
     const uint32_t abort_addr = tmem_slot + 4;
     auto bar = [&](int i) -> uint32_t { return bars + 8u * (uint32_t)i; };
-    auto kv_full = [&](int s) -> uint32_t { return bars + 8u * (uint32_t)(BAR_KV + s); };
-    auto kv_empty = [&](int s) -> uint32_t { return bars + 8u * (uint32_t)(BAR_KV + Cfg::kStages + s); };
+    auto k_full = [&](int st) -> uint32_t { return bar(kBarKv + st); };
+    auto k_empty = [&](int st) -> uint32_t { return bar(kBarKv + Cfg::kStagesK + st); };
+    auto v_full = [&](int st) -> uint32_t { return bar(kBarKv + 2 * Cfg::kStagesK + st); };
+    auto v_empty = [&](int st) -> uint32_t { return bar(kBarKv + 2 * Cfg::kStagesK + Cfg::kStagesV + st); };
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
     const int lane = tid & 31;
-#ifdef KSA_TRACE
-    const int tr_slot = (blockIdx.x == 0) ? 0 : ((blockIdx.x == 100) ? 1 : -1);
-    uint32_t tr_n = 0;
-    if (tid == 0 && blockIdx.x < 256) { unsigned long long t_; asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t_)); g_cta_span[0][blockIdx.x] = t_; }
-#endif
 
     if (tid == 0) {
-        mbar_init(bar(BAR_QFULL), 1);
-        mbar_init(bar(BAR_QEMPTY), 1);
         for (int t = 0; t < 2; ++t) {
+            mbar_init(bar(BAR_QFULL + t), 1);
+            mbar_init(bar(BAR_QEMPTY + t), 1);
             mbar_init(bar(BAR_SFULL + t), 1);
-            mbar_init(bar(BAR_PFULL + t), 4);      // one arrival per softmax warp
-            mbar_init(bar(BAR_OFULL + t), 1);
+            mbar_init(bar(BAR_LOADED + t), 4);     // one arrival per softmax warp
+            mbar_init(bar(BAR_PFULL + t), 4);
+            mbar_init(bar(BAR_PVDONE + t), 1);
+            mbar_init(bar(BAR_DRAIN + t), 1);
         }
-        mbar_init(bar(BAR_DRAIN), 1);
-        for (int s = 0; s < Cfg::kStages; ++s) { mbar_init(kv_full(s), 1); mbar_init(kv_empty(s), 1); }
+        for (int st = 0; st < Cfg::kStagesK; ++st) { mbar_init(k_full(st), 1); mbar_init(k_empty(st), 1); }
+        for (int st = 0; st < Cfg::kStagesV; ++st) { mbar_init(v_full(st), 1); mbar_init(v_empty(st), 1); }
         st_shared_u32(abort_addr, 0u);
         st_shared_u32(abort_addr + 4, 0u);     // never raised: lets the teardown waits run while aborting
         fence_mbar_init();
     }
-    if (warp == kProducerWarp) {            // one warp allocates all 512 TMEM columns (1 CTA per SM)
+    if (warp == kLoadQkWarp) {            // one warp allocates all 512 TMEM columns (1 CTA per SM)
         tmem_alloc(tmem_slot, 512);
         tmem_relinquish();
     }
@@ -149,232 +140,201 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
     auto item_index = [&](int r) -> int { return r * grid + ((r & 1) ? (grid - 1 - cta) : cta); };
 
     if (warp >= 8) {
-    // register hand-over: this warpgroup gives most of its registers to the softmax warpgroups,
-    // which keep a whole 128-column score row per thread
-    setmaxnreg_dec<kRegsOther>();
-    if (warp == kProducerWarp) {
-        // =============================== TMA producer ===============================
-        if (lane == 0) {
-            prefetch_tensormap(&maps.qt); prefetch_tensormap(&maps.kt); prefetch_tensormap(&maps.vt);
-            prefetch_tensormap(&maps.ks); prefetch_tensormap(&maps.vs);
-            uint32_t q_phase = 0, ring_phase = 0;
-            int stage = 0;
-            uint32_t armed_mask = 0, armed_parity = 0;   // per stage: a load was issued / with which parity
-            bool q_armed = false;
-            bool alive = true;
-            for (int r = 0; alive; ++r) {
-                const int idx = item_index(r);
-                if (idx >= a.num_work) break;
-                const WorkItem w = a.work[idx];
-                const SeqInfo sq = a.seqs[w.seq];
-                // the two query heads of an item share a KV head (one K and one V tile per key tile) or, where a pair
-                // straddles two KV heads (multi-head attention, odd group sizes), each has its own: then every key tile
-                // takes four ring stages, K for head 0, K for head 1, V for head 0, V for head 1
-                const int hk = w.head0 / G;
-                const int nsplit = ((w.head0 + w.n_heads - 1) / G != hk) ? 2 : 1;
-                const int T = w.ns_tiles + (w.band_hi - w.band_lo + 1);
-                if (!bounded_wait(bar(BAR_QEMPTY), q_phase ^ 1u, abort_addr, a.status, kStatusWaitQEmpty)) break;
-                mbar_arrive_expect_tx(bar(BAR_QFULL), (uint32_t)(w.n_heads * Cfg::kTileBytes));
-                q_armed = true;
-                for (int t = 0; t < w.n_heads; ++t)
-                    for (int h = 0; h < Cfg::kHalves; ++h)
-                        if (a.direct)
-                            tma_load_4d(sQ + t * Cfg::kTileBytes + h * 16384, &maps.qt, bar(BAR_QFULL),
-                                        h * 64, 0, sq.chunk0 + w.q_tile * (kTileM / a.k), w.head0 + t);
-                        else
-                            tma_load_3d(sQ + t * Cfg::kTileBytes + h * 16384, &maps.qt, bar(BAR_QFULL),
-                                        h * 64, sq.text_off + w.q_tile * kTileM, w.head0 + t);
-                q_phase ^= 1u;
-                for (int j = 0; j < T && alive; ++j) {
-                    const bool summ = j < w.ns_tiles;
-                    const int y = summ ? (sq.summ_off + j * kTileN) : (sq.text_off + (w.band_lo + j - w.ns_tiles) * kTileN);
-                    // direct views: a tile is 128/m chunks of the summary view or 128/k chunks of the text view
-                    const int zc = sq.chunk0 + (summ ? j * (kTileN / max(a.m, 1)) : (w.band_lo + j - w.ns_tiles) * (kTileN / a.k));
-                    const CUtensorMap* mk = summ ? &maps.ks : &maps.kt;
-                    const CUtensorMap* mv = summ ? &maps.vs : &maps.vt;
-                    for (int kvt = 0; kvt < 2 * nsplit && alive; ++kvt) {
-                        const int kv = kvt / nsplit, hkt = hk + kvt % nsplit;
-                        if (!bounded_wait(kv_empty(stage), ring_phase ^ 1u, abort_addr, a.status, kStatusWaitKvEmpty)) { alive = false; break; }
-                        mbar_arrive_expect_tx(kv_full(stage), (uint32_t)Cfg::kTileBytes);
-                        armed_mask |= 1u << stage;
-                        armed_parity = (armed_parity & ~(1u << stage)) | (ring_phase << stage);
+        // register hand-over: this warpgroup gives most of its registers to the softmax warpgroups,
+        // which keep a whole 128-column score row per thread
+        setmaxnreg_dec<kRegsOther>();
+        if (warp == kLoadQkWarp || warp == kLoadVWarp) {
+            // =============================== TMA producers ===============================
+            // warp 8: the Q tiles of an item and its K tiles; warp 11: its V tiles.  The two query heads of an item share
+            // a KV head (one K and one V tile per key tile) or, where a pair straddles two KV heads (multi-head attention,
+            // odd group sizes), each has its own: then a key tile takes two stages of each ring, head 0 first.
+            if (lane == 0) {
+                const bool is_v = warp == kLoadVWarp;
+                const CUtensorMap* map_t = is_v ? &maps.vt : &maps.kt;
+                const CUtensorMap* map_s = is_v ? &maps.vs : &maps.ks;
+                prefetch_tensormap(map_t); prefetch_tensormap(map_s);
+                if (!is_v) prefetch_tensormap(&maps.qt);
+                const int stages = is_v ? Cfg::kStagesV : Cfg::kStagesK;
+                const uint32_t ring = is_v ? sV : sK, full0 = is_v ? v_full(0) : k_full(0), empty0 = is_v ? v_empty(0) : k_empty(0);
+                uint32_t q_phase = 0, ring_phase = 0;        // q_phase: bit t for query tile t
+                int stage = 0;
+                uint32_t armed_mask = 0, armed_parity = 0;   // per stage: a load was issued / with which parity
+                uint32_t q_armed = 0;                        // per query tile: a load was issued
+                bool alive = true;
+                for (int r = 0; alive; ++r) {
+                    const int idx = item_index(r);
+                    if (idx >= a.num_work) break;
+                    const WorkItem w = a.work[idx];
+                    const SeqInfo sq = a.seqs[w.seq];
+                    const int hk = w.head0 / G;
+                    const int nsplit = ((w.head0 + w.n_heads - 1) / G != hk) ? 2 : 1;
+                    const int T = w.ns_tiles + (w.band_hi - w.band_lo + 1);
+                    auto load_q = [&](int t) {
+                        if (!bounded_wait(bar(BAR_QEMPTY + t), ((q_phase >> t) & 1u) ^ 1u, abort_addr, a.status, kStatusWaitQEmpty)) { alive = false; return; }
+                        q_phase ^= 1u << t;
+                        mbar_arrive_expect_tx(bar(BAR_QFULL + t), (uint32_t)Cfg::kTileBytes);
+                        q_armed |= 1u << t;
                         for (int h = 0; h < Cfg::kHalves; ++h)
                             if (a.direct)
-                                tma_load_4d(sRing + stage * Cfg::kTileBytes + h * 16384, kv ? mv : mk, kv_full(stage), h * 64, 0, zc, hkt);
+                                tma_load_4d(sQ + t * Cfg::kTileBytes + h * 16384, &maps.qt, bar(BAR_QFULL + t),
+                                            h * 64, 0, sq.chunk0 + w.q_tile * (kTileM / a.k), w.head0 + t);
                             else
-                                tma_load_3d(sRing + stage * Cfg::kTileBytes + h * 16384, kv ? mv : mk, kv_full(stage), h * 64, y, hkt);
-                        if (++stage == Cfg::kStages) { stage = 0; ring_phase ^= 1u; }
-                    }
-                }
-            }
-            if (ld_shared_u32(abort_addr) != 0u) {
-                // leave no copy in flight behind: wait (bounded) for every load that was issued
-                if (q_armed) bounded_wait(bar(BAR_QFULL), q_phase ^ 1u, abort_addr + 4, a.status, kStatusWaitQFull);
-                for (int s = 0; s < Cfg::kStages; ++s)
-                    if (armed_mask & (1u << s))
-                        bounded_wait(kv_full(s), (armed_parity >> s) & 1u, abort_addr + 4, a.status, kStatusWaitKvFull);
-            }
-        }
-    } else if (warp == kMmaWarp) {
-        // =============================== MMA issuer =================================
-        if (lane == 0) {
-            constexpr uint32_t idesc_qk = make_idesc_bf16(128, 128, false);
-            constexpr uint32_t idesc_pv = make_idesc_bf16(128, D, true);
-            uint32_t qf_phase = 0, pf_phase[2] = {0, 0}, ring_phase = 0;
-            int stage = 0;
-            bool alive = true;
-            auto issue_qk = [&](int t, int st) {
-                const uint64_t qd = make_smem_desc_sw128(sQ + t * Cfg::kTileBytes, 16, 1024);
-                const uint64_t kd = make_smem_desc_sw128(sRing + st * Cfg::kTileBytes, 16, 1024);
-#pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) {
-                    const uint32_t off = (uint32_t)((kk >> 2) * 16384 + (kk & 3) * 32) >> 4;
-                    mma_ss(tmem + t * 128, qd + off, kd + off, idesc_qk, kk > 0 ? 1u : 0u);
-                }
-            };
-            auto issue_pv = [&](int t, int st, bool acc) {
-                const uint64_t vd = make_smem_desc_sw128(sRing + st * Cfg::kTileBytes, Cfg::kVLbo, Cfg::kVSbo);
-#pragma unroll
-                for (int kk = 0; kk < kTileN / 16; ++kk)
-                    mma_ts(tmem + 256 + t * 128, tmem + t * 128 + kk * 8, vd + (uint32_t)((kk * 2048) >> 4), idesc_pv,
-                           (acc || kk > 0) ? 1u : 0u);
-            };
-            for (int r = 0; alive; ++r) {
-                const int idx = item_index(r);
-                if (idx >= a.num_work) break;
-                const WorkItem w = a.work[idx];
-                const int T = w.ns_tiles + (w.band_hi - w.band_lo + 1);
-                const int nh = w.n_heads;
-                // one K and one V stage per key tile, or one per query head where the pair straddles two KV heads
-                const int nsplit = ((w.head0 + nh - 1) / G != w.head0 / G) ? 2 : 1;
-                if (nsplit == 1) {
-                // ---- one K and one V stage per key tile (the two heads share a KV head, or a single head) ----
-                    if (!bounded_wait(bar(BAR_QFULL), qf_phase, abort_addr, a.status, kStatusWaitQFull)) break;
-                    qf_phase ^= 1u;
-                    if (!bounded_wait(kv_full(stage), ring_phase, abort_addr, a.status, kStatusWaitKvFull)) break;
-                    tc_fence_after();
-                    for (int t = 0; t < nh; ++t) { issue_qk(t, stage); tc_commit(bar(BAR_SFULL + t)); }
-                    if (++stage == Cfg::kStages) { stage = 0; ring_phase ^= 1u; }
-                    for (int j = 0; j < T && alive; ++j) {
-                        const int vstage = stage; const uint32_t vphase = ring_phase;
-                        if (++stage == Cfg::kStages) { stage = 0; ring_phase ^= 1u; }
-                        int kstage = -1; uint32_t kphase = 0;
-                        if (j + 1 < T) {
-                            kstage = stage; kphase = ring_phase;
-                            if (++stage == Cfg::kStages) { stage = 0; ring_phase ^= 1u; }
-                        }
-                        KSA_TR(0, 39);
-                        // both stages of this iteration are checked here, while the softmax warps still work on P_0: the ring
-                        // runs two tiles ahead, so neither wait depends on anything this iteration does
-                        if (!bounded_wait(kv_full(vstage), vphase, abort_addr, a.status, kStatusWaitKvFull)) { alive = false; break; }
-                        if (kstage >= 0 && !bounded_wait(kv_full(kstage), kphase, abort_addr, a.status, kStatusWaitKvFull)) { alive = false; break; }
-                        KSA_TR(0, 40);
-                        for (int t = 0; t < nh; ++t) {
-                            if (!bounded_wait(bar(BAR_PFULL + t), pf_phase[t], abort_addr, a.status, kStatusWaitPFull)) { alive = false; break; }
-                            pf_phase[t] ^= 1u;
-                            KSA_TR(0, 20 + t);
-                            tc_fence_after();
-                            issue_pv(t, vstage, j > 0);
-                            KSA_TR(0, 25 + t);
-                            if (j == T - 1) tc_commit(bar(BAR_OFULL + t));
-                            if (j + 1 < T) {
-                                issue_qk(t, kstage);
-                                tc_commit(bar(BAR_SFULL + t));
-                                KSA_TR(0, 30 + t);
-                            }
-                        }
-                        if (!alive) break;
-                    }
-                } else {
-                // ---- a pair that straddles two KV heads: every head has its own K and V stage ----
-                    if (!bounded_wait(bar(BAR_QFULL), qf_phase, abort_addr, a.status, kStatusWaitQFull)) break;
-                    qf_phase ^= 1u;
-                    // stage and phase of the K and the V tile of query tile 0 / 1 (scalars: no indexed local arrays)
-                    int kst0, kst1, vst0 = 0, vst1 = 0;
-                    uint32_t kph0, kph1, vph0 = 0, vph1 = 0;
-                    auto take = [&](int& st0, uint32_t& ph0, int& st1, uint32_t& ph1) {   // the next nsplit stages of the ring (not waited for yet)
-                        st0 = stage; ph0 = ring_phase;
-                        if (++stage == Cfg::kStages) { stage = 0; ring_phase ^= 1u; }
-                        st1 = st0; ph1 = ph0;
-                        if (nsplit == 2) {
-                            st1 = stage; ph1 = ring_phase;
-                            if (++stage == Cfg::kStages) { stage = 0; ring_phase ^= 1u; }
-                        }
+                                tma_load_3d(sQ + t * Cfg::kTileBytes + h * 16384, &maps.qt, bar(BAR_QFULL + t),
+                                            h * 64, sq.text_off + w.q_tile * kTileM, w.head0 + t);
                     };
-                    auto full = [&](int st, uint32_t ph) -> bool { return bounded_wait(kv_full(st), ph, abort_addr, a.status, kStatusWaitKvFull); };
-                    take(kst0, kph0, kst1, kph1);
-                    if (!full(kst0, kph0) || !full(kst1, kph1)) break;
-                    tc_fence_after();
-                    for (int t = 0; t < nh; ++t) { issue_qk(t, t ? kst1 : kst0); tc_commit(bar(BAR_SFULL + t)); }
+                    if (!is_v) load_q(0);
                     for (int j = 0; j < T && alive; ++j) {
-                        KSA_TR(0, 39);
-                        take(vst0, vph0, vst1, vph1);
-                        if (j + 1 < T) take(kst0, kph0, kst1, kph1);
-                        // With one K and one V stage per key tile both are checked here, while the softmax warps still work on
-                        // P_0: the ring runs two tiles ahead, so neither wait depends on anything this iteration does.  With
-                        // four stages per key tile the ring runs hardly one tile ahead: each stage is waited for where it is used.
-                        if (nsplit == 1) {
-                            if (!full(vst0, vph0)) { alive = false; break; }
-                            if (j + 1 < T && !full(kst0, kph0)) { alive = false; break; }
+                        const bool summ = j < w.ns_tiles;
+                        const CUtensorMap* map = summ ? map_s : map_t;
+                        // direct views: a tile is 128/m chunks of the summary view or 128/k chunks of the text view
+                        const int pos = a.direct ? sq.chunk0 + (summ ? j * (kTileN / max(a.m, 1)) : (w.band_lo + j - w.ns_tiles) * (kTileN / a.k))
+                                                 : (summ ? sq.summ_off + j * kTileN : sq.text_off + (w.band_lo + j - w.ns_tiles) * kTileN);
+                        for (int u = 0; u < nsplit; ++u) {
+                            if (!bounded_wait(empty0 + 8u * stage, ring_phase ^ 1u, abort_addr, a.status, kStatusWaitKvEmpty)) { alive = false; break; }
+                            mbar_arrive_expect_tx(full0 + 8u * stage, (uint32_t)Cfg::kTileBytes);
+                            armed_mask |= 1u << stage;
+                            armed_parity = (armed_parity & ~(1u << stage)) | (ring_phase << stage);
+                            for (int h = 0; h < Cfg::kHalves; ++h)
+                                if (a.direct)
+                                    tma_load_4d(ring + stage * Cfg::kTileBytes + h * 16384, map, full0 + 8u * stage, h * 64, 0, pos, hk + u);
+                                else
+                                    tma_load_3d(ring + stage * Cfg::kTileBytes + h * 16384, map, full0 + 8u * stage, h * 64, pos, hk + u);
+                            if (++stage == stages) { stage = 0; ring_phase ^= 1u; }
+                            if (j == 0 && u == 0 && !is_v && w.n_heads == 2) { load_q(1); if (!alive) break; }
                         }
-                        KSA_TR(0, 40);
-                        for (int t = 0; t < nh; ++t) {
-                            if (!bounded_wait(bar(BAR_PFULL + t), pf_phase[t], abort_addr, a.status, kStatusWaitPFull)) { alive = false; break; }
-                            pf_phase[t] ^= 1u;
-                            KSA_TR(0, 20 + t);
-                            if (nsplit == 2 && !full(t ? vst1 : vst0, t ? vph1 : vph0)) { alive = false; break; }
-                            tc_fence_after();
-                            issue_pv(t, t ? vst1 : vst0, j > 0);
-                            KSA_TR(0, 25 + t);
-                            if (j == T - 1) tc_commit(bar(BAR_OFULL + t));
-                            if (j + 1 < T) {
-                                if (nsplit == 2) {
-                                    if (!full(t ? kst1 : kst0, t ? kph1 : kph0)) { alive = false; break; }
-                                    tc_fence_after();
-                                }
-                                issue_qk(t, t ? kst1 : kst0);
-                                tc_commit(bar(BAR_SFULL + t));
-                                KSA_TR(0, 30 + t);
+                    }
+                }
+                if (ld_shared_u32(abort_addr) != 0u) {
+                    // leave no copy in flight behind: wait (bounded) for every load that was issued
+                    for (int t = 0; t < 2; ++t)
+                        if (q_armed & (1u << t)) bounded_wait(bar(BAR_QFULL + t), ((q_phase >> t) & 1u) ^ 1u, abort_addr + 4, a.status, kStatusWaitQFull);
+                    for (int st = 0; st < stages; ++st)
+                        if (armed_mask & (1u << st))
+                            bounded_wait(full0 + 8u * st, (armed_parity >> st) & 1u, abort_addr + 4, a.status, kStatusWaitKvFull);
+                }
+            }
+        } else {
+            // =============================== MMA issuers =================================
+            // the whole warp walks the loop on warp-uniform values, one lane issues
+            constexpr uint32_t hi = smem_desc_hi_sw128(1024);
+            const uint32_t leader = elect_one();
+            const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+            bool alive = true;
+            auto wait = [&](uint32_t b, uint32_t parity, int code) {
+                if (alive) alive = __all_sync(0xffffffffu, bounded_wait(b, parity, abort_addr, a.status, code));
+            };
+            uint32_t stage = 0, ring_phase = 0, phase0 = 0, phase1 = 0;
+            if (warp == kQkWarp) {
+                constexpr uint32_t idesc = make_idesc_bf16(128, 128, false);
+                const uint32_t q_lo = smem_desc_lo(sQ, 16), k_lo = smem_desc_lo(sK, 16);
+                uint32_t q_phase0 = 0, q_phase1 = 0;
+                int before = -1;                            // query tile whose scores stand in the slot
+                for (int r = 0; alive; ++r) {
+                    const int idx = item_index(r);
+                    if (idx >= a.num_work) break;
+                    const WorkItem w = a.work[idx];
+                    const int T = __shfl_sync(0xffffffffu, w.ns_tiles + (w.band_hi - w.band_lo + 1), 0);
+                    const int nh = __shfl_sync(0xffffffffu, w.n_heads, 0);
+                    const bool split = __shfl_sync(0xffffffffu, (w.head0 + w.n_heads - 1) / G - w.head0 / G, 0) != 0;
+                    for (int j = 0; j < T && alive; ++j) {
+#pragma unroll
+                        for (int t = 0; t < 2; ++t) {
+                            if (t == 1 && nh == 1) break;
+                            if (j == 0) {
+                                wait(bar(BAR_QFULL + t), t ? q_phase1 : q_phase0, kStatusWaitQFull);
+                                if (t) q_phase1 ^= 1u; else q_phase0 ^= 1u;
                             }
+                            if (t == 0 || split) wait(k_full(0) + 8u * stage, ring_phase, kStatusWaitKvFull);
+                            // the slot: the scores before are in their group's registers
+                            if (before == 0) { wait(bar(BAR_LOADED), phase0, kStatusWaitPFull); phase0 ^= 1u; }
+                            else if (before == 1) { wait(bar(BAR_LOADED + 1), phase1, kStatusWaitPFull); phase1 ^= 1u; }
+                            if (!alive) break;
+                            before = t;
+                            tc_fence_after();
+                            const uint32_t qd = q_lo + (uint32_t)(t * (Cfg::kTileBytes >> 4)), kd = k_lo + stage * (uint32_t)(Cfg::kTileBytes >> 4);
+#pragma unroll
+                            for (int kk = 0; kk < D / 16; ++kk) {
+                                const uint32_t off = (uint32_t)((kk >> 2) * 16384 + (kk & 3) * 32) >> 4;
+                                mma_ss_warp(leader, tm, qd + off, kd + off, hi, idesc, kk > 0 ? 1u : 0u);
+                            }
+                            tc_commit_warp(leader, bar(BAR_SFULL + t));
+                            if ((t == nh - 1 || split) && ++stage == (uint32_t)Cfg::kStagesK) { stage = 0; ring_phase ^= 1u; }
                         }
-                        if (!alive) break;
+                    }
+                }
+            } else {
+                constexpr uint32_t idesc = make_idesc_bf16(128, D, true);
+                const uint32_t v_lo = smem_desc_lo(sV, Cfg::kVLbo);
+                for (int r = 0; alive; ++r) {
+                    const int idx = item_index(r);
+                    if (idx >= a.num_work) break;
+                    const WorkItem w = a.work[idx];
+                    const int T = __shfl_sync(0xffffffffu, w.ns_tiles + (w.band_hi - w.band_lo + 1), 0);
+                    const int nh = __shfl_sync(0xffffffffu, w.n_heads, 0);
+                    const bool split = __shfl_sync(0xffffffffu, (w.head0 + w.n_heads - 1) / G - w.head0 / G, 0) != 0;
+                    for (int j = 0; j < T && alive; ++j) {
+#pragma unroll
+                        for (int t = 0; t < 2; ++t) {
+                            if (t == 1 && nh == 1) break;
+                            if (t == 0 || split) wait(v_full(0) + 8u * stage, ring_phase, kStatusWaitKvFull);
+                            wait(bar(BAR_PFULL + t), t ? phase1 : phase0, kStatusWaitPFull);
+                            if (t) phase1 ^= 1u; else phase0 ^= 1u;
+                            if (!alive) break;
+                            tc_fence_after();
+                            const uint32_t vd = v_lo + stage * (uint32_t)(Cfg::kTileBytes >> 4);
+#pragma unroll
+                            for (int kk = 0; kk < kTileN / 16; ++kk)
+                                mma_ts_warp(leader, tm + 256u + t * 128u, tm + 128u + t * 64u + kk * 8u, vd + (uint32_t)((kk * 2048) >> 4), hi, idesc,
+                                            (j > 0 || kk > 0) ? 1u : 0u);
+                            tc_commit_warp(leader, bar(BAR_PVDONE + t));
+                            if ((t == nh - 1 || split) && ++stage == (uint32_t)Cfg::kStagesV) { stage = 0; ring_phase ^= 1u; }
+                        }
                     }
                 }
             }
             // drain the tensor pipe before TMEM is released
-            tc_commit(bar(BAR_DRAIN));
-            bounded_wait(bar(BAR_DRAIN), 0, abort_addr + 4, a.status, kStatusWaitOFull);
+            const uint32_t drain = bar(BAR_DRAIN + (warp == kQkWarp ? 0 : 1));
+            tc_commit_warp(leader, drain);
+            bounded_wait(drain, 0, abort_addr + 4, a.status, kStatusWaitOFull);
         }
-    }
     } else {
         setmaxnreg_inc<kRegsSoftmax>();
         // =============================== softmax warpgroups =========================
         const int t = warp >> 2;
         const int row = tid & 127;
         const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t tS = tmem + lane_sel + (uint32_t)(t * 128);
+        const uint32_t tS = tmem + lane_sel;                                   // the score slot
+        const uint32_t tP = tmem + lane_sel + 128u + (uint32_t)(t * 64);
         const uint32_t tO = tmem + lane_sel + 256u + (uint32_t)(t * 128);
         const float scale_log2 = a.scale_log2;
-        uint32_t sf_phase = 0, of_phase = 0;
+        uint32_t sf_phase = 0, pv_phase = 0;
         const int s_len = a.k + a.m;
         bool alive = true;
-        // Shared-memory stages (and the Q tiles) are handed back to the producer by one thread of the
-        // LAST query tile's warpgroup: tcgen05 operations of the issuing thread complete in order, so
-        // its s_full for key tile j says that every product issued before it has finished reading --
-        // K(j) and V(j-1) for both query tiles.  This keeps those signals out of the MMA thread's
-        // instruction stream.  Every thread follows the ring position (two stages per key tile).
-        int rel_stage = 0;
-        auto release_next = [&]() {
-            mbar_arrive_relaxed(kv_empty(rel_stage));
-            if (++rel_stage == Cfg::kStages) rel_stage = 0;
-        };
+        // Shared-memory stages are handed back to the producers by the first thread of a warpgroup: of the item's LAST
+        // query tile where both share the K / V tiles (the products of an issuing warp complete in order, so its s_full
+        // for key tile j says that both have read K(j), its pv_done that both have read V(j)), of each query tile for
+        // its own stages where the pair straddles two KV heads.
+        int k_base = 0, v_base = 0;                        // ring stages of the item's first tiles
         for (int r = 0; alive; ++r) {
             const int idx = item_index(r);
             if (idx >= a.num_work) break;
             const WorkItem w = a.work[idx];
-            if (t >= w.n_heads) { rel_stage = (rel_stage + 2 * (w.ns_tiles + (w.band_hi - w.band_lo + 1))) % Cfg::kStages; continue; }
-            const bool releaser = (t == w.n_heads - 1) && (tid & 127) == 0;
             const int nsplit = ((w.head0 + w.n_heads - 1) / G != w.head0 / G) ? 2 : 1;   // ring stages per K / V tile
+            // the next stage this thread hands back, and how far on the one after it stands
+            int rel_k = (k_base + (nsplit - 1) * t) % Cfg::kStagesK, rel_v = (v_base + (nsplit - 1) * t) % Cfg::kStagesV;
+            k_base = (k_base + nsplit * (w.ns_tiles + (w.band_hi - w.band_lo + 1))) % Cfg::kStagesK;
+            v_base = (v_base + nsplit * (w.ns_tiles + (w.band_hi - w.band_lo + 1))) % Cfg::kStagesV;
+            if (t >= w.n_heads) continue;
+            const bool first_thread = (tid & 127) == 0;
+            const bool releaser = first_thread && (nsplit == 2 || t == w.n_heads - 1);
+            auto release_k = [&]() {
+                mbar_arrive_relaxed(k_empty(rel_k));
+                if ((rel_k += nsplit) >= Cfg::kStagesK) rel_k -= Cfg::kStagesK;
+            };
+            auto release_v = [&]() {
+                mbar_arrive_relaxed(v_empty(rel_v));
+                if ((rel_v += nsplit) >= Cfg::kStagesV) rel_v -= Cfg::kStagesV;
+            };
             const SeqInfo sq = a.seqs[w.seq];
             const int T = w.ns_tiles + (w.band_hi - w.band_lo + 1);
             const int i_raw = w.q_tile * kTileM + row;
@@ -391,7 +351,6 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) { alive = false; break; }
                 sf_phase ^= 1u;
-                if (row == 0) KSA_TR(1 + t, 1);
                 tc_fence_after();
                 uint32_t s[128];
                 {
@@ -402,24 +361,13 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
                     tmem_ld32(tS + 0, c0); tmem_ld32(tS + 32, c1); tmem_ld32(tS + 64, c2); tmem_ld32(tS + 96, c3);
                 }
                 // the stage hand-backs ride on the latency of the loads
-                if (nsplit == 2) {
-                    // a stage per head (ring order K_0, K_1, V_0, V_1 per key tile): each query tile's first thread hands
-                    // back its own head's stages as soon as its own scores say they were read; rel_stage stays at the
-                    // item's first stage until the epilogue
-                    if ((tid & 127) == 0) {
-                        if (j > 0) mbar_arrive_relaxed(kv_empty((rel_stage + 4 * (j - 1) + 2 + t) % Cfg::kStages));   // V_t(j-1)
-                        mbar_arrive_relaxed(kv_empty((rel_stage + 4 * j + t) % Cfg::kStages));                         // K_t(j)
-                        if (releaser && j == T - 1) mbar_arrive_relaxed(bar(BAR_QEMPTY));
-                    }
-                } else if (releaser) {
-                    if (j > 0) release_next();                   // V(j-1)
-                    release_next();                              // K(j)
-                    if (j == T - 1) mbar_arrive_relaxed(bar(BAR_QEMPTY));
-                } else if ((tid & 127) == 0) {
-                    rel_stage = (rel_stage + (j > 0 ? 2 : 1)) % Cfg::kStages;
-                }
+                if (releaser) release_k();                   // K(j)
+                if (first_thread && j == T - 1) mbar_arrive_relaxed(bar(BAR_QEMPTY + t));
                 tc_wait_ld();
-                if (row == 0) KSA_TR(1 + t, 2);
+                // the scores are in registers: the slot may take the next ones
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_relaxed(bar(BAR_LOADED + t));
                 // in-tile mask, only where the schedule says the tile is partial
                 bool masked;
                 int ca, cb;                                   // visible columns [ca, cb)
@@ -452,7 +400,6 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
                 mx0 = fmax3(mx0, __uint_as_float(s[124]), __uint_as_float(s[125]));
                 mx1 = fmax3(mx1, __uint_as_float(s[126]), __uint_as_float(s[127]));
                 const float mx_sc = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3)) * scale_log2;
-                if (row == 0) KSA_TR(1 + t, 3);
                 // lazy rescale: the reference max only moves when some row of the warp outgrew it
                 const bool need = mx_sc > m_used + kRescaleThreshold;
                 const bool need_any = __any_sync(0xffffffffu, need);
@@ -478,14 +425,21 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
                     s[q] = pack_bf16x2(pr.x, pr.y);
                 }
                 l_run += (la.x + la.y) + (lb.x + lb.y);
-                if (row == 0) KSA_TR(1 + t, 4);
+                if (j > 0) {
+                    // O_t += P_t V(j-1) has read P_t and written O_t
+                    ok = bounded_wait(bar(BAR_PVDONE + t), pv_phase, abort_addr, a.status, kStatusWaitPvDone);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) { alive = false; break; }
+                    pv_phase ^= 1u;
+                    if (releaser) release_v();               // V(j-1)
+                    tc_fence_after();
+                }
                 {
                     uint32_t (&p0)[32] = *reinterpret_cast<uint32_t (*)[32]>(&s[0]);
                     uint32_t (&p1)[32] = *reinterpret_cast<uint32_t (*)[32]>(&s[32]);
-                    tmem_st32(tS + 0, p0); tmem_st32(tS + 32, p1);
+                    tmem_st32(tP + 0, p0); tmem_st32(tP + 32, p1);
                 }
                 if (need_any && j > 0) {
-                    // O_t += P V(j-1) has completed (s_full of tile j was committed after it)
 #pragma unroll
                     for (int c = 0; c < D / 32; ++c) {
                         uint32_t o[32];
@@ -498,23 +452,16 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
                 }
                 tc_wait_st();
                 tc_fence_before();
+                __syncwarp();
                 if (lane == 0) mbar_arrive_relaxed(bar(BAR_PFULL + t));
-                if (row == 0) KSA_TR(1 + t, 6);
-                if (lane == 0 && row != 0) KSA_TR(4 + warp, 6);
             }
             if (!alive) break;
             // ---- epilogue: O / l -> bf16 at the row's augmented position (Eq. 1), LSE ----
-            bool ok = bounded_wait(bar(BAR_OFULL + t), of_phase, abort_addr, a.status, kStatusWaitOFull);
+            bool ok = bounded_wait(bar(BAR_PVDONE + t), pv_phase, abort_addr, a.status, kStatusWaitOFull);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
-            of_phase ^= 1u;
-            if (nsplit == 2) {
-                if ((tid & 127) == 0) {
-                    mbar_arrive_relaxed(kv_empty((rel_stage + 4 * (T - 1) + 2 + t) % Cfg::kStages));                   // V_t(T-1)
-                    rel_stage = (rel_stage + 4 * T) % Cfg::kStages;
-                }
-            } else if (releaser) release_next();                 // V(T-1)
-            else if ((tid & 127) == 0) rel_stage = (rel_stage + 1) % Cfg::kStages;
+            pv_phase ^= 1u;
+            if (releaser) release_v();                       // V(T-1)
             tc_fence_after();
             const float inv_l = 1.f / l_run;
             const int h = w.head0 + t;
@@ -545,28 +492,8 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
 
     tc_fence_before();
     __syncthreads();
-#ifdef KSA_TRACE
-    if (tid == 0 && blockIdx.x < 256) { unsigned long long t_; asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t_)); g_cta_span[1][blockIdx.x] = t_; }
-#endif
-    if (warp == kProducerWarp) tmem_dealloc(tmem, 512);
+    if (warp == kLoadQkWarp) tmem_dealloc(tmem, 512);
 }
-
-#ifdef KSA_TRACE
-extern "C" __attribute__((visibility("default"))) int ksa_debug_read_spans(void* spans)
-{
-    cudaDeviceSynchronize();
-    return (int)cudaMemcpyFromSymbol(spans, g_cta_span, sizeof(g_cta_span));
-}
-
-extern "C" __attribute__((visibility("default"))) int ksa_debug_read_trace(void* ev, void* cnt, int reset)
-{
-    cudaDeviceSynchronize();
-    if (ev) cudaMemcpyFromSymbol(ev, g_trace, sizeof(g_trace));
-    if (cnt) cudaMemcpyFromSymbol(cnt, g_trace_cnt, sizeof(g_trace_cnt));
-    if (reset) { static uint32_t z[2 * kTraceRoles] = {0}; cudaMemcpyToSymbol(g_trace_cnt, z, sizeof(z)); }
-    return (int)cudaGetLastError();
-}
-#endif
 
 cudaError_t setup_text_tc()
 {
