@@ -27,15 +27,20 @@
 // Warps 0-15: one accumulator row per thread, four warps per row quarter (warps w, w + 4, w + 8, w + 12
 // share the lanes 32 (w % 4) ..; each takes 32 of the 128 columns: the element-wise work has no reduction
 // across columns, and four warps per scheduler hide the TMEM load / store latencies); warp 16: TMA
-// producer; warp 17: MMA issuer.  The issuer's time is the critical path, so it waits only for the row
-// warps: row warp 0 checks that the next B1 / B2 stage has landed before it arrives.  The tensor pipe
-// works in order, so the completion of a product also tells which stage the accumulation before it has
-// finished with: in the dQ kernel row warp 0, which sees every completion of X and Y, passes that on to
-// the producer through one "empty" barrier per stage (the issuer is spared the extra commits -- except
-// for the K stages, which the early products would otherwise release too late); in the dK / dV kernel the
-// issuer commits to the "empty" barriers right behind each accumulation.  (The producer itself may fall
-// several completions behind, which a parity wait on a shared barrier cannot follow: hence one barrier
-// per stage.)  Every mbarrier wait is bounded (status word + CTA-wide abort flag).
+// producer; warp 17: MMA issuer, a converged warp of which one lane issues (operands in uniform registers:
+// from inside an `if (lane == 0)` region the instruction stream, not the tensor pipe, set the rate).  The
+// tensor pipe works in order, so the completion of a product also tells which stage the accumulation before it
+// has finished with: in the dQ kernel row warp 0, which sees every completion of X and Y, passes that on to
+// the producer through one "empty" barrier per stage (except for the K stages, which the early products would
+// otherwise release too late); in the dK / dV kernel the issuer commits to the "empty" barriers right behind
+// each accumulation.  (The producer itself may fall several completions behind, which a parity wait on a
+// shared barrier cannot follow: hence one barrier per stage.)  Every mbarrier wait is bounded (status word +
+// CTA-wide abort flag).
+//
+// What bounds them: the row warps.  Two sequences of 32,768 tokens, 32/8 heads: a 128 x 128 tile takes 3,000 cycles
+// in the dK / dV kernel and 1,950 in the dQ kernel (2,600 before: issuing thread in a divergent region, releasing
+// arrivals, scalar fp32), 1,024 of them exponentials on the special-function unit; the issuer waits for the
+// row warps 1,400 / 670 of them.  Whole backward call 12.5 -> 11.4 ms.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -68,30 +73,6 @@ struct BtMap {
 };
 enum : int { BB_AFULL = 0, BB_B1FULL = 1, BB_B2FULL = 4, BB_XFULL = 6, BB_YFULL = 7, BB_PA = 8, BB_PB = 9, BB_OFULL = 10,
              BB_B1EMPTY = 11, BB_B2EMPTY = 14, BB_YFULL2 = 16, BB_PB2 = 17 };
-
-// Optional event trace (compile with -DKSA_BWD_TRACE=1 for the dQ kernel, =3 for the dK / dV kernel over summary
-// keys): one CTA records (event id, clock) pairs for lane 0 of every row warp; ksa_debug_read_bwd_trace() copies
-// them out.  =2 / =4: no stamps, only the MMA issuer's waiting times (below).
-#ifdef KSA_BWD_TRACE
-constexpr int kBtEvents = 4096;
-__device__ uint2 g_btrace[17][kBtEvents];         // role 0: MMA issuer (sums only); 1 + w: row warp w
-__device__ uint32_t g_btrace_cnt[17];
-#define KSA_BT(role, id)                                                                         \
-    do {                                                                                         \
-        if (bt_on && bt_n < (uint32_t)kBtEvents) g_btrace[role][bt_n++] = make_uint2((uint32_t)(id), (uint32_t)clock()); \
-    } while (0)
-#else
-#define KSA_BT(role, id) do { } while (0)
-#endif
-// KSA_BWD_TRACE == 2 / 4: the MMA issuer of one CTA of the dQ / the dK/dV (summary keys) kernel sums the cycles it
-// spends waiting for the row warps (registers only, written once at the end: stamps in memory disturb the waits).
-#if defined(KSA_BWD_TRACE) && (KSA_BWD_TRACE == 2 || KSA_BWD_TRACE == 4)
-#define KSA_BT_WAIT_BEGIN() const uint32_t bt_w0 = (uint32_t)clock()
-#define KSA_BT_WAIT_END(acc) acc += (uint32_t)clock() - bt_w0
-#else
-#define KSA_BT_WAIT_BEGIN() do { } while (0)
-#define KSA_BT_WAIT_END(acc) do { } while (0)
-#endif
 
 __device__ __forceinline__ uint32_t bt_ld_shared(uint32_t addr)
 {
@@ -179,43 +160,43 @@ __device__ __forceinline__ void bt_init(const BtSmem<D>& sm, int tid, int warp)
     tc_fence_after();
 }
 
-// ---- MMA issue helpers (one thread) ---------------------------------------------------------------
+// ---- MMA issue helpers (a converged warp; `leader` != 0 in the issuing lane) -------------------------
 // D[tmem_d] = A B^T, both 128 x D tiles K-major in shared memory ([64-element half of d][128 rows][128 B]).
 template <int D>
-__device__ __forceinline__ void bt_product(uint32_t tmem_d, uint32_t a_tile, uint32_t b_tile)
+__device__ __forceinline__ void bt_product(uint32_t leader, uint32_t tmem_d, uint32_t a_tile, uint32_t b_tile)
 {
-    constexpr uint32_t idesc = make_idesc_bf16(128, 128, false);
-    const uint64_t ad = make_smem_desc_sw128(a_tile, 16, 1024), bd = make_smem_desc_sw128(b_tile, 16, 1024);
+    constexpr uint32_t idesc = make_idesc_bf16(128, 128, false), hi = smem_desc_hi_sw128(1024);
+    const uint32_t ad = smem_desc_lo(a_tile, 16), bd = smem_desc_lo(b_tile, 16);
 #pragma unroll
     for (int kk = 0; kk < D / 16; ++kk) {
         const uint32_t off = (uint32_t)(((kk >> 2) * 16384 + (kk & 3) * 32) >> 4);
-        mma_ss(tmem_d, ad + off, bd + off, idesc, kk > 0 ? 1u : 0u);
+        mma_ss_warp(leader, tmem_d, ad + off, bd + off, hi, idesc, kk > 0 ? 1u : 0u);
     }
 }
 // D[tmem_d] (+)= A B: A = 128 x 128 bf16 in TMEM (16 packed columns at the start of every 32-column chunk of
 // tmem_a), B = a 128 x D tile in shared memory read MN-major (64-element atoms of d 16384 bytes apart,
 // 8-row groups 1024 bytes apart): D accumulator columns.
 template <int D>
-__device__ __forceinline__ void bt_accumulate(uint32_t tmem_d, uint32_t tmem_a, uint32_t b_tile, bool first)
+__device__ __forceinline__ void bt_accumulate(uint32_t leader, uint32_t tmem_d, uint32_t tmem_a, uint32_t b_tile, bool first)
 {
-    constexpr uint32_t idesc = make_idesc_bf16(128, D, true);
-    const uint64_t bd = make_smem_desc_sw128(b_tile, 16384, 1024);
+    constexpr uint32_t idesc = make_idesc_bf16(128, D, true), hi = smem_desc_hi_sw128(1024);
+    const uint32_t bd = smem_desc_lo(b_tile, 16384);
 #pragma unroll
     for (int kk = 0; kk < 8; ++kk)
-        mma_ts(tmem_d, tmem_a + (kk >> 1) * 32 + (kk & 1) * 8, bd + (uint32_t)((kk * 2048) >> 4), idesc, (!first || kk > 0) ? 1u : 0u);
+        mma_ts_warp(leader, tmem_d, tmem_a + (kk >> 1) * 32 + (kk & 1) * 8, bd + (uint32_t)((kk * 2048) >> 4), hi, idesc, (!first || kk > 0) ? 1u : 0u);
 }
 
 // Half of such an accumulation for the dK / dV kernel, whose row warps hand their 32-column blocks over in two
 // halves of 16 query columns: the four k-steps 2 c + odd, whose 16 x bf16 operand stands in the 8 columns at
 // tmem_a + 32 c + 16 odd (tmem_a already points at dS^T, or 8 columns further at P^T).
 template <int D>
-__device__ __forceinline__ void bt_accumulate_half(uint32_t tmem_d, uint32_t tmem_a, uint32_t b_tile, int odd, bool first)
+__device__ __forceinline__ void bt_accumulate_half(uint32_t leader, uint32_t tmem_d, uint32_t tmem_a, uint32_t b_tile, int odd, bool first)
 {
-    constexpr uint32_t idesc = make_idesc_bf16(128, D, true);
-    const uint64_t bd = make_smem_desc_sw128(b_tile, 16384, 1024);
+    constexpr uint32_t idesc = make_idesc_bf16(128, D, true), hi = smem_desc_hi_sw128(1024);
+    const uint32_t bd = smem_desc_lo(b_tile, 16384);
 #pragma unroll
     for (int c = 0; c < 4; ++c)
-        mma_ts(tmem_d, tmem_a + c * 32 + odd * 16, bd + (uint32_t)(((2 * c + odd) * 2048) >> 4), idesc, (!first || c > 0) ? 1u : 0u);
+        mma_ts_warp(leader, tmem_d, tmem_a + c * 32 + odd * 16, bd + (uint32_t)(((2 * c + odd) * 2048) >> 4), hi, idesc, (!first || c > 0) ? 1u : 0u);
 }
 
 // ---- producer helpers (one thread) ----------------------------------------------------------------
@@ -304,7 +285,7 @@ ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__
     BtSmem<D> sm;
     if (!bt_layout(sm, bsm_raw, a.status)) return;
     uint8_t* base_ptr = bsm_raw + (sm.base - smem_u32(bsm_raw));
-    // per-query scalars of the streamed tile, double-buffered by j: [j & 1][lse, delta][128 columns]; every row
+    // per-query scalars of the streamed tile, negated, double-buffered by j: [j & 1][lse, delta][128 columns]; every row
     // warp writes the 32 columns it reads itself, one tile ahead (the four warps of a column group write the same
     // values, and each relies on its own writes only), see below
     float* rows = reinterpret_cast<float*>(base_ptr + BtMap<D>::kOffRow);
@@ -314,8 +295,8 @@ ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__
     auto fetch = [&](int qt, int g) {                                     // pair (query tile qt, head g of the group)
         const int h = hk * G + g;
         const size_t r = (size_t)h * a.text_rows + sq.text_off + (size_t)qt * 128 + 32 * cg + lane;
-        n_lse = a.lse_t[r];                                               // +inf on padding rows: P = 0 there
-        n_dl = a.delta_t[r];
+        n_lse = -a.lse_t[r];                                              // -inf on padding rows: P = 0 there
+        n_dl = -a.delta_t[r];
     };
     if (scalar_writer) {                                                  // tile 0: visible to all after the first barrier
         fetch(seg0, 0);
@@ -355,61 +336,50 @@ ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__
         }
     } else if (warp == 17) {
         // =============================== MMA issuer =================================
-        if (lane == 0) {
-            const uint32_t abort_addr = sm.abort_addr();
-            bool alive = bt_wait(sm.bar(BB_AFULL), 0, abort_addr, a.status, kStatusWaitKvFull);
-            if (alive) alive = bt_wait(sm.bar(BB_B1FULL), 0, abort_addr, a.status, kStatusWaitQFull);
-            if (alive) { bt_product<D>(tX, sm.a1(), sm.b1(0)); tc_commit(sm.bar(BB_XFULL)); }
-            if (alive) alive = bt_wait(sm.bar(BB_B2FULL), 0, abort_addr, a.status, kStatusWaitQFull);
-            if (alive) { bt_product<D>(tY, sm.a2(), sm.b2(0)); tc_commit(sm.bar(BB_YFULL)); }
-            uint32_t bt_wait_a = 0, bt_wait_b = 0, bt_wait_c = 0, bt_iss_x = 0, bt_iss_acc = 0;
-            const uint32_t bt_loop0 = (uint32_t)clock();
-            (void)bt_wait_a; (void)bt_wait_b; (void)bt_loop0; (void)bt_wait_c; (void)bt_iss_x; (void)bt_iss_acc;
-            for (int j = 0; j < J && alive; ++j) {
-                // the warps hold X_j in registers: the next S^T product may overwrite it while they exponentiate
-                { KSA_BT_WAIT_BEGIN();
-                  if (!bt_wait(sm.bar(BB_PA), j & 1, abort_addr, a.status, kStatusWaitPFull)) break;
-                  KSA_BT_WAIT_END(bt_wait_a); }
-                tc_fence_after();
-                if (j + 1 < J) {
-                    const int s1 = (j + 1) % kB1Stages;
-                    { KSA_BT_WAIT_BEGIN();
-                    if (!bt_wait(sm.bar(BB_B1FULL + s1), ((j + 1) / kB1Stages) & 1, abort_addr, a.status, kStatusWaitQFull)) break;
-                    KSA_BT_WAIT_END(bt_wait_c); }
-                    { KSA_BT_WAIT_BEGIN();
-                    bt_product<D>(tX, sm.a1(), sm.b1(s1));
-                    tc_commit(sm.bar(BB_XFULL));
-                    KSA_BT_WAIT_END(bt_iss_x); }
-                }
-                // dS^T and P^T of the first 16 queries of every block stand in Y's columns: the even k-steps
-                { KSA_BT_WAIT_BEGIN();
-                  if (!bt_wait(sm.bar(BB_PB), j & 1, abort_addr, a.status, kStatusWaitPFull)) break;
-                  KSA_BT_WAIT_END(bt_wait_b); }
-                tc_fence_after();
-                KSA_BT_WAIT_BEGIN();
-                bt_accumulate_half<D>(tDV, tY + 8, sm.b2(j & 1), 0, j == 0);                   // dV += P^T dO_j
-                bt_accumulate_half<D>(tDK, tY, sm.b1(j % kB1Stages), 0, j == 0);               // dK += dS^T Q_j
-                // ... the other 16 (row warp 0 checked the stage of Y_{j+1} before it arrived): the odd k-steps
-                if (!bt_wait(sm.bar(BB_PB2), j & 1, abort_addr, a.status, kStatusWaitPFull)) break;
-                tc_fence_after();
-                bt_accumulate_half<D>(tDV, tY + 8, sm.b2(j & 1), 1, false);
-                tc_commit(sm.bar(BB_B2EMPTY + (j & 1)));                                    // ... then its dO stage is free
-                bt_accumulate_half<D>(tDK, tY, sm.b1(j % kB1Stages), 1, false);
-                tc_commit(sm.bar(BB_B1EMPTY + j % kB1Stages));                              // ... then its Q stage is free
-                if (j + 1 < J) { bt_product<D>(tY, sm.a2(), sm.b2((j + 1) & 1)); tc_commit(sm.bar(BB_YFULL)); }
-                KSA_BT_WAIT_END(bt_iss_acc);
+        // the whole warp walks the loop on warp-uniform values, one lane issues
+        const uint32_t leader = elect_one();
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0), base = __shfl_sync(0xffffffffu, sm.base, 0);
+        const int Ju = __shfl_sync(0xffffffffu, J, 0);
+        const BtSmem<D> su{base};
+        const uint32_t uX = tm, uY = tm + 128u, uDV = tm + 256u, uDK = tm + 384u;
+        auto wait = [&](uint32_t bar, uint32_t parity, int code) -> bool {
+            return __all_sync(0xffffffffu, bt_wait(bar, parity, su.abort_addr(), a.status, code));
+        };
+        bool alive = wait(su.bar(BB_AFULL), 0, kStatusWaitKvFull);
+        if (alive) alive = wait(su.bar(BB_B1FULL), 0, kStatusWaitQFull);
+        if (alive) { bt_product<D>(leader, uX, su.a1(), su.b1(0)); tc_commit_warp(leader, su.bar(BB_XFULL)); }
+        if (alive) alive = wait(su.bar(BB_B2FULL), 0, kStatusWaitQFull);
+        if (alive) { bt_product<D>(leader, uY, su.a2(), su.b2(0)); tc_commit_warp(leader, su.bar(BB_YFULL)); }
+        int s1 = 0;                                            // j % kB1Stages
+        uint32_t b1_phase = 0;                                 // parity of tile j + 1's fill of its stage
+        for (int j = 0; j < Ju && alive; ++j) {
+            const int s1n = s1 + 1 == kB1Stages ? 0 : s1 + 1;
+            if (s1n == 0) b1_phase ^= 1u;
+            if (j + 1 < Ju && !wait(su.bar(BB_B1FULL + s1n), b1_phase, kStatusWaitQFull)) break;
+            // the warps hold X_j in registers: the next S^T product may overwrite it while they exponentiate
+            if (!wait(su.bar(BB_PA), j & 1, kStatusWaitPFull)) break;
+            tc_fence_after();
+            if (j + 1 < Ju) {
+                bt_product<D>(leader, uX, su.a1(), su.b1(s1n));
+                tc_commit_warp(leader, su.bar(BB_XFULL));
             }
-            tc_commit(sm.bar(BB_OFULL));
-#if defined(KSA_BWD_TRACE) && KSA_BWD_TRACE == 4
-            if (summ && blockIdx.x == 1 && blockIdx.y == 4 && blockIdx.z == 0) {
-                g_btrace[0][0] = make_uint2(bt_wait_a, bt_wait_b);
-                g_btrace[0][1] = make_uint2((uint32_t)clock() - bt_loop0, (uint32_t)J);
-                g_btrace[0][2] = make_uint2(bt_wait_c, bt_iss_x);
-                g_btrace[0][3] = make_uint2(bt_iss_acc, 0u);
-                g_btrace_cnt[0] = 4;
-            }
-#endif
+            // dS^T and P^T of the first 16 queries of every block stand in Y's columns: the even k-steps
+            if (!wait(su.bar(BB_PB), j & 1, kStatusWaitPFull)) break;
+            tc_fence_after();
+            bt_accumulate_half<D>(leader, uDV, uY + 8, su.b2(j & 1), 0, j == 0);            // dV += P^T dO_j
+            bt_accumulate_half<D>(leader, uDK, uY, su.b1(s1), 0, j == 0);                   // dK += dS^T Q_j
+            // ... the other 16: the odd k-steps
+            if (j + 1 < Ju && !wait(su.bar(BB_B2FULL + ((j + 1) & 1)), ((j + 1) >> 1) & 1, kStatusWaitQFull)) break;
+            if (!wait(su.bar(BB_PB2), j & 1, kStatusWaitPFull)) break;
+            tc_fence_after();
+            bt_accumulate_half<D>(leader, uDV, uY + 8, su.b2(j & 1), 1, false);
+            tc_commit_warp(leader, su.bar(BB_B2EMPTY + (j & 1)));                           // ... then its dO stage is free
+            bt_accumulate_half<D>(leader, uDK, uY, su.b1(s1), 1, false);
+            tc_commit_warp(leader, su.bar(BB_B1EMPTY + s1));                                // ... then its Q stage is free
+            if (j + 1 < Ju) { bt_product<D>(leader, uY, su.a2(), su.b2((j + 1) & 1)); tc_commit_warp(leader, su.bar(BB_YFULL)); }
+            s1 = s1n;
         }
+        tc_commit_warp(leader, su.bar(BB_OFULL));
     } else {
         // =============================== key rows ===================================
         const uint32_t lane_sel = (uint32_t)(quarter * 32) << 16;
@@ -423,22 +393,16 @@ ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__
         // query, i0 = 128 qt + 32 cg, is kept as quotient and remainder by k and advanced by 128 per query tile
         // (integer divisions are slow, and this loop is the warps' critical path).
         const int step_q = 128 / a.k, step_r = 128 - step_q * a.k, q31 = 31 / a.k, r31 = 31 - q31 * a.k;
-#ifdef KSA_BWD_TRACE
-        const bool bt_on = KSA_BWD_TRACE == 3 && summ && blockIdx.x == 1 && blockIdx.y == 4 && blockIdx.z == 0 && lane == 0;
-        const int bt_role = 1 + warp;
-        uint32_t bt_n = 0;
-#endif
         int qt = seg0, g = 0;
         int iq0 = (seg0 * 128 + 32 * cg) / a.k, ir0 = (seg0 * 128 + 32 * cg) - iq0 * a.k;
         for (int j = 0; j < J && alive; ++j) {
             if (j + 1 < J) fetch(g + 1 == G ? qt + 1 : qt, g + 1 == G ? 0 : g + 1);   // lands while this tile is worked on
-            const float* lse_c = rows + (j & 1) * 256 + 32 * cg;          // this warp's 32 columns
-            const float* dl_c = lse_c + 128;
+            const float4* lse_c = reinterpret_cast<const float4*>(rows + (j & 1) * 256 + 32 * cg);     // this warp's 32 columns
+            const float4* dl_c = lse_c + 32;
             const int i0 = qt * 128 + 32 * cg;                            // first query of the block
             const int iq1 = iq0 + q31 + (ir0 + r31 >= a.k ? 1 : 0);       // chunk of the block's last query
             // ---------------- phase A: P^T = exp2(S^T scale - lse), kept in registers ----------------
             if (!bt_wait_warp(sm.bar(BB_XFULL), j & 1, sm.abort_addr(), a.status, kStatusWaitSFull, lane)) { alive = false; break; }
-            KSA_BT(bt_role, 10);
             tc_fence_after();
             // all pairs of the block visible / none (rows past the streams drop out by themselves: zero K / V
             // rows are discarded at the end, padding queries have lse = +inf)
@@ -450,43 +414,45 @@ ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__
                 full = iq0 - kq_last > a.C;
                 none = iq1 - kq_first <= a.C;
             }
-            uint32_t x0[16], x1[16];                                      // S^T, then P^T in place (fp32 bits), kept for phase B
+            uint32_t x[32];                                               // S^T, then P^T in place (fp32 bits), kept for phase B
             if (none) {
 #pragma unroll
-                for (int c = 0; c < 16; ++c) x0[c] = x1[c] = 0u;
+                for (int c = 0; c < 32; ++c) x[c] = 0u;
             } else {
-                tmem_ld16(tXc, x0);
-                tmem_ld16(tXc + 16, x1);
+                tmem_ld32(tXc, x);
                 tc_wait_ld();
             }
-            // X_j is in registers: the issuer may start X_{j+1} while the exponentials run
+            // X_j is in registers: the issuer may start X_{j+1} while the exponentials run.  (This hand-over and those
+            // below order TMEM accesses only, which the fences and waits around them cover: relaxed arrivals.)
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(sm.bar(BB_PA));
-            KSA_BT(bt_role, 11);
+            if (lane == 0) mbar_arrive_relaxed(sm.bar(BB_PA));
             if (!none) {
                 if (full) {
+                    const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) {
-                        x0[c] = __float_as_uint(ex2_approx(fmaf(__uint_as_float(x0[c]), a.scale_log2, -lse_c[c])));
-                        x1[c] = __float_as_uint(ex2_approx(fmaf(__uint_as_float(x1[c]), a.scale_log2, -lse_c[16 + c])));
+                    for (int c = 0; c < 32; c += 4) {
+                        const float4 l4 = lse_c[c >> 2];
+                        const float2 t = ffma2(make_float2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])), sc2, make_float2(l4.x, l4.y));
+                        const float2 u = ffma2(make_float2(__uint_as_float(x[c + 2]), __uint_as_float(x[c + 3])), sc2, make_float2(l4.z, l4.w));
+                        x[c] = __float_as_uint(ex2_approx(t.x));
+                        x[c + 1] = __float_as_uint(ex2_approx(t.y));
+                        x[c + 2] = __float_as_uint(ex2_approx(u.x));
+                        x[c + 3] = __float_as_uint(ex2_approx(u.y));
                     }
                 } else {
                     int iq = iq0, ir = ir0;                               // chunk of query i0 + c, counted up from i0's
 #pragma unroll
                     for (int c = 0; c < 32; ++c) {
-                        uint32_t& xc = c < 16 ? x0[c & 15] : x1[c & 15];
                         const bool vis = summ ? (iq - kq > a.C) : (key <= i0 + c && iq - kq <= a.C);
-                        const float t = fmaf(__uint_as_float(xc), a.scale_log2, -lse_c[c]);
-                        xc = __float_as_uint(ex2_approx(vis ? t : -INFINITY));
+                        const float t = fmaf(__uint_as_float(x[c]), a.scale_log2, reinterpret_cast<const float*>(lse_c)[c]);
+                        x[c] = __float_as_uint(ex2_approx(vis ? t : -INFINITY));
                         if (++ir == a.k) { ir = 0; ++iq; }
                     }
                 }
             }
-            KSA_BT(bt_role, 12);
             // ---------------- phase B: dS^T = P^T (dP^T - delta); both as bf16 over Y's own columns ----------------
             if (!bt_wait_warp(sm.bar(BB_YFULL), j & 1, sm.abort_addr(), a.status, kStatusWaitSFull, lane)) { alive = false; break; }
-            KSA_BT(bt_role, 13);
             tc_fence_after();
             // Y_j was issued after every warp's arrival for tile j - 1: that tile's scalars may be overwritten
             if (j + 1 < J) {
@@ -506,33 +472,31 @@ ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__
                     tmem_ld16(tYc + half * 16, ys);
                     tc_wait_ld();
 #pragma unroll
-                    for (int c = 0; c < 16; c += 2) {
-                        const float p0 = __uint_as_float(half ? x1[c] : x0[c]), p1 = __uint_as_float(half ? x1[c + 1] : x0[c + 1]);
-                        o[c >> 1] = pack_bf16x2(p0 * (__uint_as_float(ys[c]) - dl_c[half * 16 + c]),
-                                                p1 * (__uint_as_float(ys[c + 1]) - dl_c[half * 16 + c + 1]));
-                        o[8 + (c >> 1)] = pack_bf16x2(p0, p1);
+                    for (int c = 0; c < 16; c += 4) {
+                        const int e = half * 16 + c;
+                        const float4 d4 = dl_c[e >> 2];
+                        const float2 p2 = make_float2(__uint_as_float(x[e]), __uint_as_float(x[e + 1]));
+                        const float2 q2 = make_float2(__uint_as_float(x[e + 2]), __uint_as_float(x[e + 3]));
+                        const float2 s2 = fmul2(p2, fadd2(make_float2(__uint_as_float(ys[c]), __uint_as_float(ys[c + 1])), make_float2(d4.x, d4.y)));
+                        const float2 r2 = fmul2(q2, fadd2(make_float2(__uint_as_float(ys[c + 2]), __uint_as_float(ys[c + 3])), make_float2(d4.z, d4.w)));
+                        o[c >> 1] = pack_bf16x2(s2.x, s2.y);
+                        o[(c >> 1) + 1] = pack_bf16x2(r2.x, r2.y);
+                        o[8 + (c >> 1)] = pack_bf16x2(p2.x, p2.y);
+                        o[9 + (c >> 1)] = pack_bf16x2(q2.x, q2.y);
                     }
                 }
-                tmem_st16(tYc + half * 16, o);                            // over the 16 columns of dP^T just read
+                tmem_st16(tYc + half * 16, o);                            // over the block's own columns of dP^T
                 tc_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) {
-                    if (half == 1 && warp == 0 && j + 1 < J)               // warp 0 vouches for the stage of Y_{j+1}
-                        bt_wait(sm.bar(BB_B2FULL + ((j + 1) & 1)), ((j + 1) >> 1) & 1, sm.abort_addr(), a.status, kStatusWaitQFull);
-                    mbar_arrive(sm.bar(half ? BB_PB2 : BB_PB));
-                }
+                if (lane == 0) mbar_arrive_relaxed(sm.bar(half ? BB_PB2 : BB_PB));
             }
-            KSA_BT(bt_role, 14);
             if (++g == G) {                                               // next query tile
                 g = 0; ++qt;
                 iq0 += step_q; ir0 += step_r;
                 if (ir0 >= a.k) { ir0 -= a.k; ++iq0; }
             }
         }
-#ifdef KSA_BWD_TRACE
-        if (bt_on) g_btrace_cnt[bt_role] = bt_n;
-#endif
         if (alive && bt_wait_warp(sm.bar(BB_OFULL), 0, sm.abort_addr(), a.status, kStatusWaitOFull, lane)) {
             tc_fence_after();
             // odd cg: scale * dK, even cg: dV; cg / 2 picks the half of the row (D / 2 elements)
@@ -634,45 +598,45 @@ ksa_bwd_dq_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ 
         }
     } else if (warp == 17) {
         // =============================== MMA issuer =================================
-        if (lane == 0) {
-            const uint32_t abort_addr = sm.abort_addr();
-            bool alive = bt_wait(sm.bar(BB_AFULL), 0, abort_addr, a.status, kStatusWaitKvFull);
-            if (alive) alive = bt_wait(sm.bar(BB_B1FULL), 0, abort_addr, a.status, kStatusWaitQFull);
-            if (alive) { bt_product<D>(tX, sm.a1(), sm.b1(0)); tc_commit(sm.bar(BB_XFULL)); }
-            if (alive) alive = bt_wait(sm.bar(BB_B2FULL), 0, abort_addr, a.status, kStatusWaitQFull);
-            if (alive) { bt_product<D>(tY(0), sm.a2(), sm.b2(0)); tc_commit(y_full(0)); }
-            uint32_t bt_wait_a = 0, bt_wait_b = 0;
-            const uint32_t bt_loop0 = (uint32_t)clock();
-            (void)bt_wait_a; (void)bt_wait_b; (void)bt_loop0;
-            for (int j = 0; j < J && alive; ++j) {
-                // later stages were checked by row warp 0 before its arrival
-                if (j + 1 < J) {
-                    // phase A of tile j has read X into registers; the other Y buffer was read by dQ += dS K_{j-1}
-                    KSA_BT_WAIT_BEGIN();
-                    if (!bt_wait(sm.bar(BB_PA), j & 1, abort_addr, a.status, kStatusWaitPFull)) break;
-                    KSA_BT_WAIT_END(bt_wait_a);
-                    tc_fence_after();
-                    bt_product<D>(tX, sm.a1(), sm.b1((j + 1) % kB1Stages));
-                    tc_commit(sm.bar(BB_XFULL));
-                    bt_product<D>(tY(j + 1), sm.a2(), sm.b2((j + 1) & 1));
-                    tc_commit(y_full(j + 1));
-                }
-                { KSA_BT_WAIT_BEGIN();
-                  if (!bt_wait(p_b(j), (j >> 1) & 1, abort_addr, a.status, kStatusWaitPFull)) break;
-                  KSA_BT_WAIT_END(bt_wait_b); }
+        // the whole warp walks the loop on warp-uniform values, one lane issues
+        const uint32_t leader = elect_one();
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0), base = __shfl_sync(0xffffffffu, sm.base, 0);
+        const int Ju = __shfl_sync(0xffffffffu, J, 0);
+        const BtSmem<D> su{base};
+        const uint32_t uX = tm, uDQ = tm + 256u;
+        auto uY = [&](int j) -> uint32_t { return tm + ((j & 1) ? 384u : 128u); };
+        auto u_full = [&](int j) -> uint32_t { return su.bar((j & 1) ? BB_YFULL2 : BB_YFULL); };
+        auto wait = [&](uint32_t bar, uint32_t parity, int code) -> bool {
+            return __all_sync(0xffffffffu, bt_wait(bar, parity, su.abort_addr(), a.status, code));
+        };
+        bool alive = wait(su.bar(BB_AFULL), 0, kStatusWaitKvFull);
+        if (alive) alive = wait(su.bar(BB_B1FULL), 0, kStatusWaitQFull);
+        if (alive) { bt_product<D>(leader, uX, su.a1(), su.b1(0)); tc_commit_warp(leader, su.bar(BB_XFULL)); }
+        if (alive) alive = wait(su.bar(BB_B2FULL), 0, kStatusWaitQFull);
+        if (alive) { bt_product<D>(leader, uY(0), su.a2(), su.b2(0)); tc_commit_warp(leader, u_full(0)); }
+        int s1 = 0;                                            // j % kB1Stages
+        uint32_t b1_phase = 0;                                 // parity of tile j + 1's fill of its stage
+        for (int j = 0; j < Ju && alive; ++j) {
+            const int s1n = s1 + 1 == kB1Stages ? 0 : s1 + 1;
+            if (j + 1 < Ju) {
+                if (s1n == 0) b1_phase ^= 1u;
+                if (!wait(su.bar(BB_B1FULL + s1n), b1_phase, kStatusWaitQFull)) break;
+                if (!wait(su.bar(BB_B2FULL + ((j + 1) & 1)), ((j + 1) >> 1) & 1, kStatusWaitQFull)) break;
+                // phase A of tile j has read X into registers; the other Y buffer was read by dQ += dS K_{j-1}
+                if (!wait(su.bar(BB_PA), j & 1, kStatusWaitPFull)) break;
                 tc_fence_after();
-                bt_accumulate<D>(tDQ, tY(j), sm.b1(j % kB1Stages), j == 0);                    // dQ += dS K_j
-                tc_commit(sm.bar(BB_B1EMPTY + j % kB1Stages));                              // K_j is free after that
+                bt_product<D>(leader, uX, su.a1(), su.b1(s1n));
+                tc_commit_warp(leader, su.bar(BB_XFULL));
+                bt_product<D>(leader, uY(j + 1), su.a2(), su.b2((j + 1) & 1));
+                tc_commit_warp(leader, u_full(j + 1));
             }
-            tc_commit(sm.bar(BB_OFULL));
-#if defined(KSA_BWD_TRACE) && KSA_BWD_TRACE == 2
-            if (blockIdx.x == 8 && blockIdx.y == 0 && blockIdx.z == 0) {
-                g_btrace[0][0] = make_uint2(bt_wait_a, bt_wait_b);
-                g_btrace[0][1] = make_uint2((uint32_t)clock() - bt_loop0, (uint32_t)J);
-                g_btrace_cnt[0] = 2;
-            }
-#endif
+            if (!wait(su.bar((j & 1) ? BB_PB2 : BB_PB), (j >> 1) & 1, kStatusWaitPFull)) break;
+            tc_fence_after();
+            bt_accumulate<D>(leader, uDQ, uY(j), su.b1(s1), j == 0);                       // dQ += dS K_j
+            tc_commit_warp(leader, su.bar(BB_B1EMPTY + s1));                               // K_j is free after that
+            s1 = s1n;
         }
+        tc_commit_warp(leader, su.bar(BB_OFULL));
     } else {
         // =============================== query rows =================================
         const int quarter = warp & 3, cg = warp >> 2;                    // lanes 32 quarter ..; columns 32 cg ..
@@ -682,11 +646,6 @@ ksa_bwd_dq_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ 
         const size_t r = (size_t)h * a.text_rows + sq.text_off + i;
         const float lse2 = a.lse_t[r], dl = a.delta_t[r];                 // +inf / 0 on padding rows: P = 0 there
         const int iq = i / a.k, iq_w0 = i_w0 / a.k, iq_w1 = (i_w0 + 31) / a.k;
-#ifdef KSA_BWD_TRACE
-        const bool bt_on = KSA_BWD_TRACE == 1 && blockIdx.x == 8 && blockIdx.y == 0 && blockIdx.z == 0 && lane == 0;
-        const int bt_role = 1 + warp;
-        uint32_t bt_n = 0;
-#endif
         bool alive = true;
         // The chunk of the block's first key, kc0 = key0 + 32 cg, is kept as quotient and remainder by the keys per
         // chunk of its stream and advanced by 128 per tile; divisions only where the stream starts (integer
@@ -719,78 +678,63 @@ ksa_bwd_dq_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ 
             }
             // ---------------- phase A: P = exp2(S scale - lse) ----------------
             if (!bt_wait_warp(sm.bar(BB_XFULL), j & 1, sm.abort_addr(), a.status, kStatusWaitSFull, lane)) { alive = false; break; }
-            KSA_BT(bt_role, 10);
             tc_fence_after();
-            uint32_t x0[16], x1[16];                                      // S, then P in place (fp32 bits)
+            uint32_t x[32];                                               // S, then P in place (fp32 bits)
             if (!none) {
-                tmem_ld16(tXc, x0);
-                tmem_ld16(tXc + 16, x1);
+                tmem_ld32(tXc, x);
                 tc_wait_ld();
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) {                                              // X may be overwritten from here on
-                if (warp == 0 && j + 1 < J) {                              // warp 0 vouches for the stages of X_{j+1} and Y_{j+1}
-                    bt_wait(sm.bar(BB_B1FULL + (j + 1) % kB1Stages), ((j + 1) / kB1Stages) & 1, sm.abort_addr(), a.status, kStatusWaitQFull);
-                    bt_wait(sm.bar(BB_B2FULL + ((j + 1) & 1)), ((j + 1) >> 1) & 1, sm.abort_addr(), a.status, kStatusWaitQFull);
-                }
-                mbar_arrive(sm.bar(BB_PA));
-            }
-            KSA_BT(bt_role, 11);
+            if (lane == 0) mbar_arrive_relaxed(sm.bar(BB_PA));            // X may be overwritten from here on
             if (!none) {
                 if (full) {
+                    const float2 sc2 = make_float2(a.scale_log2, a.scale_log2), nl2 = make_float2(-lse2, -lse2);
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) {
-                        x0[c] = __float_as_uint(ex2_approx(fmaf(__uint_as_float(x0[c]), a.scale_log2, -lse2)));
-                        x1[c] = __float_as_uint(ex2_approx(fmaf(__uint_as_float(x1[c]), a.scale_log2, -lse2)));
+                    for (int c = 0; c < 32; c += 2) {
+                        const float2 t = ffma2(make_float2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])), sc2, nl2);
+                        x[c] = __float_as_uint(ex2_approx(t.x));
+                        x[c + 1] = __float_as_uint(ex2_approx(t.y));
                     }
                 } else {
                     int kq = kq0, kr = kr0;                               // chunk of key kc0 + c, counted up from kc0's
 #pragma unroll
                     for (int c = 0; c < 32; ++c) {
-                        uint32_t& xc = c < 16 ? x0[c & 15] : x1[c & 15];
                         const bool vis = is_summ ? (iq - kq > a.C) : (kc0 + c <= i && iq - kq <= a.C);
-                        const float t = fmaf(__uint_as_float(xc), a.scale_log2, -lse2);
-                        xc = __float_as_uint(ex2_approx(vis ? t : -INFINITY));
+                        const float t = fmaf(__uint_as_float(x[c]), a.scale_log2, -lse2);
+                        x[c] = __float_as_uint(ex2_approx(vis ? t : -INFINITY));
                         if (++kr == cdiv) { kr = 0; ++kq; }
                     }
                 }
             }
-            KSA_BT(bt_role, 12);
             // ---------------- phase B: dS = P (dP - delta) ----------------
             // one barrier per Y buffer: Y_{j+1} may be complete before a warp gets here for Y_j
             if (!bt_wait_warp(y_full(j), (j >> 1) & 1, sm.abort_addr(), a.status, kStatusWaitSFull, lane)) { alive = false; break; }
-            KSA_BT(bt_role, 13);
             tc_fence_after();
-            if (warp == 0 && lane == 0) mbar_arrive(sm.bar(BB_B2EMPTY + (j & 1)));          // Y_j is complete: its V stage is free
+            if (warp == 0 && lane == 0) mbar_arrive_relaxed(sm.bar(BB_B2EMPTY + (j & 1)));          // Y_j is complete: its V stage is free
             const uint32_t tYc = tY(j) + lane_sel + cg * 32;
             uint32_t dd[16];
             if (none) {
 #pragma unroll
                 for (int c = 0; c < 16; ++c) dd[c] = 0u;
             } else {
+                uint32_t ys[32];
+                tmem_ld32(tYc, ys);
+                tc_wait_ld();
+                const float2 nd2 = make_float2(-dl, -dl);
 #pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    uint32_t ys[16];
-                    tmem_ld16(tYc + half * 16, ys);
-                    tc_wait_ld();
-#pragma unroll
-                    for (int c = 0; c < 16; c += 2) {
-                        const float p0 = __uint_as_float(half ? x1[c] : x0[c]), p1 = __uint_as_float(half ? x1[c + 1] : x0[c + 1]);
-                        dd[half * 8 + (c >> 1)] = pack_bf16x2(p0 * (__uint_as_float(ys[c]) - dl), p1 * (__uint_as_float(ys[c + 1]) - dl));
-                    }
+                for (int c = 0; c < 32; c += 2) {
+                    const float2 d2 = fmul2(make_float2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])),
+                                            fadd2(make_float2(__uint_as_float(ys[c]), __uint_as_float(ys[c + 1])), nd2));
+                    dd[c >> 1] = pack_bf16x2(d2.x, d2.y);
                 }
             }
             tmem_st16(tYc, dd);                                           // over the block's own first 16 columns
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(p_b(j));
-            KSA_BT(bt_role, 14);
+            if (lane == 0) mbar_arrive_relaxed(p_b(j));
         }
-#ifdef KSA_BWD_TRACE
-        if (bt_on) g_btrace_cnt[bt_role] = bt_n;
-#endif
         if (alive && bt_wait_warp(sm.bar(BB_OFULL), 0, sm.abort_addr(), a.status, kStatusWaitOFull, lane)) {
             tc_fence_after();
             // scale * dQ as bf16 to the row's augmented position (Eq. 1); warp group cg writes elements 32 cg ..
@@ -818,16 +762,6 @@ ksa_bwd_dq_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ 
     __syncthreads();
     if (warp == 16) tmem_dealloc(tmem, 512);
 }
-
-#ifdef KSA_BWD_TRACE
-extern "C" __attribute__((visibility("default"))) int ksa_debug_read_bwd_trace(void* events, void* counts)
-{
-    cudaDeviceSynchronize();
-    cudaError_t e = cudaMemcpyFromSymbol(events, g_btrace, sizeof(g_btrace));
-    if (e == cudaSuccess) e = cudaMemcpyFromSymbol(counts, g_btrace_cnt, sizeof(g_btrace_cnt));
-    return (int)e;
-}
-#endif
 
 cudaError_t setup_bwd_tc()
 {

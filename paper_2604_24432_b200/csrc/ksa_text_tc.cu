@@ -56,7 +56,7 @@ constexpr int kRegsOther = 72;            // ... of the TMA / MMA warpgroup
 // The CTA's register allocation is fixed at launch (65,536 / 384 threads = 170 -> 168 per thread): the softmax warps
 // can only gain what the third warpgroup gives up; a larger setmaxnreg.inc would wait forever.
 static_assert(8 * kRegsSoftmax + 4 * kRegsOther <= 12 * ((65536 / 384) / 8 * 8), "register hand-over exceeds the CTA's allocation");
-constexpr int kLoadQkWarp = 8, kQkWarp = 9, kPvWarp = 10, kLoadVWarp = 11;
+constexpr int kLoadQkWarp = 8, kQkWarp = 9, kLoadVWarp = 11;         // (10: the PV products)
 // log2 units: P stays below 2^12.  A small threshold costs rescales of O: with 1 % of the keys four times larger (the 128k
 // workload) some row of nearly every warp outgrew 2^8 once or twice per work item.  Measured at 128k: 8 -> 1,032,
 // 12 -> 1,047, 20 -> 1,058 TFLOP/s, but the error against the fp64 oracle grows with it (mean |err| 5.6e-4, 5.9e-4,
