@@ -511,7 +511,7 @@ def run_decode(args):
                      # for the default batch of 32 sequences at a 128K context
                      "traffic": 1.137e9 if (B, ctx_len) == (32, 131072) else None,
                      "peak_source": f"of {peaks['source']} (copy bandwidth)",
-                     "kernel": "ksa_decode_attn_kernel (+ append, merge, commit)",
+                     "kernel": "ksa_decode_attn_kernel (+ merge)",
                      "bytes_per_step": bytes_read / steps},
         "e2e": None, "cpu_baseline": None,
     }

@@ -143,3 +143,40 @@ def test_decode_text_step_refuses_a_pending_summary(ctx):
     cache.decode_text(q, kv, kv, out, lse)
     torch.cuda.synchronize()
     assert ctx.device_status() == 0 and cache.state.cpu().numpy().tolist() == [[5, 1]]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("D,Hq,Hkv,C", [(128, 4, 2, 3), (64, 3, 3, 0)])
+def test_decode_step_of_a_batch_in_mixed_states(ctx, D, Hq, Hkv, C):
+    """Sequence 0 takes the step, sequence 1 does not (text step: its chunk waits for the summary; summary step: nothing is
+    due): its rows of out / lse, its cache and its state stay as they are, and sequence 0's step equals a step on its own."""
+    k, n = 4, 24
+    dev = torch.device("cuda", 0)
+    g = torch.Generator("cpu").manual_seed(3)
+    draw = lambda *shape: torch.randn(shape, generator=g).to(torch.bfloat16).to(dev)
+    both = ksa.DecodeCache(ctx, ksa.CacheSpec(2, k, C, n, Hq, Hkv, D, 0.1))
+    alone = ksa.DecodeCache(ctx, ksa.CacheSpec(1, k, C, n, Hq, Hkv, D, 0.1))
+    both.kcache.copy_(draw(*both.kcache.shape)); both.vcache.copy_(draw(*both.vcache.shape))
+    alone.kcache.copy_(both.kcache[:1]); alone.vcache.copy_(both.vcache[:1])
+    for summary, state in ((False, [[22, 5], [20, 4]]), (True, [[24, 5], [23, 5]])):
+        both.state.copy_(torch.tensor(state, dtype=torch.int32)); alone.state.copy_(both.state[:1])
+        before = [t.clone() for t in (both.kcache, both.vcache, both.state)]
+        q, kn, vn = draw(2, Hq, D), draw(2, Hkv, D), draw(2, Hkv, D)
+        out = torch.full((2, Hq, D), 7.0, dtype=torch.bfloat16, device=dev); lse = torch.full((2, Hq), -3.0, device=dev)
+        out1 = torch.empty((1, Hq, D), dtype=torch.bfloat16, device=dev); lse1 = torch.empty((1, Hq), device=dev)
+        ctx.clear_device_status()
+        (both.decode_summary if summary else both.decode_text)(q, kn, vn, out, lse)
+        torch.cuda.synchronize()
+        assert ctx.device_status() == (0 if summary else 101)
+        ctx.clear_device_status()
+        (alone.decode_summary if summary else alone.decode_text)(q[:1].contiguous(), kn[:1].contiguous(), vn[:1].contiguous(), out1, lse1)
+        torch.cuda.synchronize()
+        assert ctx.device_status() == 0
+        assert (out[1] == 7.0).all() and (lse[1] == -3.0).all()
+        for t, b in zip((both.kcache, both.vcache, both.state), before):
+            assert torch.equal(t[1], b[1])
+        assert torch.equal(both.kcache[0], alone.kcache[0]) and torch.equal(both.vcache[0], alone.vcache[0])
+        assert torch.equal(both.state[0], alone.state[0]) and not torch.equal(both.state[0], before[2][0])
+        # the batch of two has its slices split differently: the same sums in another order
+        assert (out[0].float() - out1[0].float()).abs().max().item() <= 2e-2
+        assert (lse[0] - lse1[0]).abs().max().item() <= 1e-5 * 10
