@@ -936,12 +936,16 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_bwd(ksa_ctx* ctx,
     a.direct = direct ? 1 : 0;
     // The four accumulators are contiguous in the workspace: one clear.  Where one CTA of the tensor-core dK / dV kernel
     // covers every query tile that sees a text key tile, that launch stores the text keys' rows instead of adding to them:
-    // then only the summary keys' accumulators are cleared and the summary rows' kernel, which adds to both, runs after it.
+    // then only the summary keys' accumulators are cleared.
+    // The summary rows' gradients come last where their kernel also finishes the chunks' rows (it reads the accumulators
+    // and writes dk, dv), or where the text rows' kernel stores; the CUDA-core kernel otherwise adds before or after.
     const bool text_stored = !(p->flags & KSA_FLAG_BWD_MMA_SYNC_KERNELS) && bwd_text_keys_stored(a);
+    const bool summ_rows = a.m > 0 && a.max_n_summ > 0;
+    const bool summ_finishes = summ_rows && bwd_summary_mma_applies(a);
     const size_t clear0 = text_stored ? bl.dks : bl.dkt;
     if (bl.total > clear0 && (e = cudaMemsetAsync(ws + clear0, 0, bl.total - clear0, stream)) != cudaSuccess) return cuda_fail(ctx, e);
     if ((e = launch_bwd_prep(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);
-    if (!text_stored && (e = launch_bwd_summary(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);
+    if (!text_stored && !summ_finishes && (e = launch_bwd_summary(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);
     if (!(p->flags & KSA_FLAG_BWD_MMA_SYNC_KERNELS)) {
         // text rows on the tcgen05 tensor cores, fed by TMA from the packed streams or the caller's tensors
         if (!ctx->bwd_tc_ready) {
@@ -977,9 +981,13 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_bwd(ksa_ctx* ctx,
         if ((e = launch_bwd_dq(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);
         if ((e = launch_bwd_dkv(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);
     }
-    if (text_stored && (e = launch_bwd_summary(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);
-    if ((e = launch_bwd_finish(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);
-    ctx->launches += (direct ? 4 : 5) + ((a.m > 0 && a.max_n_summ > 0) ? 2 : 0);
+    if (text_stored && !summ_finishes && (e = launch_bwd_summary(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);
+    if (summ_finishes && (e = launch_bwd_summary_mma(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);
+    bool tails = false;                                                  // text rows behind a last whole chunk
+    for (const SeqInfo& sq : hs.seqs) tails = tails || sq.n_text != sq.n_chunks * a.k;
+    if ((!summ_finishes || tails) && (e = launch_bwd_finish(a, summ_finishes, stream)) != cudaSuccess) return cuda_fail(ctx, e);
+    // prep, dQ, dK / dV of the text keys; pack; dK / dV of the summary keys and the summary rows; finish
+    ctx->launches += 3 + (direct ? 0 : 1) + (summ_rows ? 2 : 0) + ((!summ_finishes || tails) ? 1 : 0);
     return KSA_OK;
 }
 

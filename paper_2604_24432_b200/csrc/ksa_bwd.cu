@@ -472,20 +472,22 @@ __global__ void __launch_bounds__(256) ksa_bwd_summary_kernel(BwdArgs a)
 }
 
 // =================================================================================================
-// finish: fp32 accumulators of the streams -> bf16 dk, dv at the augmented positions (Eq. 1)
+// finish: fp32 accumulators of the streams -> bf16 dk, dv at the augmented positions (Eq. 1).  With tails != 0 only
+// the text rows behind each sequence's last whole chunk (the summary rows' kernel has finished the chunks).
 // =================================================================================================
-__global__ void __launch_bounds__(256) ksa_bwd_finish_kernel(BwdArgs a)
+__global__ void __launch_bounds__(256) ksa_bwd_finish_kernel(BwdArgs a, int tails)
 {
     const SeqInfo sq = a.seqs[blockIdx.y];
     const bool text = (blockIdx.z == 0);
+    const int row_first = tails ? sq.n_chunks * a.k : 0;
     const int vecs = a.D / 8;
-    const int live = text ? sq.n_text : sq.n_summ;
+    const int live = (text ? sq.n_text : sq.n_summ) - row_first;
     const int64_t per_row = (int64_t)a.Hkv * vecs;
     const int64_t total = (int64_t)live * per_row;
     const int s = a.k + a.m;
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (int64_t)gridDim.x * blockDim.x) {
-        const int row = (int)(idx / per_row);
-        const int rem = (int)(idx - (int64_t)row * per_row);
+        const int row_rel = (int)(idx / per_row), row = row_first + row_rel;
+        const int rem = (int)(idx - (int64_t)row_rel * per_row);
         const int hk = rem / vecs, vv = rem - hk * vecs;
         const int64_t aug = text ? sq.aug_off + (int64_t)(row / a.k) * s + (row % a.k)
                                  : sq.aug_off + (int64_t)(row / a.m) * s + a.k + (row % a.m);
@@ -527,7 +529,6 @@ cudaError_t launch_bwd_prep(const BwdArgs& a, cudaStream_t stream)
 cudaError_t launch_bwd_summary(const BwdArgs& a, cudaStream_t stream)
 {
     if (a.m <= 0 || a.max_n_summ <= 0) return cudaSuccess;
-    if (bwd_summary_mma_applies(a)) return launch_bwd_summary_mma(a, stream);
     const int64_t warps = (int64_t)a.max_n_summ * a.Hq;
     dim3 grid((unsigned)((warps + 7) / 8), (unsigned)a.num_seqs, 1);
     if (a.D == 128) ksa_bwd_summary_kernel<128><<<grid, 256, 0, stream>>>(a);
@@ -561,15 +562,15 @@ cudaError_t launch_bwd_dkv(const BwdArgs& a, cudaStream_t stream)
     return cudaSuccess;
 }
 
-cudaError_t launch_bwd_finish(const BwdArgs& a, cudaStream_t stream)
+cudaError_t launch_bwd_finish(const BwdArgs& a, bool tails, cudaStream_t stream)
 {
     const int64_t per_row = (int64_t)a.Hkv * (a.D / 8);
-    const int64_t rows = a.max_text_pad > a.max_summ_pad ? a.max_text_pad : a.max_summ_pad;
+    const int64_t rows = tails ? a.k : a.max_text_pad > a.max_summ_pad ? a.max_text_pad : a.max_summ_pad;
     int64_t blocks = (rows * per_row + 255) / 256;
     if (blocks > 148 * 32) blocks = 148 * 32;
     if (blocks < 1) blocks = 1;
-    dim3 grid((unsigned)blocks, (unsigned)a.num_seqs, a.m > 0 ? 2u : 1u);
-    ksa_bwd_finish_kernel<<<grid, 256, 0, stream>>>(a);
+    dim3 grid((unsigned)blocks, (unsigned)a.num_seqs, a.m > 0 && !tails ? 2u : 1u);
+    ksa_bwd_finish_kernel<<<grid, 256, 0, stream>>>(a, tails ? 1 : 0);
     return cudaGetLastError();
 }
 

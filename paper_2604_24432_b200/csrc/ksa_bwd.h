@@ -37,17 +37,18 @@ struct BwdMaps { CUtensorMap qt, dot, kt, vt, ks, vs; };
 
 // Packs the text rows of dO, lse (in log2 units) and delta = <dO, O>.
 cudaError_t launch_bwd_prep(const BwdArgs& a, cudaStream_t stream);
-// Summary query rows: their dQ rows directly, their dK / dV contributions into the accumulators.
+// Summary query rows on CUDA cores: their dQ rows directly, their dK / dV contributions added to the accumulators.
 cudaError_t launch_bwd_summary(const BwdArgs& a, cudaStream_t stream);
-// The same on mma.sync tiles, one block per (chunk, KV head) or per group of short chunks; launch_bwd_summary dispatches
-// to it when bwd_summary_mma_applies (at most 128 query rows m G and 128 keys k + m per chunk).
+// The same on mma.sync tiles, one block per (chunk, KV head) or per group of short chunks, where bwd_summary_mma_applies (at
+// most 128 query rows m G and 128 keys k + m per chunk).  It also finishes the rows of every whole chunk: it must run after
+// the text rows' kernels, adds to their accumulators and writes dk / dv.
 bool bwd_summary_mma_applies(const BwdArgs& a);
 cudaError_t launch_bwd_summary_mma(const BwdArgs& a, cudaStream_t stream);
 // Text query rows: dQ (written directly), then dK / dV into the accumulators.
 cudaError_t launch_bwd_dq(const BwdArgs& a, cudaStream_t stream);
 cudaError_t launch_bwd_dkv(const BwdArgs& a, cudaStream_t stream);
-// Accumulators -> bf16 dk / dv at the augmented positions.
-cudaError_t launch_bwd_finish(const BwdArgs& a, cudaStream_t stream);
+// Accumulators -> bf16 dk / dv at the augmented positions; `tails`: only the text rows behind the last whole chunks.
+cudaError_t launch_bwd_finish(const BwdArgs& a, bool tails, cudaStream_t stream);
 cudaError_t setup_bwd();
 // dQ and dK / dV of the text rows on the tcgen05 tensor cores (head_dim 128 and 64).
 cudaError_t launch_bwd_dq_tc(const BwdArgs& a, const BwdMaps& maps, cudaStream_t stream);

@@ -9,8 +9,16 @@
 // XOR-swizzled by row for ldmatrix).  Phase 1, a warp per 16 query rows: S and dP on the tensor cores, P, delta and
 // dS in registers, dQ = dS K with dS taken from the accumulator registers as the A operand; P and dS also go to shared
 // memory as bf16.  Phase 2, a warp per 16 keys: dV and dK as products over the query rows, with P^T and dS^T read
-// through ldmatrix.trans; one vector atomic per element and block into the fp32 accumulators of the key streams (the
-// text keys of the chunk also collect from the text rows' kernels), instead of one per element and query row.
+// through ldmatrix.trans.
+//
+// A chunk's k + m rows of a KV head belong to one block, so this kernel is also the last step of the backward pass for
+// them: it runs after the text rows' kernels, adds its dV and dK to the fp32 sums these left in the key streams' accumulators
+// (asked for before the products, so that they arrive beside them) and writes the bf16 gradients.  Only the rows behind a
+// sequence's last whole chunk are left to the finish kernel.  Two sequences of 32,768 tokens, 32/8 heads, k = 8: the
+// kernel with one vector atomic per element and the finish pass over all rows took 787 + 160 us, now 468 us (64 + 8 layout at
+// 2 x 8,192: 152 + 46 -> 139 us; 16/16 heads, 7,942 ragged tokens: 113 + 47 -> 86 + 4 us).  What bounds
+// it is the latency of a block (loads, one warp per 16 query rows, then keys); its HBM traffic, 1.4 GB, would take 213 us.  Short
+// blocks (up to 64 keys) have an instance with half the score registers, which lets four instead of two of them share an SM.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -23,6 +31,7 @@ namespace ksa {
 namespace {
 
 constexpr int kBsMaxKeys = 128;       // k + m, padded to a multiple of 16
+constexpr int kBsShortKeys = 64;      // the short instance
 constexpr int kBsMaxRows = 128;       // m G, padded to a multiple of 16
 
 __device__ __forceinline__ uint32_t bs_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -61,11 +70,10 @@ __device__ __forceinline__ uint32_t bs_sw(uint32_t base, int row, int chunk)
     return base + (uint32_t)row * (uint32_t)(D * 2) + (uint32_t)(((chunk ^ (row & 7)) & (D / 8 - 1)) << 4);
 }
 
-template <int D>
-__global__ void __launch_bounds__(128, 2) ksa_bwd_summary_mma_kernel(BwdArgs a, int s_pad, int m_pad, int cpb)
+template <int D, int KT_MAX>
+__global__ void __launch_bounds__(128, KT_MAX <= 4 ? 4 : KT_MAX <= 6 ? 3 : 2) ksa_bwd_summary_mma_kernel(BwdArgs a, int s_pad, int m_pad, int cpb)
 {
     constexpr int CH = D / 8;
-    constexpr int KT_MAX = kBsMaxKeys / 16;
     extern __shared__ __align__(128) uint16_t bs_smem[];
     const SeqInfo sq = a.seqs[blockIdx.y];
     const int j = blockIdx.x * cpb, hk = blockIdx.z;                   // first chunk of the block
@@ -82,7 +90,7 @@ __global__ void __launch_bounds__(128, 2) ksa_bwd_summary_mma_kernel(BwdArgs a, 
     const uint32_t sV = sK + (uint32_t)s_pad * D * 2;
     const uint32_t sP = sV + (uint32_t)s_pad * D * 2;
     const uint32_t sS = sP + (uint32_t)m_pad * pstride;
-    const uint32_t sO = sS + (uint32_t)m_pad * pstride;                // per warp 16 rows of dQ on their way out
+    const uint32_t sO = sS + (uint32_t)m_pad * pstride;                // per warp at work 16 rows of dQ on their way out
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     // ---- stage Q, dO (row t = summary t / G, query head hk G + t % G), K, V; padding rows are zeros ----
@@ -239,48 +247,68 @@ __global__ void __launch_bounds__(128, 2) ksa_bwd_summary_mma_kernel(BwdArgs a, 
     __syncthreads();
 
     // =============================== phase 2: a warp per 16 keys ===============================
+    // K and V have been read: the rows of a key tile stage its gradients on their way out (dV over K, dK over V)
     for (int kt = warp; kt < kt_run; kt += 4) {
         // the accumulator rows of keys kt 16 + g0 and + 8: text rows of the chunk, then the chunk's own summaries
-        float* acc_k[2]; float* acc_v[2];
+        const float* acc_k[2]; const float* acc_v[2];
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
-            const int kidx = kt * 16 + g0 + 8 * half;
+            const int kidx = min(kt * 16 + g0 + 8 * half, keys - 1);   // (padding keys read a live row and are not stored)
             const int kc = kidx / s, key = kidx - kc * s;              // chunk within the block, key within the chunk
-            if (kidx < keys && key < a.k) {
+            if (key < a.k) {
                 const size_t row = (size_t)hk * a.text_rows + sq.text_off + (size_t)(j + kc) * a.k + key;
                 acc_k[half] = a.dkt + row * D; acc_v[half] = a.dvt + row * D;
-            } else if (kidx < keys) {
+            } else {
                 const size_t row = (size_t)hk * a.summ_rows + sq.summ_off + (size_t)(j + kc) * a.m + (key - a.k);
                 acc_k[half] = a.dks + row * D; acc_v[half] = a.dvs + row * D;
-            } else {
-                acc_k[half] = nullptr; acc_v[half] = nullptr;
             }
         }
 #pragma unroll
         for (int which = 0; which < 2; ++which) {                     // 0: dV = P^T dO, 1: dK = scale dS^T Q
             const uint32_t sA = which ? sS : sP, sB = which ? sQ : sG;
-            float o[D / 8][4];
+            const float mul = which ? a.scale : 1.f;
+            const uint32_t sW = (which ? sV : sK) + (uint32_t)(kt * 16) * D * 2;      // the tile's own rows of V / K
+#pragma unroll 1
+            for (int i0 = 0; i0 < D / 8; i0 += 8) {                    // 64 elements at a time: sums and products fit the registers
+                float2 sum[8][2];                                      // what the text rows' kernels have added up
 #pragma unroll
-            for (int i = 0; i < D / 8; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }
-            for (int rk = 0; rk < m_pad / 16; ++rk) {
-                uint32_t pa[4];
-                bs_ldsm_t(pa, sA + (uint32_t)(rk * 16 + r8 + 8 * (mi >> 1)) * pstride + (uint32_t)(kt * 16 + 8 * (mi & 1)) * 2);
+                for (int i = 0; i < 8; ++i)
 #pragma unroll
-                for (int n2 = 0; n2 < D / 16; ++n2) {
-                    uint32_t gb[4];
-                    bs_ldsm_t(gb, bs_sw<D>(sB, rk * 16 + r8 + 8 * (mi & 1), 2 * n2 + (mi >> 1)));
-                    bs_mma(o[2 * n2], pa, gb[0], gb[1]);
-                    bs_mma(o[2 * n2 + 1], pa, gb[2], gb[3]);
+                    for (int half = 0; half < 2; ++half)
+                        sum[i][half] = *reinterpret_cast<const float2*>((which ? acc_k[half] : acc_v[half]) + (i0 + i) * 8 + c2);
+                float o[8][4];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }
+                for (int rk = 0; rk < m_pad / 16; ++rk) {
+                    uint32_t pa[4];
+                    bs_ldsm_t(pa, sA + (uint32_t)(rk * 16 + r8 + 8 * (mi >> 1)) * pstride + (uint32_t)(kt * 16 + 8 * (mi & 1)) * 2);
+#pragma unroll
+                    for (int n2 = 0; n2 < 4; ++n2) {
+                        uint32_t gb[4];
+                        bs_ldsm_t(gb, bs_sw<D>(sB, rk * 16 + r8 + 8 * (mi & 1), i0 + 2 * n2 + (mi >> 1)));
+                        bs_mma(o[2 * n2], pa, gb[0], gb[1]);
+                        bs_mma(o[2 * n2 + 1], pa, gb[2], gb[3]);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const uint32_t w0 = bs_pack(fmaf(o[i][0], mul, sum[i][0].x), fmaf(o[i][1], mul, sum[i][0].y));
+                    const uint32_t w1 = bs_pack(fmaf(o[i][2], mul, sum[i][1].x), fmaf(o[i][3], mul, sum[i][1].y));
+                    asm volatile("st.shared.u32 [%0], %1;" ::"r"(bs_sw<D>(sW, g0, i0 + i) + (uint32_t)c2 * 2), "r"(w0) : "memory");
+                    asm volatile("st.shared.u32 [%0], %1;" ::"r"(bs_sw<D>(sW, g0 + 8, i0 + i) + (uint32_t)c2 * 2), "r"(w1) : "memory");
                 }
             }
-            const float mul = which ? a.scale : 1.f;
+            __syncwarp();
+            uint16_t* dst = (which ? a.dk + (int64_t)hk * a.dk_sh : a.dv + (int64_t)hk * a.dv_sh);
+            const int64_t dst_st = which ? a.dk_st : a.dv_st;
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                float* acc = which ? acc_k[half] : acc_v[half];
-                if (acc == nullptr) continue;
-#pragma unroll
-                for (int i = 0; i < D / 8; ++i)
-                    atomicAdd(reinterpret_cast<float2*>(acc + i * 8 + c2), make_float2(o[i][2 * half] * mul, o[i][2 * half + 1] * mul));
+            for (int it = 0; it < 16 * CH / 32; ++it) {
+                const int idx = it * 32 + lane;
+                const int rl = idx / CH, c = idx - rl * CH;
+                if (kt * 16 + rl >= keys) continue;
+                uint4 val;
+                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(val.x), "=r"(val.y), "=r"(val.z), "=r"(val.w) : "r"(bs_sw<D>(sW, rl, c)));
+                *reinterpret_cast<uint4*>(dst + (row0 + kt * 16 + rl) * dst_st + c * 8) = val;
             }
         }
     }
@@ -291,17 +319,18 @@ bool g_bs_done[64] = {};
 
 size_t bs_smem_bytes(int D, int s_pad, int m_pad)
 {
-    return (size_t)2 * (m_pad + s_pad) * D * 2 + (size_t)2 * m_pad * (s_pad + 8) * 2 + (size_t)4 * 16 * D * 2;
+    return (size_t)2 * (m_pad + s_pad) * D * 2 + (size_t)2 * m_pad * (s_pad + 8) * 2 + (size_t)std::min(4, m_pad / 16) * 16 * D * 2;
 }
 
 }  // namespace
 
-// Chunks per block: as many as it takes to fill a 16-row tile, within the kernel's row and key limits.
+// Chunks per block: as many as it takes to fill a 16-row tile, within the kernel's row and key limits -- and no more than
+// the short instance takes where a chunk fits it (many short blocks hide their latencies, long ones do not).
 static int bs_chunks_per_block(const BwdArgs& a)
 {
     const int G = a.Hq / a.Hkv, per_chunk = a.m * G, s = a.k + a.m;
     int c = (16 + per_chunk - 1) / per_chunk;
-    c = std::min(c, std::min(kBsMaxKeys / s, kBsMaxRows / per_chunk));
+    c = std::min(c, std::min((s <= kBsShortKeys ? kBsShortKeys : kBsMaxKeys) / s, kBsMaxRows / per_chunk));
     return std::max(c, 1);
 }
 
@@ -322,18 +351,31 @@ cudaError_t launch_bwd_summary_mma(const BwdArgs& a, cudaStream_t stream)
     if (dev >= 0 && dev < 64) {
         std::lock_guard<std::mutex> lock(g_bs_mutex);            // the shared-memory opt-in is a per-device setting
         if (!g_bs_done[dev]) {
-            if ((e = cudaFuncSetAttribute(ksa_bwd_summary_mma_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)bs_smem_bytes(128, kBsMaxKeys, kBsMaxRows))) != cudaSuccess) return e;
-            if ((e = cudaFuncSetAttribute(ksa_bwd_summary_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)bs_smem_bytes(64, kBsMaxKeys, kBsMaxRows))) != cudaSuccess) return e;
+            const auto opt_in = [&](auto* kernel, int D, int keys) {
+                return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bs_smem_bytes(D, keys, kBsMaxRows));
+            };
+            if ((e = opt_in(ksa_bwd_summary_mma_kernel<128, 8>, 128, kBsMaxKeys)) != cudaSuccess) return e;
+            if ((e = opt_in(ksa_bwd_summary_mma_kernel<64, 8>, 64, kBsMaxKeys)) != cudaSuccess) return e;
+            if ((e = opt_in(ksa_bwd_summary_mma_kernel<128, 6>, 128, 96)) != cudaSuccess) return e;
+            if ((e = opt_in(ksa_bwd_summary_mma_kernel<64, 6>, 64, 96)) != cudaSuccess) return e;
+            if ((e = opt_in(ksa_bwd_summary_mma_kernel<128, 4>, 128, kBsShortKeys)) != cudaSuccess) return e;
+            if ((e = opt_in(ksa_bwd_summary_mma_kernel<64, 4>, 64, kBsShortKeys)) != cudaSuccess) return e;
             g_bs_done[dev] = true;
         }
     }
     const int max_chunks = a.max_n_summ / a.m;
     dim3 grid((unsigned)((max_chunks + cpb - 1) / cpb), (unsigned)a.num_seqs, (unsigned)a.Hkv);
     const size_t smem = bs_smem_bytes(a.D, s_pad, m_pad);
-    if (a.D == 128) ksa_bwd_summary_mma_kernel<128><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
-    else            ksa_bwd_summary_mma_kernel<64><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
+    if (s_pad <= kBsShortKeys) {
+        if (a.D == 128) ksa_bwd_summary_mma_kernel<128, 4><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
+        else            ksa_bwd_summary_mma_kernel<64, 4><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
+    } else if (s_pad <= 96) {
+        if (a.D == 128) ksa_bwd_summary_mma_kernel<128, 6><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
+        else            ksa_bwd_summary_mma_kernel<64, 6><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
+    } else {
+        if (a.D == 128) ksa_bwd_summary_mma_kernel<128, 8><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
+        else            ksa_bwd_summary_mma_kernel<64, 8><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
+    }
     return cudaGetLastError();
 }
 
