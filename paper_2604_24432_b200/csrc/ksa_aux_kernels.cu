@@ -17,84 +17,66 @@ __device__ __forceinline__ uint16_t float_to_bf16_bits(float f)
 }
 
 // ---------------------------------------------------------------------------------------
-// Pack.  grid = (blocks, num_seqs, 2): z = 0 packs the text stream (Q, K, V rows of text
-// tokens), z = 1 the summary stream (K, V rows of summary tokens).  One thread moves one
-// 16-byte vector.  Text token i of a sequence sits at augmented row (i/k)*(k+m) + i%k,
-// summary (j, r) at j*(k+m) + k + r (Eq. 1).
+// Pack: the text stream (Q, K, V rows of text tokens), then the summary stream (K, V rows of summary tokens).
+// Text token i of a sequence sits at augmented row (i/k)*(k+m) + i%k, summary (j, r) at j*(k+m) + k + r (Eq. 1).
+// A block moves four neighbouring rows of a stream, all heads: a thread keeps its vector of a head and walks the heads,
+// four rows' loads in flight; the rows' places are worked out once per block.  (With a thread per 16-byte vector that
+// divided its way from a flat index to row, head and vector, and a grid for the longest sequence times the number of
+// sequences: 645 us for six sequences of 127,475 tokens, 32/8 heads, now 478 us = 6.5 TB/s, the copy bandwidth; 81 -> 31 us
+// for four of 7,942 tokens, 16/16 heads; 39 -> 22 us for one of 6,007.  Eight rows: 489, 34, 24 us; a warp per row: 962 us.)
 // ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) ksa_pack_kernel(KernelArgs a)
+constexpr int kPackRows = 4;
+
+__global__ void __launch_bounds__(256) ksa_pack_kernel(KernelArgs a, int blocks_text, int rows_text, int rows_summ)
 {
     const bool ranged = a.r_seq >= 0;
-    const SeqInfo sq = a.seqs[ranged ? a.r_seq : (int)blockIdx.y];
-    const bool text = (blockIdx.z == 0);
-    const int vecs = a.D / 8;
-    const int slots = text ? (a.Hq + 2 * a.Hkv) : (2 * a.Hkv);
-    const int row_first = ranged ? (text ? a.r_text0 : a.r_summ0) : 0;
-    const int pad_rows = (ranged ? (text ? a.r_text1 : a.r_summ1) : (text ? sq.text_pad : sq.summ_pad)) - row_first;
-    const int live_rows = text ? sq.n_text : sq.n_summ;
-    const int64_t per_row = (int64_t)slots * vecs;
-    const int64_t total = (int64_t)pad_rows * per_row;
-    const int s = a.k + a.m;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int row_rel = (int)(idx / per_row);
-        const int rem = (int)(idx - (int64_t)row_rel * per_row);
-        const int row = row_first + row_rel;
-        const int slot = rem / vecs;
-        const int vec = rem - slot * vecs;
-        int64_t aug = 0;
-        if (row < live_rows) {
-            if (text) aug = sq.aug_off + (int64_t)(row / a.k) * s + (row % a.k);
-            else      aug = sq.aug_off + (int64_t)(row / a.m) * s + a.k + (row % a.m);
-        }
-        const uint16_t* src;
-        uint16_t* dst;
-        if (text) {
-            const int64_t drow = (int64_t)sq.text_off + row;
-            if (slot < a.Hq) {
-                src = a.q + aug * a.q_st + (int64_t)slot * a.q_sh;
-                dst = a.qt + ((int64_t)slot * a.text_rows + drow) * a.D;
-            } else if (slot < a.Hq + a.Hkv) {
-                const int h = slot - a.Hq;
-                src = a.kx + aug * a.k_st + (int64_t)h * a.k_sh;
-                dst = a.kt + ((int64_t)h * a.text_rows + drow) * a.D;
-            } else {
-                const int h = slot - a.Hq - a.Hkv;
-                src = a.v + aug * a.v_st + (int64_t)h * a.v_sh;
-                dst = a.vt + ((int64_t)h * a.text_rows + drow) * a.D;
-            }
-        } else {
-            const int64_t drow = (int64_t)sq.summ_off + row;
-            if (slot < a.Hkv) {
-                src = a.kx + aug * a.k_st + (int64_t)slot * a.k_sh;
-                dst = a.ks + ((int64_t)slot * a.summ_rows + drow) * a.D;
-            } else {
-                const int h = slot - a.Hkv;
-                src = a.v + aug * a.v_st + (int64_t)h * a.v_sh;
-                dst = a.vs + ((int64_t)h * a.summ_rows + drow) * a.D;
-            }
-        }
-        uint4 val = make_uint4(0u, 0u, 0u, 0u);
+    const bool text = (int)blockIdx.x < blocks_text;
+    const int row0 = ((int)blockIdx.x - (text ? 0 : blocks_text)) * kPackRows;   // row of the stream, or of the range
+    // (a sequence's part of a stream is a whole number of 128-row tiles, so the block's rows belong to one sequence)
+    const SeqInfo sq = a.seqs[ranged ? a.r_seq : seq_of_row(a.seqs, a.num_seqs, row0, text)];
+    const int first = ranged ? row0 + (text ? a.r_text0 : a.r_summ0) : row0 - (text ? sq.text_off : sq.summ_off);
+    const int end = ranged ? (text ? a.r_text0 + rows_text : a.r_summ0 + rows_summ) : (text ? sq.text_pad : sq.summ_pad);
+    const int live = text ? sq.n_text : sq.n_summ;
+    const int s = a.k + a.m, per = text ? a.k : a.m;             // rows of a chunk in this stream
+    int64_t aug[kPackRows];
+    bool in[kPackRows];                                          // the row is to be written
+#pragma unroll
+    for (int r = 0; r < kPackRows; ++r) {
+        const int row = first + r;
+        aug[r] = row < live ? sq.aug_off + (int64_t)(row / per) * s + (text ? 0 : a.k) + row % per : -1;
         // (debug builds) the source row inside the caller's tensors, the destination row inside its stream
-        const bool in_range = ksa_in_bounds(aug >= 0 && aug < a.total_aug && row >= 0 &&
-                                            (int64_t)(text ? sq.text_off : sq.summ_off) + row < (text ? a.text_rows : a.summ_rows), a.status);
-        if (!in_range) continue;
-        if (row < live_rows) val = *reinterpret_cast<const uint4*>(src + vec * 8);
-        *reinterpret_cast<uint4*>(dst + vec * 8) = val;
+        in[r] = row < end && ksa_in_bounds(aug[r] < a.total_aug && row >= 0 &&
+                                           (int64_t)(text ? sq.text_off : sq.summ_off) + row < (text ? a.text_rows : a.summ_rows), a.status);
+    }
+    const int vecs = a.D / 8, vec = threadIdx.x % vecs;
+    const int nq = text ? a.Hq : 0, slots = nq + 2 * a.Hkv;
+    const int64_t drow = (int64_t)(text ? sq.text_off : sq.summ_off) + first, drows = text ? a.text_rows : a.summ_rows;
+    for (int slot = threadIdx.x / vecs; slot < slots; slot += 256 / vecs) {
+        const int h = slot < nq ? slot : (slot - nq < a.Hkv ? slot - nq : slot - nq - a.Hkv);
+        const uint16_t* src; uint16_t* dst; int64_t st;
+        if (slot < nq)              { src = a.q + (int64_t)h * a.q_sh;  st = a.q_st; dst = a.qt; }
+        else if (slot < nq + a.Hkv) { src = a.kx + (int64_t)h * a.k_sh; st = a.k_st; dst = text ? a.kt : a.ks; }
+        else                        { src = a.v + (int64_t)h * a.v_sh;  st = a.v_st; dst = text ? a.vt : a.vs; }
+        dst += ((int64_t)h * drows + drow) * a.D + vec * 8;
+        uint4 val[kPackRows];
+#pragma unroll
+        for (int r = 0; r < kPackRows; ++r) {
+            val[r] = make_uint4(0u, 0u, 0u, 0u);
+            if (in[r] && aug[r] >= 0) val[r] = *reinterpret_cast<const uint4*>(src + aug[r] * st + vec * 8);
+        }
+#pragma unroll
+        for (int r = 0; r < kPackRows; ++r)
+            if (in[r]) *reinterpret_cast<uint4*>(dst + r * a.D) = val[r];
     }
 }
 
 cudaError_t launch_pack(const KernelArgs& a, cudaStream_t stream)
 {
-    // grid.x covers the longest padded stream of any sequence (grid-stride loop beyond the cap).
-    const int64_t per_row = (int64_t)(a.Hq + 2 * a.Hkv) * (a.D / 8);
-    int64_t rows = a.max_text_pad > a.max_summ_pad ? a.max_text_pad : a.max_summ_pad;
-    if (a.r_seq >= 0) rows = (a.r_text1 - a.r_text0) > (a.r_summ1 - a.r_summ0) ? (a.r_text1 - a.r_text0) : (a.r_summ1 - a.r_summ0);
-    int64_t blocks = (rows * per_row + 255) / 256;
-    if (blocks > 148 * 64) blocks = 148 * 64;
-    if (blocks < 1) blocks = 1;
-    dim3 grid((unsigned)blocks, a.r_seq >= 0 ? 1u : (unsigned)a.num_seqs, a.m > 0 ? 2u : 1u);
-    ksa_pack_kernel<<<grid, 256, 0, stream>>>(a);
+    const int64_t text = a.r_seq >= 0 ? a.r_text1 - a.r_text0 : a.text_rows;
+    const int64_t summ = a.m <= 0 ? 0 : a.r_seq >= 0 ? a.r_summ1 - a.r_summ0 : a.summ_rows;
+    const int64_t bt = (text + kPackRows - 1) / kPackRows, bs = (summ + kPackRows - 1) / kPackRows;
+    if (bt + bs < 1) return cudaSuccess;
+    ksa_pack_kernel<<<(unsigned)(bt + bs), 256, 0, stream>>>(a, (int)bt, (int)text, (int)summ);
     return cudaGetLastError();
 }
 
@@ -305,8 +287,10 @@ __global__ void __launch_bounds__(256, 2) ksa_summary_staged_kernel(KernelArgs a
 // and the four groups read the very same shared-memory addresses.
 constexpr int kSummMaxKeys = 12;
 
-template <int D>
-__global__ void __launch_bounds__(256) ksa_summary_short_kernel(KernelArgs a)
+// kStreams: the rows come from the packed streams (text rows of kt / vt, summary rows of ks / vs, the summary tokens'
+// queries from qs, all head-major) instead of the caller's interleaved tensors.
+template <int D, bool kStreams>
+__global__ void __launch_bounds__(256) ksa_summary_short_kernel(KernelArgs a, const uint16_t* __restrict__ qs)
 {
     constexpr int E = D / 8;                      // elements per lane: 16 (two 16-byte vectors) or 8 (one)
     constexpr int V4 = E / 8;
@@ -330,8 +314,19 @@ __global__ void __launch_bounds__(256) ksa_summary_short_kernel(KernelArgs a)
         const int total = nch * s * vecs;
         for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
             const int rr = idx / vecs, vv = idx - rr * vecs;
-            const uint4 kx = *reinterpret_cast<const uint4*>(a.kx + (r0 + rr) * a.k_st + (int64_t)hk * a.k_sh + vv * 8);
-            const uint4 vx = *reinterpret_cast<const uint4*>(a.v + (r0 + rr) * a.v_st + (int64_t)hk * a.v_sh + vv * 8);
+            const uint16_t* kp; const uint16_t* vp;
+            if constexpr (kStreams) {
+                const int c = rr / s, off = rr - c * s, j = j0 + c;
+                const int64_t row = off < a.k ? (int64_t)hk * a.text_rows + sq.text_off + (int64_t)j * a.k + off
+                                              : (int64_t)hk * a.summ_rows + sq.summ_off + (int64_t)j * a.m + (off - a.k);
+                kp = (off < a.k ? a.kt : a.ks) + row * D;
+                vp = (off < a.k ? a.vt : a.vs) + row * D;
+            } else {
+                kp = a.kx + (r0 + rr) * a.k_st + (int64_t)hk * a.k_sh;
+                vp = a.v + (r0 + rr) * a.v_st + (int64_t)hk * a.v_sh;
+            }
+            const uint4 kx = *reinterpret_cast<const uint4*>(kp + vv * 8);
+            const uint4 vx = *reinterpret_cast<const uint4*>(vp + vv * 8);
             *reinterpret_cast<uint4*>(sK + rr * D + vv * 8) = kx;
             *reinterpret_cast<uint4*>(sV + rr * D + vv * 8) = vx;
         }
@@ -364,7 +359,8 @@ __global__ void __launch_bounds__(256) ksa_summary_short_kernel(KernelArgs a)
         const int nk = a.k + ((a.flags & 1u) ? 0 : (r + 1));           // own-chunk text (+ own summaries 0..r)
         float qv[E];
         {
-            const uint16_t* qp = a.q + qrow * a.q_st + (int64_t)h * a.q_sh + sub * 8;
+            const uint16_t* qp = (kStreams ? qs + ((int64_t)h * a.summ_rows + sq.summ_off + (int64_t)j * a.m + r) * D
+                                           : a.q + qrow * a.q_st + (int64_t)h * a.q_sh) + sub * 8;
 #pragma unroll
             for (int c = 0; c < V4; ++c) unpack(*reinterpret_cast<const uint4*>(qp + 64 * c), qv + 8 * c);
         }
@@ -440,8 +436,8 @@ cudaError_t launch_summary(const KernelArgs& a, cudaStream_t stream)
     const int chunk_groups = (max_chunks + kSummChunks - 1) / kSummChunks;
     if (a.k + a.m <= kSummMaxKeys) {
         dim3 g2((unsigned)chunk_groups, ny, (unsigned)a.Hkv);
-        if (a.D == 128) ksa_summary_short_kernel<128><<<g2, 256, 0, stream>>>(a);
-        else            ksa_summary_short_kernel<64><<<g2, 256, 0, stream>>>(a);
+        if (a.D == 128) ksa_summary_short_kernel<128, false><<<g2, 256, 0, stream>>>(a, nullptr);
+        else            ksa_summary_short_kernel<64, false><<<g2, 256, 0, stream>>>(a, nullptr);
     } else if (summary_mma_applies(a)) {
         return launch_summary_mma(a, max_chunks, ny, stream);
     } else {
@@ -641,6 +637,14 @@ __global__ void __launch_bounds__(256) ksa_summary_streams_kernel(KernelArgs a, 
 cudaError_t launch_summary_streams(const KernelArgs& a, const uint16_t* qs, cudaStream_t stream)
 {
     if (a.m <= 0 || a.max_n_summ <= 0) return cudaSuccess;
+    if (a.k + a.m <= kSummMaxKeys) {
+        // short chunks: rows staged per block as for interleaved tensors (36,000 augmented rows, 32/8 heads: 201 us in the
+        // kernel below, one warp per row with every key load waited for in turn, 72 us here)
+        dim3 g2((unsigned)((a.max_n_summ / a.m + kSummChunks - 1) / kSummChunks), (unsigned)a.num_seqs, (unsigned)a.Hkv);
+        if (a.D == 128) ksa_summary_short_kernel<128, true><<<g2, 256, 0, stream>>>(a, qs);
+        else            ksa_summary_short_kernel<64, true><<<g2, 256, 0, stream>>>(a, qs);
+        return cudaGetLastError();
+    }
     const int G = a.Hq / a.Hkv;
     int64_t blocks = ((int64_t)a.max_n_summ * a.Hkv * ((G + 3) / 4) + 7) / 8;
     if (blocks > 148 * 32) blocks = 148 * 32;

@@ -376,40 +376,62 @@ __global__ void __launch_bounds__(128) ksa_bwd_dkv_kernel(BwdArgs a, int summ)
 // =================================================================================================
 // preparation: text rows of dO into the packed layout (not in direct mode), lse in log2 units, delta = <dO, O>
 // =================================================================================================
+// A block takes four neighbouring rows of the text stream, all heads: a thread keeps its vector of a head and walks the
+// heads with eight loads in flight (HBM-bound: 2 x 32,768 tokens, 32 heads 308 -> 178 us = 6.8 TB/s; a thread
+// per vector with one load of each tensor in flight before).
+constexpr int kPrepRows = 4;
+
 __global__ void __launch_bounds__(256) ksa_bwd_prep_kernel(BwdArgs a)
 {
-    // One 16-byte vector (8 elements) per lane: D / 8 lanes make up a (row, head) unit, a warp holds 32 / (D / 8)
-    // units (consecutive heads of one row first: those are contiguous in dout / out).
-    const SeqInfo sq = a.seqs[blockIdx.y];
-    const int lane = threadIdx.x & 31;
-    const int lanes_per_unit = a.D / 8, units_per_warp = 32 / lanes_per_unit;
-    const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t unit = warp * units_per_warp + lane / lanes_per_unit;
-    const int sub = lane % lanes_per_unit;
-    const bool live = unit < (int64_t)sq.text_pad * a.Hq;
-    const int i = live ? (int)(unit / a.Hq) : 0, h = live ? (int)(unit % a.Hq) : 0;
-    const size_t prow = (size_t)h * a.text_rows + sq.text_off + i;
-    float d = 0.f;
-    float lse2 = INFINITY;
-    uint4 gv = make_uint4(0u, 0u, 0u, 0u);
-    const bool real = live && i < sq.n_text;
-    if (real) {
-        const int64_t aug = sq.aug_off + (int64_t)(i / a.k) * (a.k + a.m) + (i % a.k);
-        gv = *reinterpret_cast<const uint4*>(a.dout + aug * a.do_st + (int64_t)h * a.do_sh + sub * 8);
-        const uint4 ov = *reinterpret_cast<const uint4*>(a.out + aug * a.o_st + (int64_t)h * a.o_sh + sub * 8);
-        const uint32_t gw[4] = {gv.x, gv.y, gv.z, gv.w}, ow[4] = {ov.x, ov.y, ov.z, ov.w};
+    const int srow = blockIdx.x * kPrepRows;                             // row of the text stream
+    const SeqInfo sq = a.seqs[seq_of_row(a.seqs, a.num_seqs, srow, true)];
+    const int first = srow - sq.text_off;
+    int64_t aug[kPrepRows];                                              // -1: a padding row
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            d = fmaf(__uint_as_float(gw[e] << 16), __uint_as_float(ow[e] << 16), d);
-            d = fmaf(__uint_as_float(gw[e] & 0xffff0000u), __uint_as_float(ow[e] & 0xffff0000u), d);
-        }
-        if (sub == 0) lse2 = a.lse[(int64_t)h * a.total_aug + aug] * 1.4426950408889634f;
+    for (int r = 0; r < kPrepRows; ++r) {
+        const int i = first + r;
+        aug[r] = i < sq.n_text ? sq.aug_off + (int64_t)(i / a.k) * (a.k + a.m) + (i % a.k) : -1;
     }
-    // sum over the lanes of the unit (whole warps take part: no early exit above)
-    for (int s = lanes_per_unit >> 1; s > 0; s >>= 1) d += __shfl_xor_sync(0xffffffffu, d, s);
-    if (!live) return;
-    if (!a.direct) *reinterpret_cast<uint4*>(a.dot + prow * a.D + sub * 8) = gv;        // zeros on padding rows
-    if (sub == 0) { a.lse_t[prow] = lse2; a.delta_t[prow] = real ? d : 0.f; }
+    const int vecs = a.D / 8, vec = threadIdx.x % vecs;
+    // every thread of a warp takes the same number of steps (the shuffles below)
+    const int steps = (a.Hq + 256 / vecs - 1) / (256 / vecs);
+    for (int it = 0; it < steps; ++it) {
+        const int h = it * (256 / vecs) + threadIdx.x / vecs;
+        const bool live = h < a.Hq;
+        const size_t prow = (size_t)h * a.text_rows + srow;
+        uint4 gv[kPrepRows], ov[kPrepRows];
+        float lse2[kPrepRows], d[kPrepRows];
+#pragma unroll
+        for (int r = 0; r < kPrepRows; ++r) {
+            gv[r] = ov[r] = make_uint4(0u, 0u, 0u, 0u);
+            lse2[r] = INFINITY;
+            if (live && aug[r] >= 0) {
+                gv[r] = *reinterpret_cast<const uint4*>(a.dout + aug[r] * a.do_st + (int64_t)h * a.do_sh + vec * 8);
+                ov[r] = *reinterpret_cast<const uint4*>(a.out + aug[r] * a.o_st + (int64_t)h * a.o_sh + vec * 8);
+                if (vec == 0) lse2[r] = a.lse[(int64_t)h * a.total_aug + aug[r]] * 1.4426950408889634f;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < kPrepRows; ++r) {
+            const uint32_t gw[4] = {gv[r].x, gv[r].y, gv[r].z, gv[r].w}, ow[4] = {ov[r].x, ov[r].y, ov[r].z, ov[r].w};
+            d[r] = 0.f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                d[r] = fmaf(__uint_as_float(gw[e] << 16), __uint_as_float(ow[e] << 16), d[r]);
+                d[r] = fmaf(__uint_as_float(gw[e] & 0xffff0000u), __uint_as_float(ow[e] & 0xffff0000u), d[r]);
+            }
+            for (int s = vecs >> 1; s > 0; s >>= 1) d[r] += __shfl_xor_sync(0xffffffffu, d[r], s);
+        }
+        if (!live) continue;
+        if (!a.direct) {
+#pragma unroll
+            for (int r = 0; r < kPrepRows; ++r) *reinterpret_cast<uint4*>(a.dot + (prow + r) * a.D + vec * 8) = gv[r];     // zeros on padding rows
+        }
+        if (vec == 0) {                                                  // text_rows and srow are multiples of four
+            *reinterpret_cast<float4*>(a.lse_t + prow) = make_float4(lse2[0], lse2[1], lse2[2], lse2[3]);
+            *reinterpret_cast<float4*>(a.delta_t + prow) = make_float4(d[0], d[1], d[2], d[3]);
+        }
+    }
 }
 
 // =================================================================================================
@@ -519,10 +541,7 @@ cudaError_t setup_bwd()
 
 cudaError_t launch_bwd_prep(const BwdArgs& a, cudaStream_t stream)
 {
-    const int64_t units = (int64_t)a.max_text_pad * a.Hq;                // (row, head) units, 32 / (D / 8) per warp
-    const int64_t warps = (units * (a.D / 8) + 31) / 32;
-    dim3 grid((unsigned)((warps + 7) / 8), (unsigned)a.num_seqs, 1);
-    ksa_bwd_prep_kernel<<<grid, 256, 0, stream>>>(a);
+    ksa_bwd_prep_kernel<<<(unsigned)(a.text_rows / kPrepRows), 256, 0, stream>>>(a);
     return cudaGetLastError();
 }
 

@@ -93,6 +93,16 @@ __device__ __forceinline__ bool ksa_in_bounds(bool ok, int32_t* status)
 #else
 __device__ __forceinline__ bool ksa_in_bounds(bool, int32_t*) { return true; }
 #endif
+// The sequence that holds row `row` of the packed text (summary) stream: the last one that starts at or before it.
+__device__ __forceinline__ int seq_of_row(const SeqInfo* seqs, int n, int row, bool text)
+{
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if ((text ? seqs[mid].text_off : seqs[mid].summ_off) <= row) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
 // a row of out (and its lse entry) addressed by augmented row and query head
 __device__ __forceinline__ bool ksa_out_row_ok(const KernelArgs& a, int64_t aug, int h)
 {

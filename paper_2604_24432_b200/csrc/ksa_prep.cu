@@ -136,31 +136,26 @@ __global__ void __launch_bounds__(256, kPrepMinBlocks) ksa_prep_kernel(PrepArgs 
 }
 
 // Padding rows of the streams: rows [n_text, text_pad) of every sequence's part of qt, kt, vt and rows
-// [n_summ, summ_pad) of ks, vs, qs.  One block per (sequence, stream); at most 127 rows each.
+// [n_summ, summ_pad) of ks, vs, qs; at most 127 each.  A warp per row, all heads of the three streams.  (One block per
+// (sequence, stream) took 59 us for three sequences, 5 us now.)
 __global__ void __launch_bounds__(256) ksa_zero_stream_pads_kernel(PrepArgs a)
 {
     const SeqInfo sq = a.seqs[blockIdx.y];
-    const int which = blockIdx.x;                                  // 0 qt, 1 kt, 2 vt, 3 ks_out, 4 vs_out, 5 qs_out
-    const bool text = which < 3;
-    uint16_t* base = which == 0 ? a.qt : which == 1 ? a.kt : which == 2 ? a.vt : which == 3 ? a.ks_out : which == 4 ? a.vs_out : a.qs_out;
-    const int H = (which == 0 || which == 5) ? a.Hq : a.Hkv;
-    const int64_t rows = text ? a.text_rows : a.summ_rows;
-    const int64_t r0 = text ? (int64_t)sq.text_off + sq.n_text : (int64_t)sq.summ_off + sq.n_summ;
-    const int64_t r1 = text ? (int64_t)sq.text_off + sq.text_pad : (int64_t)sq.summ_off + sq.summ_pad;
-    const int vecs = a.D / 8;
-    const int64_t total = (r1 - r0) * H * vecs;
-    for (int64_t idx = threadIdx.x; idx < total; idx += blockDim.x) {
-        const int vec = (int)(idx % vecs);
-        const int64_t t = idx / vecs;
-        const int h = (int)(t % H);
-        const int64_t row = r0 + t / H;
-        *reinterpret_cast<uint4*>(base + ((int64_t)h * rows + row) * a.D + vec * 8) = make_uint4(0u, 0u, 0u, 0u);
+    const bool text = blockIdx.z == 0;
+    const int lane = threadIdx.x & 31, vecs = a.D / 8;
+    const int row = (text ? sq.n_text : sq.n_summ) + (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5);
+    if (row >= (text ? sq.text_pad : sq.summ_pad)) return;
+    const int64_t rows = text ? a.text_rows : a.summ_rows, r = (int64_t)(text ? sq.text_off : sq.summ_off) + row;
+    for (int slot = lane / vecs; slot < a.Hq + 2 * a.Hkv; slot += 32 / vecs) {
+        uint16_t* base = slot < a.Hq ? (text ? a.qt : a.qs_out) : slot < a.Hq + a.Hkv ? (text ? a.kt : a.ks_out) : (text ? a.vt : a.vs_out);
+        const int h = slot < a.Hq ? slot : slot < a.Hq + a.Hkv ? slot - a.Hq : slot - a.Hq - a.Hkv;
+        *reinterpret_cast<uint4*>(base + ((int64_t)h * rows + r) * a.D + (lane % vecs) * 8) = make_uint4(0u, 0u, 0u, 0u);
     }
 }
 
 cudaError_t launch_zero_stream_pads(const PrepArgs& a, int num_seqs, cudaStream_t stream)
 {
-    dim3 grid(6u, (unsigned)num_seqs, 1u);
+    dim3 grid(16u, (unsigned)num_seqs, 2u);
     ksa_zero_stream_pads_kernel<<<grid, 256, 0, stream>>>(a);
     return cudaGetLastError();
 }
