@@ -243,3 +243,32 @@ def test_q_zero_gives_log_count(ctx):
     out, lse = parity.run_gpu(ctx, prob, q, k, v)
     cnt = np.array([orc.visible_count(1500, 8, 1, 16, p) for p in range(total)])
     assert np.abs(lse - np.log(cnt)[:, None]).max() < 1e-4
+
+
+def test_changing_lengths_between_calls_in_flight(ctx):
+    """Calls with other lengths every time, on two streams and without waiting in between, past the point where the
+    context's schedule memory is reused: every result has the bits of the same call on its own."""
+    dev = torch.device("cuda", 0)
+    Hq, Hkv, D = 32, 4, 64
+    lens = [[700], [30_000], [333, 1290], [64_000], [1024], [52_011]]                 # schedules of up to 384 KB
+    cases = []
+    for i, ls in enumerate(lens):
+        prob = ksa.Problem(ls, 8, 1, 16, Hq, Hkv, D, 0.125)
+        total = ksa.total_aug_len(prob)
+        g = torch.Generator("cuda").manual_seed(i)
+        q, kk, v = (torch.randn((total, h, D), generator=g, device=dev).to(torch.bfloat16) for h in (Hq, Hkv, Hkv))
+        ws = [torch.empty(max(256, ksa.workspace_bytes(prob)), dtype=torch.uint8, device=dev) for _ in range(2)]
+        outs = [(torch.zeros_like(q), torch.zeros((Hq, total), device=dev)) for _ in range(2)]
+        ctx.attn_fwd(prob, q, kk, v, *outs[0], ws[0])
+        torch.cuda.synchronize()
+        cases.append((prob, q, kk, v, ws, outs, outs[0][0].clone(), outs[0][1].clone()))
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for rep in range(12):                                                             # some 10 MB of schedules
+        for i, (prob, q, kk, v, ws, outs, _, _) in enumerate(cases):
+            s = (i + rep) % 2
+            ctx.attn_fwd(prob, q, kk, v, *outs[s], ws[s], stream=streams[s].cuda_stream)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    for prob, q, kk, v, ws, outs, out, lse in cases:
+        for o, l in outs:
+            assert torch.equal(o.view(torch.int16), out.view(torch.int16)) and torch.equal(l.view(torch.int32), lse.view(torch.int32))
