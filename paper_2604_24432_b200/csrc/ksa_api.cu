@@ -221,13 +221,13 @@ static BaseItem schedule_q_tile(const Eq3& e, const SeqInfo& s, int seq, int qt)
     return it;
 }
 
-void build_schedule(const ksa_params* p, HostSchedule& hs, int target_chunks)
+void build_schedule(const ksa_params* p, HostSchedule& hs, int target_chunks, int num_sms)
 {
     const Eq3 e{p->chunk_len, p->summaries_per_chunk, p->window_chunks};
     const int k = p->chunk_len, m = p->summaries_per_chunk, s = k + m;
     // two query heads per work item: a pair inside a GQA group shares its K / V tiles; a pair that straddles two KV
     // heads (multi-head attention, odd group sizes) streams K / V per head; a single head only if the count is odd
-    const int heads_per_item = (p->num_q_heads % 2 == 0) ? 2 : 1;
+    int heads_per_item = (p->num_q_heads % 2 == 0) ? 2 : 1;
     struct Tagged { BaseItem it; int32_t chunk; };
     std::vector<Tagged> base;
     hs.chunks.clear();
@@ -263,6 +263,11 @@ void build_schedule(const ksa_params* p, HostSchedule& hs, int target_chunks)
         if (x.chunk != y.chunk) return x.chunk < y.chunk;
         return (x.it.ns_tiles + x.it.band_hi - x.it.band_lo) > (y.it.ns_tiles + y.it.band_hi - y.it.band_lo);
     });
+    // A single head gets through its key tiles sooner than a pair does, but a pair costs little more than one head: single
+    // heads where each still has an SM of its own (1,024 tokens: 4 heads of 64 17.9 -> 14.7 us, 16 heads of 128, 128 items,
+    // 20.4 -> 18.4 us; 517 tokens, 32 heads, 160 items: 18.3 against 21.1 us).  The CTA-pair kernel wants pairs.
+    if (heads_per_item == 2 && target_chunks == 0 && !(p->flags & KSA_FLAG_CTA_PAIR_KERNEL) &&
+        (int64_t)base.size() * p->num_q_heads <= num_sms) heads_per_item = 1;
     hs.work.clear();
     hs.work.reserve(base.size() * (p->num_q_heads / heads_per_item));
     for (const Tagged& tg : base) {
@@ -318,6 +323,7 @@ static std::vector<int32_t> schedule_key(const ksa_params* p)
     for (int b = 0; b <= p->num_seqs; ++b) key.push_back(p->cu_text_lens[b]);
     key.push_back(p->chunk_len); key.push_back(p->summaries_per_chunk); key.push_back(p->window_chunks);
     key.push_back(p->num_q_heads); key.push_back(p->num_kv_heads); key.push_back(p->head_dim);
+    key.push_back((int32_t)(p->flags & KSA_FLAG_CTA_PAIR_KERNEL));       // its work items have two heads
     return key;
 }
 
@@ -518,7 +524,7 @@ static int ensure_schedule(ksa_ctx* ctx, const ksa_params* p, bool upload, int t
         HostSchedule hs;
         try {
             build_layout(p, hs);
-            build_schedule(p, hs, target_chunks);
+            build_schedule(p, hs, target_chunks, ctx->num_sms);
         } catch (const std::bad_alloc&) { return KSA_ERR_NOMEM; }
         if (!schedule_in_range(p, hs)) return KSA_ERR_INTERNAL;
         hs.key = key;
@@ -746,6 +752,12 @@ static int launch_text(ksa_ctx* ctx, const KernelArgs& a, uint32_t flags, const 
     return KSA_OK;
 }
 
+// Where the text rows' kernel is short, the SMs that it leaves idle (small calls) or leaves early (its last round of work
+// items) are worth the summary rows' time: 1,024 tokens 24.6 -> 19.7 us, 8,192 tokens (seven rounds) 222 -> 214 us.  A call of
+// a hundred rounds gains nothing (127,475 tokens: 6,890 and 6,950 us): the line lies between the two.
+static constexpr int kBehindTextRounds = 16;
+static bool behind_text_pays(const ksa_ctx* ctx, const KernelArgs& a) { return a.num_work <= kBehindTextRounds * ctx->num_sms; }
+
 extern "C" __attribute__((visibility("default"))) int ksa_attn_fwd(ksa_ctx* ctx, const void* q, const void* k, const void* v, void* out, float* lse,
                             void* workspace, size_t workspace_bytes, const ksa_params* p, void* cuda_stream)
 {
@@ -768,15 +780,18 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_fwd(ksa_ctx* ctx,
         if ((e = launch_pack(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);
         ctx->launches += 1;
     }
-    if (a.m > 0 && a.max_n_summ > 0) {
-        if ((e = launch_summary(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);
-        ctx->launches += 1;
-    }
+    // The summary rows beside the end of the text rows' kernel: launched behind it, they take the SMs it leaves (in front
+    // of it where their kernel cannot, and where the text kernel is timed between two events).
+    const bool summ_rows = a.m > 0 && a.max_n_summ > 0;
+    const bool behind = summ_rows && !ctx->timing && behind_text_pays(ctx, a) && summary_behind_text_ok(a, false);
+    if (summ_rows && !behind && (e = launch_summary(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);
     if (ctx->timing) cudaEventRecord(ctx->ev0, stream);
     FwdMaps maps;
     if ((rc = prepare_text(ctx, a, p->flags, maps)) != KSA_OK) return rc;
     if ((rc = launch_text(ctx, a, p->flags, maps, stream)) != KSA_OK) return rc;
     if (ctx->timing) { cudaEventRecord(ctx->ev1, stream); ctx->timing_valid = true; }
+    if (behind && (e = launch_summary(a, stream, true)) != cudaSuccess) return cuda_fail(ctx, e);
+    if (summ_rows) ctx->launches += 1;
     return KSA_OK;
 }
 
@@ -1162,15 +1177,16 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_fwd_prepared(ksa_
     if ((e = launch_zero_stream_pads(pa, p->num_seqs, stream)) != cudaSuccess) return cuda_fail(ctx, e);
     if ((e = launch_prep(pa, max_aug_len, p->num_seqs, stream)) != cudaSuccess) return cuda_fail(ctx, e);
     ctx->launches += 2;
-    if (a.m > 0 && a.max_n_summ > 0) {
-        if ((e = launch_summary_streams(a, qs, stream)) != cudaSuccess) return cuda_fail(ctx, e);
-        ctx->launches += 1;
-    }
+    const bool summ_rows = a.m > 0 && a.max_n_summ > 0;
+    const bool behind = summ_rows && !ctx->timing && behind_text_pays(ctx, a) && summary_behind_text_ok(a, true);      // as in ksa_attn_fwd
+    if (summ_rows && !behind && (e = launch_summary_streams(a, qs, stream, false)) != cudaSuccess) return cuda_fail(ctx, e);
     if (ctx->timing) cudaEventRecord(ctx->ev0, stream);
     FwdMaps maps;
     if ((rc = prepare_text(ctx, a, p->flags, maps)) != KSA_OK) return rc;
     if ((rc = launch_text(ctx, a, p->flags, maps, stream)) != KSA_OK) return rc;
     if (ctx->timing) { cudaEventRecord(ctx->ev1, stream); ctx->timing_valid = true; }
+    if (behind && (e = launch_summary_streams(a, qs, stream, true)) != cudaSuccess) return cuda_fail(ctx, e);
+    if (summ_rows) ctx->launches += 1;
     return KSA_OK;
 }
 

@@ -6,6 +6,7 @@
 #include <type_traits>
 
 #include "ksa_launch.h"
+#include "ksa_ptx.cuh"
 
 namespace ksa {
 
@@ -29,6 +30,7 @@ constexpr int kPackRows = 4;
 
 __global__ void __launch_bounds__(256) ksa_pack_kernel(KernelArgs a, int blocks_text, int rows_text, int rows_summ)
 {
+    ptx::pdl_launch_dependents();                                // the text kernel sets itself up meanwhile
     const bool ranged = a.r_seq >= 0;
     const bool text = (int)blockIdx.x < blocks_text;
     const int row0 = ((int)blockIdx.x - (text ? 0 : blocks_text)) * kPackRows;   // row of the stream, or of the range
@@ -290,7 +292,7 @@ constexpr int kSummMaxKeys = 12;
 // kStreams: the rows come from the packed streams (text rows of kt / vt, summary rows of ks / vs, the summary tokens'
 // queries from qs, all head-major) instead of the caller's interleaved tensors.
 template <int D, bool kStreams>
-__global__ void __launch_bounds__(256) ksa_summary_short_kernel(KernelArgs a, const uint16_t* __restrict__ qs)
+__device__ __forceinline__ void summary_short_block(const KernelArgs& a, const uint16_t* __restrict__ qs)
 {
     constexpr int E = D / 8;                      // elements per lane: 16 (two 16-byte vectors) or 8 (one)
     constexpr int V4 = E / 8;
@@ -425,7 +427,26 @@ __global__ void __launch_bounds__(256) ksa_summary_short_kernel(KernelArgs a, co
     }
 }
 
-cudaError_t launch_summary(const KernelArgs& a, cudaStream_t stream)
+// The first block ends after the kernel in front (where this one was launched beside it): see launch_summary.
+template <int D, bool kStreams>
+__global__ void __launch_bounds__(256) ksa_summary_short_kernel(KernelArgs a, const uint16_t* __restrict__ qs)
+{
+    summary_short_block<D, kStreams>(a, qs);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) ptx::pdl_wait();
+}
+
+template <bool kStreams>
+static cudaError_t launch_summary_short(const KernelArgs& a, const uint16_t* qs, dim3 grid, cudaStream_t stream, bool behind_text)
+{
+    auto* kernel = a.D == 128 ? ksa_summary_short_kernel<128, kStreams> : ksa_summary_short_kernel<64, kStreams>;
+    if (behind_text) return launch_dependent(kernel, grid, 256, 0, stream, a, qs);
+    kernel<<<grid, 256, 0, stream>>>(a, qs);
+    return cudaGetLastError();
+}
+
+bool summary_behind_text_ok(const KernelArgs& a, bool streams) { return a.k + a.m <= kSummMaxKeys || (!streams && summary_mma_applies(a)); }
+
+cudaError_t launch_summary(const KernelArgs& a, cudaStream_t stream, bool behind_text)
 {
     if (a.m <= 0 || a.max_n_summ <= 0) return cudaSuccess;
     // grid.x covers the sequence with the most summary rows; shorter ones exit early.
@@ -436,10 +457,9 @@ cudaError_t launch_summary(const KernelArgs& a, cudaStream_t stream)
     const int chunk_groups = (max_chunks + kSummChunks - 1) / kSummChunks;
     if (a.k + a.m <= kSummMaxKeys) {
         dim3 g2((unsigned)chunk_groups, ny, (unsigned)a.Hkv);
-        if (a.D == 128) ksa_summary_short_kernel<128, false><<<g2, 256, 0, stream>>>(a, nullptr);
-        else            ksa_summary_short_kernel<64, false><<<g2, 256, 0, stream>>>(a, nullptr);
+        return launch_summary_short<false>(a, nullptr, g2, stream, behind_text);
     } else if (summary_mma_applies(a)) {
-        return launch_summary_mma(a, max_chunks, ny, stream);
+        return launch_summary_mma(a, max_chunks, ny, stream, behind_text);
     } else {
         const int tasks = a.m * (a.Hq / a.Hkv);
         const int task_blocks = (tasks + kSummTaskBlock - 1) / kSummTaskBlock;
@@ -634,16 +654,14 @@ __global__ void __launch_bounds__(256) ksa_summary_streams_kernel(KernelArgs a, 
     }
 }
 
-cudaError_t launch_summary_streams(const KernelArgs& a, const uint16_t* qs, cudaStream_t stream)
+cudaError_t launch_summary_streams(const KernelArgs& a, const uint16_t* qs, cudaStream_t stream, bool behind_text)
 {
     if (a.m <= 0 || a.max_n_summ <= 0) return cudaSuccess;
     if (a.k + a.m <= kSummMaxKeys) {
         // short chunks: rows staged per block as for interleaved tensors (36,000 augmented rows, 32/8 heads: 201 us in the
         // kernel below, one warp per row with every key load waited for in turn, 72 us here)
         dim3 g2((unsigned)((a.max_n_summ / a.m + kSummChunks - 1) / kSummChunks), (unsigned)a.num_seqs, (unsigned)a.Hkv);
-        if (a.D == 128) ksa_summary_short_kernel<128, true><<<g2, 256, 0, stream>>>(a, qs);
-        else            ksa_summary_short_kernel<64, true><<<g2, 256, 0, stream>>>(a, qs);
-        return cudaGetLastError();
+        return launch_summary_short<true>(a, qs, g2, stream, behind_text);
     }
     const int G = a.Hq / a.Hkv;
     int64_t blocks = ((int64_t)a.max_n_summ * a.Hkv * ((G + 3) / 4) + 7) / 8;

@@ -22,6 +22,8 @@
 
 #include "../../include/ksa_decode.h"
 #include "ksa_host.h"
+#include "ksa_launch.h"
+#include "ksa_ptx.cuh"
 
 namespace ksa {
 
@@ -106,11 +108,6 @@ __device__ __forceinline__ float fast_ex2(float x)
     return y;
 }
 
-// Programmatic dependent launch: the kernels of this file are launched with the attribute, i.e. possibly before the
-// kernel in front of them in the stream has finished; nothing may be read or written before pdl_wait() returns.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // In place of a split's reference maximum: the sequence does not take this step (a NaN that no maximum can be).
 constexpr uint32_t kDecSkipped = 0x7fdec0deu;
 
@@ -148,8 +145,8 @@ __global__ void __launch_bounds__(kDecThreads) ksa_decode_attn_kernel(DecodeArgs
     const int split = blockIdx.x;
     const int b = blockIdx.y / a.Hkv, hk = blockIdx.y - b * a.Hkv;
     int reason = 0;
-    pdl_launch_dependents();
-    pdl_wait();
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const StepPlan p = plan_step(a, b, &reason);
     if (!p.run) {
         if (reason && split == 0 && hk == 0 && threadIdx.x == 0) atomicCAS(a.status, 0, reason);
@@ -312,8 +309,8 @@ __global__ void __launch_bounds__(kDecThreads) ksa_decode_attn_kernel(DecodeArgs
 template <int D>
 __global__ void __launch_bounds__(D) ksa_decode_merge_kernel(DecodeArgs a)
 {
-    pdl_launch_dependents();
-    pdl_wait();
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
     const int b = blockIdx.x / a.Hq, h = blockIdx.x - b * a.Hq;
     const int hk = h / a.G, g = h - hk * a.G;
     const int lane = threadIdx.x & 31;
@@ -573,17 +570,10 @@ static int decode_step(ksa_ctx* ctx, int summary_step, void* kcache, void* vcach
             return ksa_ctx_cuda_fail(ctx, (int)e);
         attr_done = true;
     }
-    // programmatic dependent launches: see pdl_wait()
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.stream = stream; cfg.attrs = &attr; cfg.numAttrs = 1;
-    cfg.gridDim = dim3((unsigned)a.nsplit, (unsigned)(a.B * a.Hkv), 1); cfg.blockDim = dim3(kDecThreads); cfg.dynamicSmemBytes = smem;
-    e = a.D == 128 ? cudaLaunchKernelEx(&cfg, ksa_decode_attn_kernel<128>, a) : cudaLaunchKernelEx(&cfg, ksa_decode_attn_kernel<64>, a);
+    const dim3 grid((unsigned)a.nsplit, (unsigned)(a.B * a.Hkv), 1);
+    e = launch_dependent(a.D == 128 ? ksa_decode_attn_kernel<128> : ksa_decode_attn_kernel<64>, grid, kDecThreads, (size_t)smem, stream, a);
     if (e != cudaSuccess) return ksa_ctx_cuda_fail(ctx, (int)e);
-    cfg.gridDim = dim3((unsigned)(a.B * a.Hq)); cfg.blockDim = dim3((unsigned)a.D); cfg.dynamicSmemBytes = 0;
-    e = a.D == 128 ? cudaLaunchKernelEx(&cfg, ksa_decode_merge_kernel<128>, a) : cudaLaunchKernelEx(&cfg, ksa_decode_merge_kernel<64>, a);
+    e = launch_dependent(a.D == 128 ? ksa_decode_merge_kernel<128> : ksa_decode_merge_kernel<64>, dim3((unsigned)(a.B * a.Hq)), a.D, 0, stream, a);
     if (e != cudaSuccess) return ksa_ctx_cuda_fail(ctx, (int)e);
     ksa_ctx_add_launches(ctx, 2);
     return KSA_OK;

@@ -37,7 +37,8 @@ void build_layout(const ksa_params* p, HostSchedule& hs);
 // Fills hs.work (longest first) from p and the layout already in hs.
 // target_chunks > 0 additionally splits the query tiles into about that many row chunks (in
 // sequence order) and orders the work list chunk by chunk.
-void build_schedule(const ksa_params* p, HostSchedule& hs, int target_chunks = 0);
+// A call whose query heads are no more than num_sms tiles gets work items of a single query head.
+void build_schedule(const ksa_params* p, HostSchedule& hs, int target_chunks = 0, int num_sms = 0);
 // Offsets of the packed streams inside the workspace, and its total size.
 WorkspaceLayout workspace_layout(const ksa_params* p, const HostSchedule& hs);
 

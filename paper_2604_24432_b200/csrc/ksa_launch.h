@@ -7,17 +7,35 @@
 
 namespace ksa {
 
+// Launch with the programmatic-dependent-launch attribute: the kernel may start while the one in front of it in the stream
+// still runs, if that one allows it (pdl_launch_dependents), and calls pdl_wait before it touches what that one writes.
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, const A&... args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // De-interleaves text Q/K/V rows and summary K/V rows of the augmented layout (Eq. 1)
 // into dense head-major streams; padding rows are written as zeros.
 cudaError_t launch_pack(const KernelArgs& a, cudaStream_t stream);
 
-// Summary rows: each attends to the (at most k + m) keys of its own chunk.
-cudaError_t launch_summary(const KernelArgs& a, cudaStream_t stream);
+// Summary rows: each attends to the (at most k + m) keys of its own chunk.  behind_text: launched behind the text rows'
+// kernel, beside which it runs (the two read the same inputs and write different rows; its first block waits for the text
+// kernel's end, so that the work behind it finds both done).
+cudaError_t launch_summary(const KernelArgs& a, cudaStream_t stream, bool behind_text = false);
+// The kernels that can run there: the short-chunk and the mma.sync kernel (from the streams: the short-chunk kernel).
+bool summary_behind_text_ok(const KernelArgs& a, bool streams);
 // The same on mma.sync tiles: one block per (chunk, KV head), or per group of chunks stacked up to 64 query rows;
 // launch_summary dispatches to it for chunks of more than 12 keys when summary_mma_applies (at most 128 query rows m G
 // and 128 keys k + m per chunk).  Chunks of up to 12 keys are faster on the short-chunk kernel (measured).
 bool summary_mma_applies(const KernelArgs& a);
-cudaError_t launch_summary_mma(const KernelArgs& a, int max_chunks, unsigned ny, cudaStream_t stream);
+cudaError_t launch_summary_mma(const KernelArgs& a, int max_chunks, unsigned ny, cudaStream_t stream, bool behind_text);
 
 // Text rows, CUDA-core cross-check kernel (KSA_FLAG_REFERENCE_KERNEL).
 cudaError_t launch_text_ref(const KernelArgs& a, cudaStream_t stream);
@@ -63,6 +81,6 @@ cudaError_t launch_prep(const PrepArgs& a, int64_t max_aug_len, int num_seqs, cu
 // does not write.
 cudaError_t launch_zero_stream_pads(const PrepArgs& a, int num_seqs, cudaStream_t stream);
 // Summary rows from the packed streams (query rows in qs): each attends to the keys of its own chunk.
-cudaError_t launch_summary_streams(const KernelArgs& a, const uint16_t* qs, cudaStream_t stream);
+cudaError_t launch_summary_streams(const KernelArgs& a, const uint16_t* qs, cudaStream_t stream, bool behind_text);
 
 }  // namespace ksa

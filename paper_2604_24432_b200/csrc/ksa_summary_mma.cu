@@ -19,6 +19,7 @@
 #include <mutex>
 
 #include "ksa_launch.h"
+#include "ksa_ptx.cuh"
 
 namespace ksa {
 
@@ -65,7 +66,7 @@ __device__ __forceinline__ uint32_t sw_addr(uint32_t base, int row, int chunk)
 }
 
 template <int D>
-__global__ void __launch_bounds__(128, 3) ksa_summary_mma_kernel(KernelArgs a, int s_pad, int m_pad, int cpb)
+__device__ __forceinline__ void summary_mma_block(const KernelArgs& a, int s_pad, int m_pad, int cpb)
 {
     constexpr int CH = D / 8;                     // 16-byte chunks per row
     constexpr int KT_MAX = kMmaMaxKeys / 16;
@@ -248,6 +249,14 @@ __global__ void __launch_bounds__(128, 3) ksa_summary_mma_kernel(KernelArgs a, i
     }
 }
 
+// The first block ends after the kernel in front (where this one was launched beside it): see launch_summary.
+template <int D>
+__global__ void __launch_bounds__(128, 3) ksa_summary_mma_kernel(KernelArgs a, int s_pad, int m_pad, int cpb)
+{
+    summary_mma_block<D>(a, s_pad, m_pad, cpb);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) ptx::pdl_wait();
+}
+
 std::mutex g_attr_mutex;
 bool g_attr_done[64] = {};
 
@@ -269,7 +278,7 @@ bool summary_mma_applies(const KernelArgs& a)
     return a.m > 0 && a.k + a.m <= kMmaMaxKeys && a.m * G <= kMmaMaxRows;
 }
 
-cudaError_t launch_summary_mma(const KernelArgs& a, int max_chunks, unsigned ny, cudaStream_t stream)
+cudaError_t launch_summary_mma(const KernelArgs& a, int max_chunks, unsigned ny, cudaStream_t stream, bool behind_text)
 {
     const int G = a.Hq / a.Hkv;
     const int cpb = summ_chunks_per_block(a);
@@ -290,8 +299,9 @@ cudaError_t launch_summary_mma(const KernelArgs& a, int max_chunks, unsigned ny,
     // aligned groups of cpb chunks that the chunk range [j_first, j_first + max_chunks) touches
     const int j_first = a.r_seq >= 0 ? a.r_summ0 / a.m : 0;
     dim3 grid((unsigned)((j_first + max_chunks - 1) / cpb - j_first / cpb + 1), ny, (unsigned)a.Hkv);
-    if (a.D == 128) ksa_summary_mma_kernel<128><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
-    else            ksa_summary_mma_kernel<64><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
+    auto* kernel = a.D == 128 ? ksa_summary_mma_kernel<128> : ksa_summary_mma_kernel<64>;
+    if (behind_text) return launch_dependent(kernel, grid, 128, smem, stream, a, s_pad, m_pad, cpb);
+    kernel<<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
     return cudaGetLastError();
 }
 

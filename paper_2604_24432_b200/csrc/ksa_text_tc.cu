@@ -131,6 +131,11 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = ld_shared_u32(tmem_slot);
+    // Launched while the kernel in front (the pack) drains: nothing is read before it has finished.  From then on -- not
+    // before: it does not wait for that kernel itself -- the summary rows' kernel behind may start as soon as every CTA is
+    // resident; it takes the SMs that this kernel leaves.
+    pdl_wait();
+    pdl_launch_dependents();
 
     const int G = a.Hq / a.Hkv;
     const int grid = (int)gridDim.x;
@@ -508,11 +513,8 @@ cudaError_t launch_text_tc(const KernelArgs& a, const TextMaps& maps, int num_sm
 {
     if (a.num_work <= 0) return cudaSuccess;
     const int grid = a.num_work < num_sms ? a.num_work : num_sms;
-    if (a.D == 128)
-        ksa_text_tc_kernel<128><<<grid, kThreadsTc, TcCfg<128>::kSmemBytes, stream>>>(a, maps);
-    else
-        ksa_text_tc_kernel<64><<<grid, kThreadsTc, TcCfg<64>::kSmemBytes, stream>>>(a, maps);
-    return cudaGetLastError();
+    return a.D == 128 ? launch_dependent(ksa_text_tc_kernel<128>, dim3((unsigned)grid), kThreadsTc, TcCfg<128>::kSmemBytes, stream, a, maps)
+                      : launch_dependent(ksa_text_tc_kernel<64>, dim3((unsigned)grid), kThreadsTc, TcCfg<64>::kSmemBytes, stream, a, maps);
 }
 
 }  // namespace ksa

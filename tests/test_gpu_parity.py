@@ -272,3 +272,38 @@ def test_changing_lengths_between_calls_in_flight(ctx):
     for prob, q, kk, v, ws, outs, out, lse in cases:
         for o, l in outs:
             assert torch.equal(o.view(torch.int16), out.view(torch.int16)) and torch.equal(l.view(torch.int32), lse.view(torch.int32))
+
+
+@pytest.mark.parametrize("lens,k,m,C,Hq,Hkv,D", [
+    ([1], 8, 1, 2, 4, 4, 64),                     # no summary rows; one work item per head
+    ([5, 8, 640], 8, 1, 4, 4, 4, 64),             # the first sequence has no chunk: the summary grid's first block ends at once
+    ([1024], 8, 1, 16, 6, 2, 128),                # 48 heads' tiles: work items of single heads
+    ([1216], 8, 1, 16, 16, 4, 128),               # 160 of them, more than the SMs: pairs
+    ([3000, 777], 64, 8, 4, 8, 2, 128),           # summary rows on mma.sync tiles
+    ([6007], 8, 1, 128, 16, 2, 128),              # several rounds of work items
+])
+def test_work_behind_a_call_finds_all_rows(ctx, lens, k, m, C, Hq, Hkv, D):
+    """The summary rows' kernel runs beside the text rows': what is enqueued behind the call (here a copy of the outputs,
+    call after call on the same buffers, with the buffers overwritten in between) must see the rows of both."""
+    dev = torch.device("cuda", 0)
+    prob = ksa.Problem(lens, k, m, C, Hq, Hkv, D, float(D) ** -0.5)
+    total = ksa.total_aug_len(prob)
+    ws = torch.empty(max(256, ksa.workspace_bytes(prob)), dtype=torch.uint8, device=dev)
+    inputs, want = [], []
+    for i in range(2):
+        g = torch.Generator("cuda").manual_seed(i)
+        inputs.append(tuple(torch.randn((total, h, D), generator=g, device=dev).to(torch.bfloat16) for h in (Hq, Hkv, Hkv)))
+        out = torch.empty((total, Hq, D), dtype=torch.bfloat16, device=dev); lse = torch.empty((Hq, total), device=dev)
+        ctx.attn_fwd(prob, *inputs[i], out, lse, ws)
+        torch.cuda.synchronize()
+        want.append((out.clone(), lse.clone()))
+    got = []
+    for rep in range(16):
+        out.fill_(7.0); lse.fill_(7.0)
+        ctx.attn_fwd(prob, *inputs[rep % 2], out, lse, ws)
+        got.append((out.clone(), lse.clone()))
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    for rep, (o, l) in enumerate(got):
+        assert torch.equal(o.view(torch.int16), want[rep % 2][0].view(torch.int16)), rep
+        assert torch.equal(l.view(torch.int32), want[rep % 2][1].view(torch.int32)), rep
