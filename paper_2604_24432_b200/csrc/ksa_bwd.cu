@@ -357,16 +357,16 @@ __global__ void __launch_bounds__(128) ksa_bwd_dkv_kernel(BwdArgs a, int summ)
     }
     b_cp_wait<0>();
     // add this segment's partial sums to the fp32 accumulators of the stream
-    float* acc_k = (summ ? a.dks : a.dkt) + krow0 * D;
-    float* acc_v = (summ ? a.dvs : a.dvt) + krow0 * D;
+    float* acc_k = summ ? a.dks : a.dkt;
+    float* acc_v = summ ? a.dvs : a.dvt;
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
         const int rr = warp * 16 + g0 + half * 8;
         if (kt * kBT + rr >= n_keys) continue;
 #pragma unroll
         for (int nt = 0; nt < D / 8; ++nt) {
-            float* pk = acc_k + (size_t)rr * D + nt * 8 + c2;
-            float* pv = acc_v + (size_t)rr * D + nt * 8 + c2;
+            float* pk = acc_k + acc_at(krow0 + rr, nt * 8 + c2, D);
+            float* pv = acc_v + acc_at(krow0 + rr, nt * 8 + c2, D);
             atomicAdd(reinterpret_cast<float2*>(pk), make_float2(dk[nt][half * 2] * a.scale, dk[nt][half * 2 + 1] * a.scale));
             atomicAdd(reinterpret_cast<float2*>(pv), make_float2(dv[nt][half * 2], dv[nt][half * 2 + 1]));
         }
@@ -476,15 +476,15 @@ __global__ void __launch_bounds__(256) ksa_bwd_summary_kernel(BwdArgs a)
         float* ak; float* av;
         if (t < a.k) {
             const size_t row = (size_t)hk * a.text_rows + sq.text_off + (size_t)j * a.k + t;
-            ak = a.dkt + row * D; av = a.dvt + row * D;
+            ak = a.dkt + acc_at(row, lane * E, D); av = a.dvt + acc_at(row, lane * E, D);
         } else {
             const size_t row = (size_t)hk * a.summ_rows + sq.summ_off + (size_t)j * a.m + (t - a.k);
-            ak = a.dks + row * D; av = a.dvs + row * D;
+            ak = a.dks + acc_at(row, lane * E, D); av = a.dvs + acc_at(row, lane * E, D);
         }
 #pragma unroll
         for (int e = 0; e < E; e += 2) {
-            atomicAdd(reinterpret_cast<float2*>(ak + lane * E + e), make_float2(ds * qv[e], ds * qv[e + 1]));
-            atomicAdd(reinterpret_cast<float2*>(av + lane * E + e), make_float2(p * gv[e], p * gv[e + 1]));
+            atomicAdd(reinterpret_cast<float2*>(ak + e), make_float2(ds * qv[e], ds * qv[e + 1]));
+            atomicAdd(reinterpret_cast<float2*>(av + e), make_float2(p * gv[e], p * gv[e + 1]));
             dqv[e] = fmaf(ds, kf[e], dqv[e]); dqv[e + 1] = fmaf(ds, kf[e + 1], dqv[e + 1]);
         }
     }
@@ -502,25 +502,29 @@ __global__ void __launch_bounds__(256) ksa_bwd_finish_kernel(BwdArgs a, int tail
     const SeqInfo sq = a.seqs[blockIdx.y];
     const bool text = (blockIdx.z == 0);
     const int row_first = tails ? sq.n_chunks * a.k : 0;
-    const int vecs = a.D / 8;
+    // a warp takes four rows x 64 elements: 64 contiguous bytes of an accumulator, 128 of a row of dk / dv at a time
     const int live = (text ? sq.n_text : sq.n_summ) - row_first;
-    const int64_t per_row = (int64_t)a.Hkv * vecs;
-    const int64_t total = (int64_t)live * per_row;
-    const int s = a.k + a.m;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (int64_t)gridDim.x * blockDim.x) {
-        const int row_rel = (int)(idx / per_row), row = row_first + row_rel;
-        const int rem = (int)(idx - (int64_t)row_rel * per_row);
-        const int hk = rem / vecs, vv = rem - hk * vecs;
+    const int lane = threadIdx.x & 31, halves = a.D / 64;
+    const int per_group = a.Hkv * halves, s = a.k + a.m;
+    const int64_t units = (int64_t)((live + 3) / 4) * per_group;
+    for (int64_t u = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); u < units; u += (int64_t)gridDim.x * 8) {
+        const int group = (int)(u / per_group), rem = (int)(u - (int64_t)group * per_group);
+        const int hk = rem / halves, d = (rem - hk * halves) * 64 + (lane & 7) * 8;
+        const int row_rel = group * 4 + (lane >> 3), row = row_first + row_rel;
+        if (row_rel >= live) continue;
         const int64_t aug = text ? sq.aug_off + (int64_t)(row / a.k) * s + (row % a.k)
                                  : sq.aug_off + (int64_t)(row / a.m) * s + a.k + (row % a.m);
         const size_t srow = text ? ((size_t)hk * a.text_rows + sq.text_off + row) : ((size_t)hk * a.summ_rows + sq.summ_off + row);
-        const float* fk = (text ? a.dkt : a.dks) + srow * a.D + vv * 8;
-        const float* fv = (text ? a.dvt : a.dvs) + srow * a.D + vv * 8;
+        const size_t at = acc_at(srow, d, a.D);
+        const float* fk = (text ? a.dkt : a.dks) + at;
+        const float* fv = (text ? a.dvt : a.dvs) + at;
+        const float4 k0 = *reinterpret_cast<const float4*>(fk), k1 = *reinterpret_cast<const float4*>(fk + 512);
+        const float4 v0 = *reinterpret_cast<const float4*>(fv), v1 = *reinterpret_cast<const float4*>(fv + 512);
         uint4 ok, ov;
-        ok.x = b_pack2(fk[0], fk[1]); ok.y = b_pack2(fk[2], fk[3]); ok.z = b_pack2(fk[4], fk[5]); ok.w = b_pack2(fk[6], fk[7]);
-        ov.x = b_pack2(fv[0], fv[1]); ov.y = b_pack2(fv[2], fv[3]); ov.z = b_pack2(fv[4], fv[5]); ov.w = b_pack2(fv[6], fv[7]);
-        *reinterpret_cast<uint4*>(a.dk + aug * a.dk_st + (int64_t)hk * a.dk_sh + vv * 8) = ok;
-        *reinterpret_cast<uint4*>(a.dv + aug * a.dv_st + (int64_t)hk * a.dv_sh + vv * 8) = ov;
+        ok.x = b_pack2(k0.x, k0.y); ok.y = b_pack2(k0.z, k0.w); ok.z = b_pack2(k1.x, k1.y); ok.w = b_pack2(k1.z, k1.w);
+        ov.x = b_pack2(v0.x, v0.y); ov.y = b_pack2(v0.z, v0.w); ov.z = b_pack2(v1.x, v1.y); ov.w = b_pack2(v1.z, v1.w);
+        *reinterpret_cast<uint4*>(a.dk + aug * a.dk_st + (int64_t)hk * a.dk_sh + d) = ok;
+        *reinterpret_cast<uint4*>(a.dv + aug * a.dv_st + (int64_t)hk * a.dv_sh + d) = ov;
     }
 }
 
@@ -583,9 +587,9 @@ cudaError_t launch_bwd_dkv(const BwdArgs& a, cudaStream_t stream)
 
 cudaError_t launch_bwd_finish(const BwdArgs& a, bool tails, cudaStream_t stream)
 {
-    const int64_t per_row = (int64_t)a.Hkv * (a.D / 8);
+    const int64_t per_group = (int64_t)a.Hkv * (a.D / 64);               // warps per four rows
     const int64_t rows = tails ? a.k : a.max_text_pad > a.max_summ_pad ? a.max_text_pad : a.max_summ_pad;
-    int64_t blocks = (rows * per_row + 255) / 256;
+    int64_t blocks = ((rows + 3) / 4 * per_group + 7) / 8;
     if (blocks > 148 * 32) blocks = 148 * 32;
     if (blocks < 1) blocks = 1;
     dim3 grid((unsigned)blocks, (unsigned)a.num_seqs, a.m > 0 && !tails ? 2u : 1u);

@@ -24,11 +24,19 @@ struct BwdArgs {
     uint16_t* dot;              // [Hq][text_rows][D]
     float* lse_t;               // [Hq][text_rows], times log2(e); +inf on padding rows
     float* delta_t;             // [Hq][text_rows], <dO, O>
-    float* dkt; float* dvt;     // [Hkv][text_rows][D] fp32
-    float* dks; float* dvs;     // [Hkv][summ_rows][D] fp32
+    float* dkt; float* dvt;     // [Hkv][text_rows][D] fp32, elements as acc_at() places them
+    float* dks; float* dvs;     // [Hkv][summ_rows][D] fp32, likewise
     int32_t* status;            // device status word of the context (bounded waits report here)
     int32_t direct;             // tensor-core kernels read q, k, v, dout through chunked views: no packed copies
 };
+
+// Place of element d of a row in the accumulators: 128-row tiles (the streams' parts are whole tiles), in a tile four
+// elements of a row, then the next row, then the next four elements.  A warp of the tensor-core kernel holds 32 rows, one to a
+// lane: its 16-byte stores and atomics fill whole lines (row-major they touched 32 lines each, 8,192 line accesses a CTA).
+__host__ __device__ inline size_t acc_at(size_t row, int d, int D)
+{
+    return ((row >> 7) * (size_t)(D / 4) + (size_t)(d >> 2)) * 512 + (row & 127) * 4 + (size_t)(d & 3);
+}
 
 // Tensor maps for the tensor-core kernels (128-byte swizzle, boxes of 64 elements x 128 rows): Q and dO per query
 // head, K and V of the text and the summary rows per KV head -- of the packed streams, or (direct mode) chunked

@@ -257,10 +257,10 @@ __global__ void __launch_bounds__(128, KT_MAX <= 4 ? 4 : KT_MAX <= 6 ? 3 : 2) ks
             const int kc = kidx / s, key = kidx - kc * s;              // chunk within the block, key within the chunk
             if (key < a.k) {
                 const size_t row = (size_t)hk * a.text_rows + sq.text_off + (size_t)(j + kc) * a.k + key;
-                acc_k[half] = a.dkt + row * D; acc_v[half] = a.dvt + row * D;
+                acc_k[half] = a.dkt + acc_at(row, c2, D); acc_v[half] = a.dvt + acc_at(row, c2, D);
             } else {
                 const size_t row = (size_t)hk * a.summ_rows + sq.summ_off + (size_t)(j + kc) * a.m + (key - a.k);
-                acc_k[half] = a.dks + row * D; acc_v[half] = a.dvs + row * D;
+                acc_k[half] = a.dks + acc_at(row, c2, D); acc_v[half] = a.dvs + acc_at(row, c2, D);
             }
         }
 #pragma unroll
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(128, KT_MAX <= 4 ? 4 : KT_MAX <= 6 ? 3 : 2) ks
                 for (int i = 0; i < 8; ++i)
 #pragma unroll
                     for (int half = 0; half < 2; ++half)
-                        sum[i][half] = *reinterpret_cast<const float2*>((which ? acc_k[half] : acc_v[half]) + (i0 + i) * 8 + c2);
+                        sum[i][half] = *reinterpret_cast<const float2*>((which ? acc_k[half] : acc_v[half]) + (i0 + i) * 1024);
                 float o[8][4];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }

@@ -40,7 +40,10 @@
 // What bounds them: the row warps.  Two sequences of 32,768 tokens, 32/8 heads: a 128 x 128 tile takes 3,000 cycles
 // in the dK / dV kernel and 1,950 in the dQ kernel (2,600 before: issuing thread in a divergent region, releasing
 // arrivals, scalar fp32), 1,024 of them exponentials on the special-function unit; the issuer waits for the
-// row warps 1,400 / 670 of them.  Whole backward call 12.5 -> 11.4 ms.
+// row warps 1,400 / 670 of them.  Whole backward call 12.5 -> 11.4 ms.  A CTA's start and end cost the dQ kernel some 10,000
+// cycles (16 tiles at 16,384 tokens): 1,600 until the next CTA is there, 4,600 until the first products are under way (the
+// producer's loads start beside the rest of the set-up), 3,800 for the last product and the epilogue, whose stores take
+// four lanes a row (dQ 732 -> 723 us) or go to accumulators laid out for them (dK / dV of the text keys 575 -> 539 us).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -136,25 +139,29 @@ __device__ __forceinline__ bool bt_layout(BtSmem<D>& sm, const uint8_t* raw, int
     return true;
 }
 
+// The barriers, by the producer's thread, which goes on to its first loads at once: they run beside the rest of the
+// set-up (TMEM, the row warps' scalars).  bt_ready() is where everybody meets.
 template <int D>
-__device__ __forceinline__ void bt_init(const BtSmem<D>& sm, int tid, int warp)
+__device__ __forceinline__ void bt_init_barriers(const BtSmem<D>& sm)
 {
-    if (tid == 0) {
-        mbar_init(sm.bar(BB_AFULL), 1);
-        for (int s = 0; s < kB1Stages; ++s) { mbar_init(sm.bar(BB_B1FULL + s), 1); mbar_init(sm.bar(BB_B1EMPTY + s), 1); }
-        for (int s = 0; s < kB2Stages; ++s) { mbar_init(sm.bar(BB_B2FULL + s), 1); mbar_init(sm.bar(BB_B2EMPTY + s), 1); }
-        mbar_init(sm.bar(BB_XFULL), 1);
-        mbar_init(sm.bar(BB_YFULL), 1);
-        mbar_init(sm.bar(BB_YFULL2), 1);
-        mbar_init(sm.bar(BB_PA), 16);
-        mbar_init(sm.bar(BB_PB), 16);
-        mbar_init(sm.bar(BB_PB2), 16);
-        mbar_init(sm.bar(BB_OFULL), 1);
-        bt_st_shared(sm.abort_addr(), 0u);
-        bt_st_shared(sm.abort_addr() + 4, 0u);
-        fence_mbar_init();
-    }
-    if (warp == 16) { tmem_alloc(sm.tmem_slot(), 512); tmem_relinquish(); }
+    mbar_init(sm.bar(BB_AFULL), 1);
+    for (int s = 0; s < kB1Stages; ++s) { mbar_init(sm.bar(BB_B1FULL + s), 1); mbar_init(sm.bar(BB_B1EMPTY + s), 1); }
+    for (int s = 0; s < kB2Stages; ++s) { mbar_init(sm.bar(BB_B2FULL + s), 1); mbar_init(sm.bar(BB_B2EMPTY + s), 1); }
+    mbar_init(sm.bar(BB_XFULL), 1);
+    mbar_init(sm.bar(BB_YFULL), 1);
+    mbar_init(sm.bar(BB_YFULL2), 1);
+    mbar_init(sm.bar(BB_PA), 16);
+    mbar_init(sm.bar(BB_PB), 16);
+    mbar_init(sm.bar(BB_PB2), 16);
+    mbar_init(sm.bar(BB_OFULL), 1);
+    bt_st_shared(sm.abort_addr(), 0u);
+    bt_st_shared(sm.abort_addr() + 4, 0u);
+    fence_mbar_init();
+}
+template <int D>
+__device__ __forceinline__ void bt_ready(const BtSmem<D>& sm, int warp)
+{
+    if (warp == 17) { tmem_alloc(sm.tmem_slot(), 512); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -253,7 +260,7 @@ __global__ void __maxnreg__(kBwdTcRegs)
 ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ BwdMaps maps, const int summ, const int seg_tiles, const int store)
 {
     extern __shared__ uint8_t bsm_raw[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     // ---- which keys, which queries (Eq. 3) ------------------------------------------------------
     const int G = a.Hq / a.Hkv;
@@ -298,38 +305,48 @@ ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__
         n_lse = -a.lse_t[r];                                              // -inf on padding rows: P = 0 there
         n_dl = -a.delta_t[r];
     };
+    // loads of streamed tile j (the producer's thread)
+    const bool direct = a.direct != 0;
+    auto load_b1 = [&](int j) {
+        int qt, h;
+        pair_of(j, qt, h);
+        bt_load_tile<D>(sm.b1(j % kB1Stages), sm.bar(BB_B1FULL + j % kB1Stages), &maps.qt,
+                        direct ? sq.chunk0 + qt * (128 / a.k) : sq.text_off + qt * 128, h, direct);
+    };
+    auto load_b2 = [&](int j) {
+        int qt, h;
+        pair_of(j, qt, h);
+        bt_load_tile<D>(sm.b2(j & 1), sm.bar(BB_B2FULL + (j & 1)), &maps.dot,
+                        direct ? sq.chunk0 + qt * (128 / a.k) : sq.text_off + qt * 128, h, direct);
+    };
+    if (warp == 16 && lane == 0) {
+        bt_init_barriers(sm);
+        mbar_arrive_expect_tx(sm.bar(BB_AFULL), 2u * BtMap<D>::kTile);
+        const int kpos = direct ? sq.chunk0 + kt * (128 / (summ ? a.m : a.k)) : krow0;
+        bt_issue_tile<D>(sm.a1(), sm.bar(BB_AFULL), summ ? &maps.ks : &maps.kt, kpos, hk, direct);
+        load_b1(0);
+        bt_issue_tile<D>(sm.a2(), sm.bar(BB_AFULL), summ ? &maps.vs : &maps.vt, kpos, hk, direct);
+        load_b2(0);
+    }
     if (scalar_writer) {                                                  // tile 0: visible to all after the first barrier
         fetch(seg0, 0);
         rows[32 * cg + lane] = n_lse;
         rows[128 + 32 * cg + lane] = n_dl;
     }
-    bt_init(sm, tid, warp);
+    bt_ready(sm, warp);
     const uint32_t tmem = bt_ld_shared(sm.tmem_slot());
     const uint32_t tX = tmem, tY = tmem + 128u, tDV = tmem + 256u, tDK = tmem + 384u;
 
     if (warp == 16) {
         // =============================== TMA producer ===============================
         if (lane == 0) {
-            prefetch_tensormap(&maps.qt); prefetch_tensormap(&maps.dot);
-            const bool direct = a.direct != 0;
-            const int q_step = direct ? 128 / a.k : 128, q_base = direct ? sq.chunk0 : sq.text_off;   // position of a query tile
-            mbar_arrive_expect_tx(sm.bar(BB_AFULL), 2u * BtMap<D>::kTile);
-            {
-                const int kpos = direct ? sq.chunk0 + kt * (128 / (summ ? a.m : a.k)) : krow0;
-                bt_issue_tile<D>(sm.a1(), sm.bar(BB_AFULL), summ ? &maps.ks : &maps.kt, kpos, hk, direct);
-                bt_issue_tile<D>(sm.a2(), sm.bar(BB_AFULL), summ ? &maps.vs : &maps.vt, kpos, hk, direct);
-            }
-            int filled1 = 0, filled2 = 0;
-            bool ok = true;
-            for (int j = 0; j < J && ok; ++j) {
-                int qt, h;
-                pair_of(j, qt, h);
-                const int pos = q_base + qt * q_step;
-                if (!(ok = bt_stage_free(sm, BB_B1EMPTY, kB1Stages, j, a.status))) break;
-                bt_load_tile<D>(sm.b1(j % kB1Stages), sm.bar(BB_B1FULL + j % kB1Stages), &maps.qt, pos, h, direct);
+            int filled1 = 1, filled2 = 1;                                 // tile 0 is on its way
+            for (int j = 1; j < J; ++j) {
+                if (!bt_stage_free(sm, BB_B1EMPTY, kB1Stages, j, a.status)) break;
+                load_b1(j);
                 ++filled1;
-                if (!(ok = bt_stage_free(sm, BB_B2EMPTY, kB2Stages, j, a.status))) break;
-                bt_load_tile<D>(sm.b2(j & 1), sm.bar(BB_B2FULL + (j & 1)), &maps.dot, pos, h, direct);
+                if (!bt_stage_free(sm, BB_B2EMPTY, kB2Stages, j, a.status)) break;
+                load_b2(j);
                 ++filled2;
             }
             if (bt_ld_shared(sm.abort_addr()) != 0u) bt_drain(sm, filled1, filled2, a.status);
@@ -504,7 +521,7 @@ ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__
             const bool is_dk = (cg & 1) != 0;
             const int d0 = (cg >> 1) * (D / 2);
             const size_t arow = (size_t)hk * (summ ? a.summ_rows : a.text_rows) + (size_t)krow0 + quarter * 32 + lane;
-            float* acc = (is_dk ? (summ ? a.dks : a.dkt) : (summ ? a.dvs : a.dvt)) + arow * D + d0;
+            float* acc = (is_dk ? (summ ? a.dks : a.dkt) : (summ ? a.dvs : a.dvt)) + acc_at(arow, d0, D);
             const float mul = is_dk ? a.scale : 1.f;
             const uint32_t tacc = (is_dk ? tDK : tDV) + lane_sel + d0;
 #pragma unroll
@@ -518,8 +535,9 @@ ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__
                     for (int e = 0; e < 32; e += 4) {
                         const float4 val = make_float4(__uint_as_float(o[e]) * mul, __uint_as_float(o[e + 1]) * mul,
                                                        __uint_as_float(o[e + 2]) * mul, __uint_as_float(o[e + 3]) * mul);
-                        if (store) *reinterpret_cast<float4*>(acc + c * 32 + e) = val;
-                        else atomicAdd(reinterpret_cast<float4*>(acc + c * 32 + e), val);
+                        float4* at = reinterpret_cast<float4*>(acc + (c * 32 + e) / 4 * 512);        // (acc_at)
+                        if (store) *at = val;
+                        else atomicAdd(at, val);
                     }
                 }
             }
@@ -527,7 +545,7 @@ ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 16) tmem_dealloc(tmem, 512);
+    if (warp == 17) tmem_dealloc(tmem, 512);
 }
 
 // =====================================================================================================
@@ -538,7 +556,7 @@ __global__ void __maxnreg__(kBwdTcRegs)
 ksa_bwd_dq_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ BwdMaps maps)
 {
     extern __shared__ uint8_t bsm_raw[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     // ---- which queries, which keys (Eq. 3) ------------------------------------------------------
     const int h = blockIdx.y, hk = h / (a.Hq / a.Hkv);
@@ -559,7 +577,27 @@ ksa_bwd_dq_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ 
 
     BtSmem<D> sm;
     if (!bt_layout(sm, bsm_raw, a.status)) return;
-    bt_init(sm, tid, warp);
+    // loads of streamed tile j (the producer's thread): key0 / 128 tiles into its stream, rows of the packed stream or
+    // chunks of the caller's tensor
+    const bool direct = a.direct != 0;
+    auto load_kv = [&](int j, uint32_t dst, uint32_t bar, const CUtensorMap* map_s, const CUtensorMap* map_t) {
+        bool is_summ; int key0;
+        tile_of(j, is_summ, key0);
+        bt_load_tile<D>(dst, bar, is_summ ? map_s : map_t,
+                        direct ? sq.chunk0 + (key0 >> 7) * (128 / (is_summ ? a.m : a.k)) : (is_summ ? sq.summ_off : sq.text_off) + key0, hk, direct);
+    };
+    auto load_b1 = [&](int j) { load_kv(j, sm.b1(j % kB1Stages), sm.bar(BB_B1FULL + j % kB1Stages), &maps.ks, &maps.kt); };
+    auto load_b2 = [&](int j) { load_kv(j, sm.b2(j & 1), sm.bar(BB_B2FULL + (j & 1)), &maps.vs, &maps.vt); };
+    if (warp == 16 && lane == 0) {
+        bt_init_barriers(sm);
+        mbar_arrive_expect_tx(sm.bar(BB_AFULL), 2u * BtMap<D>::kTile);
+        const int qpos = direct ? sq.chunk0 + qt * (128 / a.k) : sq.text_off + qt * 128;
+        bt_issue_tile<D>(sm.a1(), sm.bar(BB_AFULL), &maps.qt, qpos, h, direct);
+        load_b1(0);
+        bt_issue_tile<D>(sm.a2(), sm.bar(BB_AFULL), &maps.dot, qpos, h, direct);
+        load_b2(0);
+    }
+    bt_ready(sm, warp);
     const uint32_t tmem = bt_ld_shared(sm.tmem_slot());
     const uint32_t tX = tmem, tDQ = tmem + 256u;
     auto tY = [&](int j) -> uint32_t { return tmem + ((j & 1) ? 384u : 128u); };   // dP of tile j, then dS in place
@@ -571,27 +609,13 @@ ksa_bwd_dq_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ 
     if (warp == 16) {
         // =============================== TMA producer ===============================
         if (lane == 0) {
-            prefetch_tensormap(&maps.kt); prefetch_tensormap(&maps.vt);
-            const bool direct = a.direct != 0;
-            mbar_arrive_expect_tx(sm.bar(BB_AFULL), 2u * BtMap<D>::kTile);
-            {
-                const int qpos = direct ? sq.chunk0 + qt * (128 / a.k) : sq.text_off + qt * 128;
-                bt_issue_tile<D>(sm.a1(), sm.bar(BB_AFULL), &maps.qt, qpos, h, direct);
-                bt_issue_tile<D>(sm.a2(), sm.bar(BB_AFULL), &maps.dot, qpos, h, direct);
-            }
-            int filled1 = 0, filled2 = 0;
-            bool ok = true;
-            for (int j = 0; j < J && ok; ++j) {
-                bool is_summ; int key0;
-                tile_of(j, is_summ, key0);
-                // key0 / 128 tiles into its stream: rows of the packed stream, or chunks of the caller's tensor
-                const int pos = direct ? sq.chunk0 + (key0 >> 7) * (128 / (is_summ ? a.m : a.k))
-                                       : (is_summ ? sq.summ_off : sq.text_off) + key0;
-                if (!(ok = bt_stage_free(sm, BB_B1EMPTY, kB1Stages, j, a.status))) break;
-                bt_load_tile<D>(sm.b1(j % kB1Stages), sm.bar(BB_B1FULL + j % kB1Stages), is_summ ? &maps.ks : &maps.kt, pos, hk, direct);
+            int filled1 = 1, filled2 = 1;                                 // tile 0 is on its way
+            for (int j = 1; j < J; ++j) {
+                if (!bt_stage_free(sm, BB_B1EMPTY, kB1Stages, j, a.status)) break;
+                load_b1(j);
                 ++filled1;
-                if (!(ok = bt_stage_free(sm, BB_B2EMPTY, kB2Stages, j, a.status))) break;
-                bt_load_tile<D>(sm.b2(j & 1), sm.bar(BB_B2FULL + (j & 1)), is_summ ? &maps.vs : &maps.vt, pos, hk, direct);
+                if (!bt_stage_free(sm, BB_B2EMPTY, kB2Stages, j, a.status)) break;
+                load_b2(j);
                 ++filled2;
             }
             if (bt_ld_shared(sm.abort_addr()) != 0u) bt_drain(sm, filled1, filled2, a.status);
@@ -738,29 +762,33 @@ ksa_bwd_dq_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ 
         if (alive && bt_wait_warp(sm.bar(BB_OFULL), 0, sm.abort_addr(), a.status, kStatusWaitOFull, lane)) {
             tc_fence_after();
             // scale * dQ as bf16 to the row's augmented position (Eq. 1); warp group cg writes elements 32 cg ..
-            const int64_t aug = sq.aug_off + (int64_t)iq * (a.k + a.m) + (i - iq * a.k);
-            uint16_t* dst = a.dq + aug * a.dq_st + (int64_t)h * a.dq_sh + cg * 32;
-            uint32_t o[32];
             if (cg * 32 < D) {                                            // warp-uniform: the row has D elements
+                int64_t off = -1;                                         // -1: a padding row
+                if (i < sq.n_text)
+                    off = (sq.aug_off + (int64_t)iq * (a.k + a.m) + (i - iq * a.k)) * a.dq_st + (int64_t)h * a.dq_sh + cg * 32;
+                uint32_t o[32];
                 tmem_ld32(tDQ + lane_sel + cg * 32, o);
                 tc_wait_ld();
-            }
-            if (cg * 32 < D && i < sq.n_text) {
+                uint4 w[4];
 #pragma unroll
-                for (int e = 0; e < 32; e += 8) {
-                    uint4 w;
-                    w.x = pack_bf16x2(__uint_as_float(o[e]) * a.scale, __uint_as_float(o[e + 1]) * a.scale);
-                    w.y = pack_bf16x2(__uint_as_float(o[e + 2]) * a.scale, __uint_as_float(o[e + 3]) * a.scale);
-                    w.z = pack_bf16x2(__uint_as_float(o[e + 4]) * a.scale, __uint_as_float(o[e + 5]) * a.scale);
-                    w.w = pack_bf16x2(__uint_as_float(o[e + 6]) * a.scale, __uint_as_float(o[e + 7]) * a.scale);
-                    *reinterpret_cast<uint4*>(dst + e) = w;
+                for (int e = 0; e < 4; ++e) {
+                    w[e].x = pack_bf16x2(__uint_as_float(o[8 * e]) * a.scale, __uint_as_float(o[8 * e + 1]) * a.scale);
+                    w[e].y = pack_bf16x2(__uint_as_float(o[8 * e + 2]) * a.scale, __uint_as_float(o[8 * e + 3]) * a.scale);
+                    w[e].z = pack_bf16x2(__uint_as_float(o[8 * e + 4]) * a.scale, __uint_as_float(o[8 * e + 5]) * a.scale);
+                    w[e].w = pack_bf16x2(__uint_as_float(o[8 * e + 6]) * a.scale, __uint_as_float(o[8 * e + 7]) * a.scale);
+                }
+                quad_transpose(w, lane);                                  // w[j]: 16 bytes of the group's row j
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int64_t at = __shfl_sync(0xffffffffu, off, (lane & 28) + j);
+                    if (at >= 0) *reinterpret_cast<uint4*>(a.dq + at + (lane & 3) * 8) = w[j];
                 }
             }
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 16) tmem_dealloc(tmem, 512);
+    if (warp == 17) tmem_dealloc(tmem, 512);
 }
 
 cudaError_t setup_bwd_tc()

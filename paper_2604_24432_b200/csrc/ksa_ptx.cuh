@@ -404,5 +404,25 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
     return r;
 }
 
+// 4 x 4 transposition of 16-byte vectors in every group of four lanes: lane l of the group comes with v[j] of its own and
+// leaves with v[j] = what lane j's v[l] was.  Rows that stand one to a lane leave as 64 contiguous bytes per four lanes: a
+// store of 16 bytes a lane then touches 8 lines instead of 32 (the store path takes a line per cycle).
+__device__ __forceinline__ void quad_transpose(uint4 (&v)[4], int lane)
+{
+#pragma unroll
+    for (int s = 1; s <= 2; s <<= 1) {
+        const bool up = (lane & s) != 0;
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            uint4& lo = v[s == 1 ? 2 * p : p];
+            uint4& hi = v[s == 1 ? 2 * p + 1 : p + 2];
+            uint4 x = up ? lo : hi;
+            x.x = __shfl_xor_sync(0xffffffffu, x.x, s); x.y = __shfl_xor_sync(0xffffffffu, x.y, s);
+            x.z = __shfl_xor_sync(0xffffffffu, x.z, s); x.w = __shfl_xor_sync(0xffffffffu, x.w, s);
+            if (up) lo = x; else hi = x;
+        }
+    }
+}
+
 }  // namespace ptx
 }  // namespace ksa

@@ -471,23 +471,28 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
             const float inv_l = 1.f / l_run;
             const int h = w.head0 + t;
             const int64_t aug = sq.aug_off + (int64_t)(i / a.k) * s_len + (i % a.k);
-            uint16_t* orow = a.out + aug * a.o_st + (int64_t)h * a.o_sh;
             const bool store = valid && ksa_out_row_ok(a, aug, h);
+            // a row stands in one lane: four lanes exchange 64 bytes of their rows, so that a store touches 8 lines, not 32
+            // (the epilogues took 246 of 3,207 cycles a key tile at 32,768 tokens: the store path takes a line per cycle)
+            const int64_t off = store ? aug * a.o_st + (int64_t)h * a.o_sh : -1;
 #pragma unroll
             for (int c = 0; c < D / 32; ++c) {
                 uint32_t o[32];
                 tmem_ld32(tO + c * 32, o);
                 tc_wait_ld();
-                if (store) {
+                uint4 pk[4];
 #pragma unroll
-                    for (int e = 0; e < 32; e += 8) {
-                        uint4 pk;
-                        pk.x = pack_bf16x2(__uint_as_float(o[e]) * inv_l, __uint_as_float(o[e + 1]) * inv_l);
-                        pk.y = pack_bf16x2(__uint_as_float(o[e + 2]) * inv_l, __uint_as_float(o[e + 3]) * inv_l);
-                        pk.z = pack_bf16x2(__uint_as_float(o[e + 4]) * inv_l, __uint_as_float(o[e + 5]) * inv_l);
-                        pk.w = pack_bf16x2(__uint_as_float(o[e + 6]) * inv_l, __uint_as_float(o[e + 7]) * inv_l);
-                        *reinterpret_cast<uint4*>(orow + c * 32 + e) = pk;
-                    }
+                for (int e = 0; e < 4; ++e) {
+                    pk[e].x = pack_bf16x2(__uint_as_float(o[8 * e]) * inv_l, __uint_as_float(o[8 * e + 1]) * inv_l);
+                    pk[e].y = pack_bf16x2(__uint_as_float(o[8 * e + 2]) * inv_l, __uint_as_float(o[8 * e + 3]) * inv_l);
+                    pk[e].z = pack_bf16x2(__uint_as_float(o[8 * e + 4]) * inv_l, __uint_as_float(o[8 * e + 5]) * inv_l);
+                    pk[e].w = pack_bf16x2(__uint_as_float(o[8 * e + 6]) * inv_l, __uint_as_float(o[8 * e + 7]) * inv_l);
+                }
+                quad_transpose(pk, lane);                             // pk[e]: 16 bytes of the group's row e
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int64_t at = __shfl_sync(0xffffffffu, off, (lane & 28) + e);
+                    if (at >= 0) *reinterpret_cast<uint4*>(a.out + at + c * 32 + (lane & 3) * 8) = pk[e];
                 }
             }
             if (store) a.lse[(int64_t)h * a.total_aug + aug] = (m_used + log2f(l_run)) * 0.6931471805599453f;
