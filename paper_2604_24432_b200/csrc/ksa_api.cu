@@ -1015,8 +1015,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_bwd(ksa_ctx* ctx,
             for (auto& t : streams)
                 if ((rc = encode_stream_map(ctx, t.map, const_cast<void*>(t.base), a.D, t.rows, t.H)) != KSA_OK) return rc;
         }
-        if ((e = launch_bwd_dq_tc(a, bm, stream)) != cudaSuccess) return cuda_fail(ctx, e);
-        if ((e = launch_bwd_dkv_tc(a, bm, stream)) != cudaSuccess) return cuda_fail(ctx, e);
+        if ((e = launch_bwd_tc(a, bm, stream)) != cudaSuccess) return cuda_fail(ctx, e);
     } else {
         if ((e = launch_bwd_dq(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);
         if ((e = launch_bwd_dkv(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);

@@ -49,6 +49,7 @@
 #include <algorithm>
 
 #include "ksa_bwd.h"
+#include "ksa_launch.h"
 #include "ksa_ptx.cuh"
 
 namespace ksa {
@@ -256,8 +257,7 @@ __device__ __forceinline__ bool bt_stage_free(const BtSmem<D>& sm, int empty0, i
 // dK / dV
 // =====================================================================================================
 template <int D>
-__global__ void __maxnreg__(kBwdTcRegs)
-ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ BwdMaps maps, const int summ, const int seg_tiles, const int store)
+__device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& maps, const int summ, const int seg_tiles, const int store)
 {
     extern __shared__ uint8_t bsm_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -552,8 +552,7 @@ ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__
 // dQ
 // =====================================================================================================
 template <int D>
-__global__ void __maxnreg__(kBwdTcRegs)
-ksa_bwd_dq_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ BwdMaps maps)
+__device__ __forceinline__ void bt_dq_block(const BwdArgs& a, const BwdMaps& maps)
 {
     extern __shared__ uint8_t bsm_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -791,6 +790,32 @@ ksa_bwd_dq_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ 
     if (warp == 17) tmem_dealloc(tmem, 512);
 }
 
+// The three launches -- dK / dV of the summary keys, of the text keys, dQ -- do not depend on each other: each one's CTAs take
+// the SMs that the one in front leaves (programmatic dependent launches), longest CTAs first (64, about 40 and 9 + 16 tiles
+// each at 32,768 tokens), so that the tails of the first two are filled (training layer of 7,942 ragged tokens, 16/16 heads
+// 610 -> 573 us, 2 x 8,192 tokens 2,140 -> 2,070 us; nothing at 2 x 32,768).
+// Nothing here waits for the launch in front, which was itself started behind the preparation; only the last block of each
+// waits for its end, so that the kernel behind the three, an ordinary launch, finds all of them done.
+__device__ __forceinline__ void bt_end_behind_front()
+{
+    if (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1) pdl_wait();
+}
+template <int D>
+__global__ void __maxnreg__(kBwdTcRegs)
+ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ BwdMaps maps, const int summ, const int seg_tiles, const int store)
+{
+    pdl_launch_dependents();
+    bt_dkv_block<D>(a, maps, summ, seg_tiles, store);
+    bt_end_behind_front();
+}
+template <int D>
+__global__ void __maxnreg__(kBwdTcRegs)
+ksa_bwd_dq_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ BwdMaps maps)
+{
+    bt_dq_block<D>(a, maps);
+    bt_end_behind_front();
+}
+
 cudaError_t setup_bwd_tc()
 {
     cudaError_t e = cudaFuncSetAttribute(ksa_bwd_dkv_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, BtMap<128>::kSmem);
@@ -798,14 +823,6 @@ cudaError_t setup_bwd_tc()
     if ((e = cudaFuncSetAttribute(ksa_bwd_dq_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, BtMap<128>::kSmem)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(ksa_bwd_dkv_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, BtMap<64>::kSmem)) != cudaSuccess) return e;
     return cudaFuncSetAttribute(ksa_bwd_dq_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, BtMap<64>::kSmem);
-}
-
-cudaError_t launch_bwd_dq_tc(const BwdArgs& a, const BwdMaps& maps, cudaStream_t stream)
-{
-    dim3 grid((unsigned)(a.max_text_pad / 128), (unsigned)a.Hq, (unsigned)a.num_seqs);
-    if (a.D == 128) ksa_bwd_dq_tc_kernel<128><<<grid, kBwdTcThreads, BtMap<128>::kSmem, stream>>>(a, maps);
-    else            ksa_bwd_dq_tc_kernel<64><<<grid, kBwdTcThreads, BtMap<64>::kSmem, stream>>>(a, maps);
-    return cudaGetLastError();
 }
 
 // Query tiles that see a text key tile (an upper bound), and the query tiles a CTA of the dK / dV kernel walks.
@@ -819,25 +836,33 @@ static int bwd_seg_tiles(const BwdArgs& a) { return std::max(16, kBwdSegPairs / 
 // accumulators with plain stores -- it must be their first writer (no clear needed; the summary rows' kernel adds later).
 bool bwd_text_keys_stored(const BwdArgs& a) { return bwd_text_span(a) <= bwd_seg_tiles(a); }
 
-cudaError_t launch_bwd_dkv_tc(const BwdArgs& a, const BwdMaps& maps, cudaStream_t stream)
+cudaError_t launch_bwd_tc(const BwdArgs& a, const BwdMaps& maps, cudaStream_t stream)
 {
     const int n_qt = a.max_text_pad / 128;
-    const long long text_span = bwd_text_span(a);
-    for (int summ = 0; summ < 2; ++summ) {
+    const size_t smem = a.D == 128 ? BtMap<128>::kSmem : BtMap<64>::kSmem;
+    bool first = true;                                                    // behind the preparation: an ordinary launch
+    for (int summ = 1; summ >= 0; --summ) {
         if (summ && (a.m <= 0 || a.max_n_summ <= 0)) continue;
-        const long long span = summ ? n_qt : text_span;
+        const long long span = summ ? n_qt : bwd_text_span(a);
         const int tiles = summ ? (a.max_n_summ + 127) / 128 : n_qt;
         // a CTA walks seg query tiles x G heads: 16 tiles with four or more heads per KV head, more with fewer (the
         // start-up and the final atomics of a CTA are spread over about 64 streamed tiles either way)
         const int seg = bwd_seg_tiles(a);
         const int store = (!summ && bwd_text_keys_stored(a)) ? 1 : 0;
-        dim3 grid((unsigned)((span + seg - 1) / seg), (unsigned)tiles, (unsigned)(a.num_seqs * a.Hkv));
-        if (a.D == 128) ksa_bwd_dkv_tc_kernel<128><<<grid, kBwdTcThreads, BtMap<128>::kSmem, stream>>>(a, maps, summ, seg, store);
-        else            ksa_bwd_dkv_tc_kernel<64><<<grid, kBwdTcThreads, BtMap<64>::kSmem, stream>>>(a, maps, summ, seg, store);
-        cudaError_t e = cudaGetLastError();
+        const dim3 grid((unsigned)((span + seg - 1) / seg), (unsigned)tiles, (unsigned)(a.num_seqs * a.Hkv));
+        auto* kernel = a.D == 128 ? ksa_bwd_dkv_tc_kernel<128> : ksa_bwd_dkv_tc_kernel<64>;
+        cudaError_t e;
+        if (first) {
+            kernel<<<grid, kBwdTcThreads, smem, stream>>>(a, maps, summ, seg, store);
+            e = cudaGetLastError();
+        } else {
+            e = launch_dependent(kernel, grid, kBwdTcThreads, smem, stream, a, maps, summ, seg, store);
+        }
         if (e != cudaSuccess) return e;
+        first = false;
     }
-    return cudaSuccess;
+    return launch_dependent(a.D == 128 ? ksa_bwd_dq_tc_kernel<128> : ksa_bwd_dq_tc_kernel<64>,
+                            dim3((unsigned)n_qt, (unsigned)a.Hq, (unsigned)a.num_seqs), kBwdTcThreads, smem, stream, a, maps);
 }
 
 }  // namespace ksa

@@ -270,3 +270,44 @@ def test_full_causal_mode_against_torch_attention(ctx):
         err = (mine.float().transpose(0, 1) - theirs).abs()
         assert err.max().item() <= 2e-2 * theirs.abs().max().item() + 1e-5, name
         assert err.mean().item() <= 1e-2 * theirs.abs().mean().item() + 1e-5, name
+
+
+@pytest.mark.parametrize("lens,k,m,C,Hq,Hkv,D", [
+    ([900, 77], 8, 1, 4, 4, 4, 128),               # all three launches, rows behind the last whole chunk
+    ([1280], 16, 0, 7, 4, 2, 64),                  # no summaries: two launches, the finish kernel over all rows
+    ([2100], 120, 16, 3, 16, 2, 128),              # summary rows beyond the tile kernel's limits: CUDA-core kernel
+])
+def test_work_behind_a_backward_call_finds_all_gradients(ctx, lens, k, m, C, Hq, Hkv, D):
+    """The kernels of a call overlap: what is enqueued behind it (a copy of the gradients, call after call on the same
+    buffers, overwritten in between) must see all of them.  dq has the bits of the call on its own; dk, dv are sums of
+    fp32 atomics in any order, rounded to bf16: equal to within one rounding of the largest element."""
+    dev = torch.device("cuda", 0)
+    prob = ksa.Problem(lens, k, m, C, Hq, Hkv, D, float(D) ** -0.5)
+    total = ksa.total_aug_len(prob)
+    ws = torch.empty(max(256, ksa.workspace_bytes(prob)), dtype=torch.uint8, device=dev)
+    wsb = torch.full((ksa.bwd_workspace_bytes(prob),), 0xFF, dtype=torch.uint8, device=dev)
+    sets = []
+    for i in range(2):
+        g = torch.Generator("cuda").manual_seed(i)
+        q, kk, v, go = (torch.randn((total, h, D), generator=g, device=dev).to(torch.bfloat16) for h in (Hq, Hkv, Hkv, Hq))
+        out = torch.empty_like(q); lse = torch.empty((Hq, total), device=dev)
+        ctx.attn_fwd(prob, q, kk, v, out, lse, ws)
+        sets.append((q, kk, v, out, lse, go))
+    dq, dk, dv = torch.empty_like(q), torch.empty_like(kk), torch.empty_like(v)
+    want, got = [], []
+    for s in sets:
+        ctx.attn_bwd(prob, *s, dq, dk, dv, wsb)
+        torch.cuda.synchronize()
+        want.append([t.clone() for t in (dq, dk, dv)])
+    for rep in range(12):
+        for t in (dq, dk, dv):
+            t.fill_(7.0)
+        ctx.attn_bwd(prob, *sets[rep % 2], dq, dk, dv, wsb)
+        got.append([t.clone() for t in (dq, dk, dv)])
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    for rep, (a, b, c) in enumerate(got):
+        wq, wk, wv = want[rep % 2]
+        assert torch.equal(a.view(torch.int16), wq.view(torch.int16)), rep
+        for x, w in ((b, wk), (c, wv)):
+            assert (x.float() - w.float()).abs().max().item() <= 2.0 ** -7 * w.float().abs().max().item(), rep
