@@ -14,11 +14,14 @@
 // A chunk's k + m rows of a KV head belong to one block, so this kernel is also the last step of the backward pass for
 // them: it runs after the text rows' kernels, adds its dV and dK to the fp32 sums these left in the key streams' accumulators
 // (asked for before the products, so that they arrive beside them) and writes the bf16 gradients.  Only the rows behind a
-// sequence's last whole chunk are left to the finish kernel.  Two sequences of 32,768 tokens, 32/8 heads, k = 8: the
-// kernel with one vector atomic per element and the finish pass over all rows took 787 + 160 us, now 468 us (64 + 8 layout at
-// 2 x 8,192: 152 + 46 -> 139 us; 16/16 heads, 7,942 ragged tokens: 113 + 47 -> 86 + 4 us).  What bounds
-// it is the latency of a block (loads, one warp per 16 query rows, then keys); its HBM traffic, 1.4 GB, would take 213 us.  Short
-// blocks (up to 64 keys) have an instance with half the score registers, which lets four instead of two of them share an SM.
+// sequence's last whole chunk are left to the finish kernel.
+//
+// Instances: by key tiles (fewer score registers, more blocks an SM), and for blocks of one query tile and at most 64 keys one
+// whose phase 1 gives each warp a key tile and, for dQ, a quarter of the head, instead of everything to one warp (a row's
+// delta is then the sum of the key tiles' shares in a fixed order).  Two sequences of 32,768 tokens, 32/8 heads, k = 8: 787 us
+// with one vector atomic per element + 160 us for a finish pass over all rows, 476 us as one kernel, 356 us with the one-tile
+// instance; 16/16 heads, 7,942 ragged tokens: 113 + 47, 98 + 4, 85 + 4 us; 64 + 8 layout at 2 x 8,192: 152 + 46 -> 139 us.
+// What bounds it is the latency of a block's steps; its HBM traffic, 1.4 GB in the first case, would take 213 us.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -70,8 +73,8 @@ __device__ __forceinline__ uint32_t bs_sw(uint32_t base, int row, int chunk)
     return base + (uint32_t)row * (uint32_t)(D * 2) + (uint32_t)(((chunk ^ (row & 7)) & (D / 8 - 1)) << 4);
 }
 
-template <int D, int KT_MAX>
-__global__ void __launch_bounds__(128, KT_MAX <= 4 ? 4 : KT_MAX <= 6 ? 3 : 2) ksa_bwd_summary_mma_kernel(BwdArgs a, int s_pad, int m_pad, int cpb)
+template <int D, int KT_MAX, bool kOneTile>
+__global__ void __launch_bounds__(128, kOneTile ? 5 : KT_MAX <= 4 ? 4 : KT_MAX <= 6 ? 3 : 2) ksa_bwd_summary_mma_kernel(BwdArgs a, int s_pad, int m_pad, int cpb)
 {
     constexpr int CH = D / 8;
     extern __shared__ __align__(128) uint16_t bs_smem[];
@@ -129,6 +132,116 @@ __global__ void __launch_bounds__(128, KT_MAX <= 4 ? 4 : KT_MAX <= 6 ? 3 : 2) ks
     const int kt_run = s_pad / 16;
     const float sl2 = a.scale * 1.4426950408889634f;
 
+    // rows t: visible keys [lo, lo + nk) of the stacked keys -- the row's own chunk (Sec. 2.2.1) --, lse of the forward pass
+    // in log2 units
+    auto row_of = [&](int t, int& lo, uint32_t& nk, float& l) {
+        lo = 0; nk = 0; l = 0.f;
+        if (t < tasks) {
+            const int cc = t / per_chunk, tt = t - cc * per_chunk;
+            const int r = tt / G, h = hk * G + (tt - r * G);
+            lo = cc * s; nk = (uint32_t)(a.k + own * (r + 1));
+            l = a.lse[(int64_t)h * a.total_aug + row0 + (int64_t)cc * s + a.k + r] * 1.4426950408889634f;
+        }
+    };
+    // dQ row rl of the tile at query row t0, its 16-byte chunk c, from the staging rows at sOw to its augmented position (Eq. 1)
+    auto put_dq = [&](uint32_t sOw, int t0, int rl, int c) {
+        const int t = t0 + rl;
+        if (t >= tasks) return;
+        const int cc = t / per_chunk, tt = t - cc * per_chunk;
+        const int r = tt / G, h = hk * G + (tt - r * G);
+        uint4 val;
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(val.x), "=r"(val.y), "=r"(val.z), "=r"(val.w) : "r"(bs_sw<D>(sOw, rl, c)));
+        *reinterpret_cast<uint4*>(a.dq + (row0 + (int64_t)cc * s + a.k + r) * a.dq_st + (int64_t)h * a.dq_sh + c * 8) = val;
+    };
+
+    if constexpr (kOneTile) {
+        // =============================== phase 1, one tile of 16 query rows: a warp per key tile ===============================
+        // (with a warp per 16 query rows three of the four would wait for the one that forms everything)
+        float sc[2][4], dp[2][4];
+        const int n0 = 2 * warp, t0 = g0, t1 = g0 + 8;
+        float* sD = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bs_smem) + (sO - sQ)) + 16 * D / 2;      // [4][16], behind the staging rows
+        if (warp < kt_run) {
+#pragma unroll
+            for (int n = 0; n < 2; ++n) { sc[n][0] = sc[n][1] = sc[n][2] = sc[n][3] = 0.f; dp[n][0] = dp[n][1] = dp[n][2] = dp[n][3] = 0.f; }
+#pragma unroll
+            for (int kk = 0; kk < D / 16; ++kk) {
+                uint32_t qa[4], ga[4], kb[4], vb[4];
+                bs_ldsm(qa, bs_sw<D>(sQ, r8 + 8 * (mi & 1), 2 * kk + (mi >> 1)));
+                bs_ldsm(ga, bs_sw<D>(sG, r8 + 8 * (mi & 1), 2 * kk + (mi >> 1)));
+                bs_ldsm(kb, bs_sw<D>(sK, warp * 16 + r8 + 8 * (mi >> 1), 2 * kk + (mi & 1)));
+                bs_ldsm(vb, bs_sw<D>(sV, warp * 16 + r8 + 8 * (mi >> 1), 2 * kk + (mi & 1)));
+                bs_mma(sc[0], qa, kb[0], kb[1]);
+                bs_mma(sc[1], qa, kb[2], kb[3]);
+                bs_mma(dp[0], ga, vb[0], vb[1]);
+                bs_mma(dp[1], ga, vb[2], vb[3]);
+            }
+            int lo0, lo1; uint32_t nk0, nk1; float l0, l1;
+            row_of(t0, lo0, nk0, l0);
+            row_of(t1, lo1, nk1, l1);
+            float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                const int key = (n0 + n) * 8 + c2;
+                sc[n][0] = (uint32_t)(key - lo0) < nk0 ? bs_ex2(fmaf(sc[n][0], sl2, -l0)) : 0.f;
+                sc[n][1] = (uint32_t)(key + 1 - lo0) < nk0 ? bs_ex2(fmaf(sc[n][1], sl2, -l0)) : 0.f;
+                sc[n][2] = (uint32_t)(key - lo1) < nk1 ? bs_ex2(fmaf(sc[n][2], sl2, -l1)) : 0.f;
+                sc[n][3] = (uint32_t)(key + 1 - lo1) < nk1 ? bs_ex2(fmaf(sc[n][3], sl2, -l1)) : 0.f;
+                d0 = fmaf(sc[n][0], dp[n][0], fmaf(sc[n][1], dp[n][1], d0));
+                d1 = fmaf(sc[n][2], dp[n][2], fmaf(sc[n][3], dp[n][3], d1));
+            }
+            d0 += __shfl_xor_sync(0xffffffffu, d0, 1); d0 += __shfl_xor_sync(0xffffffffu, d0, 2);
+            d1 += __shfl_xor_sync(0xffffffffu, d1, 1); d1 += __shfl_xor_sync(0xffffffffu, d1, 2);
+            if ((lane & 3) == 0) { sD[warp * 16 + t0] = d0; sD[warp * 16 + t1] = d1; }
+        }
+        __syncthreads();
+        if (warp < kt_run) {
+            float d0 = 0.f, d1 = 0.f;                                  // delta: the key tiles' shares, always in this order
+            for (int kt = 0; kt < kt_run; ++kt) { d0 += sD[kt * 16 + t0]; d1 += sD[kt * 16 + t1]; }
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                const uint32_t p_lo = bs_pack(sc[n][0], sc[n][1]), p_hi = bs_pack(sc[n][2], sc[n][3]);
+                const uint32_t s_lo = bs_pack(sc[n][0] * (dp[n][0] - d0), sc[n][1] * (dp[n][1] - d0));
+                const uint32_t s_hi = bs_pack(sc[n][2] * (dp[n][2] - d1), sc[n][3] * (dp[n][3] - d1));
+                const uint32_t off0 = (uint32_t)t0 * pstride + (uint32_t)((n0 + n) * 8 + c2) * 2, off1 = (uint32_t)t1 * pstride + (uint32_t)((n0 + n) * 8 + c2) * 2;
+                asm volatile("st.shared.u32 [%0], %1;" ::"r"(sP + off0), "r"(p_lo) : "memory");
+                asm volatile("st.shared.u32 [%0], %1;" ::"r"(sP + off1), "r"(p_hi) : "memory");
+                asm volatile("st.shared.u32 [%0], %1;" ::"r"(sS + off0), "r"(s_lo) : "memory");
+                asm volatile("st.shared.u32 [%0], %1;" ::"r"(sS + off1), "r"(s_hi) : "memory");
+            }
+        }
+        __syncthreads();
+        // ---- dQ = scale dS K: a quarter of the head's elements per warp ----
+        constexpr int kN2 = D / 64;                                    // 16-element steps of a warp
+        float o[2 * kN2][4];
+#pragma unroll
+        for (int i = 0; i < 2 * kN2; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }
+#pragma unroll
+        for (int kt = 0; kt < KT_MAX; ++kt) {
+            if (kt < kt_run) {
+                uint32_t da[4];
+                bs_ldsm(da, sS + (uint32_t)(r8 + 8 * (mi & 1)) * pstride + (uint32_t)(kt * 16 + 8 * (mi >> 1)) * 2);
+#pragma unroll
+                for (int n2 = 0; n2 < kN2; ++n2) {
+                    uint32_t kb[4];
+                    bs_ldsm_t(kb, bs_sw<D>(sK, kt * 16 + r8 + 8 * (mi & 1), 2 * (warp * kN2 + n2) + (mi >> 1)));
+                    bs_mma(o[2 * n2], da, kb[0], kb[1]);
+                    bs_mma(o[2 * n2 + 1], da, kb[2], kb[3]);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2 * kN2; ++i) {
+            const uint32_t w0 = bs_pack(o[i][0] * a.scale, o[i][1] * a.scale), w1 = bs_pack(o[i][2] * a.scale, o[i][3] * a.scale);
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(bs_sw<D>(sO, g0, warp * 2 * kN2 + i) + (uint32_t)c2 * 2), "r"(w0) : "memory");
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(bs_sw<D>(sO, g0 + 8, warp * 2 * kN2 + i) + (uint32_t)c2 * 2), "r"(w1) : "memory");
+        }
+        __syncwarp();
+#pragma unroll
+        for (int it = 0; it < kN2; ++it) {                             // 16 rows x 2 kN2 chunks of 16 bytes
+            const int idx = it * 32 + lane;
+            put_dq(sO, 0, idx / (2 * kN2), warp * 2 * kN2 + idx % (2 * kN2));
+        }
+    } else
     // =============================== phase 1: a warp per 16 query rows ===============================
     for (int mt = warp; mt < m_pad / 16; mt += 4) {
         float sc[2 * KT_MAX][4], dp[2 * KT_MAX][4];
@@ -152,24 +265,10 @@ __global__ void __launch_bounds__(128, KT_MAX <= 4 ? 4 : KT_MAX <= 6 ? 3 : 2) ks
                 }
             }
         }
-        // rows t0 = 16 mt + g0 and t0 + 8: visible keys [lo, lo + nk) of the stacked keys -- the row's own chunk
-        // (Sec. 2.2.1) --, lse of the forward pass in log2 units
         const int t0 = mt * 16 + g0, t1 = t0 + 8;
-        int lo0 = 0, lo1 = 0;
-        uint32_t nk0 = 0, nk1 = 0;
-        float l0 = 0.f, l1 = 0.f;
-        if (t0 < tasks) {
-            const int cc = t0 / per_chunk, tt = t0 - cc * per_chunk;
-            const int r = tt / G, h = hk * G + (tt - r * G);
-            lo0 = cc * s; nk0 = (uint32_t)(a.k + own * (r + 1));
-            l0 = a.lse[(int64_t)h * a.total_aug + row0 + (int64_t)cc * s + a.k + r] * 1.4426950408889634f;
-        }
-        if (t1 < tasks) {
-            const int cc = t1 / per_chunk, tt = t1 - cc * per_chunk;
-            const int r = tt / G, h = hk * G + (tt - r * G);
-            lo1 = cc * s; nk1 = (uint32_t)(a.k + own * (r + 1));
-            l1 = a.lse[(int64_t)h * a.total_aug + row0 + (int64_t)cc * s + a.k + r] * 1.4426950408889634f;
-        }
+        int lo0, lo1; uint32_t nk0, nk1; float l0, l1;
+        row_of(t0, lo0, nk0, l0);
+        row_of(t1, lo1, nk1, l1);
         float d0 = 0.f, d1 = 0.f;
 #pragma unroll
         for (int n = 0; n < 2 * KT_MAX; ++n) {
@@ -233,14 +332,7 @@ __global__ void __launch_bounds__(128, KT_MAX <= 4 ? 4 : KT_MAX <= 6 ? 3 : 2) ks
 #pragma unroll
             for (int it = 0; it < 16 * CH / 32; ++it) {
                 const int idx = it * 32 + lane;
-                const int rl = idx / CH, c = idx - rl * CH;
-                const int t = mt * 16 + rl;
-                if (t >= tasks) continue;
-                const int cc = t / per_chunk, tt = t - cc * per_chunk;
-                const int r = tt / G, h = hk * G + (tt - r * G);
-                uint4 val;
-                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(val.x), "=r"(val.y), "=r"(val.z), "=r"(val.w) : "r"(bs_sw<D>(sOw, rl, c)));
-                *reinterpret_cast<uint4*>(a.dq + (row0 + (int64_t)cc * s + a.k + r) * a.dq_st + (int64_t)h * a.dq_sh + c * 8) = val;
+                put_dq(sOw, mt * 16, idx / CH, idx % CH);
             }
         }
     }
@@ -319,7 +411,7 @@ bool g_bs_done[64] = {};
 
 size_t bs_smem_bytes(int D, int s_pad, int m_pad)
 {
-    return (size_t)2 * (m_pad + s_pad) * D * 2 + (size_t)2 * m_pad * (s_pad + 8) * 2 + (size_t)std::min(4, m_pad / 16) * 16 * D * 2;
+    return (size_t)2 * (m_pad + s_pad) * D * 2 + (size_t)2 * m_pad * (s_pad + 8) * 2 + (size_t)std::min(4, m_pad / 16) * 16 * D * 2 + 256;
 }
 
 }  // namespace
@@ -354,28 +446,25 @@ cudaError_t launch_bwd_summary_mma(const BwdArgs& a, cudaStream_t stream)
             const auto opt_in = [&](auto* kernel, int D, int keys) {
                 return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bs_smem_bytes(D, keys, kBsMaxRows));
             };
-            if ((e = opt_in(ksa_bwd_summary_mma_kernel<128, 8>, 128, kBsMaxKeys)) != cudaSuccess) return e;
-            if ((e = opt_in(ksa_bwd_summary_mma_kernel<64, 8>, 64, kBsMaxKeys)) != cudaSuccess) return e;
-            if ((e = opt_in(ksa_bwd_summary_mma_kernel<128, 6>, 128, 96)) != cudaSuccess) return e;
-            if ((e = opt_in(ksa_bwd_summary_mma_kernel<64, 6>, 64, 96)) != cudaSuccess) return e;
-            if ((e = opt_in(ksa_bwd_summary_mma_kernel<128, 4>, 128, kBsShortKeys)) != cudaSuccess) return e;
-            if ((e = opt_in(ksa_bwd_summary_mma_kernel<64, 4>, 64, kBsShortKeys)) != cudaSuccess) return e;
+            if ((e = opt_in(ksa_bwd_summary_mma_kernel<128, 8, false>, 128, kBsMaxKeys)) != cudaSuccess) return e;
+            if ((e = opt_in(ksa_bwd_summary_mma_kernel<64, 8, false>, 64, kBsMaxKeys)) != cudaSuccess) return e;
+            if ((e = opt_in(ksa_bwd_summary_mma_kernel<128, 6, false>, 128, 96)) != cudaSuccess) return e;
+            if ((e = opt_in(ksa_bwd_summary_mma_kernel<64, 6, false>, 64, 96)) != cudaSuccess) return e;
+            if ((e = opt_in(ksa_bwd_summary_mma_kernel<128, 4, false>, 128, kBsShortKeys)) != cudaSuccess) return e;
+            if ((e = opt_in(ksa_bwd_summary_mma_kernel<64, 4, false>, 64, kBsShortKeys)) != cudaSuccess) return e;
+            if ((e = opt_in(ksa_bwd_summary_mma_kernel<128, 4, true>, 128, kBsShortKeys)) != cudaSuccess) return e;
+            if ((e = opt_in(ksa_bwd_summary_mma_kernel<64, 4, true>, 64, kBsShortKeys)) != cudaSuccess) return e;
             g_bs_done[dev] = true;
         }
     }
     const int max_chunks = a.max_n_summ / a.m;
     dim3 grid((unsigned)((max_chunks + cpb - 1) / cpb), (unsigned)a.num_seqs, (unsigned)a.Hkv);
     const size_t smem = bs_smem_bytes(a.D, s_pad, m_pad);
-    if (s_pad <= kBsShortKeys) {
-        if (a.D == 128) ksa_bwd_summary_mma_kernel<128, 4><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
-        else            ksa_bwd_summary_mma_kernel<64, 4><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
-    } else if (s_pad <= 96) {
-        if (a.D == 128) ksa_bwd_summary_mma_kernel<128, 6><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
-        else            ksa_bwd_summary_mma_kernel<64, 6><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
-    } else {
-        if (a.D == 128) ksa_bwd_summary_mma_kernel<128, 8><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
-        else            ksa_bwd_summary_mma_kernel<64, 8><<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
-    }
+    auto* kernel = s_pad > 96 ? (a.D == 128 ? ksa_bwd_summary_mma_kernel<128, 8, false> : ksa_bwd_summary_mma_kernel<64, 8, false>)
+                 : s_pad > kBsShortKeys ? (a.D == 128 ? ksa_bwd_summary_mma_kernel<128, 6, false> : ksa_bwd_summary_mma_kernel<64, 6, false>)
+                 : m_pad > 16 ? (a.D == 128 ? ksa_bwd_summary_mma_kernel<128, 4, false> : ksa_bwd_summary_mma_kernel<64, 4, false>)
+                              : (a.D == 128 ? ksa_bwd_summary_mma_kernel<128, 4, true> : ksa_bwd_summary_mma_kernel<64, 4, true>);
+    kernel<<<grid, 128, smem, stream>>>(a, s_pad, m_pad, cpb);
     return cudaGetLastError();
 }
 
