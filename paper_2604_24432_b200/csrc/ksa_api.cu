@@ -438,6 +438,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_create(ksa_ctx** out, 
     ctx->encode = (EncodeTiledFn)fn;
     if ((e = cudaMalloc(&ctx->d_status, sizeof(int32_t))) != cudaSuccess) { delete ctx; return KSA_ERR_CUDA; }
     if ((e = cudaMemset(ctx->d_status, 0, sizeof(int32_t))) != cudaSuccess) { cudaFree(ctx->d_status); delete ctx; return KSA_ERR_CUDA; }
+    if ((e = cudaStreamCreateWithFlags(&ctx->s_sched, cudaStreamNonBlocking)) != cudaSuccess) { cudaFree(ctx->d_status); delete ctx; return KSA_ERR_CUDA; }
     cudaEventCreate(&ctx->ev0);
     cudaEventCreate(&ctx->ev1);
     *out = ctx;
@@ -536,13 +537,8 @@ static int ensure_schedule(ksa_ctx* ctx, const ksa_params* p, bool upload, int t
         cudaError_t e;
         const size_t sb = (size_t)round_up((int64_t)(hs.seqs.size() * sizeof(SeqInfo)), 256), wb = hs.work.size() * sizeof(WorkItem);
         const size_t need = (size_t)round_up((int64_t)(sb + wb), 256);
-        // a context that stays with its first lengths needs neither the stream nor room for more (a new stream and a
-        // large allocation cost milliseconds)
+        // (a context that stays with its first lengths needs no room for more: a large allocation costs milliseconds)
         const bool again = ctx->arena != nullptr;
-        if (again && !ctx->s_sched && (e = cudaStreamCreateWithFlags(&ctx->s_sched, cudaStreamNonBlocking)) != cudaSuccess) {
-            ctx->s_sched = nullptr;
-            return cuda_fail(ctx, e);
-        }
         if (ctx->arena_used + need > ctx->arena_cap) {
             if (again && (e = cudaDeviceSynchronize()) != cudaSuccess) return cuda_fail(ctx, e);   // nothing reads the old parts any more
             ctx->arena_used = 0;
@@ -559,8 +555,7 @@ static int ensure_schedule(ksa_ctx* ctx, const ksa_params* p, bool upload, int t
         // on a stream of its own and waited for: whatever stream the caller uses next finds the schedule in place, and
         // the copy does not wait for kernels in flight
         char* dst = ctx->arena + ctx->arena_used;
-        if (!again) e = cudaMemcpy(dst, ctx->sched_bytes.data(), sb + wb, cudaMemcpyHostToDevice);
-        else if ((e = cudaMemcpyAsync(dst, ctx->sched_bytes.data(), sb + wb, cudaMemcpyHostToDevice, ctx->s_sched)) == cudaSuccess)
+        if ((e = cudaMemcpyAsync(dst, ctx->sched_bytes.data(), sb + wb, cudaMemcpyHostToDevice, ctx->s_sched)) == cudaSuccess)
             e = cudaStreamSynchronize(ctx->s_sched);
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         ctx->arena_used += need;
