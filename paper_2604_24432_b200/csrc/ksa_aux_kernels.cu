@@ -291,8 +291,11 @@ constexpr int kSummMaxKeys = 12;
 
 // kStreams: the rows come from the packed streams (text rows of kt / vt, summary rows of ks / vs, the summary tokens'
 // queries from qs, all head-major) instead of the caller's interleaved tensors.
+// Launched behind the text rows' kernel, a block reads its rows without waiting (ptx::pdl_wait) for any kernel: the one that
+// wrote them ended before the text kernel triggered this launch, so they stand in L2, but nothing has told this SM's L1 to drop
+// what it holds of those addresses from earlier calls.  Hence loads that bypass L1 (each row is read once).
 template <int D, bool kStreams>
-__device__ __forceinline__ void summary_short_block(const KernelArgs& a, const uint16_t* __restrict__ qs)
+__device__ __forceinline__ void summary_short_block(const KernelArgs& a, const uint16_t* qs)
 {
     constexpr int E = D / 8;                      // elements per lane: 16 (two 16-byte vectors) or 8 (one)
     constexpr int V4 = E / 8;
@@ -327,8 +330,8 @@ __device__ __forceinline__ void summary_short_block(const KernelArgs& a, const u
                 kp = a.kx + (r0 + rr) * a.k_st + (int64_t)hk * a.k_sh;
                 vp = a.v + (r0 + rr) * a.v_st + (int64_t)hk * a.v_sh;
             }
-            const uint4 kx = *reinterpret_cast<const uint4*>(kp + vv * 8);
-            const uint4 vx = *reinterpret_cast<const uint4*>(vp + vv * 8);
+            const uint4 kx = __ldcg(reinterpret_cast<const uint4*>(kp + vv * 8));
+            const uint4 vx = __ldcg(reinterpret_cast<const uint4*>(vp + vv * 8));
             *reinterpret_cast<uint4*>(sK + rr * D + vv * 8) = kx;
             *reinterpret_cast<uint4*>(sV + rr * D + vv * 8) = vx;
         }
@@ -364,7 +367,7 @@ __device__ __forceinline__ void summary_short_block(const KernelArgs& a, const u
             const uint16_t* qp = (kStreams ? qs + ((int64_t)h * a.summ_rows + sq.summ_off + (int64_t)j * a.m + r) * D
                                            : a.q + qrow * a.q_st + (int64_t)h * a.q_sh) + sub * 8;
 #pragma unroll
-            for (int c = 0; c < V4; ++c) unpack(*reinterpret_cast<const uint4*>(qp + 64 * c), qv + 8 * c);
+            for (int c = 0; c < V4; ++c) unpack(__ldcg(reinterpret_cast<const uint4*>(qp + 64 * c)), qv + 8 * c);
         }
         float x[kSummMaxKeys];
 #pragma unroll
@@ -429,7 +432,7 @@ __device__ __forceinline__ void summary_short_block(const KernelArgs& a, const u
 
 // The first block ends after the kernel in front (where this one was launched beside it): see launch_summary.
 template <int D, bool kStreams>
-__global__ void __launch_bounds__(256) ksa_summary_short_kernel(KernelArgs a, const uint16_t* __restrict__ qs)
+__global__ void __launch_bounds__(256) ksa_summary_short_kernel(KernelArgs a, const uint16_t* qs)
 {
     summary_short_block<D, kStreams>(a, qs);
     if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) ptx::pdl_wait();

@@ -302,8 +302,8 @@ __device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& ma
     auto fetch = [&](int qt, int g) {                                     // pair (query tile qt, head g of the group)
         const int h = hk * G + g;
         const size_t r = (size_t)h * a.text_rows + sq.text_off + (size_t)qt * 128 + 32 * cg + lane;
-        n_lse = -a.lse_t[r];                                              // -inf on padding rows: P = 0 there
-        n_dl = -a.delta_t[r];
+        n_lse = -__ldcg(a.lse_t + r);                                     // -inf on padding rows: P = 0 there
+        n_dl = -__ldcg(a.delta_t + r);                                    // (past L1: see the launches)
     };
     // loads of streamed tile j (the producer's thread)
     const bool direct = a.direct != 0;
@@ -667,7 +667,7 @@ __device__ __forceinline__ void bt_dq_block(const BwdArgs& a, const BwdMaps& map
         const uint32_t tXc = tX + lane_sel + cg * 32;                     // this warp's 32 x 32 block
         const int i_w0 = i_first + quarter * 32, i = i_w0 + lane;         // this thread's query row
         const size_t r = (size_t)h * a.text_rows + sq.text_off + i;
-        const float lse2 = a.lse_t[r], dl = a.delta_t[r];                 // +inf / 0 on padding rows: P = 0 there
+        const float lse2 = __ldcg(a.lse_t + r), dl = __ldcg(a.delta_t + r);      // +inf / 0 on padding rows: P = 0 there
         const int iq = i / a.k, iq_w0 = i_w0 / a.k, iq_w1 = (i_w0 + 31) / a.k;
         bool alive = true;
         // The chunk of the block's first key, kc0 = key0 + 32 cg, is kept as quotient and remainder by the keys per
@@ -795,7 +795,10 @@ __device__ __forceinline__ void bt_dq_block(const BwdArgs& a, const BwdMaps& map
 // each at 32,768 tokens), so that the tails of the first two are filled (training layer of 7,942 ragged tokens, 16/16 heads
 // 610 -> 573 us, 2 x 8,192 tokens 2,140 -> 2,070 us; nothing at 2 x 32,768).
 // Nothing here waits for the launch in front, which was itself started behind the preparation; only the last block of each
-// waits for its end, so that the kernel behind the three, an ordinary launch, finds all of them done.
+// waits for its end, so that the kernel behind the three, an ordinary launch, finds all of them done.  What the preparation and
+// the pack wrote stands in L2 by then, but without a wait of its own (pdl_wait) a kernel has no promise that its L1 has dropped
+// those addresses' old contents: the tiles come by TMA, lse and delta by loads that bypass L1, the sums are added in L2
+// (nothing measurable: 2 x 32,768 tokens 14.60 ms, before 14.64; a fence.acq_rel.gpu at the start instead costs 0.7 - 1.6 %).
 __device__ __forceinline__ void bt_end_behind_front()
 {
     if (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1) pdl_wait();

@@ -91,7 +91,8 @@ __device__ __forceinline__ void summary_mma_block(const KernelArgs& a, int s_pad
     const uint32_t sK = sQ + (uint32_t)m_pad * D * 2;
     const uint32_t sV = sK + (uint32_t)s_pad * D * 2;
     // ---- stage Q (row t = summary t / G of the chunk, query head hk G + t % G), K, V; padding rows are zeros.
-    //      Asynchronous 16-byte copies: every load of the block is in flight before the first one is waited for. ----
+    //      Asynchronous 16-byte copies: every load of the block is in flight before the first one is waited for.  They come
+    //      from L2 (.cg): launched behind the text rows' kernel, the block reads rows without waiting for any kernel ----
     for (int idx = threadIdx.x; idx < (m_pad + 2 * s_pad) * CH; idx += blockDim.x) {
         const int rr = idx / CH, c = idx - rr * CH;
         const uint16_t* src = a.kx + row0 * a.k_st + (int64_t)hk * a.k_sh;   // a valid address for the zero-filled rows
