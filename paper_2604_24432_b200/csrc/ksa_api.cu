@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -38,7 +39,7 @@ struct ksa_ctx {
     // Device memory of the schedules: a new set of lengths takes the next part of the arena, so that work in flight keeps
     // reading the part it was launched with; only when the arena is full does the host wait for the device.
     char* arena = nullptr; size_t arena_cap = 0, arena_used = 0;
-    cudaStream_t s_sched = nullptr;   // the uploads' own stream
+    cudaStream_t s_sched = nullptr;   // the uploads' stream, from the second set of lengths on (shared: upload_stream_take)
     std::vector<char> sched_bytes;    // seqs, then work, as they are uploaded
     int32_t* d_status = nullptr;
     bool timing = false;
@@ -53,6 +54,34 @@ struct ksa_ctx {
     std::vector<cudaEvent_t> ev_in, ev_done;
     cudaEvent_t ev_start = nullptr;
 };
+
+// The stream of the schedules' uploads: one per device, made when a first context's lengths change, gone with the last context
+// that took it.  (A stream costs 65 - 80 us to create, four times a call of 1,024 tokens: not in ksa_create, where contexts
+// that only decode or stay with their lengths would pay for it, nor once for every context.)
+namespace {
+struct UploadStream { cudaStream_t stream = nullptr; int users = 0; };
+std::mutex g_upload_mutex;
+UploadStream g_upload[64];                               // by device
+}  // namespace
+static cudaError_t upload_stream_take(int device, cudaStream_t* out)
+{
+    std::lock_guard<std::mutex> lock(g_upload_mutex);
+    if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
+    UploadStream& u = g_upload[device];
+    if (!u.stream) {
+        const cudaError_t e = cudaStreamCreateWithFlags(&u.stream, cudaStreamNonBlocking);
+        if (e != cudaSuccess) { u.stream = nullptr; return e; }
+    }
+    ++u.users;
+    *out = u.stream;
+    return cudaSuccess;
+}
+static void upload_stream_give(int device)
+{
+    std::lock_guard<std::mutex> lock(g_upload_mutex);
+    UploadStream& u = g_upload[device];
+    if (--u.users == 0) { cudaStreamDestroy(u.stream); u.stream = nullptr; }
+}
 
 static int cuda_fail(ksa_ctx* ctx, cudaError_t e)
 {
@@ -438,7 +467,6 @@ extern "C" __attribute__((visibility("default"))) int ksa_create(ksa_ctx** out, 
     ctx->encode = (EncodeTiledFn)fn;
     if ((e = cudaMalloc(&ctx->d_status, sizeof(int32_t))) != cudaSuccess) { delete ctx; return KSA_ERR_CUDA; }
     if ((e = cudaMemset(ctx->d_status, 0, sizeof(int32_t))) != cudaSuccess) { cudaFree(ctx->d_status); delete ctx; return KSA_ERR_CUDA; }
-    if ((e = cudaStreamCreateWithFlags(&ctx->s_sched, cudaStreamNonBlocking)) != cudaSuccess) { cudaFree(ctx->d_status); delete ctx; return KSA_ERR_CUDA; }
     cudaEventCreate(&ctx->ev0);
     cudaEventCreate(&ctx->ev1);
     *out = ctx;
@@ -450,7 +478,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_destroy(ksa_ctx* ctx)
     if (!ctx) return KSA_OK;
     cudaSetDevice(ctx->device);
     if (ctx->arena) cudaFree(ctx->arena);
-    if (ctx->s_sched) cudaStreamDestroy(ctx->s_sched);
+    if (ctx->s_sched) upload_stream_give(ctx->device);
     if (ctx->d_status) cudaFree(ctx->d_status);
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);
     if (ctx->ev1) cudaEventDestroy(ctx->ev1);
@@ -552,8 +580,9 @@ static int ensure_schedule(ksa_ctx* ctx, const ksa_params* p, bool upload, int t
         try { ctx->sched_bytes.resize(need); } catch (const std::bad_alloc&) { return KSA_ERR_NOMEM; }
         std::memcpy(ctx->sched_bytes.data(), hs.seqs.data(), hs.seqs.size() * sizeof(SeqInfo));
         if (wb) std::memcpy(ctx->sched_bytes.data() + sb, hs.work.data(), wb);
-        // on a stream of its own and waited for: whatever stream the caller uses next finds the schedule in place, and
-        // the copy does not wait for kernels in flight
+        // waited for: whatever stream the caller uses next finds the schedule in place.  From the second set of lengths on the
+        // copies have a stream of their own and do not wait for kernels in flight
+        if (again && !ctx->s_sched && (e = upload_stream_take(ctx->device, &ctx->s_sched)) != cudaSuccess) return cuda_fail(ctx, e);
         char* dst = ctx->arena + ctx->arena_used;
         if ((e = cudaMemcpyAsync(dst, ctx->sched_bytes.data(), sb + wb, cudaMemcpyHostToDevice, ctx->s_sched)) == cudaSuccess)
             e = cudaStreamSynchronize(ctx->s_sched);
