@@ -23,8 +23,10 @@
  *     call with a new set of lengths builds and uploads it with a blocking copy).
  *     The same holds for ksa_attn_bwd, ksa_attn_fwd_part and ksa_qkv_prepare: after
  *     that first call they may be recorded into a CUDA graph (stream capture) and
- *     replayed on the same buffers (the graph reads the context's device copy of that
- *     schedule: replay it before the context goes on to other lengths).
+ *     replayed on the same buffers, also after the context has gone on to other
+ *     lengths, heads, layouts or parts: the context keeps the device copy of the schedule
+ *     that the graph reads until the graph is destroyed.  The context must outlive the
+ *     last replay.
  *   - There is no CPU fallback: on a machine without an sm_100 device ksa_create fails.
  *
  * Layout of one packed batch (Eq. 1, generalised to m summaries per chunk):

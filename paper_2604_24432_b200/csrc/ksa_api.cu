@@ -1,8 +1,10 @@
 // C ABI of the KSA forward library: argument validation, sequence layout (Eq. 1), the
 // block-sparse tile schedule (Eq. 3 at tile granularity) and the kernel launches.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -39,6 +41,11 @@ struct ksa_ctx {
     // Device memory of the schedules: a new set of lengths takes the next part of the arena, so that work in flight keeps
     // reading the part it was launched with; only when the arena is full does the host wait for the device.
     char* arena = nullptr; size_t arena_cap = 0, arena_used = 0;
+    // CUDA graphs that hold calls whose schedules stand in the arena (counted down when a graph is gone); while there are any,
+    // a full arena is not started over but set aside, and freed once they are gone.
+    std::shared_ptr<std::atomic<int>> arena_graphs;
+    struct Aside { char* mem; std::shared_ptr<std::atomic<int>> graphs; };
+    std::vector<Aside> aside;
     cudaStream_t s_sched = nullptr;   // the uploads' stream, from the second set of lengths on (shared: upload_stream_take)
     std::vector<char> sched_bytes;    // seqs, then work, as they are uploaded
     int32_t* d_status = nullptr;
@@ -478,6 +485,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_destroy(ksa_ctx* ctx)
     if (!ctx) return KSA_OK;
     cudaSetDevice(ctx->device);
     if (ctx->arena) cudaFree(ctx->arena);
+    for (const ksa_ctx::Aside& b : ctx->aside) cudaFree(b.mem);
     if (ctx->s_sched) upload_stream_give(ctx->device);
     if (ctx->d_status) cudaFree(ctx->d_status);
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);
@@ -545,7 +553,62 @@ extern "C" __attribute__((visibility("default"))) int ksa_text_kernel_ms(ksa_ctx
 // A server's calls have other lengths every time: with cudaFree, cudaMalloc and a blocking copy for each new set of lengths
 // the host waited for the device in every call (four prompts of 517 - 6,007 tokens, 310 us of kernels: 434 us, now 340 us).
 static constexpr size_t kScheduleArena = 256 << 10;
-static int ensure_schedule(ksa_ctx* ctx, const ksa_params* p, bool upload, int target_chunks = 0)
+
+// Room for `need` bytes behind arena_used.  A full arena starts over once nothing in flight reads it, or, if graphs may read it
+// again, makes way for a new one; a schedule of more than a quarter of it gets a larger one.
+static int arena_room(ksa_ctx* ctx, size_t need)
+{
+    if (ctx->arena_used + need <= ctx->arena_cap) return KSA_OK;
+    cudaError_t e;
+    // (a context that stays with its first lengths needs no room for more: a large allocation costs milliseconds)
+    size_t cap = std::max(kScheduleArena, need);
+    if (ctx->arena) {
+        if ((e = cudaDeviceSynchronize()) != cudaSuccess) return cuda_fail(ctx, e);
+        size_t n = 0;
+        for (const ksa_ctx::Aside& b : ctx->aside) {
+            if (b.graphs->load() == 0) cudaFree(b.mem); else ctx->aside[n++] = b;
+        }
+        ctx->aside.resize(n);
+        const bool recorded = ctx->arena_graphs->load() > 0;
+        ctx->arena_used = 0;
+        if (!recorded && need <= ctx->arena_cap / 4) return KSA_OK;
+        if (recorded) {
+            try { ctx->aside.push_back({ctx->arena, ctx->arena_graphs}); } catch (const std::bad_alloc&) { ctx->arena_used = ctx->arena_cap; return KSA_ERR_NOMEM; }
+        } else {
+            cudaFree(ctx->arena);
+        }
+        cap = need > ctx->arena_cap / 4 ? std::max(kScheduleArena, 4 * need) : ctx->arena_cap;
+        ctx->arena = nullptr; ctx->arena_cap = 0;
+    }
+    try { ctx->arena_graphs = std::make_shared<std::atomic<int>>(0); } catch (const std::bad_alloc&) { return KSA_ERR_NOMEM; }
+    if ((e = cudaMalloc(&ctx->arena, cap)) != cudaSuccess) { ctx->arena = nullptr; return cuda_fail(ctx, e); }
+    ctx->arena_cap = cap;
+    return KSA_OK;
+}
+
+// If the caller's stream is being recorded into a graph, the graph holds on to the arena as it stands: it counts as one of its
+// graphs until it and everything instantiated from it are destroyed.
+static int arena_keep_for_graph(ksa_ctx* ctx, cudaStream_t stream)
+{
+    cudaStreamCaptureStatus status;
+    cudaError_t e = cudaStreamIsCapturing(stream, &status);
+    if (e != cudaSuccess) return cuda_fail(ctx, e);
+    if (status != cudaStreamCaptureStatusActive) return KSA_OK;
+    cudaGraph_t graph = nullptr;
+    if ((e = cudaStreamGetCaptureInfo(stream, &status, nullptr, &graph)) != cudaSuccess) return cuda_fail(ctx, e);
+    using Count = std::shared_ptr<std::atomic<int>>;
+    Count* held = new (std::nothrow) Count(ctx->arena_graphs);
+    if (!held) return KSA_ERR_NOMEM;
+    const auto gone = [](void* ptr) { Count* c = static_cast<Count*>(ptr); (*c)->fetch_sub(1); delete c; };
+    cudaUserObject_t object;
+    (*held)->fetch_add(1);
+    if ((e = cudaUserObjectCreate(&object, held, gone, 1, cudaUserObjectNoDestructorSync)) != cudaSuccess) { gone(held); return cuda_fail(ctx, e); }
+    if ((e = cudaGraphRetainUserObject(graph, object, 1, cudaGraphUserObjectMove)) != cudaSuccess) { cudaUserObjectRelease(object, 1); return cuda_fail(ctx, e); }
+    return KSA_OK;
+}
+
+// The schedule of these lengths, in the context and (upload) on the device for work on `stream`.
+static int ensure_schedule(ksa_ctx* ctx, const ksa_params* p, bool upload, int target_chunks = 0, cudaStream_t stream = nullptr)
 {
     std::vector<int32_t> key = schedule_key(p);
     key.push_back(target_chunks);
@@ -565,18 +628,9 @@ static int ensure_schedule(ksa_ctx* ctx, const ksa_params* p, bool upload, int t
         cudaError_t e;
         const size_t sb = (size_t)round_up((int64_t)(hs.seqs.size() * sizeof(SeqInfo)), 256), wb = hs.work.size() * sizeof(WorkItem);
         const size_t need = (size_t)round_up((int64_t)(sb + wb), 256);
-        // (a context that stays with its first lengths needs no room for more: a large allocation costs milliseconds)
         const bool again = ctx->arena != nullptr;
-        if (ctx->arena_used + need > ctx->arena_cap) {
-            if (again && (e = cudaDeviceSynchronize()) != cudaSuccess) return cuda_fail(ctx, e);   // nothing reads the old parts any more
-            ctx->arena_used = 0;
-            if (need > ctx->arena_cap / 4) {
-                if (ctx->arena) { cudaFree(ctx->arena); ctx->arena = nullptr; ctx->arena_cap = 0; }
-                const size_t cap = std::max(kScheduleArena, again ? 4 * need : need);
-                if ((e = cudaMalloc(&ctx->arena, cap)) != cudaSuccess) { ctx->arena = nullptr; return cuda_fail(ctx, e); }
-                ctx->arena_cap = cap;
-            }
-        }
+        const int rc = arena_room(ctx, need);
+        if (rc != KSA_OK) return rc;
         try { ctx->sched_bytes.resize(need); } catch (const std::bad_alloc&) { return KSA_ERR_NOMEM; }
         std::memcpy(ctx->sched_bytes.data(), hs.seqs.data(), hs.seqs.size() * sizeof(SeqInfo));
         if (wb) std::memcpy(ctx->sched_bytes.data() + sb, hs.work.data(), wb);
@@ -591,7 +645,7 @@ static int ensure_schedule(ksa_ctx* ctx, const ksa_params* p, bool upload, int t
         ctx->d_seqs = reinterpret_cast<SeqInfo*>(dst);
         ctx->d_work = reinterpret_cast<WorkItem*>(dst + sb);
     }
-    return KSA_OK;
+    return upload ? arena_keep_for_graph(ctx, stream) : KSA_OK;
 }
 
 extern "C" __attribute__((visibility("default"))) int ksa_schedule_dump(ksa_ctx* ctx, const ksa_params* p, ksa_tile_rec* recs, int64_t cap,
@@ -791,7 +845,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_fwd(ksa_ctx* ctx,
     if ((rc = validate_strides(p)) != KSA_OK) return rc;
     const uintptr_t ptrs[5] = {(uintptr_t)q, (uintptr_t)k, (uintptr_t)v, (uintptr_t)out, (uintptr_t)lse};
     for (int i = 0; i < 5; ++i) if (ptrs[i] & 15) return KSA_ERR_INVALID_ARG;
-    if ((rc = ensure_schedule(ctx, p, true)) != KSA_OK) return rc;
+    if ((rc = ensure_schedule(ctx, p, true, 0, (cudaStream_t)cuda_stream)) != KSA_OK) return rc;
     const HostSchedule& hs = ctx->sched;
     const bool direct = direct_ok(p);
     const WorkspaceLayout wl = workspace_layout(p, hs);
@@ -874,7 +928,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_fwd_part(ksa_ctx*
     if ((rc = validate_strides(p)) != KSA_OK) return rc;
     const uintptr_t ptrs[5] = {(uintptr_t)q, (uintptr_t)k, (uintptr_t)v, (uintptr_t)out, (uintptr_t)lse};
     for (int i = 0; i < 5; ++i) if (ptrs[i] & 15) return KSA_ERR_INVALID_ARG;
-    if ((rc = ensure_schedule(ctx, p, true, num_parts * kPartChunkFactor)) != KSA_OK) return rc;
+    if ((rc = ensure_schedule(ctx, p, true, num_parts * kPartChunkFactor, (cudaStream_t)cuda_stream)) != KSA_OK) return rc;
     const HostSchedule& hs = ctx->sched;
     const bool direct = direct_ok(p);
     const WorkspaceLayout wl = workspace_layout(p, hs);
@@ -963,7 +1017,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_bwd(ksa_ctx* ctx,
     const uintptr_t ptrs[9] = {(uintptr_t)q, (uintptr_t)k, (uintptr_t)v, (uintptr_t)out, (uintptr_t)lse, (uintptr_t)dout,
                                (uintptr_t)dq, (uintptr_t)dk, (uintptr_t)dv};
     for (int i = 0; i < 9; ++i) if (ptrs[i] & 15) return KSA_ERR_INVALID_ARG;
-    if ((rc = ensure_schedule(ctx, p, true)) != KSA_OK) return rc;
+    if ((rc = ensure_schedule(ctx, p, true, 0, (cudaStream_t)cuda_stream)) != KSA_OK) return rc;
     const HostSchedule& hs = ctx->sched;
     const BwdLayout bl = bwd_layout(p, hs);
     if (!workspace || workspace_bytes < bl.total || ((uintptr_t)workspace & 255)) return KSA_ERR_WORKSPACE;
@@ -1108,7 +1162,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_qkv_prepare(ksa_ctx* c
     const uintptr_t ptrs[9] = {(uintptr_t)q_main, (uintptr_t)k_main, (uintptr_t)v_main, (uintptr_t)q_summ, (uintptr_t)k_summ,
                                (uintptr_t)v_summ, (uintptr_t)q_out, (uintptr_t)k_out, (uintptr_t)v_out};
     for (int i = 0; i < 9; ++i) if (ptrs[i] & 15) return KSA_ERR_INVALID_ARG;
-    if ((rc = ensure_schedule(ctx, p, true)) != KSA_OK) return rc;
+    if ((rc = ensure_schedule(ctx, p, true, 0, (cudaStream_t)cuda_stream)) != KSA_OK) return rc;
     const HostSchedule& hs = ctx->sched;
     PrepArgs a{};
     a.seqs = ctx->d_seqs;
@@ -1169,7 +1223,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_fwd_prepared(ksa_
     const uintptr_t ptrs[8] = {(uintptr_t)q_main, (uintptr_t)k_main, (uintptr_t)v_main, (uintptr_t)q_summ, (uintptr_t)k_summ,
                                (uintptr_t)v_summ, (uintptr_t)out, (uintptr_t)lse};
     for (int i = 0; i < 8; ++i) if (ptrs[i] & 15) return KSA_ERR_INVALID_ARG;
-    if ((rc = ensure_schedule(ctx, p, true)) != KSA_OK) return rc;
+    if ((rc = ensure_schedule(ctx, p, true, 0, (cudaStream_t)cuda_stream)) != KSA_OK) return rc;
     const HostSchedule& hs = ctx->sched;
     size_t qs_off = 0;
     const size_t need = prepared_ws_bytes(p, hs, &qs_off);
@@ -1267,7 +1321,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_fwd_host(ksa_ctx*
     // earlier stages have already uploaded and packed; its rows of out are contiguous too.
     // Stage c: copy-in stream uploads chunk c -> caller's stream packs it, runs its summary rows and
     // its share of the work list -> copy-out stream downloads its out / lse rows.
-    if ((rc = ensure_schedule(ctx, &pc, true, kHostPipelineChunks)) != KSA_OK) return rc;
+    if ((rc = ensure_schedule(ctx, &pc, true, kHostPipelineChunks, stream)) != KSA_OK) return rc;
     const HostSchedule& hs = ctx->sched;
     const WorkspaceLayout wl = workspace_layout(&pc, hs);
     cudaError_t e;

@@ -16,8 +16,20 @@ struct Counts { int streams_made, streams_gone, mallocs, frees, device_syncs, up
 Counts g_n{};
 const ksa::SeqInfo* g_seqs = nullptr;
 int g_num_seqs = 0;
+struct Retained { void* graph; cudaHostFn_t destroy; void* ptr; };
+std::vector<Retained> g_retained;
+void* g_graph = nullptr;                                 // the graph that calls are recorded into, null: none
 }  // namespace
 
+FAKE void fake_capture(void* graph) { g_graph = graph; }
+FAKE void fake_graph_destroy(void* graph)
+{
+    for (size_t i = g_retained.size(); i-- > 0;)
+        if (g_retained[i].graph == graph) {
+            g_retained[i].destroy(g_retained[i].ptr);
+            g_retained.erase(g_retained.begin() + (long)i);
+        }
+}
 // what the last ksa_qkv_prepare was launched with
 FAKE Counts fake_counts() { return g_n; }
 FAKE const void* fake_seqs() { return g_seqs; }
@@ -60,3 +72,28 @@ FAKE cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned)
     return cudaSuccess;
 }
 FAKE cudaError_t cudaStreamDestroy(cudaStream_t s) { ++g_n.streams_gone; std::free(s); return cudaSuccess; }
+
+// ---- stream capture: a user object's destructor runs when the graph that holds its one reference goes --------------------
+FAKE cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s)
+{
+    *s = g_graph ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
+FAKE cudaError_t cudaStreamGetCaptureInfo(cudaStream_t stream, cudaStreamCaptureStatus* s, unsigned long long*, cudaGraph_t* graph,
+                                          const cudaGraphNode_t**, size_t*)
+{
+    *graph = static_cast<cudaGraph_t>(g_graph);
+    return cudaStreamIsCapturing(stream, s);
+}
+namespace { Retained g_object; }
+FAKE cudaError_t cudaUserObjectCreate(cudaUserObject_t* o, void* ptr, cudaHostFn_t destroy, unsigned, unsigned)
+{
+    g_object = Retained{nullptr, destroy, ptr};
+    *o = reinterpret_cast<cudaUserObject_t>(&g_object);
+    return cudaSuccess;
+}
+FAKE cudaError_t cudaGraphRetainUserObject(cudaGraph_t graph, cudaUserObject_t, unsigned, unsigned)
+{
+    g_retained.push_back(Retained{graph, g_object.destroy, g_object.ptr});
+    return cudaSuccess;
+}

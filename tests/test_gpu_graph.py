@@ -84,3 +84,45 @@ def test_forward_backward_replayed_from_a_graph(ctx, lens, k, m, C, Hq, Hkv, D):
                 # dk, dv are sums of fp32 atomic adds whose order is not fixed: equal up to rounding order
                 d = (t.float() - want[i][name].float()).abs().max().item()
                 assert d <= 2e-2 * want[i][name].float().abs().max().item(), (name, i, d)
+
+
+def test_a_graph_is_replayed_after_the_context_went_on_to_other_lengths(ctx):
+    """The captured call reads its schedule from the context's device memory at every replay: calls with other lengths, which
+    fill that memory several times over, leave it in place, and it is given back when the graphs are gone."""
+    dev = torch.device("cuda", 0)
+    Hq, Hkv, D = 32, 4, 64
+    g = torch.Generator("cuda").manual_seed(5)
+
+    def case(lens):
+        prob = ksa.Problem(lens, 8, 1, 16, Hq, Hkv, D, 0.125)
+        total = ksa.total_aug_len(prob)
+        q, k, v = (torch.randn((total, h, D), generator=g, device=dev).to(torch.bfloat16) for h in (Hq, Hkv, Hkv))
+        return prob, q, k, v, torch.empty_like(q), torch.empty((Hq, total), device=dev), torch.empty(max(256, ksa.workspace_bytes(prob)), dtype=torch.uint8, device=dev)
+
+    cases = [case([5000, 1290]), case([640])]
+    others = [case([n]) for n in (30_001, 40_000, 700)]                               # schedules of up to 240 KB
+    free = []
+    for rep in range(6):
+        graphs = []
+        for c in cases:
+            ctx.attn_fwd(*c)                                                          # the first call with these lengths: not captured
+            torch.cuda.synchronize()
+            want = (c[4].clone(), c[5].clone())
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                ctx.attn_fwd(*c)
+            graphs.append((graph, c, want))
+        for _ in range(4):
+            for c in others:
+                ctx.attn_fwd(*c)
+        for graph, c, want in graphs:
+            c[4].fill_(7.0); c[5].fill_(7.0)
+            graph.replay()
+            torch.cuda.synchronize()
+            assert ctx.device_status() == 0
+            assert torch.equal(c[4].view(torch.int16), want[0].view(torch.int16)) and torch.equal(c[5].view(torch.int32), want[1].view(torch.int32))
+        del graph, graphs
+        torch.cuda.synchronize()
+        free.append(torch.cuda.mem_get_info()[0])
+    # each round records into two arenas of 256 KB - 1 MB; a driver page is 2 MB
+    assert free[2] - free[-1] <= 4 << 20, free

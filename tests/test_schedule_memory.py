@@ -42,6 +42,7 @@ def fake(tmp_path_factory):
     L = ctypes.CDLL(lib)
     L.fake_counts.restype = Counts
     L.fake_seqs.restype = ctypes.c_void_p
+    L.fake_capture.argtypes = L.fake_graph_destroy.argtypes = [ctypes.c_void_p]
     L.fake_seqs_text.argtypes = [ctypes.c_void_p, ctypes.c_int]
     return L
 
@@ -100,3 +101,44 @@ def test_a_full_arena_waits_once_and_starts_over(fake):
     assert 1 <= c.count("device_syncs") <= 4                                     # ... after the device has been waited for
     c.close()
     assert c.count("mallocs") == c.count("frees")
+
+
+@pytest.mark.parametrize("n", [4096, 70_000])                                    # schedules of 10 KB, and larger than the arena
+def test_a_graph_keeps_the_schedule_it_was_recorded_with(fake, n):
+    """A call recorded into a graph reads its schedule at every replay: the context's later calls, however many, leave that
+    memory alone until the graph is gone, and then take it back."""
+    c = FakeContext(fake)
+    kept = {}
+    for graph in (1, 2, 3):
+        lens = [n + 8 * graph, 77]
+        at = c.call(lens, Hq=16)
+        fake.fake_capture(graph)
+        assert c.call(lens, Hq=16) == at
+        fake.fake_capture(None)
+        kept[graph] = (at, ctypes.string_at(at, 8192))
+    def others(count):
+        for i in range(count):
+            c.call([n + 1000 + 8 * i], Hq=16)
+            c.call([64 + i, 5], Hq=2)
+            for at, was in kept.values():
+                assert ctypes.string_at(at, 8192) == was
+    others(40)
+    assert c.count("device_syncs") > 0                                           # the arena did go round
+    for graph in (2, 1, 3):
+        fake.fake_graph_destroy(graph)
+        del kept[graph]
+        others(20)
+    assert c.count("mallocs") - c.count("frees") <= 3                            # status word, arena, one block to be freed next
+    c.close()
+    assert c.count("mallocs") == c.count("frees")
+
+
+def test_a_graph_may_outlive_its_context(fake):
+    c = FakeContext(fake)
+    c.call([500])
+    fake.fake_capture(9)
+    c.call([500])
+    fake.fake_capture(None)
+    c.close()
+    assert c.count("mallocs") == c.count("frees")
+    fake.fake_graph_destroy(9)
