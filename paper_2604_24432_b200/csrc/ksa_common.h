@@ -51,8 +51,6 @@ struct KernelArgs {
     int64_t total_aug;
     int64_t text_rows;      // padded rows of the packed text stream
     int64_t summ_rows;      // padded rows of the packed summary stream
-    int32_t max_text_pad;   // largest per-sequence padded text rows
-    int32_t max_summ_pad;   // largest per-sequence padded summary rows
     int32_t max_n_summ;     // largest per-sequence summary count
     // Row range (pack and summary kernels): r_seq < 0 means every sequence in full; otherwise only
     // sequence r_seq, packed text rows [r_text0, r_text1), summary-stream rows [r_summ0, r_summ1)
