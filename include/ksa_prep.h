@@ -54,7 +54,8 @@ int ksa_qkv_prepare(ksa_ctx* ctx, const void* q_main, const void* k_main, const 
  * straight into the packed streams the tensor-core kernel reads -- no prepared copy of q, k, v is ever
  * stored in the interleaved layout, and the whole step moves q, k and v through HBM once in and once out
  * (what ksa_qkv_prepare alone costs).  Works for any lengths; results equal
- * ksa_qkv_prepare followed by ksa_attn_fwd bit for bit (same arithmetic on the same rows).
+ * ksa_qkv_prepare followed by ksa_attn_fwd bit for bit (same arithmetic on the same rows), except the
+ * summary rows of chunks of more than 12 keys, which come from another kernel: equal up to the order of sums.
  * q_main .. v_summ, lambda, rope_theta, prep_flags: as for ksa_qkv_prepare; out, lse, p, cuda_stream: as for
  * ksa_attn_fwd (KSA_FLAG_REFERENCE_KERNEL is not accepted).  workspace: DEVICE, 256-byte aligned,
  * >= ksa_prepared_workspace_bytes (the packed streams plus the prepared query rows of the summary tokens).

@@ -16,8 +16,8 @@
 //            read, with one arrival per half: the accumulations over the first halves (k-steps 0, 2, 4, 6)
 //            run beside the arithmetic of the second.  Pipe order per j: X_{j+1}, dV += P^T dO_j and
 //            dK += dS^T Q_j (even k-steps, then odd), Y_{j+1}.  At the end each key row adds dV and
-//            scale * dK to the fp32 accumulators of its stream (vector atomics: several segments and the
-//            summary-row kernel add to the same rows).
+//            scale * dK to the fp32 accumulators of its stream: vector atomics where several segments cover a key
+//            tile, plain stores where one CTA does (text keys, bwd_text_keys_stored).
 //   dQ       query-stationary: A1 = Q tile, A2 = dO tile, B1 = K tile, B2 = V tile over the visible
 //            summary tiles, then the visible text tiles (Eq. 3); X = S, Y = dP.  One accumulator leaves
 //            room for a second Y buffer (columns from 384), so both products of tile j + 1 are issued
@@ -302,8 +302,8 @@ __device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& ma
     auto fetch = [&](int qt, int g) {                                     // pair (query tile qt, head g of the group)
         const int h = hk * G + g;
         const size_t r = (size_t)h * a.text_rows + sq.text_off + (size_t)qt * 128 + 32 * cg + lane;
-        n_lse = -__ldcg(a.lse_t + r);                                     // -inf on padding rows: P = 0 there
-        n_dl = -__ldcg(a.delta_t + r);                                    // (past L1: see the launches)
+        n_lse = -(summ ? a.lse_t[r] : __ldcg(a.lse_t + r));              // -inf on padding rows: P = 0 there
+        n_dl = -(summ ? a.delta_t[r] : __ldcg(a.delta_t + r));           // (text keys: past L1, see the launches)
     };
     // loads of streamed tile j (the producer's thread)
     const bool direct = a.direct != 0;
@@ -793,12 +793,13 @@ __device__ __forceinline__ void bt_dq_block(const BwdArgs& a, const BwdMaps& map
 // The three launches -- dK / dV of the summary keys, of the text keys, dQ -- do not depend on each other: each one's CTAs take
 // the SMs that the one in front leaves (programmatic dependent launches), longest CTAs first (64, about 40 and 9 + 16 tiles
 // each at 32,768 tokens), so that the tails of the first two are filled (training layer of 7,942 ragged tokens, 16/16 heads
-// 610 -> 573 us, 2 x 8,192 tokens 2,140 -> 2,070 us; nothing at 2 x 32,768).
+// 619 -> 590 us, 2 x 8,192 tokens 2,132 -> 2,064 us; nothing at 2 x 32,768).
 // Nothing here waits for the launch in front, which was itself started behind the preparation; only the last block of each
 // waits for its end, so that the kernel behind the three, an ordinary launch, finds all of them done.  What the preparation and
 // the pack wrote stands in L2 by then, but without a wait of its own (pdl_wait) a kernel has no promise that its L1 has dropped
-// those addresses' old contents: the tiles come by TMA, lse and delta by loads that bypass L1, the sums are added in L2
-// (nothing measurable: 2 x 32,768 tokens 14.60 ms, before 14.64; a fence.acq_rel.gpu at the start instead costs 0.7 - 1.6 %).
+// those addresses' old contents: the tiles come by TMA, lse and delta by loads that bypass L1 (but in the first launch, an
+// ordinary one), the sums are added in L2.  2 x 32,768 tokens, backward alone: 9,692 us with every load through L1, 9,725 with
+// every one past it, 9,711 so; a fence.acq_rel.gpu at the start of each CTA instead costs 0.7 - 1.6 % of a training layer.
 __device__ __forceinline__ void bt_end_behind_front()
 {
     if (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1) pdl_wait();
