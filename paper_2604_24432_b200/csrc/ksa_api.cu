@@ -354,7 +354,7 @@ static bool schedule_in_range(const ksa_params* p, const HostSchedule& hs)
 static std::vector<int32_t> schedule_key(const ksa_params* p)
 {
     std::vector<int32_t> key;
-    key.reserve(p->num_seqs + 8);
+    key.reserve(p->num_seqs + 10);                                       // one more: the caller's part count
     key.push_back(p->num_seqs);
     for (int b = 0; b <= p->num_seqs; ++b) key.push_back(p->cu_text_lens[b]);
     key.push_back(p->chunk_len); key.push_back(p->summaries_per_chunk); key.push_back(p->window_chunks);
