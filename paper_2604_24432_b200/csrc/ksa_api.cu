@@ -46,7 +46,7 @@ struct ksa_ctx {
     std::shared_ptr<std::atomic<int>> arena_graphs;
     struct Aside { char* mem; std::shared_ptr<std::atomic<int>> graphs; };
     std::vector<Aside> aside;
-    cudaStream_t s_sched = nullptr;   // the uploads' stream, from the second set of lengths on (shared: upload_stream_take)
+    cudaStream_t s_sched = nullptr;   // the uploads' stream, from the first upload on (shared: upload_stream_take)
     std::vector<char> sched_bytes;    // seqs, then work, as they are uploaded
     int32_t* d_status = nullptr;
     bool timing = false;
@@ -62,9 +62,9 @@ struct ksa_ctx {
     cudaEvent_t ev_start = nullptr;
 };
 
-// The stream of the schedules' uploads: one per device, made when a first context's lengths change, gone with the last context
-// that took it.  (A stream costs 65 - 80 us to create, four times a call of 1,024 tokens: not in ksa_create, where contexts
-// that only decode or stay with their lengths would pay for it, nor once for every context.)
+// The stream of the schedules' uploads, on which they wait for no work in flight: one per device, made for a first context's first
+// upload, gone with the last context that took it.  (A stream costs 65 - 80 us to create, four times a call of 1,024 tokens: not
+// in ksa_create, where contexts that only decode would pay for it, nor once for every context.)
 namespace {
 struct UploadStream { cudaStream_t stream = nullptr; int users = 0; };
 std::mutex g_upload_mutex;
@@ -628,15 +628,14 @@ static int ensure_schedule(ksa_ctx* ctx, const ksa_params* p, bool upload, int t
         cudaError_t e;
         const size_t sb = (size_t)round_up((int64_t)(hs.seqs.size() * sizeof(SeqInfo)), 256), wb = hs.work.size() * sizeof(WorkItem);
         const size_t need = (size_t)round_up((int64_t)(sb + wb), 256);
-        const bool again = ctx->arena != nullptr;
         const int rc = arena_room(ctx, need);
         if (rc != KSA_OK) return rc;
         try { ctx->sched_bytes.resize(need); } catch (const std::bad_alloc&) { return KSA_ERR_NOMEM; }
         std::memcpy(ctx->sched_bytes.data(), hs.seqs.data(), hs.seqs.size() * sizeof(SeqInfo));
         if (wb) std::memcpy(ctx->sched_bytes.data() + sb, hs.work.data(), wb);
-        // waited for: whatever stream the caller uses next finds the schedule in place.  From the second set of lengths on the
-        // copies have a stream of their own and do not wait for kernels in flight
-        if (again && !ctx->s_sched && (e = upload_stream_take(ctx->device, &ctx->s_sched)) != cudaSuccess) return cuda_fail(ctx, e);
+        // on the uploads' stream and waited for: whatever stream the caller uses next finds the schedule in place, and the copy does
+        // not wait for kernels in flight
+        if (!ctx->s_sched && (e = upload_stream_take(ctx->device, &ctx->s_sched)) != cudaSuccess) return cuda_fail(ctx, e);
         char* dst = ctx->arena + ctx->arena_used;
         if ((e = cudaMemcpyAsync(dst, ctx->sched_bytes.data(), sb + wb, cudaMemcpyHostToDevice, ctx->s_sched)) == cudaSuccess)
             e = cudaStreamSynchronize(ctx->s_sched);

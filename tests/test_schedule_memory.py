@@ -72,19 +72,16 @@ class FakeContext:
         assert self.L.ksa_destroy(self.handle) == ksa.KSA_OK
 
 
-def test_an_upload_stream_only_where_lengths_change(fake):
-    """A context that decodes, or stays with its first lengths, takes no stream; those whose lengths change share one, which
-    goes with the last of them."""
+def test_the_upload_stream_is_made_once_and_shared(fake):
+    """A context that uploads no schedule (one that decodes) takes no stream; the others share one, which goes with the last of
+    them.  No upload waits for the default stream."""
     a, b, c = (FakeContext(fake) for _ in range(3))
     assert a.count("streams_made") == 0
-    for ctx in (a, b):
-        ctx.call([100, 37])
-        ctx.call([100, 37])
-    assert a.count("streams_made") == 0 and a.count("uploads_default") == 2
     for i in range(5):
         for ctx in (a, b):
             ctx.call([64 + i])
-    assert a.count("streams_made") == 1 and a.count("uploads_own") == 10 and a.count("uploads_default") == 2
+            ctx.call([64 + i])
+    assert a.count("streams_made") == 1 and a.count("uploads_own") == 10 and a.count("uploads_default") == 0
     assert a.count("device_syncs") == 0
     a.close()
     c.close()
