@@ -596,6 +596,15 @@ __device__ __forceinline__ void bt_dq_block(const BwdArgs& a, const BwdMaps& map
         bt_issue_tile<D>(sm.a2(), sm.bar(BB_AFULL), &maps.dot, qpos, h, direct);
         load_b2(0);
     }
+    // row warps: this thread's query row and its scalars, on their way beside the set-up
+    const int quarter = warp & 3, cg = warp >> 2;                        // lanes 32 quarter ..; columns 32 cg ..
+    const int i_w0 = i_first + quarter * 32, i = i_w0 + lane;
+    float lse2 = 0.f, dl = 0.f;
+    if (warp < 16) {
+        const size_t r = (size_t)h * a.text_rows + sq.text_off + i;
+        lse2 = __ldcg(a.lse_t + r);                                      // +inf / 0 on padding rows: P = 0 there
+        dl = __ldcg(a.delta_t + r);                                      // (past L1: see the launches)
+    }
     bt_ready(sm, warp);
     const uint32_t tmem = bt_ld_shared(sm.tmem_slot());
     const uint32_t tX = tmem, tDQ = tmem + 256u;
@@ -662,12 +671,8 @@ __device__ __forceinline__ void bt_dq_block(const BwdArgs& a, const BwdMaps& map
         tc_commit_warp(leader, su.bar(BB_OFULL));
     } else {
         // =============================== query rows =================================
-        const int quarter = warp & 3, cg = warp >> 2;                    // lanes 32 quarter ..; columns 32 cg ..
         const uint32_t lane_sel = (uint32_t)(quarter * 32) << 16;
         const uint32_t tXc = tX + lane_sel + cg * 32;                     // this warp's 32 x 32 block
-        const int i_w0 = i_first + quarter * 32, i = i_w0 + lane;         // this thread's query row
-        const size_t r = (size_t)h * a.text_rows + sq.text_off + i;
-        const float lse2 = __ldcg(a.lse_t + r), dl = __ldcg(a.delta_t + r);      // +inf / 0 on padding rows: P = 0 there
         const int iq = i / a.k, iq_w0 = i_w0 / a.k, iq_w1 = (i_w0 + 31) / a.k;
         bool alive = true;
         // The chunk of the block's first key, kc0 = key0 + 32 cg, is kept as quotient and remainder by the keys per
@@ -799,7 +804,8 @@ __device__ __forceinline__ void bt_dq_block(const BwdArgs& a, const BwdMaps& map
 // the pack wrote stands in L2 by then, but without a wait of its own (pdl_wait) a kernel has no promise that its L1 has dropped
 // those addresses' old contents: the tiles come by TMA, lse and delta by loads that bypass L1 (but in the first launch, an
 // ordinary one), the sums are added in L2.  2 x 32,768 tokens, backward alone: 9,692 us with every load through L1, 9,725 with
-// every one past it, 9,711 so; a fence.acq_rel.gpu at the start of each CTA instead costs 0.7 - 1.6 % of a training layer.
+// every one past it, 9,711 so, and another 16 less with dQ's rows on their way beside the set-up; a fence.acq_rel.gpu at the
+// start of each CTA instead costs 0.7 - 1.6 % of a training layer.
 __device__ __forceinline__ void bt_end_behind_front()
 {
     if (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1) pdl_wait();
