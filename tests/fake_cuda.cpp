@@ -15,7 +15,6 @@ namespace {
 struct Counts { int streams_made, streams_gone, mallocs, frees, device_syncs, uploads_default, uploads_own; };
 Counts g_n{};
 const ksa::SeqInfo* g_seqs = nullptr;
-int g_num_seqs = 0;
 struct Retained { void* graph; cudaHostFn_t destroy; void* ptr; };
 std::vector<Retained> g_retained;
 void* g_graph = nullptr;                                 // the graph that calls are recorded into, null: none
@@ -30,14 +29,14 @@ FAKE void fake_graph_destroy(void* graph)
             g_retained.erase(g_retained.begin() + (long)i);
         }
 }
-// what the last ksa_qkv_prepare was launched with
 FAKE Counts fake_counts() { return g_n; }
+// the schedule that the last ksa_qkv_prepare was launched with
 FAKE const void* fake_seqs() { return g_seqs; }
 FAKE int fake_seqs_text(const void* seqs, int i) { return static_cast<const ksa::SeqInfo*>(seqs)[i].n_text; }
 
-cudaError_t ksa::launch_prep(const PrepArgs& a, int64_t, int num_seqs, cudaStream_t)
+cudaError_t ksa::launch_prep(const PrepArgs& a, int64_t, int, cudaStream_t)
 {
-    g_seqs = a.seqs; g_num_seqs = num_seqs;
+    g_seqs = a.seqs;
     return cudaSuccess;
 }
 
