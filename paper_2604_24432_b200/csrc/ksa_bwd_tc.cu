@@ -24,11 +24,17 @@
 //            as soon as the warps have read X_j, and the warps never wait for the pipe: order per j:
 //            X_{j+1}, Y_{j+1}, dQ += dS K_j.  At the end scale * dQ goes to the caller's tensor as bf16.
 //
+// A CTA (one per SM) works through many units -- a key tile with a segment of query tiles, or a query tile of one head -- one
+// after the other; see "the units of a CTA" below.  The streams of tiles run on across units: stages, barriers and the Y buffers
+// are counted over all tiles of the CTA, and the next unit's loads and first products run beside the last unit's epilogue.
+//
 // Warps 0-15: one accumulator row per thread, four warps per row quarter (warps w, w + 4, w + 8, w + 12
 // share the lanes 32 (w % 4) ..; each takes 32 of the 128 columns: the element-wise work has no reduction
 // across columns, and four warps per scheduler hide the TMEM load / store latencies); warp 16: TMA
-// producer; warp 17: MMA issuer, a converged warp of which one lane issues (operands in uniform registers:
-// from inside an `if (lane == 0)` region the instruction stream, not the tensor pipe, set the rate).  The
+// producer and the unit descriptors; warp 17: MMA issuer, a converged warp of which one lane issues; warps 18, 19 only make the
+// fifth warpgroup whole, for the register hand-over.  Role, loop counts and waits are known to the compiler as the same in all
+// lanes (votes and reductions of the warp), so that addresses, descriptors and loop control stay in uniform registers: with the
+// warp number as threadIdx.x / 32 and waits of single lanes the two kernels took 12 - 14 % longer.  The
 // tensor pipe works in order, so the completion of a product also tells which stage the accumulation before it
 // has finished with: in the dQ kernel row warp 0, which sees every completion of X and Y, passes that on to
 // the producer through one "empty" barrier per stage (except for the K stages, which the early products would
@@ -37,13 +43,14 @@
 // shared barrier cannot follow: hence one barrier per stage.)  Every mbarrier wait is bounded (status word +
 // CTA-wide abort flag).
 //
-// What bounds them: the row warps.  Two sequences of 32,768 tokens, 32/8 heads: a 128 x 128 tile takes 3,000 cycles
-// in the dK / dV kernel and 1,950 in the dQ kernel (2,600 before: issuing thread in a divergent region, releasing
-// arrivals, scalar fp32), 1,024 of them exponentials on the special-function unit; the issuer waits for the
-// row warps 1,400 / 670 of them.  Whole backward call 12.5 -> 11.4 ms.  A CTA's start and end cost the dQ kernel some 10,000
-// cycles (16 tiles at 16,384 tokens): 1,600 until the next CTA is there, 4,600 until the first products are under way (the
-// producer's loads start beside the rest of the set-up), 3,800 for the last product and the epilogue, whose stores take
-// four lanes a row (dQ 732 -> 723 us) or go to accumulators laid out for them (dK / dV of the text keys 575 -> 539 us).
+// What bounds them: the row warps and the shared-memory reads of the products (X and Y read both operands from there: 160 KB a
+// tile of dQ and 192 KB of dK / dV beside 64 KB that TMA writes, at 128 bytes a cycle).  Thousand cycles of 148 SMs, a CTA per
+// unit -> CTAs that stay: 2 x 8,192 tokens in 64 + 8 chunks, 32/8 heads: dQ 961 -> 810, dK / dV 454 + 878 -> 388 + 752; 7,942
+// ragged tokens, 16/16 heads: 206 -> 155, 77 + 270 -> 70 + 217.  A training layer 2,107 -> 1,983 us, 585 -> 548 us; 2 x 32,768
+// tokens 14.5 -> 13.9 ms (power cap).  A unit's end costs about 3,500 cycles (last product, epilogue, first loads of the next
+// unit's scalars) where the end of a CTA and the start of the next took some 10,000.  The scalars of the next tile
+// are negated when they are stored and not beside their load, which stalled every tile of dK / dV for it (5 - 7 %).
+// Tried and taken back: a second issuing warp (dQ 811 -> 841), the Q / K stage checked a tile ahead (759 -> 943).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -56,8 +63,10 @@ namespace ksa {
 
 using namespace ptx;
 
-constexpr int kBwdTcThreads = 576;
-constexpr int kBwdTcRegs = 96;                  // 18 warps: five on a scheduler, 5 x 32 x 96 registers fit its file
+constexpr int kBwdTcThreads = 640;              // five warpgroups
+constexpr int kBwdTcRegs = 96;                  // five warps on a scheduler, 5 x 32 x 96 registers fit its file
+constexpr int kBwdRegsRows = 104, kBwdRegsOther = 64;        // after the hand-over
+static_assert(16 * kBwdRegsRows + 4 * kBwdRegsOther <= 20 * kBwdTcRegs, "register hand-over exceeds the CTA's allocation");
 constexpr int kBwdSegPairs = 64;                // dK / dV: (query tile, query head) pairs per CTA, at least 16 query tiles
 constexpr int kB1Stages = 3, kB2Stages = 2;
 
@@ -66,17 +75,21 @@ template <int D>
 struct BtMap {
     static constexpr int kTile = 128 * D * 2;   // one 128 x D bf16 tile: [64-element half of d][128 rows][128 B]
     static constexpr int kOffA1 = 0, kOffA2 = kTile, kOffB1 = 2 * kTile, kOffB2 = kOffB1 + kB1Stages * kTile;
-    static constexpr int kOffBars = kOffB2 + kB2Stages * kTile;                        // 18 barriers
-    static constexpr int kOffMisc = kOffBars + 192;                                    // TMEM slot, abort flags
+    static constexpr int kOffBars = kOffB2 + kB2Stages * kTile;                        // 25 barriers
+    static constexpr int kOffMisc = kOffBars + 256;                                    // TMEM slot, abort flags, next block
     static constexpr int kOffRow = kOffMisc + 64;                                      // dK / dV: [2][lse, delta][128] per-query scalars
-    static constexpr int kLayoutBytes = kOffRow + 2 * 2 * 128 * 4;
-    // head_dim 128: the whole opt-in window (the layout needs all but 768 bytes of it); 64: the layout and the slack
+    static constexpr int kOffUnit = kOffRow + 2 * 2 * 128 * 4;                         // two unit descriptors of 64 bytes
+    static constexpr int kLayoutBytes = kOffUnit + 128;
+    // head_dim 128: the whole opt-in window (the layout needs all but 576 bytes of it); 64: the layout and the slack
     // for its 1024-byte alignment
     static constexpr int kSmem = D == 128 ? 232448 : kLayoutBytes + 1024;
     static_assert(kLayoutBytes <= kSmem, "shared memory layout");
 };
 enum : int { BB_AFULL = 0, BB_B1FULL = 1, BB_B2FULL = 4, BB_XFULL = 6, BB_YFULL = 7, BB_PA = 8, BB_PB = 9, BB_OFULL = 10,
-             BB_B1EMPTY = 11, BB_B2EMPTY = 14, BB_YFULL2 = 16, BB_PB2 = 17 };
+             BB_B1EMPTY = 11, BB_B2EMPTY = 14, BB_YFULL2 = 16, BB_PB2 = 17,
+             BB_AEMPTY = 18, BB_UFULL = 19, BB_UEMPTY = 21, BB_CLC = 23, BB_DRAIN = 24 };
+// words of a unit descriptor
+enum : int { U_J = 0, U_TEXT_OFF = 1, U_TILE = 2, U_HEAD = 3, U_A = 4, U_B = 5, U_C = 6, U_AUG = 8 };
 
 __device__ __forceinline__ uint32_t bt_ld_shared(uint32_t addr)
 {
@@ -104,12 +117,23 @@ __device__ __forceinline__ bool bt_wait(uint32_t bar, uint32_t parity, uint32_t 
         }
     }
 }
-// One lane polls for the warp (hundreds of polling threads would crowd the barrier unit).
-__device__ __forceinline__ bool bt_wait_warp(uint32_t bar, uint32_t parity, uint32_t abort_addr, int32_t* status, int code, int lane)
+// A converged warp waits, every branch on a vote of the whole warp: after a wait of each lane, or of one lane, for itself the
+// compiler no longer takes the warp for converged (dK / dV 822 -> 759 thousand cycles; cases of the head comment)
+__device__ __forceinline__ bool bt_wait_converged(uint32_t bar, uint32_t parity, uint32_t abort_addr, int32_t* status, int code)
 {
-    bool ok = true;
-    if (lane == 0) ok = bt_wait(bar, parity, abort_addr, status, code);
-    return __shfl_sync(0xffffffffu, ok, 0);
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const long long t0 = clock64();
+    for (uint32_t it = 1;; ++it) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if ((it & 63u) == 0u) {
+            if (__any_sync(0xffffffffu, bt_ld_shared(abort_addr) != 0u)) return false;
+            if (__any_sync(0xffffffffu, clock64() - t0 > (1ll << 31))) {
+                atomicCAS(status, 0, code);
+                bt_st_shared(abort_addr, 1u);
+                return false;
+            }
+        }
+    }
 }
 
 // Shared-memory layout and barrier addresses of one CTA.
@@ -124,6 +148,8 @@ struct BtSmem {
     __device__ __forceinline__ uint32_t bar(int i) const { return base + M::kOffBars + 8u * (uint32_t)i; }
     __device__ __forceinline__ uint32_t tmem_slot() const { return base + M::kOffMisc; }
     __device__ __forceinline__ uint32_t abort_addr() const { return base + M::kOffMisc + 4; }
+    __device__ __forceinline__ uint32_t next_block() const { return base + M::kOffMisc + 16; }
+    __device__ __forceinline__ uint32_t unit(int n, int word) const { return base + M::kOffUnit + (uint32_t)(n & 1) * 64u + 4u * (uint32_t)word; }
 };
 
 // The layout starts on the first 1024-byte boundary of the dynamic window; false (and a status code) if it
@@ -155,6 +181,10 @@ __device__ __forceinline__ void bt_init_barriers(const BtSmem<D>& sm)
     mbar_init(sm.bar(BB_PB), 16);
     mbar_init(sm.bar(BB_PB2), 16);
     mbar_init(sm.bar(BB_OFULL), 1);
+    mbar_init(sm.bar(BB_AEMPTY), 1);
+    for (int s = 0; s < 2; ++s) { mbar_init(sm.bar(BB_UFULL + s), 1); mbar_init(sm.bar(BB_UEMPTY + s), 17); }   // read by 16 row warps and two issuers
+    mbar_init(sm.bar(BB_CLC), 1);
+    mbar_init(sm.bar(BB_DRAIN), 1);
     bt_st_shared(sm.abort_addr(), 0u);
     bt_st_shared(sm.abort_addr() + 4, 0u);
     fence_mbar_init();
@@ -229,12 +259,14 @@ __device__ __forceinline__ void bt_load_tile(uint32_t dst, uint32_t bar, const C
     bt_issue_tile<D>(dst, bar, map, pos, head, direct);
 }
 // After an abort: leave no copy in flight.  Bounded waits (the second flag is never set) for the last fill of
-// every stage; filled1 / filled2 = B1 / B2 tiles whose load was issued.
+// every stage; filled_a / filled1 / filled2 = A pairs / B1 / B2 tiles whose load was issued; asked = requests for a block that
+// were answered, pending: one more is on its way.
 template <int D>
-__device__ __forceinline__ void bt_drain(const BtSmem<D>& sm, int filled1, int filled2, int32_t* status)
+__device__ __forceinline__ void bt_drain(const BtSmem<D>& sm, int filled_a, int filled1, int filled2, bool pending, int asked, int32_t* status)
 {
     const uint32_t never = sm.abort_addr() + 4;
-    bt_wait(sm.bar(BB_AFULL), 0, never, status, kStatusWaitKvFull);
+    if (pending) bt_wait(sm.bar(BB_CLC), (uint32_t)(asked & 1), never, status, kStatusWaitNextBlock);
+    if (filled_a > 0) bt_wait(sm.bar(BB_AFULL), (uint32_t)((filled_a - 1) & 1), never, status, kStatusWaitKvFull);
     for (int s = 0; s < kB1Stages; ++s) {
         const int fills = (filled1 + kB1Stages - 1 - s) / kB1Stages;     // tiles j < filled1 with j % 3 == s
         if (fills > 0) bt_wait(sm.bar(BB_B1FULL + s), (uint32_t)((fills - 1) & 1), never, status, kStatusWaitQFull);
@@ -245,7 +277,15 @@ __device__ __forceinline__ void bt_drain(const BtSmem<D>& sm, int filled1, int f
     }
 }
 
-// Stage `stage` (of `stages`) is about to take tile j: wait until its previous tile (j - stages) was released.
+// The issuer's end: no product is in flight when TMEM is freed (after an abort, too).
+template <int D>
+__device__ __forceinline__ void bt_drain_pipe(uint32_t leader, const BtSmem<D>& su, int32_t* status)
+{
+    tc_commit_warp(leader, su.bar(BB_DRAIN));
+    bt_wait(su.bar(BB_DRAIN), 0, su.abort_addr() + 4, status, kStatusWaitOFull);
+}
+
+// A stage is about to take tile j of the CTA (tiles are counted over its units): wait until its previous tile was released.
 template <int D>
 __device__ __forceinline__ bool bt_stage_free(const BtSmem<D>& sm, int empty0, int stages, int j, int32_t* status)
 {
@@ -253,275 +293,388 @@ __device__ __forceinline__ bool bt_stage_free(const BtSmem<D>& sm, int empty0, i
     return bt_wait(sm.bar(empty0 + j % stages), (uint32_t)((j / stages - 1) & 1), sm.abort_addr(), status, kStatusWaitQEmpty);
 }
 
+// ---- the units of a CTA ---------------------------------------------------------------------------
+// The grid has a block for every unit of work, and a CTA that is through with its own unit takes over the next block that has
+// not started (cluster launch control: the block is cancelled, its index comes back through shared memory) until none is left.
+// The producer's thread does that, works out what the unit is, and hands it to the other warps as a descriptor in shared memory
+// (two slots); J = 0 ends the CTA.
+struct BtBlock { int x, y, z; };
+template <int D>
+__device__ __forceinline__ void bt_request_block(const BtSmem<D>& sm)
+{
+    fence_proxy_async();                                                  // the slot was read by this thread
+    mbar_arrive_expect_tx(sm.bar(BB_CLC), 16u);
+    clc_try_cancel(sm.next_block(), sm.bar(BB_CLC));
+}
+// The answer to request number `n` of the CTA: 1 and the block, 0 if none was left (nothing is asked for after that), -1 if the
+// wait gave up.
+template <int D>
+__device__ __forceinline__ int bt_take_block(const BtSmem<D>& sm, int n, BtBlock& blk, int32_t* status)
+{
+    if (!bt_wait(sm.bar(BB_CLC), (uint32_t)(n & 1), sm.abort_addr(), status, kStatusWaitNextBlock)) return -1;
+    return clc_query(sm.next_block(), blk.x, blk.y, blk.z) ? 1 : 0;
+}
+// A word of descriptor n for a whole warp, known to the compiler as the same in every lane: loop counts and addresses that come
+// of it stay in uniform registers.
+template <int D>
+__device__ __forceinline__ int bt_unit_word(const BtSmem<D>& sm, int n, int word)
+{
+    return (int)__reduce_or_sync(0xffffffffu, bt_ld_shared(sm.unit(n, word)));
+}
+// The producer's side of the slots: descriptor n may be written / has been written.
+template <int D>
+__device__ __forceinline__ bool bt_unit_free(const BtSmem<D>& sm, int n, int32_t* status)
+{
+    if (n < 2) return true;
+    return bt_wait(sm.bar(BB_UEMPTY + (n & 1)), (uint32_t)(((n >> 1) - 1) & 1), sm.abort_addr(), status, kStatusWaitUnit);
+}
+
 // =====================================================================================================
 // dK / dV
 // =====================================================================================================
-template <int D>
-__device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& maps, const int summ, const int seg_tiles, const int store)
+// A unit: one key tile, one KV head, a segment of the query tiles that see the keys.  Block (x, y): segment x % segs of key tile
+// x / segs of the packed stream (its rows are numbered over all sequences), KV head y.  (Segments first: the units in flight
+// then share their query tiles.  Tiles first, the launch over the summary keys at 32,768 tokens read them from memory again and
+// again and took 4,060 instead of 3,390 us.)
+struct BtDkvUnit { int J, kt, hk, seg0, n_keys, krow0, text_off, chunk0; };
+__device__ __forceinline__ bool bt_dkv_unit(const BwdArgs& a, const BtBlock& blk, const int summ, const int seg_tiles, const int segs, BtDkvUnit& u)
 {
-    extern __shared__ uint8_t bsm_raw[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-    // ---- which keys, which queries (Eq. 3) ------------------------------------------------------
-    const int G = a.Hq / a.Hkv;
-    const int hk = blockIdx.z % a.Hkv, b = blockIdx.z / a.Hkv;
-    const SeqInfo sq = a.seqs[b];
-    const int kt = blockIdx.y;
-    const int n_keys = summ ? sq.n_summ : sq.n_text;
-    if (kt * 128 >= n_keys) return;
+    const int tile = blk.x / segs;
+    const SeqInfo sq = a.seqs[seq_of_row(a.seqs, a.num_seqs, tile * 128, !summ)];
+    u.krow0 = tile * 128;
+    u.kt = tile - (summ ? sq.summ_off : sq.text_off) / 128;
+    u.hk = blk.y;
+    u.n_keys = summ ? sq.n_summ : sq.n_text;
+    u.text_off = sq.text_off; u.chunk0 = sq.chunk0;
+    if (u.kt * 128 >= u.n_keys) return false;
     const int n_qt = (sq.n_text + 127) / 128;
-    int qt_lo, qt_hi;
+    int qt_lo, qt_hi;                                                     // the query tiles that see the keys (Eq. 3)
     if (!summ) {
-        const int key_last = min(n_keys, kt * 128 + 128) - 1;
-        qt_lo = kt;
+        const int key_last = min(u.n_keys, u.kt * 128 + 128) - 1;
+        qt_lo = u.kt;
         const long long i_max = ((long long)(key_last / a.k) + a.C + 1) * a.k - 1;
         qt_hi = (int)min((long long)(n_qt - 1), i_max / 128);
     } else {
-        const long long i_min = ((long long)(kt * 128) / a.m + 1 + a.C) * a.k;     // first row that sees summary kt*128
-        if (i_min >= sq.n_text) return;
+        const long long i_min = ((long long)(u.kt * 128) / a.m + 1 + a.C) * a.k;     // first row that sees summary kt*128
+        if (i_min >= sq.n_text) return false;
         qt_lo = (int)(i_min / 128);
         qt_hi = n_qt - 1;
     }
-    const int seg0 = qt_lo + (int)blockIdx.x * seg_tiles;
-    if (seg0 > qt_hi) return;
-    const int seg1 = min(qt_hi + 1, seg0 + seg_tiles);
-    const int J = (seg1 - seg0) * G;                                      // streamed tiles: (query tile, query head) pairs
-    const int krow0 = (summ ? sq.summ_off : sq.text_off) + kt * 128;      // first row of the key tile in its packed stream
-    auto pair_of = [&](int j, int& qt, int& h) { qt = seg0 + j / G; h = hk * G + j % G; };
+    u.seg0 = qt_lo + (blk.x - tile * segs) * seg_tiles;
+    if (u.seg0 > qt_hi) return false;
+    u.J = (min(qt_hi + 1, u.seg0 + seg_tiles) - u.seg0) * (a.Hq / a.Hkv);            // streamed tiles: (query tile, query head) pairs
+    return true;
+}
 
+template <int D>
+__device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& maps, const int summ, const int seg_tiles, const int segs, const int store)
+{
+    extern __shared__ uint8_t bsm_raw[];
+    const int warp = (int)__reduce_or_sync(0xffffffffu, threadIdx.x >> 5), lane = threadIdx.x & 31;       // (uniform to the compiler)
+    const int G = a.Hq / a.Hkv;
     BtSmem<D> sm;
     if (!bt_layout(sm, bsm_raw, a.status)) return;
-    uint8_t* base_ptr = bsm_raw + (sm.base - smem_u32(bsm_raw));
-    // per-query scalars of the streamed tile, negated, double-buffered by j: [j & 1][lse, delta][128 columns]; every row
-    // warp writes the 32 columns it reads itself, one tile ahead (the four warps of a column group write the same
-    // values, and each relies on its own writes only), see below
-    float* rows = reinterpret_cast<float*>(base_ptr + BtMap<D>::kOffRow);
-    const int quarter = warp & 3, cg = warp >> 2;                        // row warps: lanes 32 quarter ..; columns 32 cg ..
-    const bool scalar_writer = warp < 16 && quarter == 0;
-    float n_lse = 0.f, n_dl = 0.f;                                        // the writer lane's values for the next tile
-    auto fetch = [&](int qt, int g) {                                     // pair (query tile qt, head g of the group)
-        const int h = hk * G + g;
-        const size_t r = (size_t)h * a.text_rows + sq.text_off + (size_t)qt * 128 + 32 * cg + lane;
-        n_lse = -(summ ? a.lse_t[r] : __ldcg(a.lse_t + r));              // -inf on padding rows: P = 0 there
-        n_dl = -(summ ? a.delta_t[r] : __ldcg(a.delta_t + r));           // (text keys: past L1, see the launches)
-    };
-    // loads of streamed tile j (the producer's thread)
+
+    // ---- the producer's thread: descriptor and loads of a unit ------------------------------------
     const bool direct = a.direct != 0;
-    auto load_b1 = [&](int j) {
-        int qt, h;
-        pair_of(j, qt, h);
-        bt_load_tile<D>(sm.b1(j % kB1Stages), sm.bar(BB_B1FULL + j % kB1Stages), &maps.qt,
-                        direct ? sq.chunk0 + qt * (128 / a.k) : sq.text_off + qt * 128, h, direct);
+    BtDkvUnit u{};
+    bool started = false;                                                 // unit 0: described, first tile on its way
+    auto publish = [&](int n) {
+        bt_st_shared(sm.unit(n, U_TEXT_OFF), (uint32_t)u.text_off); bt_st_shared(sm.unit(n, U_TILE), (uint32_t)u.kt);
+        bt_st_shared(sm.unit(n, U_HEAD), (uint32_t)u.hk); bt_st_shared(sm.unit(n, U_A), (uint32_t)u.seg0);
+        bt_st_shared(sm.unit(n, U_B), (uint32_t)u.n_keys); bt_st_shared(sm.unit(n, U_C), (uint32_t)u.krow0);
+        bt_st_shared(sm.unit(n, U_J), (uint32_t)u.J);
+        mbar_arrive(sm.bar(BB_UFULL + (n & 1)));
     };
-    auto load_b2 = [&](int j) {
-        int qt, h;
-        pair_of(j, qt, h);
-        bt_load_tile<D>(sm.b2(j & 1), sm.bar(BB_B2FULL + (j & 1)), &maps.dot,
-                        direct ? sq.chunk0 + qt * (128 / a.k) : sq.text_off + qt * 128, h, direct);
+    auto load_a = [&]() {                                                 // K and V tile
+        mbar_arrive_expect_tx(sm.bar(BB_AFULL), 2u * BtMap<D>::kTile);
+        const int kpos = direct ? u.chunk0 + u.kt * (128 / (summ ? a.m : a.k)) : u.krow0;
+        bt_issue_tile<D>(sm.a1(), sm.bar(BB_AFULL), summ ? &maps.ks : &maps.kt, kpos, u.hk, direct);
+        bt_issue_tile<D>(sm.a2(), sm.bar(BB_AFULL), summ ? &maps.vs : &maps.vt, kpos, u.hk, direct);
+    };
+    auto load_b = [&](int j, uint32_t dst, uint32_t bar, const CUtensorMap* map) {   // pair (query tile, head of the group) j
+        const int qt = u.seg0 + j / G;
+        bt_load_tile<D>(dst, bar, map, direct ? u.chunk0 + qt * (128 / a.k) : u.text_off + qt * 128, u.hk * G + j % G, direct);
     };
     if (warp == 16 && lane == 0) {
         bt_init_barriers(sm);
-        mbar_arrive_expect_tx(sm.bar(BB_AFULL), 2u * BtMap<D>::kTile);
-        const int kpos = direct ? sq.chunk0 + kt * (128 / (summ ? a.m : a.k)) : krow0;
-        bt_issue_tile<D>(sm.a1(), sm.bar(BB_AFULL), summ ? &maps.ks : &maps.kt, kpos, hk, direct);
-        load_b1(0);
-        bt_issue_tile<D>(sm.a2(), sm.bar(BB_AFULL), summ ? &maps.vs : &maps.vt, kpos, hk, direct);
-        load_b2(0);
-    }
-    if (scalar_writer) {                                                  // tile 0: visible to all after the first barrier
-        fetch(seg0, 0);
-        rows[32 * cg + lane] = n_lse;
-        rows[128 + 32 * cg + lane] = n_dl;
+        started = bt_dkv_unit(a, BtBlock{(int)blockIdx.x, (int)blockIdx.y, 0}, summ, seg_tiles, segs, u);
+        if (started) {
+            load_b(0, sm.b1(0), sm.bar(BB_B1FULL), &maps.qt);
+            load_a();
+            load_b(0, sm.b2(0), sm.bar(BB_B2FULL), &maps.dot);
+            publish(0);
+        }
     }
     bt_ready(sm, warp);
     const uint32_t tmem = bt_ld_shared(sm.tmem_slot());
     const uint32_t tX = tmem, tY = tmem + 128u, tDV = tmem + 256u, tDK = tmem + 384u;
 
-    if (warp == 16) {
-        // =============================== TMA producer ===============================
-        if (lane == 0) {
-            int filled1 = 1, filled2 = 1;                                 // tile 0 is on its way
-            for (int j = 1; j < J; ++j) {
-                if (!bt_stage_free(sm, BB_B1EMPTY, kB1Stages, j, a.status)) break;
-                load_b1(j);
-                ++filled1;
-                if (!bt_stage_free(sm, BB_B2EMPTY, kB2Stages, j, a.status)) break;
-                load_b2(j);
-                ++filled2;
+    if (warp >= 16) {
+        setmaxnreg_dec<kBwdRegsOther>();
+        if (warp == 16) { if (lane == 0) {
+            // =============================== TMA producer ===============================
+            int na = started ? 1 : 0, g1 = na, g2 = na, asked = 0;        // A pairs, B1 and B2 tiles loaded; answered requests
+            bool alive = true, pending = false, took_first = false;      // ... the grid's first block among them
+            for (int n = 0; alive; ++n) {
+                if (!started) {                                           // the next block that holds work
+                    u.J = 0;
+                    for (;;) {
+                        if (!pending) { bt_request_block(sm); pending = true; }
+                        BtBlock blk;
+                        const int got = bt_take_block(sm, asked, blk, a.status);
+                        if (got < 0) { alive = false; break; }
+                        ++asked; pending = false;
+                        took_first |= got > 0 && blk.x + blk.y == 0;
+                        if (got == 0 || bt_dkv_unit(a, blk, summ, seg_tiles, segs, u)) break;
+                        u.J = 0;
+                    }
+                    if (!alive || !bt_unit_free(sm, n, a.status)) { alive = false; break; }
+                    publish(n);
+                    if (u.J == 0) break;                                  // none left: the CTA ends
+                }
+                for (int j = started ? 1 : 0; j < u.J; ++j) {
+                    if (j + 1 == u.J) { bt_request_block(sm); pending = true; }          // comes while the stages are waited for
+                    if (!bt_stage_free(sm, BB_B1EMPTY, kB1Stages, g1, a.status)) { alive = false; break; }
+                    load_b(j, sm.b1(g1 % kB1Stages), sm.bar(BB_B1FULL + g1 % kB1Stages), &maps.qt);
+                    ++g1;
+                    if (j == 0) {                                         // the unit before has formed its last products
+                        if (na > 0 && !bt_wait(sm.bar(BB_AEMPTY), (uint32_t)((na - 1) & 1), sm.abort_addr(), a.status, kStatusWaitQEmpty)) { alive = false; break; }
+                        load_a();
+                        ++na;
+                    }
+                    if (!bt_stage_free(sm, BB_B2EMPTY, kB2Stages, g2, a.status)) { alive = false; break; }
+                    load_b(j, sm.b2(g2 & 1), sm.bar(BB_B2FULL + (g2 & 1)), &maps.dot);
+                    ++g2;
+                }
+                started = false;
             }
-            if (bt_ld_shared(sm.abort_addr()) != 0u) bt_drain(sm, filled1, filled2, a.status);
-        }
-    } else if (warp == 17) {
-        // =============================== MMA issuer =================================
-        // the whole warp walks the loop on warp-uniform values, one lane issues
-        const uint32_t leader = elect_one();
-        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0), base = __shfl_sync(0xffffffffu, sm.base, 0);
-        const int Ju = __shfl_sync(0xffffffffu, J, 0);
-        const BtSmem<D> su{base};
-        const uint32_t uX = tm, uY = tm + 128u, uDV = tm + 256u, uDK = tm + 384u;
-        auto wait = [&](uint32_t bar, uint32_t parity, int code) -> bool {
-            return __all_sync(0xffffffffu, bt_wait(bar, parity, su.abort_addr(), a.status, code));
-        };
-        bool alive = wait(su.bar(BB_AFULL), 0, kStatusWaitKvFull);
-        if (alive) alive = wait(su.bar(BB_B1FULL), 0, kStatusWaitQFull);
-        if (alive) { bt_product<D>(leader, uX, su.a1(), su.b1(0)); tc_commit_warp(leader, su.bar(BB_XFULL)); }
-        if (alive) alive = wait(su.bar(BB_B2FULL), 0, kStatusWaitQFull);
-        if (alive) { bt_product<D>(leader, uY, su.a2(), su.b2(0)); tc_commit_warp(leader, su.bar(BB_YFULL)); }
-        int s1 = 0;                                            // j % kB1Stages
-        uint32_t b1_phase = 0;                                 // parity of tile j + 1's fill of its stage
-        for (int j = 0; j < Ju && alive; ++j) {
-            const int s1n = s1 + 1 == kB1Stages ? 0 : s1 + 1;
-            if (s1n == 0) b1_phase ^= 1u;
-            if (j + 1 < Ju && !wait(su.bar(BB_B1FULL + s1n), b1_phase, kStatusWaitQFull)) break;
-            // the warps hold X_j in registers: the next S^T product may overwrite it while they exponentiate
-            if (!wait(su.bar(BB_PA), j & 1, kStatusWaitPFull)) break;
-            tc_fence_after();
-            if (j + 1 < Ju) {
-                bt_product<D>(leader, uX, su.a1(), su.b1(s1n));
+            if (bt_ld_shared(sm.abort_addr()) != 0u) bt_drain(sm, na, g1, g2, pending, asked, a.status);
+            if (took_first) pdl_wait();                                    // (see the launches)
+        } } else if (warp == 17) {
+            // =============================== MMA issuer =================================
+            // the whole warp walks the loop on warp-uniform values, one lane issues
+            const uint32_t leader = elect_one();
+            const uint32_t tm = __reduce_or_sync(0xffffffffu, tmem), base = __reduce_or_sync(0xffffffffu, sm.base);
+            const BtSmem<D> su{base};
+            const uint32_t uX = tm, uY = tm + 128u, uDV = tm + 256u, uDK = tm + 384u;
+            auto wait = [&](uint32_t bar, uint32_t parity, int code) -> bool {
+                return bt_wait_converged(bar, parity, su.abort_addr(), a.status, code);
+            };
+            bool alive = true;
+            int g = 0, s1 = 0;                                            // tiles of the units before; the next tile's B1 stage ...
+            uint32_t b1_phase = 0;                                        // ... and the parity of its fill
+            for (int n = 0; alive; ++n) {
+                if (!wait(su.bar(BB_UFULL + (n & 1)), (n >> 1) & 1, kStatusWaitUnit)) break;
+                const int Ju = bt_unit_word(su, n, U_J);
+                mbar_arrive_warp(leader, su.bar(BB_UEMPTY + (n & 1)));
+                if (Ju == 0) break;
+                alive = wait(su.bar(BB_AFULL), n & 1, kStatusWaitKvFull) && wait(su.bar(BB_B1FULL + s1), b1_phase, kStatusWaitQFull);
+                if (!alive) break;
+                // (X and Y are free: every row warp has handed over the last tile of the unit before)
+                bt_product<D>(leader, uX, su.a1(), su.b1(s1));
                 tc_commit_warp(leader, su.bar(BB_XFULL));
+                if (!wait(su.bar(BB_B2FULL + (g & 1)), (g >> 1) & 1, kStatusWaitQFull)) break;
+                bt_product<D>(leader, uY, su.a2(), su.b2(g & 1));
+                tc_commit_warp(leader, su.bar(BB_YFULL));
+                if (Ju == 1) tc_commit_warp(leader, su.bar(BB_AEMPTY));
+                for (int j = 0; j < Ju; ++j, ++g) {
+                    const int s1n = s1 + 1 == kB1Stages ? 0 : s1 + 1;
+                    if (s1n == 0) b1_phase ^= 1u;
+                    if (j + 1 < Ju && !(alive = wait(su.bar(BB_B1FULL + s1n), b1_phase, kStatusWaitQFull))) break;
+                    // the warps hold X_j in registers: the next S^T product may overwrite it while they exponentiate
+                    if (!(alive = wait(su.bar(BB_PA), g & 1, kStatusWaitPFull))) break;
+                    tc_fence_after();
+                    if (j + 1 < Ju) {
+                        bt_product<D>(leader, uX, su.a1(), su.b1(s1n));
+                        tc_commit_warp(leader, su.bar(BB_XFULL));
+                    }
+                    // dS^T and P^T of the first 16 queries of every block stand in Y's columns: the even k-steps
+                    if (!(alive = wait(su.bar(BB_PB), g & 1, kStatusWaitPFull))) break;
+                    tc_fence_after();
+                    bt_accumulate_half<D>(leader, uDV, uY + 8, su.b2(g & 1), 0, j == 0);            // dV += P^T dO_j
+                    bt_accumulate_half<D>(leader, uDK, uY, su.b1(s1), 0, j == 0);                   // dK += dS^T Q_j
+                    // ... the other 16: the odd k-steps
+                    if (j + 1 < Ju && !(alive = wait(su.bar(BB_B2FULL + ((g + 1) & 1)), ((g + 1) >> 1) & 1, kStatusWaitQFull))) break;
+                    if (!(alive = wait(su.bar(BB_PB2), g & 1, kStatusWaitPFull))) break;
+                    tc_fence_after();
+                    bt_accumulate_half<D>(leader, uDV, uY + 8, su.b2(g & 1), 1, false);
+                    tc_commit_warp(leader, su.bar(BB_B2EMPTY + (g & 1)));                           // ... then its dO stage is free
+                    bt_accumulate_half<D>(leader, uDK, uY, su.b1(s1), 1, false);
+                    tc_commit_warp(leader, su.bar(BB_B1EMPTY + s1));                                // ... then its Q stage is free
+                    if (j + 1 < Ju) {
+                        bt_product<D>(leader, uY, su.a2(), su.b2((g + 1) & 1));
+                        tc_commit_warp(leader, su.bar(BB_YFULL));
+                        if (j + 2 == Ju) tc_commit_warp(leader, su.bar(BB_AEMPTY));                 // K and V may make way for the next unit's
+                    }
+                    s1 = s1n;
+                }
+                if (alive) tc_commit_warp(leader, su.bar(BB_OFULL));
             }
-            // dS^T and P^T of the first 16 queries of every block stand in Y's columns: the even k-steps
-            if (!wait(su.bar(BB_PB), j & 1, kStatusWaitPFull)) break;
-            tc_fence_after();
-            bt_accumulate_half<D>(leader, uDV, uY + 8, su.b2(j & 1), 0, j == 0);            // dV += P^T dO_j
-            bt_accumulate_half<D>(leader, uDK, uY, su.b1(s1), 0, j == 0);                   // dK += dS^T Q_j
-            // ... the other 16: the odd k-steps
-            if (j + 1 < Ju && !wait(su.bar(BB_B2FULL + ((j + 1) & 1)), ((j + 1) >> 1) & 1, kStatusWaitQFull)) break;
-            if (!wait(su.bar(BB_PB2), j & 1, kStatusWaitPFull)) break;
-            tc_fence_after();
-            bt_accumulate_half<D>(leader, uDV, uY + 8, su.b2(j & 1), 1, false);
-            tc_commit_warp(leader, su.bar(BB_B2EMPTY + (j & 1)));                           // ... then its dO stage is free
-            bt_accumulate_half<D>(leader, uDK, uY, su.b1(s1), 1, false);
-            tc_commit_warp(leader, su.bar(BB_B1EMPTY + s1));                                // ... then its Q stage is free
-            if (j + 1 < Ju) { bt_product<D>(leader, uY, su.a2(), su.b2((j + 1) & 1)); tc_commit_warp(leader, su.bar(BB_YFULL)); }
-            s1 = s1n;
+            bt_drain_pipe(leader, su, a.status);
         }
-        tc_commit_warp(leader, su.bar(BB_OFULL));
     } else {
+        setmaxnreg_inc<kBwdRegsRows>();
         // =============================== key rows ===================================
+        uint8_t* base_ptr = bsm_raw + (sm.base - smem_u32(bsm_raw));
+        // per-query scalars of the streamed tile, negated, double-buffered by tile: [tile & 1][lse, delta][128 columns]; every
+        // row warp writes the 32 columns it reads itself, one tile ahead (the four warps of a column group write the same
+        // values, and each relies on its own writes only), see below
+        float* rows = reinterpret_cast<float*>(base_ptr + BtMap<D>::kOffRow);
+        const int quarter = warp & 3, cg = warp >> 2;                        // lanes 32 quarter ..; columns 32 cg ..
         const uint32_t lane_sel = (uint32_t)(quarter * 32) << 16;
         const uint32_t tXc = tX + lane_sel + cg * 32, tYc = tY + lane_sel + cg * 32;    // this warp's 32 x 32 block
-        const int key_raw = kt * 128 + quarter * 32 + lane;
-        const int key = key_raw < n_keys ? key_raw : 0x3fffffff;        // rows past the stream: never visible
-        const int kq = key / (summ ? a.m : a.k);                          // the key's chunk
-        const int kq_first = (kt * 128) / (summ ? a.m : a.k), kq_last = (kt * 128 + 127) / (summ ? a.m : a.k);
-        bool alive = true;
+        const int kdiv = summ ? a.m : a.k;
         // The streamed tiles walk the pairs (query tile, head of the group) in order; the chunk of the block's first
         // query, i0 = 128 qt + 32 cg, is kept as quotient and remainder by k and advanced by 128 per query tile
         // (integer divisions are slow, and this loop is the warps' critical path).
         const int step_q = 128 / a.k, step_r = 128 - step_q * a.k, q31 = 31 / a.k, r31 = 31 - q31 * a.k;
-        int qt = seg0, g = 0;
-        int iq0 = (seg0 * 128 + 32 * cg) / a.k, ir0 = (seg0 * 128 + 32 * cg) - iq0 * a.k;
-        for (int j = 0; j < J && alive; ++j) {
-            if (j + 1 < J) fetch(g + 1 == G ? qt + 1 : qt, g + 1 == G ? 0 : g + 1);   // lands while this tile is worked on
-            const float4* lse_c = reinterpret_cast<const float4*>(rows + (j & 1) * 256 + 32 * cg);     // this warp's 32 columns
-            const float4* dl_c = lse_c + 32;
-            const int i0 = qt * 128 + 32 * cg;                            // first query of the block
-            const int iq1 = iq0 + q31 + (ir0 + r31 >= a.k ? 1 : 0);       // chunk of the block's last query
-            // ---------------- phase A: P^T = exp2(S^T scale - lse), kept in registers ----------------
-            if (!bt_wait_warp(sm.bar(BB_XFULL), j & 1, sm.abort_addr(), a.status, kStatusWaitSFull, lane)) { alive = false; break; }
-            tc_fence_after();
-            // all pairs of the block visible / none (rows past the streams drop out by themselves: zero K / V
-            // rows are discarded at the end, padding queries have lse = +inf)
-            bool full, none;
-            if (!summ) {
-                full = kt * 128 + 127 <= i0 && iq1 - kq_first <= a.C;
-                none = kt * 128 > i0 + 31 || iq0 - kq_last > a.C;
-            } else {
-                full = iq0 - kq_last > a.C;
-                none = iq1 - kq_first <= a.C;
-            }
-            uint32_t x[32];                                               // S^T, then P^T in place (fp32 bits), kept for phase B
-            if (none) {
-#pragma unroll
-                for (int c = 0; c < 32; ++c) x[c] = 0u;
-            } else {
-                tmem_ld32(tXc, x);
-                tc_wait_ld();
-            }
-            // X_j is in registers: the issuer may start X_{j+1} while the exponentials run.  (This hand-over and those
-            // below order TMEM accesses only, which the fences and waits around them cover: relaxed arrivals.)
-            tc_fence_before();
+        int J = 0, kt = 0, hk = 0, qt = 0, text_off = 0, krow0 = 0, key = 0;       // the unit; the next pair's query tile
+        bool alive = true;
+        auto take_unit = [&](int n) -> bool {
+            if (!bt_wait_converged(sm.bar(BB_UFULL + (n & 1)), (n >> 1) & 1, sm.abort_addr(), a.status, kStatusWaitUnit)) return false;
             __syncwarp();
-            if (lane == 0) mbar_arrive_relaxed(sm.bar(BB_PA));
-            if (!none) {
-                if (full) {
-                    const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
-#pragma unroll
-                    for (int c = 0; c < 32; c += 4) {
-                        const float4 l4 = lse_c[c >> 2];
-                        const float2 t = ffma2(make_float2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])), sc2, make_float2(l4.x, l4.y));
-                        const float2 u = ffma2(make_float2(__uint_as_float(x[c + 2]), __uint_as_float(x[c + 3])), sc2, make_float2(l4.z, l4.w));
-                        x[c] = __float_as_uint(ex2_approx(t.x));
-                        x[c + 1] = __float_as_uint(ex2_approx(t.y));
-                        x[c + 2] = __float_as_uint(ex2_approx(u.x));
-                        x[c + 3] = __float_as_uint(ex2_approx(u.y));
-                    }
+            J = bt_unit_word(sm, n, U_J); text_off = bt_unit_word(sm, n, U_TEXT_OFF);
+            kt = bt_unit_word(sm, n, U_TILE); hk = bt_unit_word(sm, n, U_HEAD);
+            qt = bt_unit_word(sm, n, U_A); krow0 = bt_unit_word(sm, n, U_C);
+            const int key_raw = kt * 128 + quarter * 32 + lane;
+            key = key_raw < bt_unit_word(sm, n, U_B) ? key_raw : 0x3fffffff;      // rows past the stream: never visible
+            __syncwarp();
+            if (lane == 0) mbar_arrive(sm.bar(BB_UEMPTY + (n & 1)));
+            return true;
+        };
+        // This lane's scalars for the next tile, untouched until they are stored: the negation beside the load would wait for it
+        // there and then, in front of every tile.
+        float n_lse = 0.f, n_dl = 0.f;
+        auto fetch = [&](int qt_, int g_) {                               // pair (query tile, head of the group)
+            const size_t r = (size_t)(hk * G + g_) * a.text_rows + text_off + (size_t)qt_ * 128 + 32 * cg + lane;
+            n_lse = __ldcg(a.lse_t + r);                                 // +inf on padding rows: P = 0 there
+            n_dl = __ldcg(a.delta_t + r);                                // (past L1: see the launches)
+        };
+        auto put_scalars = [&](int tile) {
+            rows[(tile & 1) * 256 + 32 * cg + lane] = -n_lse;
+            rows[(tile & 1) * 256 + 128 + 32 * cg + lane] = -n_dl;
+        };
+        alive = take_unit(0);
+        if (alive && J > 0) { fetch(qt, 0); put_scalars(0); __syncwarp(); }
+        int t = 0;                                                        // tile, counted over the units
+        for (int n = 0; alive && J > 0; ++n) {
+            const int kq = key / kdiv;                                    // the key's chunk
+            const int kq_first = (kt * 128) / kdiv, kq_last = (kt * 128 + 127) / kdiv;
+            int g = 0;
+            int iq0 = (qt * 128 + 32 * cg) / a.k, ir0 = (qt * 128 + 32 * cg) - iq0 * a.k;
+            const int t_end = t + J;
+            for (; t < t_end; ++t) {
+                if (t + 1 < t_end) fetch(g + 1 == G ? qt + 1 : qt, g + 1 == G ? 0 : g + 1);   // lands while this tile is worked on
+                const float4* lse_c = reinterpret_cast<const float4*>(rows + (t & 1) * 256 + 32 * cg);     // this warp's 32 columns
+                const float4* dl_c = lse_c + 32;
+                const int i0 = qt * 128 + 32 * cg;                            // first query of the block
+                const int iq1 = iq0 + q31 + (ir0 + r31 >= a.k ? 1 : 0);       // chunk of the block's last query
+                // ---------------- phase A: P^T = exp2(S^T scale - lse), kept in registers ----------------
+                if (!bt_wait_converged(sm.bar(BB_XFULL), t & 1, sm.abort_addr(), a.status, kStatusWaitSFull)) { alive = false; break; }
+                tc_fence_after();
+                // all pairs of the block visible / none (rows past the streams drop out by themselves: zero K / V
+                // rows are discarded at the end, padding queries have lse = +inf)
+                bool full, none;
+                if (!summ) {
+                    full = kt * 128 + 127 <= i0 && iq1 - kq_first <= a.C;
+                    none = kt * 128 > i0 + 31 || iq0 - kq_last > a.C;
                 } else {
-                    int iq = iq0, ir = ir0;                               // chunk of query i0 + c, counted up from i0's
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) {
-                        const bool vis = summ ? (iq - kq > a.C) : (key <= i0 + c && iq - kq <= a.C);
-                        const float t = fmaf(__uint_as_float(x[c]), a.scale_log2, reinterpret_cast<const float*>(lse_c)[c]);
-                        x[c] = __float_as_uint(ex2_approx(vis ? t : -INFINITY));
-                        if (++ir == a.k) { ir = 0; ++iq; }
-                    }
+                    full = iq0 - kq_last > a.C;
+                    none = iq1 - kq_first <= a.C;
                 }
-            }
-            // ---------------- phase B: dS^T = P^T (dP^T - delta); both as bf16 over Y's own columns ----------------
-            if (!bt_wait_warp(sm.bar(BB_YFULL), j & 1, sm.abort_addr(), a.status, kStatusWaitSFull, lane)) { alive = false; break; }
-            tc_fence_after();
-            // Y_j was issued after every warp's arrival for tile j - 1: that tile's scalars may be overwritten
-            if (j + 1 < J) {
-                rows[((j + 1) & 1) * 256 + 32 * cg + lane] = n_lse;
-                rows[((j + 1) & 1) * 256 + 128 + 32 * cg + lane] = n_dl;
-            }
-            // handed over in two halves of 16 queries, so that the accumulations of the first run beside the
-            // arithmetic of the second: columns 16 half + 0 .. 7 take dS^T, 16 half + 8 .. 15 take P^T
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                uint32_t o[16];
+                uint32_t x[32];                                               // S^T, then P^T in place (fp32 bits), kept for phase B
                 if (none) {
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) o[c] = 0u;
+                    for (int c = 0; c < 32; ++c) x[c] = 0u;
                 } else {
-                    uint32_t ys[16];
-                    tmem_ld16(tYc + half * 16, ys);
+                    tmem_ld32(tXc, x);
                     tc_wait_ld();
-#pragma unroll
-                    for (int c = 0; c < 16; c += 4) {
-                        const int e = half * 16 + c;
-                        const float4 d4 = dl_c[e >> 2];
-                        const float2 p2 = make_float2(__uint_as_float(x[e]), __uint_as_float(x[e + 1]));
-                        const float2 q2 = make_float2(__uint_as_float(x[e + 2]), __uint_as_float(x[e + 3]));
-                        const float2 s2 = fmul2(p2, fadd2(make_float2(__uint_as_float(ys[c]), __uint_as_float(ys[c + 1])), make_float2(d4.x, d4.y)));
-                        const float2 r2 = fmul2(q2, fadd2(make_float2(__uint_as_float(ys[c + 2]), __uint_as_float(ys[c + 3])), make_float2(d4.z, d4.w)));
-                        o[c >> 1] = pack_bf16x2(s2.x, s2.y);
-                        o[(c >> 1) + 1] = pack_bf16x2(r2.x, r2.y);
-                        o[8 + (c >> 1)] = pack_bf16x2(p2.x, p2.y);
-                        o[9 + (c >> 1)] = pack_bf16x2(q2.x, q2.y);
-                    }
                 }
-                tmem_st16(tYc + half * 16, o);                            // over the block's own columns of dP^T
-                tc_wait_st();
+                // X_j is in registers: the issuer may start X_{j+1} while the exponentials run.  (This hand-over and those
+                // below order TMEM accesses only, which the fences and waits around them cover: relaxed arrivals.)
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive_relaxed(sm.bar(half ? BB_PB2 : BB_PB));
+                if (lane == 0) mbar_arrive_relaxed(sm.bar(BB_PA));
+                if (!none) {
+                    if (full) {
+                        const float2 sc2 = make_float2(a.scale_log2, a.scale_log2);
+#pragma unroll
+                        for (int c = 0; c < 32; c += 4) {
+                            const float4 l4 = lse_c[c >> 2];
+                            const float2 v = ffma2(make_float2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])), sc2, make_float2(l4.x, l4.y));
+                            const float2 w = ffma2(make_float2(__uint_as_float(x[c + 2]), __uint_as_float(x[c + 3])), sc2, make_float2(l4.z, l4.w));
+                            x[c] = __float_as_uint(ex2_approx(v.x));
+                            x[c + 1] = __float_as_uint(ex2_approx(v.y));
+                            x[c + 2] = __float_as_uint(ex2_approx(w.x));
+                            x[c + 3] = __float_as_uint(ex2_approx(w.y));
+                        }
+                    } else {
+                        int iq = iq0, ir = ir0;                               // chunk of query i0 + c, counted up from i0's
+#pragma unroll
+                        for (int c = 0; c < 32; ++c) {
+                            const bool vis = summ ? (iq - kq > a.C) : (key <= i0 + c && iq - kq <= a.C);
+                            const float v = fmaf(__uint_as_float(x[c]), a.scale_log2, reinterpret_cast<const float*>(lse_c)[c]);
+                            x[c] = __float_as_uint(ex2_approx(vis ? v : -INFINITY));
+                            if (++ir == a.k) { ir = 0; ++iq; }
+                        }
+                    }
+                }
+                // ---------------- phase B: dS^T = P^T (dP^T - delta); both as bf16 over Y's own columns ----------------
+                if (!bt_wait_converged(sm.bar(BB_YFULL), t & 1, sm.abort_addr(), a.status, kStatusWaitSFull)) { alive = false; break; }
+                tc_fence_after();
+                // Y_j was issued after every warp's arrival for tile j - 1: that tile's scalars may be overwritten
+                if (t + 1 < t_end) put_scalars(t + 1);
+                // handed over in two halves of 16 queries, so that the accumulations of the first run beside the
+                // arithmetic of the second: columns 16 half + 0 .. 7 take dS^T, 16 half + 8 .. 15 take P^T
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    uint32_t o[16];
+                    if (none) {
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) o[c] = 0u;
+                    } else {
+                        uint32_t ys[16];
+                        tmem_ld16(tYc + half * 16, ys);
+                        tc_wait_ld();
+#pragma unroll
+                        for (int c = 0; c < 16; c += 4) {
+                            const int e = half * 16 + c;
+                            const float4 d4 = dl_c[e >> 2];
+                            const float2 p2 = make_float2(__uint_as_float(x[e]), __uint_as_float(x[e + 1]));
+                            const float2 q2 = make_float2(__uint_as_float(x[e + 2]), __uint_as_float(x[e + 3]));
+                            const float2 s2 = fmul2(p2, fadd2(make_float2(__uint_as_float(ys[c]), __uint_as_float(ys[c + 1])), make_float2(d4.x, d4.y)));
+                            const float2 r2 = fmul2(q2, fadd2(make_float2(__uint_as_float(ys[c + 2]), __uint_as_float(ys[c + 3])), make_float2(d4.z, d4.w)));
+                            o[c >> 1] = pack_bf16x2(s2.x, s2.y);
+                            o[(c >> 1) + 1] = pack_bf16x2(r2.x, r2.y);
+                            o[8 + (c >> 1)] = pack_bf16x2(p2.x, p2.y);
+                            o[9 + (c >> 1)] = pack_bf16x2(q2.x, q2.y);
+                        }
+                    }
+                    tmem_st16(tYc + half * 16, o);                            // over the block's own columns of dP^T
+                    tc_wait_st();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_relaxed(sm.bar(half ? BB_PB2 : BB_PB));
+                }
+                if (++g == G) {                                               // next query tile
+                    g = 0; ++qt;
+                    iq0 += step_q; ir0 += step_r;
+                    if (ir0 >= a.k) { ir0 -= a.k; ++iq0; }
+                }
             }
-            if (++g == G) {                                               // next query tile
-                g = 0; ++qt;
-                iq0 += step_q; ir0 += step_r;
-                if (ir0 >= a.k) { ir0 -= a.k; ++iq0; }
-            }
-        }
-        if (alive && bt_wait_warp(sm.bar(BB_OFULL), 0, sm.abort_addr(), a.status, kStatusWaitOFull, lane)) {
-            tc_fence_after();
+            if (!alive) break;
             // odd cg: scale * dK, even cg: dV; cg / 2 picks the half of the row (D / 2 elements)
             // (tcgen05.ld is warp-collective: rows past the stream load, too)
-            const bool is_dk = (cg & 1) != 0;
+            const bool is_dk = (cg & 1) != 0, row_ok = key != 0x3fffffff;
             const int d0 = (cg >> 1) * (D / 2);
             const size_t arow = (size_t)hk * (summ ? a.summ_rows : a.text_rows) + (size_t)krow0 + quarter * 32 + lane;
             float* acc = (is_dk ? (summ ? a.dks : a.dkt) : (summ ? a.dvs : a.dvt)) + acc_at(arow, d0, D);
+            // the next unit and its first scalars, beside the last products (every warp's tile before the last is done: see above)
+            if (!take_unit(n + 1)) break;
+            if (J > 0) fetch(qt, 0);
+            if (!bt_wait_converged(sm.bar(BB_OFULL), n & 1, sm.abort_addr(), a.status, kStatusWaitOFull)) break;
+            tc_fence_after();
             const float mul = is_dk ? a.scale : 1.f;
             const uint32_t tacc = (is_dk ? tDK : tDV) + lane_sel + d0;
 #pragma unroll
@@ -529,7 +682,7 @@ __device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& ma
                 uint32_t o[32];
                 tmem_ld32(tacc + c * 32, o);
                 tc_wait_ld();
-                if (key_raw < n_keys) {
+                if (row_ok) {
                     // store: this CTA is the only one of its launch for these keys and the first writer of their rows
 #pragma unroll
                     for (int e = 0; e < 32; e += 4) {
@@ -541,6 +694,9 @@ __device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& ma
                     }
                 }
             }
+            // the accumulators are read before this warp's first hand-over of the next unit, behind which they are overwritten
+            tc_fence_before();
+            if (J > 0) { put_scalars(t); __syncwarp(); }
         }
     }
     tc_fence_before();
@@ -551,228 +707,295 @@ __device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& ma
 // =====================================================================================================
 // dQ
 // =====================================================================================================
+// A unit: one query tile and one query head, over the visible summary tiles, then the visible text tiles (Eq. 3).  Block
+// (x, y): x-th query tile of the packed stream from its end (a sequence's long rows first), head y.
+struct BtDqUnit { int J, n_s, t_lo, qt, h, n_text, text_off, summ_off, chunk0; long long aug_off; };
+__device__ __forceinline__ void bt_dq_unit(const BwdArgs& a, const BtBlock& blk, BtDqUnit& u)
+{
+    const int row0 = (int)a.text_rows - 128 - blk.x * 128;
+    const SeqInfo sq = a.seqs[seq_of_row(a.seqs, a.num_seqs, row0, true)];
+    u.qt = (row0 - sq.text_off) / 128;
+    u.h = blk.y;
+    u.n_text = sq.n_text; u.text_off = sq.text_off; u.summ_off = sq.summ_off; u.chunk0 = sq.chunk0; u.aug_off = sq.aug_off;
+    const int i_first = u.qt * 128, i_last = min(sq.n_text, i_first + 128) - 1;
+    const int far_first = max(0, i_first / a.k - a.C), far_last = max(0, i_last / a.k - a.C);
+    u.n_s = a.m > 0 ? (min(sq.n_summ, far_last * a.m) + 127) / 128 : 0;               // summary tiles seen by the last row
+    u.t_lo = (int)(((long long)far_first * a.k) / 128);                                // first text tile seen by the first row
+    u.J = u.n_s + u.qt - u.t_lo + 1;
+}
+
 template <int D>
 __device__ __forceinline__ void bt_dq_block(const BwdArgs& a, const BwdMaps& maps)
 {
     extern __shared__ uint8_t bsm_raw[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-    // ---- which queries, which keys (Eq. 3) ------------------------------------------------------
-    const int h = blockIdx.y, hk = h / (a.Hq / a.Hkv);
-    const SeqInfo sq = a.seqs[blockIdx.z];
-    const int n_qt = (sq.n_text + 127) / 128;
-    if ((int)blockIdx.x >= n_qt) return;
-    const int qt = n_qt - 1 - (int)blockIdx.x;                            // long rows first
-    const int i_first = qt * 128, i_last = min(sq.n_text, i_first + 128) - 1;
-    const int far_first = max(0, i_first / a.k - a.C), far_last = max(0, i_last / a.k - a.C);
-    const int n_s = a.m > 0 ? (min(sq.n_summ, far_last * a.m) + 127) / 128 : 0;     // summary tiles seen by the last row
-    const int t_lo = (int)(((long long)far_first * a.k) / 128);                      // first text tile seen by the first row
-    const int J = n_s + qt - t_lo + 1;
-    // streamed tile j: summary tile j while j < n_s, then text tile t_lo + j - n_s
-    auto tile_of = [&](int j, bool& is_summ, int& key0) {
-        is_summ = j < n_s;
-        key0 = (is_summ ? j : t_lo + j - n_s) * 128;
-    };
-
+    const int warp = (int)__reduce_or_sync(0xffffffffu, threadIdx.x >> 5), lane = threadIdx.x & 31;       // (uniform to the compiler)
+    const int G = a.Hq / a.Hkv;
     BtSmem<D> sm;
     if (!bt_layout(sm, bsm_raw, a.status)) return;
-    // loads of streamed tile j (the producer's thread): key0 / 128 tiles into its stream, rows of the packed stream or
-    // chunks of the caller's tensor
+
+    // ---- the producer's thread: descriptor and loads of a unit ------------------------------------
     const bool direct = a.direct != 0;
-    auto load_kv = [&](int j, uint32_t dst, uint32_t bar, const CUtensorMap* map_s, const CUtensorMap* map_t) {
-        bool is_summ; int key0;
-        tile_of(j, is_summ, key0);
-        bt_load_tile<D>(dst, bar, is_summ ? map_s : map_t,
-                        direct ? sq.chunk0 + (key0 >> 7) * (128 / (is_summ ? a.m : a.k)) : (is_summ ? sq.summ_off : sq.text_off) + key0, hk, direct);
+    BtDqUnit u{};
+    auto publish = [&](int n) {
+        bt_st_shared(sm.unit(n, U_TEXT_OFF), (uint32_t)u.text_off); bt_st_shared(sm.unit(n, U_TILE), (uint32_t)u.qt);
+        bt_st_shared(sm.unit(n, U_HEAD), (uint32_t)u.h); bt_st_shared(sm.unit(n, U_A), (uint32_t)u.n_s);
+        bt_st_shared(sm.unit(n, U_B), (uint32_t)u.t_lo); bt_st_shared(sm.unit(n, U_C), (uint32_t)u.n_text);
+        bt_st_shared(sm.unit(n, U_AUG), (uint32_t)u.aug_off); bt_st_shared(sm.unit(n, U_AUG + 1), (uint32_t)(u.aug_off >> 32));
+        bt_st_shared(sm.unit(n, U_J), (uint32_t)u.J);
+        mbar_arrive(sm.bar(BB_UFULL + (n & 1)));
     };
-    auto load_b1 = [&](int j) { load_kv(j, sm.b1(j % kB1Stages), sm.bar(BB_B1FULL + j % kB1Stages), &maps.ks, &maps.kt); };
-    auto load_b2 = [&](int j) { load_kv(j, sm.b2(j & 1), sm.bar(BB_B2FULL + (j & 1)), &maps.vs, &maps.vt); };
+    auto load_a = [&]() {                                                 // Q and dO tile
+        mbar_arrive_expect_tx(sm.bar(BB_AFULL), 2u * BtMap<D>::kTile);
+        const int qpos = direct ? u.chunk0 + u.qt * (128 / a.k) : u.text_off + u.qt * 128;
+        bt_issue_tile<D>(sm.a1(), sm.bar(BB_AFULL), &maps.qt, qpos, u.h, direct);
+        bt_issue_tile<D>(sm.a2(), sm.bar(BB_AFULL), &maps.dot, qpos, u.h, direct);
+    };
+    auto load_b = [&](int j, uint32_t dst, uint32_t bar, const CUtensorMap* map_s, const CUtensorMap* map_t) {
+        const bool is_summ = j < u.n_s;
+        const int tile = is_summ ? j : u.t_lo + j - u.n_s;
+        bt_load_tile<D>(dst, bar, is_summ ? map_s : map_t,
+                        direct ? u.chunk0 + tile * (128 / (is_summ ? a.m : a.k)) : (is_summ ? u.summ_off : u.text_off) + tile * 128, u.h / G, direct);
+    };
     if (warp == 16 && lane == 0) {
         bt_init_barriers(sm);
-        mbar_arrive_expect_tx(sm.bar(BB_AFULL), 2u * BtMap<D>::kTile);
-        const int qpos = direct ? sq.chunk0 + qt * (128 / a.k) : sq.text_off + qt * 128;
-        bt_issue_tile<D>(sm.a1(), sm.bar(BB_AFULL), &maps.qt, qpos, h, direct);
-        load_b1(0);
-        bt_issue_tile<D>(sm.a2(), sm.bar(BB_AFULL), &maps.dot, qpos, h, direct);
-        load_b2(0);
-    }
-    // row warps: this thread's query row and its scalars, on their way beside the set-up
-    const int quarter = warp & 3, cg = warp >> 2;                        // lanes 32 quarter ..; columns 32 cg ..
-    const int i_w0 = i_first + quarter * 32, i = i_w0 + lane;
-    float lse2 = 0.f, dl = 0.f;
-    if (warp < 16) {
-        const size_t r = (size_t)h * a.text_rows + sq.text_off + i;
-        lse2 = __ldcg(a.lse_t + r);                                      // +inf / 0 on padding rows: P = 0 there
-        dl = __ldcg(a.delta_t + r);                                      // (past L1: see the launches)
+        bt_dq_unit(a, BtBlock{(int)blockIdx.x, (int)blockIdx.y, 0}, u);
+        load_b(0, sm.b1(0), sm.bar(BB_B1FULL), &maps.ks, &maps.kt);
+        load_a();
+        load_b(0, sm.b2(0), sm.bar(BB_B2FULL), &maps.vs, &maps.vt);
+        publish(0);
     }
     bt_ready(sm, warp);
     const uint32_t tmem = bt_ld_shared(sm.tmem_slot());
     const uint32_t tX = tmem, tDQ = tmem + 256u;
-    auto tY = [&](int j) -> uint32_t { return tmem + ((j & 1) ? 384u : 128u); };   // dP of tile j, then dS in place
+    // dP of tile j (counted over the CTA's units), then dS in place
+    auto tY = [&](int j) -> uint32_t { return tmem + ((j & 1) ? 384u : 128u); };
     auto y_full = [&](int j) -> uint32_t { return sm.bar((j & 1) ? BB_YFULL2 : BB_YFULL); };
     // likewise one phase B barrier per Y buffer: with both products of tile j + 1 issued early, a warp may finish
     // tile j + 1 before another has finished tile j, and must not arrive in its phase
     auto p_b = [&](int j) -> uint32_t { return sm.bar((j & 1) ? BB_PB2 : BB_PB); };
 
-    if (warp == 16) {
-        // =============================== TMA producer ===============================
-        if (lane == 0) {
-            int filled1 = 1, filled2 = 1;                                 // tile 0 is on its way
-            for (int j = 1; j < J; ++j) {
-                if (!bt_stage_free(sm, BB_B1EMPTY, kB1Stages, j, a.status)) break;
-                load_b1(j);
-                ++filled1;
-                if (!bt_stage_free(sm, BB_B2EMPTY, kB2Stages, j, a.status)) break;
-                load_b2(j);
-                ++filled2;
+    if (warp >= 16) {
+        setmaxnreg_dec<kBwdRegsOther>();
+        if (warp == 16) { if (lane == 0) {
+            // =============================== TMA producer ===============================
+            int na = 1, g1 = 1, g2 = 1, asked = 0;                        // A pairs, B1 and B2 tiles loaded; answered requests
+            bool alive = true, pending = false, took_first = false;      // ... the grid's first block among them
+            for (int n = 0; alive; ++n) {
+                if (n > 0) {                                              // the next block
+                    if (!pending) { bt_request_block(sm); pending = true; }
+                    BtBlock blk;
+                    const int got = bt_take_block(sm, asked, blk, a.status);
+                    if (got < 0) break;
+                    ++asked; pending = false;
+                    took_first |= got > 0 && blk.x + blk.y == 0;
+                    if (got > 0) bt_dq_unit(a, blk, u); else u.J = 0;
+                    if (!bt_unit_free(sm, n, a.status)) break;
+                    publish(n);
+                    if (u.J == 0) break;                                  // none left: the CTA ends
+                }
+                for (int j = n > 0 ? 0 : 1; j < u.J; ++j) {
+                    if (j + 1 == u.J) { bt_request_block(sm); pending = true; }          // comes while the stages are waited for
+                    if (!bt_stage_free(sm, BB_B1EMPTY, kB1Stages, g1, a.status)) { alive = false; break; }
+                    load_b(j, sm.b1(g1 % kB1Stages), sm.bar(BB_B1FULL + g1 % kB1Stages), &maps.ks, &maps.kt);
+                    ++g1;
+                    if (j == 0) {                                         // the unit before has formed its last products
+                        if (!bt_wait(sm.bar(BB_AEMPTY), (uint32_t)((na - 1) & 1), sm.abort_addr(), a.status, kStatusWaitQEmpty)) { alive = false; break; }
+                        load_a();
+                        ++na;
+                    }
+                    if (!bt_stage_free(sm, BB_B2EMPTY, kB2Stages, g2, a.status)) { alive = false; break; }
+                    load_b(j, sm.b2(g2 & 1), sm.bar(BB_B2FULL + (g2 & 1)), &maps.vs, &maps.vt);
+                    ++g2;
+                }
             }
-            if (bt_ld_shared(sm.abort_addr()) != 0u) bt_drain(sm, filled1, filled2, a.status);
-        }
-    } else if (warp == 17) {
-        // =============================== MMA issuer =================================
-        // the whole warp walks the loop on warp-uniform values, one lane issues
-        const uint32_t leader = elect_one();
-        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0), base = __shfl_sync(0xffffffffu, sm.base, 0);
-        const int Ju = __shfl_sync(0xffffffffu, J, 0);
-        const BtSmem<D> su{base};
-        const uint32_t uX = tm, uDQ = tm + 256u;
-        auto uY = [&](int j) -> uint32_t { return tm + ((j & 1) ? 384u : 128u); };
-        auto u_full = [&](int j) -> uint32_t { return su.bar((j & 1) ? BB_YFULL2 : BB_YFULL); };
-        auto wait = [&](uint32_t bar, uint32_t parity, int code) -> bool {
-            return __all_sync(0xffffffffu, bt_wait(bar, parity, su.abort_addr(), a.status, code));
-        };
-        bool alive = wait(su.bar(BB_AFULL), 0, kStatusWaitKvFull);
-        if (alive) alive = wait(su.bar(BB_B1FULL), 0, kStatusWaitQFull);
-        if (alive) { bt_product<D>(leader, uX, su.a1(), su.b1(0)); tc_commit_warp(leader, su.bar(BB_XFULL)); }
-        if (alive) alive = wait(su.bar(BB_B2FULL), 0, kStatusWaitQFull);
-        if (alive) { bt_product<D>(leader, uY(0), su.a2(), su.b2(0)); tc_commit_warp(leader, u_full(0)); }
-        int s1 = 0;                                            // j % kB1Stages
-        uint32_t b1_phase = 0;                                 // parity of tile j + 1's fill of its stage
-        for (int j = 0; j < Ju && alive; ++j) {
-            const int s1n = s1 + 1 == kB1Stages ? 0 : s1 + 1;
-            if (j + 1 < Ju) {
-                if (s1n == 0) b1_phase ^= 1u;
-                if (!wait(su.bar(BB_B1FULL + s1n), b1_phase, kStatusWaitQFull)) break;
-                if (!wait(su.bar(BB_B2FULL + ((j + 1) & 1)), ((j + 1) >> 1) & 1, kStatusWaitQFull)) break;
-                // phase A of tile j has read X into registers; the other Y buffer was read by dQ += dS K_{j-1}
-                if (!wait(su.bar(BB_PA), j & 1, kStatusWaitPFull)) break;
-                tc_fence_after();
-                bt_product<D>(leader, uX, su.a1(), su.b1(s1n));
+            if (bt_ld_shared(sm.abort_addr()) != 0u) bt_drain(sm, na, g1, g2, pending, asked, a.status);
+            if (took_first) pdl_wait();                                    // (see the launches)
+        } } else if (warp == 17) {
+            // =============================== MMA issuer =================================
+            // the whole warp walks the loop on warp-uniform values, one lane issues
+            const uint32_t leader = elect_one();
+            const uint32_t tm = __reduce_or_sync(0xffffffffu, tmem), base = __reduce_or_sync(0xffffffffu, sm.base);
+            const BtSmem<D> su{base};
+            const uint32_t uX = tm, uDQ = tm + 256u;
+            auto uY = [&](int j) -> uint32_t { return tm + ((j & 1) ? 384u : 128u); };
+            auto u_full = [&](int j) -> uint32_t { return su.bar((j & 1) ? BB_YFULL2 : BB_YFULL); };
+            auto wait = [&](uint32_t bar, uint32_t parity, int code) -> bool {
+                return bt_wait_converged(bar, parity, su.abort_addr(), a.status, code);
+            };
+            bool alive = true;
+            int g = 0, s1 = 0;                                            // tiles of the units before; the next tile's B1 stage ...
+            uint32_t b1_phase = 0;                                        // ... and the parity of its fill
+            for (int n = 0; alive; ++n) {
+                if (!wait(su.bar(BB_UFULL + (n & 1)), (n >> 1) & 1, kStatusWaitUnit)) break;
+                const int Ju = bt_unit_word(su, n, U_J);
+                mbar_arrive_warp(leader, su.bar(BB_UEMPTY + (n & 1)));
+                if (Ju == 0) break;
+                alive = wait(su.bar(BB_AFULL), n & 1, kStatusWaitKvFull) && wait(su.bar(BB_B1FULL + s1), b1_phase, kStatusWaitQFull);
+                if (!alive) break;
+                // (X is free: every row warp has handed over the last tile of the unit before)
+                bt_product<D>(leader, uX, su.a1(), su.b1(s1));
                 tc_commit_warp(leader, su.bar(BB_XFULL));
-                bt_product<D>(leader, uY(j + 1), su.a2(), su.b2((j + 1) & 1));
-                tc_commit_warp(leader, u_full(j + 1));
+                if (!wait(su.bar(BB_B2FULL + (g & 1)), (g >> 1) & 1, kStatusWaitQFull)) break;
+                bt_product<D>(leader, uY(g), su.a2(), su.b2(g & 1));
+                tc_commit_warp(leader, u_full(g));
+                if (Ju == 1) tc_commit_warp(leader, su.bar(BB_AEMPTY));
+                for (int j = 0; j < Ju; ++j, ++g) {
+                    const int s1n = s1 + 1 == kB1Stages ? 0 : s1 + 1;
+                    if (s1n == 0) b1_phase ^= 1u;
+                    if (j + 1 < Ju) {
+                        if (!(alive = wait(su.bar(BB_B1FULL + s1n), b1_phase, kStatusWaitQFull))) break;
+                        if (!(alive = wait(su.bar(BB_B2FULL + ((g + 1) & 1)), ((g + 1) >> 1) & 1, kStatusWaitQFull))) break;
+                        // phase A of tile j has read X into registers; the other Y buffer was read by dQ += dS K_{j-1}
+                        if (!(alive = wait(su.bar(BB_PA), g & 1, kStatusWaitPFull))) break;
+                        tc_fence_after();
+                        bt_product<D>(leader, uX, su.a1(), su.b1(s1n));
+                        tc_commit_warp(leader, su.bar(BB_XFULL));
+                        bt_product<D>(leader, uY(g + 1), su.a2(), su.b2((g + 1) & 1));
+                        tc_commit_warp(leader, u_full(g + 1));
+                        if (j + 2 == Ju) tc_commit_warp(leader, su.bar(BB_AEMPTY));                // Q and dO may make way for the next unit's
+                    }
+                    if (!(alive = wait(su.bar((g & 1) ? BB_PB2 : BB_PB), (g >> 1) & 1, kStatusWaitPFull))) break;
+                    tc_fence_after();
+                    bt_accumulate<D>(leader, uDQ, uY(g), su.b1(s1), j == 0);                       // dQ += dS K_j
+                    tc_commit_warp(leader, su.bar(BB_B1EMPTY + s1));                               // K_j is free after that
+                    s1 = s1n;
+                }
+                if (alive) tc_commit_warp(leader, su.bar(BB_OFULL));
             }
-            if (!wait(su.bar((j & 1) ? BB_PB2 : BB_PB), (j >> 1) & 1, kStatusWaitPFull)) break;
-            tc_fence_after();
-            bt_accumulate<D>(leader, uDQ, uY(j), su.b1(s1), j == 0);                       // dQ += dS K_j
-            tc_commit_warp(leader, su.bar(BB_B1EMPTY + s1));                               // K_j is free after that
-            s1 = s1n;
+            bt_drain_pipe(leader, su, a.status);
         }
-        tc_commit_warp(leader, su.bar(BB_OFULL));
     } else {
+        setmaxnreg_inc<kBwdRegsRows>();
         // =============================== query rows =================================
+        const int quarter = warp & 3, cg = warp >> 2;                     // lanes 32 quarter ..; columns 32 cg ..
         const uint32_t lane_sel = (uint32_t)(quarter * 32) << 16;
         const uint32_t tXc = tX + lane_sel + cg * 32;                     // this warp's 32 x 32 block
-        const int iq = i / a.k, iq_w0 = i_w0 / a.k, iq_w1 = (i_w0 + 31) / a.k;
-        bool alive = true;
-        // The chunk of the block's first key, kc0 = key0 + 32 cg, is kept as quotient and remainder by the keys per
-        // chunk of its stream and advanced by 128 per tile; divisions only where the stream starts (integer
-        // divisions are slow, and this loop is the warps' critical path).
-        int cdiv = 1, kq0 = 0, kr0 = 0, step_q = 0, step_r = 0, q31 = 0, r31 = 0;
-        for (int j = 0; j < J; ++j) {
-            bool is_summ; int key0;
-            tile_of(j, is_summ, key0);
-            const int kc0 = key0 + 32 * cg;                               // first key of this warp's block
-            if (j == 0 || j == n_s) {                                     // first tile of the summary / the text stream
-                cdiv = is_summ ? a.m : a.k;                               // keys per chunk in this stream
-                kq0 = kc0 / cdiv; kr0 = kc0 - kq0 * cdiv;
-                step_q = 128 / cdiv; step_r = 128 - step_q * cdiv;
-                q31 = 31 / cdiv; r31 = 31 - q31 * cdiv;
-            } else {
-                kq0 += step_q; kr0 += step_r;
-                if (kr0 >= cdiv) { kr0 -= cdiv; ++kq0; }
-            }
-            const int kq1 = kq0 + q31 + (kr0 + r31 >= cdiv ? 1 : 0);      // chunk of the block's last key
-            // the warp's 32 x 32 block: all visible, none, or mixed (zero rows past a stream add nothing to dQ).
-            // Text key t is visible to row i iff t <= i and chunk(i) - chunk(t) <= C; summary key s iff
-            // chunk(i) - chunk(s) > C (Eq. 3)
-            bool full, none;
-            if (is_summ) {
-                full = iq_w0 - kq1 > a.C;
-                none = iq_w1 - kq0 <= a.C;
-            } else {
-                full = kc0 + 31 <= i_w0 && iq_w1 - kq0 <= a.C;
-                none = kc0 > i_w0 + 31 || iq_w0 - kq1 > a.C;
-            }
-            // ---------------- phase A: P = exp2(S scale - lse) ----------------
-            if (!bt_wait_warp(sm.bar(BB_XFULL), j & 1, sm.abort_addr(), a.status, kStatusWaitSFull, lane)) { alive = false; break; }
-            tc_fence_after();
-            uint32_t x[32];                                               // S, then P in place (fp32 bits)
-            if (!none) {
-                tmem_ld32(tXc, x);
-                tc_wait_ld();
-            }
-            tc_fence_before();
+        int J = 0, n_s = 0, i_w0 = 0;
+        float lse2 = 0.f, dl = 0.f;
+        // (the slot is handed back when the unit's output rows have been worked out, see below)
+        auto take_unit = [&](int n) -> bool {
+            if (!bt_wait_converged(sm.bar(BB_UFULL + (n & 1)), (n >> 1) & 1, sm.abort_addr(), a.status, kStatusWaitUnit)) return false;
             __syncwarp();
-            if (lane == 0) mbar_arrive_relaxed(sm.bar(BB_PA));            // X may be overwritten from here on
-            if (!none) {
-                if (full) {
-                    const float2 sc2 = make_float2(a.scale_log2, a.scale_log2), nl2 = make_float2(-lse2, -lse2);
+            J = bt_unit_word(sm, n, U_J);
+            if (J == 0) return true;
+            n_s = bt_unit_word(sm, n, U_A);
+            i_w0 = bt_unit_word(sm, n, U_TILE) * 128 + quarter * 32;
+            const size_t r = (size_t)bt_unit_word(sm, n, U_HEAD) * a.text_rows + bt_unit_word(sm, n, U_TEXT_OFF) + i_w0 + lane;
+            lse2 = __ldcg(a.lse_t + r);                                  // +inf / 0 on padding rows: P = 0 there
+            dl = __ldcg(a.delta_t + r);                                  // (past L1: see the launches)
+            return true;
+        };
+        bool alive = take_unit(0);
+        int j = 0;                                                        // tile, counted over the units
+        for (int n = 0; alive && J > 0; ++n) {
+            const int i = i_w0 + lane;
+            const int iq = i / a.k, iq_w0 = i_w0 / a.k, iq_w1 = (i_w0 + 31) / a.k;
+            // The chunk of the block's first key, kc0 = key0 + 32 cg, is kept as quotient and remainder by the keys per
+            // chunk of its stream and advanced by 128 per tile (kc0: the key); divisions only where the stream starts (integer
+            // divisions are slow, and this loop is the warps' critical path).
+            int cdiv = 0, kc0 = 32 * cg, kq0 = 0, kr0 = 0, step_q = 0, step_r = 0, q31 = 0, r31 = 0;
+            const int j_text = j + n_s, j_end = j + J;                    // first text tile, first tile of the next unit
+            for (; j < j_end; ++j, kc0 += 128) {
+                const bool is_summ = j < j_text;
+                if (cdiv == 0 || j == j_text) {                               // first tile of the summary / the text stream
+                    if (!is_summ) kc0 = bt_unit_word(sm, n, U_B) * 128 + 32 * cg;
+                    cdiv = is_summ ? a.m : a.k;                               // keys per chunk in this stream
+                    kq0 = kc0 / cdiv; kr0 = kc0 - kq0 * cdiv;
+                    step_q = 128 / cdiv; step_r = 128 - step_q * cdiv;
+                    q31 = 31 / cdiv; r31 = 31 - q31 * cdiv;
+                } else {
+                    kq0 += step_q; kr0 += step_r;
+                    if (kr0 >= cdiv) { kr0 -= cdiv; ++kq0; }
+                }
+                const int kq1 = kq0 + q31 + (kr0 + r31 >= cdiv ? 1 : 0);      // chunk of the block's last key
+                // the warp's 32 x 32 block: all visible, none, or mixed (zero rows past a stream add nothing to dQ).
+                // Text key t is visible to row i iff t <= i and chunk(i) - chunk(t) <= C; summary key s iff
+                // chunk(i) - chunk(s) > C (Eq. 3)
+                bool full, none;
+                if (is_summ) {
+                    full = iq_w0 - kq1 > a.C;
+                    none = iq_w1 - kq0 <= a.C;
+                } else {
+                    full = kc0 + 31 <= i_w0 && iq_w1 - kq0 <= a.C;
+                    none = kc0 > i_w0 + 31 || iq_w0 - kq1 > a.C;
+                }
+                // ---------------- phase A: P = exp2(S scale - lse) ----------------
+                if (!bt_wait_converged(sm.bar(BB_XFULL), j & 1, sm.abort_addr(), a.status, kStatusWaitSFull)) { alive = false; break; }
+                tc_fence_after();
+                uint32_t x[32];                                               // S, then P in place (fp32 bits)
+                if (!none) {
+                    tmem_ld32(tXc, x);
+                    tc_wait_ld();
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_relaxed(sm.bar(BB_PA));            // X may be overwritten from here on
+                if (!none) {
+                    if (full) {
+                        const float2 sc2 = make_float2(a.scale_log2, a.scale_log2), nl2 = make_float2(-lse2, -lse2);
+#pragma unroll
+                        for (int c = 0; c < 32; c += 2) {
+                            const float2 v = ffma2(make_float2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])), sc2, nl2);
+                            x[c] = __float_as_uint(ex2_approx(v.x));
+                            x[c + 1] = __float_as_uint(ex2_approx(v.y));
+                        }
+                    } else {
+                        int kq = kq0, kr = kr0;                               // chunk of key kc0 + c, counted up from kc0's
+#pragma unroll
+                        for (int c = 0; c < 32; ++c) {
+                            const bool vis = is_summ ? (iq - kq > a.C) : (kc0 + c <= i && iq - kq <= a.C);
+                            const float v = fmaf(__uint_as_float(x[c]), a.scale_log2, -lse2);
+                            x[c] = __float_as_uint(ex2_approx(vis ? v : -INFINITY));
+                            if (++kr == cdiv) { kr = 0; ++kq; }
+                        }
+                    }
+                }
+                // ---------------- phase B: dS = P (dP - delta) ----------------
+                // one barrier per Y buffer: Y_{j+1} may be complete before a warp gets here for Y_j
+                if (!bt_wait_converged(y_full(j), (j >> 1) & 1, sm.abort_addr(), a.status, kStatusWaitSFull)) { alive = false; break; }
+                tc_fence_after();
+                if (warp == 0 && lane == 0) mbar_arrive_relaxed(sm.bar(BB_B2EMPTY + (j & 1)));          // Y_j is complete: its V stage is free
+                const uint32_t tYc = tY(j) + lane_sel + cg * 32;
+                uint32_t dd[16];
+                if (none) {
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) dd[c] = 0u;
+                } else {
+                    uint32_t ys[32];
+                    tmem_ld32(tYc, ys);
+                    tc_wait_ld();
+                    const float2 nd2 = make_float2(-dl, -dl);
 #pragma unroll
                     for (int c = 0; c < 32; c += 2) {
-                        const float2 t = ffma2(make_float2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])), sc2, nl2);
-                        x[c] = __float_as_uint(ex2_approx(t.x));
-                        x[c + 1] = __float_as_uint(ex2_approx(t.y));
-                    }
-                } else {
-                    int kq = kq0, kr = kr0;                               // chunk of key kc0 + c, counted up from kc0's
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) {
-                        const bool vis = is_summ ? (iq - kq > a.C) : (kc0 + c <= i && iq - kq <= a.C);
-                        const float t = fmaf(__uint_as_float(x[c]), a.scale_log2, -lse2);
-                        x[c] = __float_as_uint(ex2_approx(vis ? t : -INFINITY));
-                        if (++kr == cdiv) { kr = 0; ++kq; }
+                        const float2 d2 = fmul2(make_float2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])),
+                                                fadd2(make_float2(__uint_as_float(ys[c]), __uint_as_float(ys[c + 1])), nd2));
+                        dd[c >> 1] = pack_bf16x2(d2.x, d2.y);
                     }
                 }
+                tmem_st16(tYc, dd);                                           // over the block's own first 16 columns
+                tc_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_relaxed(p_b(j));
             }
-            // ---------------- phase B: dS = P (dP - delta) ----------------
-            // one barrier per Y buffer: Y_{j+1} may be complete before a warp gets here for Y_j
-            if (!bt_wait_warp(y_full(j), (j >> 1) & 1, sm.abort_addr(), a.status, kStatusWaitSFull, lane)) { alive = false; break; }
-            tc_fence_after();
-            if (warp == 0 && lane == 0) mbar_arrive_relaxed(sm.bar(BB_B2EMPTY + (j & 1)));          // Y_j is complete: its V stage is free
-            const uint32_t tYc = tY(j) + lane_sel + cg * 32;
-            uint32_t dd[16];
-            if (none) {
-#pragma unroll
-                for (int c = 0; c < 16; ++c) dd[c] = 0u;
-            } else {
-                uint32_t ys[32];
-                tmem_ld32(tYc, ys);
-                tc_wait_ld();
-                const float2 nd2 = make_float2(-dl, -dl);
-#pragma unroll
-                for (int c = 0; c < 32; c += 2) {
-                    const float2 d2 = fmul2(make_float2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])),
-                                            fadd2(make_float2(__uint_as_float(ys[c]), __uint_as_float(ys[c + 1])), nd2));
-                    dd[c >> 1] = pack_bf16x2(d2.x, d2.y);
-                }
-            }
-            tmem_st16(tYc, dd);                                           // over the block's own first 16 columns
-            tc_wait_st();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_relaxed(p_b(j));
-        }
-        if (alive && bt_wait_warp(sm.bar(BB_OFULL), 0, sm.abort_addr(), a.status, kStatusWaitOFull, lane)) {
-            tc_fence_after();
+            if (!alive) break;
             // scale * dQ as bf16 to the row's augmented position (Eq. 1); warp group cg writes elements 32 cg ..
+            int64_t off = -1;                                             // -1: a padding row
+            const int n_text = bt_unit_word(sm, n, U_C), h = bt_unit_word(sm, n, U_HEAD);
+            const int64_t aug_off = (int64_t)(((unsigned long long)(uint32_t)bt_unit_word(sm, n, U_AUG + 1) << 32) | (uint32_t)bt_unit_word(sm, n, U_AUG));
+            if (i < n_text) off = (aug_off + (int64_t)iq * (a.k + a.m) + (i - iq * a.k)) * a.dq_st + (int64_t)h * a.dq_sh + cg * 32;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(sm.bar(BB_UEMPTY + (n & 1)));
+            // the next unit and its rows' scalars, beside the last product
+            if (!take_unit(n + 1)) break;
+            if (!bt_wait_converged(sm.bar(BB_OFULL), n & 1, sm.abort_addr(), a.status, kStatusWaitOFull)) break;
+            tc_fence_after();
             if (cg * 32 < D) {                                            // warp-uniform: the row has D elements
-                int64_t off = -1;                                         // -1: a padding row
-                if (i < sq.n_text)
-                    off = (sq.aug_off + (int64_t)iq * (a.k + a.m) + (i - iq * a.k)) * a.dq_st + (int64_t)h * a.dq_sh + cg * 32;
                 uint32_t o[32];
                 tmem_ld32(tDQ + lane_sel + cg * 32, o);
                 tc_wait_ld();
+                // (the accumulators are read before this warp's first hand-over of the next unit, behind which they are overwritten)
+                tc_fence_before();
                 uint4 w[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -781,11 +1004,11 @@ __device__ __forceinline__ void bt_dq_block(const BwdArgs& a, const BwdMaps& map
                     w[e].z = pack_bf16x2(__uint_as_float(o[8 * e + 4]) * a.scale, __uint_as_float(o[8 * e + 5]) * a.scale);
                     w[e].w = pack_bf16x2(__uint_as_float(o[8 * e + 6]) * a.scale, __uint_as_float(o[8 * e + 7]) * a.scale);
                 }
-                quad_transpose(w, lane);                                  // w[j]: 16 bytes of the group's row j
+                quad_transpose(w, lane);                                  // w[e]: 16 bytes of the group's row e
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int64_t at = __shfl_sync(0xffffffffu, off, (lane & 28) + j);
-                    if (at >= 0) *reinterpret_cast<uint4*>(a.dq + at + (lane & 3) * 8) = w[j];
+                for (int e = 0; e < 4; ++e) {
+                    const int64_t at = __shfl_sync(0xffffffffu, off, (lane & 28) + e);
+                    if (at >= 0) *reinterpret_cast<uint4*>(a.dq + at + (lane & 3) * 8) = w[e];
                 }
             }
         }
@@ -799,23 +1022,22 @@ __device__ __forceinline__ void bt_dq_block(const BwdArgs& a, const BwdMaps& map
 // the SMs that the one in front leaves (programmatic dependent launches), longest CTAs first (64, about 40 and 9 + 16 tiles
 // each at 32,768 tokens), so that the tails of the first two are filled (training layer of 7,942 ragged tokens, 16/16 heads
 // 619 -> 590 us, 2 x 8,192 tokens 2,132 -> 2,064 us; nothing at 2 x 32,768).
-// Nothing here waits for the launch in front, which was itself started behind the preparation; only the last block of each
-// waits for its end, so that the kernel behind the three, an ordinary launch, finds all of them done.  What the preparation and
-// the pack wrote stands in L2 by then, but without a wait of its own (pdl_wait) a kernel has no promise that its L1 has dropped
-// those addresses' old contents: the tiles come by TMA, lse and delta by loads that bypass L1 (but in the first launch, an
-// ordinary one), the sums are added in L2.  2 x 32,768 tokens, backward alone: 9,692 us with every load through L1, 9,725 with
-// every one past it, 9,711 so, and another 16 less with dQ's rows on their way beside the set-up; a fence.acq_rel.gpu at the
-// start of each CTA instead costs 0.7 - 1.6 % of a training layer.
+// Nothing here waits for the launch in front, which was itself started behind the preparation; only the CTA that has the first
+// block of each waits for its end when it is through, so that the kernel behind the three, an ordinary launch, finds all of them
+// done.  What the preparation and the pack wrote stands in L2 by then, but without a wait of its own (pdl_wait) a kernel has no
+// promise that its L1 has dropped those addresses' old contents: the tiles come by TMA, lse and delta by loads that bypass L1,
+// the sums are added in L2.  A fence.acq_rel.gpu at the start of each CTA instead costs 0.7 - 1.6 % of a training layer.
+// The CTA that started as the grid's first block; the producer's thread of a CTA that took that block over waits there.
 __device__ __forceinline__ void bt_end_behind_front()
 {
-    if (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1) pdl_wait();
+    if (blockIdx.x + blockIdx.y == 0) pdl_wait();
 }
 template <int D>
 __global__ void __maxnreg__(kBwdTcRegs)
-ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ BwdMaps maps, const int summ, const int seg_tiles, const int store)
+ksa_bwd_dkv_tc_kernel(const __grid_constant__ BwdArgs a, const __grid_constant__ BwdMaps maps, const int summ, const int seg_tiles, const int segs, const int store)
 {
     pdl_launch_dependents();
-    bt_dkv_block<D>(a, maps, summ, seg_tiles, store);
+    bt_dkv_block<D>(a, maps, summ, seg_tiles, segs, store);
     bt_end_behind_front();
 }
 template <int D>
@@ -848,31 +1070,31 @@ bool bwd_text_keys_stored(const BwdArgs& a) { return bwd_text_span(a) <= bwd_seg
 
 cudaError_t launch_bwd_tc(const BwdArgs& a, const BwdMaps& maps, cudaStream_t stream)
 {
-    const int n_qt = a.max_text_pad / 128;
     const size_t smem = a.D == 128 ? BtMap<128>::kSmem : BtMap<64>::kSmem;
     bool first = true;                                                    // behind the preparation: an ordinary launch
     for (int summ = 1; summ >= 0; --summ) {
         if (summ && (a.m <= 0 || a.max_n_summ <= 0)) continue;
-        const long long span = summ ? n_qt : bwd_text_span(a);
-        const int tiles = summ ? (a.max_n_summ + 127) / 128 : n_qt;
-        // a CTA walks seg query tiles x G heads: 16 tiles with four or more heads per KV head, more with fewer (the
-        // start-up and the final atomics of a CTA are spread over about 64 streamed tiles either way)
+        const long long span = summ ? a.max_text_pad / 128 : bwd_text_span(a);
+        // a unit walks seg query tiles x G heads: 16 tiles with four or more heads per KV head, more with fewer (the
+        // final atomics of a unit are spread over about 64 streamed tiles either way)
         const int seg = bwd_seg_tiles(a);
         const int store = (!summ && bwd_text_keys_stored(a)) ? 1 : 0;
-        const dim3 grid((unsigned)((span + seg - 1) / seg), (unsigned)tiles, (unsigned)(a.num_seqs * a.Hkv));
+        const long long segs = (span + seg - 1) / seg, blocks = (summ ? a.summ_rows : a.text_rows) / 128 * segs;
+        if (blocks > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+        const dim3 grid((unsigned)blocks, (unsigned)a.Hkv);
         auto* kernel = a.D == 128 ? ksa_bwd_dkv_tc_kernel<128> : ksa_bwd_dkv_tc_kernel<64>;
         cudaError_t e;
         if (first) {
-            kernel<<<grid, kBwdTcThreads, smem, stream>>>(a, maps, summ, seg, store);
+            kernel<<<grid, kBwdTcThreads, smem, stream>>>(a, maps, summ, seg, (int)segs, store);
             e = cudaGetLastError();
         } else {
-            e = launch_dependent(kernel, grid, kBwdTcThreads, smem, stream, a, maps, summ, seg, store);
+            e = launch_dependent(kernel, grid, kBwdTcThreads, smem, stream, a, maps, summ, seg, (int)segs, store);
         }
         if (e != cudaSuccess) return e;
         first = false;
     }
     return launch_dependent(a.D == 128 ? ksa_bwd_dq_tc_kernel<128> : ksa_bwd_dq_tc_kernel<64>,
-                            dim3((unsigned)n_qt, (unsigned)a.Hq, (unsigned)a.num_seqs), kBwdTcThreads, smem, stream, a, maps);
+                            dim3((unsigned)(a.text_rows / 128), (unsigned)a.Hq), kBwdTcThreads, smem, stream, a, maps);
 }
 
 }  // namespace ksa

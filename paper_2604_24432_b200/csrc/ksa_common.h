@@ -76,6 +76,8 @@ enum DeviceStatus : int32_t {
     kStatusWaitRowSums = 11,    // CTA-pair kernel: the other softmax group's row sums
     kStatusWaitPvDone = 12,     // CTA-pair kernel: completion of O += P V
     kStatusWaitOEmpty = 13,     // CTA-pair kernel: the epilogue's read of O
+    kStatusWaitUnit = 15,       // persistent kernels: a unit descriptor, or its slot
+    kStatusWaitNextBlock = 16,  // persistent kernels: the answer to a request for another block
     kStatusBounds = 14,         // KSA_DEBUG builds: a global output index was outside its tensor; the access was skipped
 };
 

@@ -106,6 +106,30 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // The kernel behind this one may be launched once every block has come here (or ended).
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// ---- cluster launch control ------------------------------------------------------------------
+// Asks for a block of this grid that has not started: if there is one it will not be launched, and its index is the caller's.
+// The 16-byte answer arrives at `dst` (shared memory), counted on `bar`.  Nothing is asked for after a refusal.
+__device__ __forceinline__ void clc_try_cancel(uint32_t dst, uint32_t bar)
+{
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(dst), "r"(bar) : "memory");
+}
+// Reads the answer: true and the block's index, or false.
+__device__ __forceinline__ bool clc_query(uint32_t src, int& x, int& y, int& z)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b128 h;\n\t"
+        "ld.shared.b128 h, [%4];\n\t"
+        "mov.b32 %0, 0;\n\tmov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\t"
+        "selp.u32 %3, 1, 0, p;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%0, %1, %2, _}, h;\n\t}"
+        : "=&r"(x), "=&r"(y), "=&r"(z), "=&r"(ok) : "r"(src) : "memory");
+    return ok != 0;
+}
+// Orders this thread's accesses to shared memory before later asynchronous ones (TMA, the answers above)
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 // ---- tcgen05: TMEM allocation ---------------------------------------------------------
 __device__ __forceinline__ void tmem_alloc(uint32_t smem_dst, uint32_t ncols)
 {
@@ -156,6 +180,14 @@ __device__ __forceinline__ void tc_commit_warp(uint32_t leader, uint32_t bar)
     asm volatile(
         "{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %0, 0;\n\t"
         "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%1];\n\t}"
+        ::"r"(leader), "r"(bar) : "memory");
+}
+// Arrival of the issuing lane of a converged warp (no branch: the warp's operands stay in uniform registers)
+__device__ __forceinline__ void mbar_arrive_warp(uint32_t leader, uint32_t bar)
+{
+    asm volatile(
+        "{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %0, 0;\n\t"
+        "@e mbarrier.arrive.shared::cta.b64 _, [%1];\n\t}"
         ::"r"(leader), "r"(bar) : "memory");
 }
 // One lane of a converged warp (1 there, 0 elsewhere)

@@ -96,6 +96,16 @@ def test_backward_matches_oracle(ctx, lens, k, m, C, Hq, Hkv, D, flags):
     _check("dv", dv.double().cpu().numpy(), rdv)
 
 
+@pytest.mark.parametrize("lens,k,m,C,Hq,Hkv,D", [
+    ([7, 1, 90, 128, 129, 3, 64, 256, 5] * 6, 8, 1, 4, 8, 4, 64),      # units of one and two tiles, several to a CTA
+    ([3, 1500, 5, 7, 900, 2], 8, 1, 16, 16, 8, 128),                   # sequences without summary rows between others
+    ([2300, 300], 8, 1, 1000, 4, 1, 128),                              # two segments of query tiles, most second ones empty
+])
+def test_backward_many_units_per_cta(ctx, lens, k, m, C, Hq, Hkv, D):
+    """More units of work than SMs: CTAs go on to the blocks that have not started."""
+    test_backward_matches_oracle(ctx, lens, k, m, C, Hq, Hkv, D, 0)
+
+
 @pytest.mark.parametrize("workload", ["32k", "128k", "varlen"])
 def test_backward_full_size_identities(ctx, workload):
     """Full-size workloads, in the launch configuration the bench times: two identities that hold for the exact
