@@ -304,6 +304,7 @@ void build_schedule(const ksa_params* p, HostSchedule& hs, int target_chunks, in
     // 20.4 -> 18.4 us; 517 tokens, 32 heads, 160 items: 18.3 against 21.1 us).  The CTA-pair kernel wants pairs.
     if (heads_per_item == 2 && target_chunks == 0 && !(p->flags & KSA_FLAG_CTA_PAIR_KERNEL) &&
         (int64_t)base.size() * p->num_q_heads <= num_sms) heads_per_item = 1;
+    const int G = p->num_q_heads / p->num_kv_heads;
     hs.work.clear();
     hs.work.reserve(base.size() * (p->num_q_heads / heads_per_item));
     for (const Tagged& tg : base) {
@@ -319,6 +320,7 @@ void build_schedule(const ksa_params* p, HostSchedule& hs, int target_chunks, in
             w.ns_tiles = bi.ns_tiles; w.ns_nomask = bi.ns_nomask;
             w.band_lo = bi.band_lo; w.band_hi = bi.band_hi;
             w.band_nomask_lo = bi.nm_lo; w.band_nomask_hi = bi.nm_hi;
+            w.kv_head = h / G; w.kv_per_tile = (h + heads_per_item - 1) / G != w.kv_head ? 2 : 1;
             hs.work.push_back(w);
         }
     }
@@ -341,7 +343,8 @@ static bool schedule_in_range(const ksa_params* p, const HostSchedule& hs)
         const SeqInfo& s = hs.seqs[w.seq];
         if (w.q_tile < 0 || (int64_t)w.q_tile * kTileM >= s.text_pad) return false;
         if (w.n_heads < 1 || w.n_heads > 2 || w.head0 < 0 || w.head0 + w.n_heads > p->num_q_heads) return false;
-        if ((w.head0 + w.n_heads - 1) / G - w.head0 / G > 1) return false;                  // one KV head per item, or one per head
+        // one KV head per item, or one per head
+        if (w.kv_head != w.head0 / G || w.kv_per_tile != 1 + (w.head0 + w.n_heads - 1) / G - w.kv_head || w.kv_per_tile > 2) return false;
         if (w.ns_tiles < 0 || (int64_t)w.ns_tiles * kTileN > s.summ_pad || w.ns_nomask < 0 || w.ns_nomask > w.ns_tiles) return false;
         if (w.band_lo < 0 || w.band_hi < w.band_lo || w.band_hi != w.q_tile) return false;
         if (w.band_nomask_lo < w.band_lo || w.band_nomask_hi > w.band_hi + 1 || w.band_nomask_hi < w.band_nomask_lo) return false;

@@ -33,7 +33,8 @@ struct WorkItem {
     int32_t band_lo, band_hi; // text-stream tiles [band_lo, band_hi] are visited
     int32_t band_nomask_lo;   // text tiles [band_nomask_lo, band_nomask_hi) need no mask
     int32_t band_nomask_hi;
-    int32_t reserved0, reserved1;
+    int32_t kv_head;          // KV head of head0
+    int32_t kv_per_tile;      // K (V) tiles per key tile: 1, or 2 where the two heads belong to two KV heads
 };
 static_assert(sizeof(WorkItem) == 48, "WorkItem layout");
 
@@ -48,6 +49,7 @@ struct KernelArgs {
     uint32_t flags;
     float scale;            // softmax scale
     float scale_log2;       // scale * log2(e)
+    uint64_t k_inverse;     // floor(2^64 / k) + 1, for i / k as a product (0 where k is 1); set by the text kernel's launch
     int64_t total_aug;
     int64_t text_rows;      // padded rows of the packed text stream
     int64_t summ_rows;      // padded rows of the packed summary stream

@@ -34,8 +34,13 @@
 // tile, 1.477 ms with the shared slot and one issuing thread, 1.466 ms with a converged issuing warp, 1.328 ms with
 // two.  131,072 tokens, 32/4 heads: 18.9 -> 16.6 ms a call (the clock falls from 1,700 to 1,430 MHz under the
 // power limit as the pipes fill), 8,192 tokens: 258 -> 229 us.
-// What bounds it now: the softmax warps.  A key tile and pair of query tiles takes 2,920 cycles, 2,048 of them
-// exponentials on the special-function unit; the issuing warps wait 60 % of the time.
+// What bounds it now: the round trip of the score slot (product 560 cycles, hand-over 300, load 300 - 400, hand-over 100, for
+// each query tile in turn) and the softmax warps' own loop (1,700 - 1,900 cycles of maximum and exponentials while the other
+// group's run beside them, 300 for each hand-over).  A key tile and pair of query tiles takes 2,850 cycles.  One to three of
+// eight exponential pairs as polynomials on the FMA pipe: 317 -> 319, 317, 343 thousand cycles (8,192 tokens, 32/8 heads), so
+// the special-function unit is not what it waits for.  A work item's start and end cost 5,000 more: its entry and divisions
+// (KV head and division by k come prepared: 325 -> 318), O's last product and the epilogue.  The epilogue in four warps of
+// its own (208 / 48 registers) took 6,400 cycles a tile beside the softmax and held up the next item's first product: 353.
 //
 // Every mbarrier wait is bounded: on timeout the thread records which wait gave up in the
 // status word, raises a CTA-wide abort flag, all roles leave their loops, the producer
@@ -104,7 +109,7 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
     auto v_empty = [&](int st) -> uint32_t { return bar(kBarKv + 2 * Cfg::kStagesK + Cfg::kStagesV + st); };
 
     const int tid = threadIdx.x;
-    const int warp = tid >> 5;
+    const int warp = (int)__reduce_or_sync(0xffffffffu, (unsigned)tid >> 5);     // (uniform to the compiler: 330 -> 325 thousand cycles)
     const int lane = tid & 31;
 
     if (tid == 0) {
@@ -137,7 +142,6 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
     pdl_wait();
     pdl_launch_dependents();
 
-    const int G = a.Hq / a.Hkv;
     const int grid = (int)gridDim.x;
     const int cta = (int)blockIdx.x;
     // items are taken in snake order over the longest-first list: round r gives this CTA
@@ -171,8 +175,7 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
                     if (idx >= a.num_work) break;
                     const WorkItem w = a.work[idx];
                     const SeqInfo sq = a.seqs[w.seq];
-                    const int hk = w.head0 / G;
-                    const int nsplit = ((w.head0 + w.n_heads - 1) / G != hk) ? 2 : 1;
+                    const int hk = w.kv_head, nsplit = w.kv_per_tile;
                     const int T = w.ns_tiles + (w.band_hi - w.band_lo + 1);
                     auto load_q = [&](int t) {
                         if (!bounded_wait(bar(BAR_QEMPTY + t), ((q_phase >> t) & 1u) ^ 1u, abort_addr, a.status, kStatusWaitQEmpty)) { alive = false; return; }
@@ -240,7 +243,7 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
                     const WorkItem w = a.work[idx];
                     const int T = __shfl_sync(0xffffffffu, w.ns_tiles + (w.band_hi - w.band_lo + 1), 0);
                     const int nh = __shfl_sync(0xffffffffu, w.n_heads, 0);
-                    const bool split = __shfl_sync(0xffffffffu, (w.head0 + w.n_heads - 1) / G - w.head0 / G, 0) != 0;
+                    const bool split = __shfl_sync(0xffffffffu, w.kv_per_tile, 0) == 2;
                     for (int j = 0; j < T && alive; ++j) {
 #pragma unroll
                         for (int t = 0; t < 2; ++t) {
@@ -276,7 +279,7 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
                     const WorkItem w = a.work[idx];
                     const int T = __shfl_sync(0xffffffffu, w.ns_tiles + (w.band_hi - w.band_lo + 1), 0);
                     const int nh = __shfl_sync(0xffffffffu, w.n_heads, 0);
-                    const bool split = __shfl_sync(0xffffffffu, (w.head0 + w.n_heads - 1) / G - w.head0 / G, 0) != 0;
+                    const bool split = __shfl_sync(0xffffffffu, w.kv_per_tile, 0) == 2;
                     for (int j = 0; j < T && alive; ++j) {
 #pragma unroll
                         for (int t = 0; t < 2; ++t) {
@@ -324,7 +327,7 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
             const int idx = item_index(r);
             if (idx >= a.num_work) break;
             const WorkItem w = a.work[idx];
-            const int nsplit = ((w.head0 + w.n_heads - 1) / G != w.head0 / G) ? 2 : 1;   // ring stages per K / V tile
+            const int nsplit = w.kv_per_tile;                // ring stages per K / V tile
             // the next stage this thread hands back, and how far on the one after it stands
             int rel_k = (k_base + (nsplit - 1) * t) % Cfg::kStagesK, rel_v = (v_base + (nsplit - 1) * t) % Cfg::kStagesV;
             k_base = (k_base + nsplit * (w.ns_tiles + (w.band_hi - w.band_lo + 1))) % Cfg::kStagesK;
@@ -345,16 +348,22 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
             const int i_raw = w.q_tile * kTileM + row;
             const bool valid = i_raw < sq.n_text;
             const int i = valid ? i_raw : sq.n_text - 1;     // padding rows mimic the last row; never stored
-            const int chunk = i / a.k;
+            const int chunk = a.k_inverse ? (int)__umul64hi((unsigned long long)i, a.k_inverse) : i;      // i / k
             const int far = max(0, chunk - a.C);
             const int lo_i = far * a.k;                      // Eq. 3: first visible text token
             const int cnt_i = far * a.m;                     // Eq. 3: summaries [0, cnt_i) visible
             float m_used = -INFINITY, l_run = 0.f;
 
+            // Both barriers of a tile are asked for ahead of their waits: a passed wait costs some 300 cycles beside the other
+            // group's exponentials (8,192 tokens, 32/8 heads: 317 -> 312 thousand cycles; 32,413 ragged tokens 1,304 -> 1,287).
+            bool s_ok = false;                               // the scores of this tile are known to be there
             for (int j = 0; j < T; ++j) {
-                bool ok = bounded_wait(bar(BAR_SFULL + t), sf_phase, abort_addr, a.status, kStatusWaitSFull);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) { alive = false; break; }
+                bool ok;
+                if (!__all_sync(0xffffffffu, s_ok)) {
+                    ok = bounded_wait(bar(BAR_SFULL + t), sf_phase, abort_addr, a.status, kStatusWaitSFull);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) { alive = false; break; }
+                }
                 sf_phase ^= 1u;
                 tc_fence_after();
                 uint32_t s[128];
@@ -418,6 +427,7 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
                 const float neg_m = (m_used == -INFINITY) ? 0.f : -m_used;
                 const float2 sc2 = make_float2(scale_log2, scale_log2);
                 const float2 nm2 = make_float2(neg_m, neg_m);
+                bool pv_ok = false;                           // the product before is known to be done
                 float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
                 // probabilities of the column pair (2q, 2q+1), packed into s[q]; the scale-and-shift
                 // and the row sum work on packed pairs (half the FMA-pipe instructions)
@@ -427,18 +437,22 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
                     float2 pr;
                     pr.x = ex2_approx(x.x); pr.y = ex2_approx(x.y);
                     if (q & 1) lb = fadd2(lb, pr); else la = fadd2(la, pr);
+                    if (q == 48 && j > 0) pv_ok = mbar_test_wait(bar(BAR_PVDONE + t), pv_phase);
                     s[q] = pack_bf16x2(pr.x, pr.y);
                 }
                 l_run += (la.x + la.y) + (lb.x + lb.y);
                 if (j > 0) {
                     // O_t += P_t V(j-1) has read P_t and written O_t
-                    ok = bounded_wait(bar(BAR_PVDONE + t), pv_phase, abort_addr, a.status, kStatusWaitPvDone);
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) { alive = false; break; }
+                    if (!__all_sync(0xffffffffu, pv_ok)) {
+                        ok = bounded_wait(bar(BAR_PVDONE + t), pv_phase, abort_addr, a.status, kStatusWaitPvDone);
+                        ok = __all_sync(0xffffffffu, ok);
+                        if (!ok) { alive = false; break; }
+                    }
                     pv_phase ^= 1u;
                     if (releaser) release_v();               // V(j-1)
                     tc_fence_after();
                 }
+                s_ok = j + 1 < T && mbar_test_wait(bar(BAR_SFULL + t), sf_phase);
                 {
                     uint32_t (&p0)[32] = *reinterpret_cast<uint32_t (*)[32]>(&s[0]);
                     uint32_t (&p1)[32] = *reinterpret_cast<uint32_t (*)[32]>(&s[32]);
@@ -470,7 +484,7 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
             tc_fence_after();
             const float inv_l = 1.f / l_run;
             const int h = w.head0 + t;
-            const int64_t aug = sq.aug_off + (int64_t)(i / a.k) * s_len + (i % a.k);
+            const int64_t aug = sq.aug_off + (int64_t)chunk * s_len + (i - chunk * a.k);
             const bool store = valid && ksa_out_row_ok(a, aug, h);
             // a row stands in one lane: four lanes exchange 64 bytes of their rows, so that a store touches 8 lines, not 32
             // (the epilogues took 246 of 3,207 cycles a key tile at 32,768 tokens: the store path takes a line per cycle)
@@ -518,8 +532,11 @@ cudaError_t launch_text_tc(const KernelArgs& a, const TextMaps& maps, int num_sm
 {
     if (a.num_work <= 0) return cudaSuccess;
     const int grid = a.num_work < num_sms ? a.num_work : num_sms;
-    return a.D == 128 ? launch_dependent(ksa_text_tc_kernel<128>, dim3((unsigned)grid), kThreadsTc, TcCfg<128>::kSmemBytes, stream, a, maps)
-                      : launch_dependent(ksa_text_tc_kernel<64>, dim3((unsigned)grid), kThreadsTc, TcCfg<64>::kSmemBytes, stream, a, maps);
+    KernelArgs ka = a;
+    // exact for the rows of a sequence: the product is off by less than i / 2^64, and i / k by 1 / k or more from the next integer
+    ka.k_inverse = a.k > 1 ? ~0ull / (uint64_t)a.k + 1 : 0;
+    return a.D == 128 ? launch_dependent(ksa_text_tc_kernel<128>, dim3((unsigned)grid), kThreadsTc, TcCfg<128>::kSmemBytes, stream, ka, maps)
+                      : launch_dependent(ksa_text_tc_kernel<64>, dim3((unsigned)grid), kThreadsTc, TcCfg<64>::kSmemBytes, stream, ka, maps);
 }
 
 }  // namespace ksa
