@@ -157,6 +157,18 @@ bool direct_ok(const ksa_params* p)
     return true;
 }
 
+// Batches that need the workspace all the same (some length is no whole number of chunks): where the tiles are whole chunks in
+// both views, the kernels read full tiles in place and only each sequence's last text and summary tile is packed, so that no
+// sequence sees rows of its neighbour.  Packing all rows took 478 us of 7.0 ms for 127,475 tokens of 32/8 heads, 12 - 25 % of a
+// prompt of a few thousand tokens and, of a ragged training layer of 7,942 tokens with 16/16 heads, 64 of 550 us.
+static int read_mode(const ksa_params* p)
+{
+    if (direct_ok(p)) return kReadInPlace;
+    const int k = p->chunk_len, m = p->summaries_per_chunk;
+    if (p->flags & (KSA_FLAG_REFERENCE_KERNEL | KSA_FLAG_CTA_PAIR_KERNEL | KSA_FLAG_BWD_MMA_SYNC_KERNELS)) return kReadPacked;      // those kernels know the streams only
+    return kTileM % k == 0 && (m == 0 || kTileN % m == 0) ? kReadTails : kReadPacked;
+}
+
 void build_layout(const ksa_params* p, HostSchedule& hs)
 {
     const int k = p->chunk_len, m = p->summaries_per_chunk;
@@ -723,9 +735,26 @@ static int encode_chunk_map(ksa_ctx* ctx, CUtensorMap* map, const void* base, in
     return KSA_OK;
 }
 
+// The same for sequences that start anywhere: dims {D, rows_per_chunk, start, chunks, H}, `start` the row of the [chunk,
+// chunk_rows] grid at which a sequence's chunks start.  (The extents describe more rows than the tensor has; a box is only asked
+// for where all its rows are rows of one sequence.)
+static int encode_start_map(ksa_ctx* ctx, CUtensorMap* map, const void* base, int D, int rows_per_chunk, int chunk_rows,
+                            int64_t total_rows, int H, int64_t st, int64_t sh)
+{
+    const cuuint64_t dims[5] = {(cuuint64_t)D, (cuuint64_t)rows_per_chunk, (cuuint64_t)chunk_rows, (cuuint64_t)(total_rows / chunk_rows + 1), (cuuint64_t)H};
+    const cuuint64_t strides[4] = {(cuuint64_t)st * 2, (cuuint64_t)st * 2, (cuuint64_t)chunk_rows * st * 2, (cuuint64_t)sh * 2};
+    const cuuint32_t box[5] = {64, (cuuint32_t)rows_per_chunk, 1, (cuuint32_t)(kTileN / rows_per_chunk), 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    CUresult r = ctx->encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
+                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) { ctx->last_cuda_error = (int)r; return KSA_ERR_CUDA; }
+    return KSA_OK;
+}
+
 // Kernel arguments of a whole problem (schedule already cached and uploaded in ctx).
 static KernelArgs make_args(ksa_ctx* ctx, const ksa_params* p, const void* q, const void* k, const void* v, void* out,
-                            float* lse, void* workspace, const WorkspaceLayout& wl, bool direct = false)
+                            float* lse, void* workspace, const WorkspaceLayout& wl, int mode = kReadPacked)
 {
     const HostSchedule& hs = ctx->sched;
     char* ws = (char*)workspace;
@@ -740,7 +769,7 @@ static KernelArgs make_args(ksa_ctx* ctx, const ksa_params* p, const void* q, co
     a.total_aug = hs.total_aug; a.text_rows = hs.text_rows; a.summ_rows = hs.summ_rows;
     a.max_n_summ = hs.max_n_summ;
     a.r_seq = -1;
-    a.direct = direct ? 1 : 0;
+    a.direct = mode;
     a.q = (const uint16_t*)q; a.kx = (const uint16_t*)k; a.v = (const uint16_t*)v;
     a.out = (uint16_t*)out; a.lse = lse;
     a.q_st = p->q_stride_tok; a.q_sh = p->q_stride_head; a.k_st = p->k_stride_tok; a.k_sh = p->k_stride_head;
@@ -787,6 +816,21 @@ static int prepare_text(ksa_ctx* ctx, const KernelArgs& a, uint32_t flags, FwdMa
     }
     if (fm.pair && ctx->max_pairs < 1) fm.pair = false;
     int rc;
+    if (a.direct == kReadTails) {
+        const int s_len = a.k + a.m;
+        struct { CUtensorMap* map; const uint16_t* base; int per; int H; int64_t st, sh; CUtensorMap* tail; uint16_t* stream; int64_t rows; } t[5] = {
+            {&maps.qt, a.q, a.k, a.Hq, a.q_st, a.q_sh, &maps.qt_tail, a.qt, a.text_rows},
+            {&maps.kt, a.kx, a.k, a.Hkv, a.k_st, a.k_sh, &maps.kt_tail, a.kt, a.text_rows},
+            {&maps.vt, a.v, a.k, a.Hkv, a.v_st, a.v_sh, &maps.vt_tail, a.vt, a.text_rows},
+            {&maps.ks, a.kx + (int64_t)a.k * a.k_st, a.m, a.Hkv, a.k_st, a.k_sh, &maps.ks_tail, a.ks, a.summ_rows},      // summary rows start k rows into each chunk
+            {&maps.vs, a.v + (int64_t)a.k * a.v_st, a.m, a.Hkv, a.v_st, a.v_sh, &maps.vs_tail, a.vs, a.summ_rows}};
+        for (int i = 0; i < (a.m > 0 ? 5 : 3); ++i) {
+            if ((rc = encode_start_map(ctx, t[i].map, t[i].base, a.D, t[i].per, s_len, a.total_aug, t[i].H, t[i].st, t[i].sh)) != KSA_OK) return rc;
+            if ((rc = encode_stream_map(ctx, t[i].tail, t[i].stream, a.D, t[i].rows, t[i].H)) != KSA_OK) return rc;
+        }
+        if (a.m == 0) { maps.ks = maps.kt; maps.vs = maps.vt; maps.ks_tail = maps.kt_tail; maps.vs_tail = maps.vt_tail; }    // never used
+        return KSA_OK;
+    }
     if (a.direct) {
         const int s_len = a.k + a.m;
         const int64_t chunks = a.total_aug / s_len;
@@ -852,14 +896,14 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_fwd(ksa_ctx* ctx,
     for (int i = 0; i < 5; ++i) if (ptrs[i] & 15) return KSA_ERR_INVALID_ARG;
     if ((rc = ensure_schedule(ctx, p, true, 0, (cudaStream_t)cuda_stream)) != KSA_OK) return rc;
     const HostSchedule& hs = ctx->sched;
-    const bool direct = direct_ok(p);
+    const int mode = read_mode(p);
     const WorkspaceLayout wl = workspace_layout(p, hs);
-    if (!direct && (!workspace || workspace_bytes < wl.total || ((uintptr_t)workspace & 255))) return KSA_ERR_WORKSPACE;
+    if (mode != kReadInPlace && (!workspace || workspace_bytes < wl.total || ((uintptr_t)workspace & 255))) return KSA_ERR_WORKSPACE;
 
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    KernelArgs a = make_args(ctx, p, q, k, v, out, lse, workspace, wl, direct);
+    KernelArgs a = make_args(ctx, p, q, k, v, out, lse, workspace, wl, mode);
     cudaError_t e;
-    if (!direct) {
+    if (mode != kReadInPlace) {
         if ((e = launch_pack(a, stream)) != cudaSuccess) return cuda_fail(ctx, e);
         ctx->launches += 1;
     }
@@ -943,7 +987,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_fwd_part(ksa_ctx*
     if (c0 == c1) return KSA_OK;
 
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    KernelArgs a = make_args(ctx, p, q, k, v, out, lse, workspace, wl, direct);
+    KernelArgs a = make_args(ctx, p, q, k, v, out, lse, workspace, wl, direct ? kReadInPlace : kReadPacked);
     cudaError_t e;
     if (!direct) {
         // the packed streams of the whole batch (rows after the part's last row are never read unmasked, but
@@ -1036,7 +1080,8 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_bwd(ksa_ctx* ctx,
     // packed streams of the forward pass (text Q, K, V and summary K, V) -- not needed when the tensor-core kernels
     // can read whole tiles straight from the caller's tensors (the no-pack case of the forward pass)
     const bool direct = direct_ok(p) && !(p->flags & KSA_FLAG_BWD_MMA_SYNC_KERNELS);
-    KernelArgs fa = make_args(ctx, p, q, k, v, dq /* unused */, const_cast<float*>(lse), workspace, bl.fwd);
+    const int mode = direct ? kReadInPlace : read_mode(p) == kReadTails ? kReadTails : kReadPacked;
+    KernelArgs fa = make_args(ctx, p, q, k, v, dq /* unused */, const_cast<float*>(lse), workspace, bl.fwd, mode);
     if (!direct && (e = launch_pack(fa, stream)) != cudaSuccess) return cuda_fail(ctx, e);
     BwdArgs a{};
     a.seqs = ctx->d_seqs; a.num_seqs = p->num_seqs;
@@ -1056,7 +1101,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_bwd(ksa_ctx* ctx,
     a.dot = (uint16_t*)(ws + bl.dot); a.lse_t = (float*)(ws + bl.lse_t); a.delta_t = (float*)(ws + bl.delta_t);
     a.dkt = (float*)(ws + bl.dkt); a.dvt = (float*)(ws + bl.dvt); a.dks = (float*)(ws + bl.dks); a.dvs = (float*)(ws + bl.dvs);
     a.status = ctx->d_status;
-    a.direct = direct ? 1 : 0;
+    a.direct = mode;
     // The four accumulators are contiguous in the workspace: one clear.  Where one CTA of the tensor-core dK / dV kernel
     // covers every query tile that sees a text key tile, that launch stores the text keys' rows instead of adding to them:
     // then only the summary keys' accumulators are cleared.
@@ -1076,7 +1121,21 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_bwd(ksa_ctx* ctx,
             ctx->bwd_tc_ready = true;
         }
         BwdMaps bm;
-        if (direct) {
+        if (mode == kReadTails) {
+            const int s_len = a.k + a.m;
+            struct { CUtensorMap* map; const uint16_t* base; int per; int H; int64_t st, sh; CUtensorMap* tail; const uint16_t* stream; int64_t rows; } t[6] = {
+                {&bm.qt, a.q, a.k, a.Hq, a.q_st, a.q_sh, &bm.qt_tail, a.qt, a.text_rows},
+                {&bm.dot, a.dout, a.k, a.Hq, a.do_st, a.do_sh, &bm.dot_tail, a.dot, a.text_rows},
+                {&bm.kt, a.kx, a.k, a.Hkv, a.k_st, a.k_sh, &bm.kt_tail, a.kt, a.text_rows},
+                {&bm.vt, a.v, a.k, a.Hkv, a.v_st, a.v_sh, &bm.vt_tail, a.vt, a.text_rows},
+                {&bm.ks, a.kx + (int64_t)a.k * a.k_st, a.m, a.Hkv, a.k_st, a.k_sh, &bm.ks_tail, a.ks, a.summ_rows},
+                {&bm.vs, a.v + (int64_t)a.k * a.v_st, a.m, a.Hkv, a.v_st, a.v_sh, &bm.vs_tail, a.vs, a.summ_rows}};
+            for (int i = 0; i < (a.m > 0 ? 6 : 4); ++i) {
+                if ((rc = encode_start_map(ctx, t[i].map, t[i].base, a.D, t[i].per, s_len, a.total_aug, t[i].H, t[i].st, t[i].sh)) != KSA_OK) return rc;
+                if ((rc = encode_stream_map(ctx, t[i].tail, const_cast<uint16_t*>(t[i].stream), a.D, t[i].rows, t[i].H)) != KSA_OK) return rc;
+            }
+            if (a.m == 0) { bm.ks = bm.kt; bm.vs = bm.vt; bm.ks_tail = bm.kt_tail; bm.vs_tail = bm.vt_tail; }    // never used
+        } else if (direct) {
             // chunked views [D, rows per chunk, chunk, head] of the caller's tensors; summary rows start k rows into a chunk
             const int s_len = a.k + a.m;
             const int64_t chunks = a.total_aug / s_len;
@@ -1236,7 +1295,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_fwd_prepared(ksa_
     const WorkspaceLayout wl = workspace_layout(p, hs);
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     // the attention kernels read the packed streams only (a.direct = 0); q, k, v of the arguments are the projections
-    KernelArgs a = make_args(ctx, p, q_main, k_main, v_main, out, lse, workspace, wl, false);
+    KernelArgs a = make_args(ctx, p, q_main, k_main, v_main, out, lse, workspace, wl, kReadPacked);
     uint16_t* qs = (uint16_t*)((char*)workspace + qs_off);
 
     PrepArgs pa{};

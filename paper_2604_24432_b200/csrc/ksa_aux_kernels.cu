@@ -28,15 +28,21 @@ __device__ __forceinline__ uint16_t float_to_bf16_bits(float f)
 // ---------------------------------------------------------------------------------------
 constexpr int kPackRows = 4;
 
+// kReadTails: 32 blocks for each sequence's last text tile, where that is not full, and 32 for its last summary tile.
+constexpr int kTailBlocks = kTileM / kPackRows;
+
 __global__ void __launch_bounds__(256) ksa_pack_kernel(KernelArgs a, int blocks_text, int rows_text, int rows_summ)
 {
     ptx::pdl_launch_dependents();                                // the text kernel sets itself up meanwhile
-    const bool ranged = a.r_seq >= 0;
+    const bool ranged = a.r_seq >= 0, tails = a.direct == kReadTails;
     const bool text = (int)blockIdx.x < blocks_text;
-    const int row0 = ((int)blockIdx.x - (text ? 0 : blocks_text)) * kPackRows;   // row of the stream, or of the range
+    const int block = (int)blockIdx.x - (text ? 0 : blocks_text);
+    const int row0 = block * kPackRows;                          // row of the stream, or of the range
     // (a sequence's part of a stream is a whole number of 128-row tiles, so the block's rows belong to one sequence)
-    const SeqInfo sq = a.seqs[ranged ? a.r_seq : seq_of_row(a.seqs, a.num_seqs, row0, text)];
-    const int first = ranged ? row0 + (text ? a.r_text0 : a.r_summ0) : row0 - (text ? sq.text_off : sq.summ_off);
+    const SeqInfo sq = a.seqs[tails ? block / kTailBlocks : ranged ? a.r_seq : seq_of_row(a.seqs, a.num_seqs, row0, text)];
+    if (tails && (text ? sq.n_text : sq.n_summ) % kTileM == 0) return;
+    const int first = tails ? (text ? sq.n_text : sq.n_summ) / kTileM * kTileM + block % kTailBlocks * kPackRows
+                    : ranged ? row0 + (text ? a.r_text0 : a.r_summ0) : row0 - (text ? sq.text_off : sq.summ_off);
     const int end = ranged ? (text ? a.r_text0 + rows_text : a.r_summ0 + rows_summ) : (text ? sq.text_pad : sq.summ_pad);
     const int live = text ? sq.n_text : sq.n_summ;
     const int s = a.k + a.m, per = text ? a.k : a.m;             // rows of a chunk in this stream
@@ -76,7 +82,9 @@ cudaError_t launch_pack(const KernelArgs& a, cudaStream_t stream)
 {
     const int64_t text = a.r_seq >= 0 ? a.r_text1 - a.r_text0 : a.text_rows;
     const int64_t summ = a.m <= 0 ? 0 : a.r_seq >= 0 ? a.r_summ1 - a.r_summ0 : a.summ_rows;
-    const int64_t bt = (text + kPackRows - 1) / kPackRows, bs = (summ + kPackRows - 1) / kPackRows;
+    const bool tails = a.direct == kReadTails;
+    const int64_t bt = tails ? (int64_t)a.num_seqs * kTailBlocks : (text + kPackRows - 1) / kPackRows;
+    const int64_t bs = tails ? (a.m > 0 ? bt : 0) : (summ + kPackRows - 1) / kPackRows;
     if (bt + bs < 1) return cudaSuccess;
     ksa_pack_kernel<<<(unsigned)(bt + bs), 256, 0, stream>>>(a, (int)bt, (int)text, (int)summ);
     return cudaGetLastError();

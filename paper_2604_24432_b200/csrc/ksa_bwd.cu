@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(256) ksa_bwd_prep_kernel(BwdArgs a)
             for (int s = vecs >> 1; s > 0; s >>= 1) d[r] += __shfl_xor_sync(0xffffffffu, d[r], s);
         }
         if (!live) continue;
-        if (!a.direct) {
+        if (a.direct == kReadPacked || (a.direct == kReadTails && first >= sq.n_text / kTileM * kTileM)) {
 #pragma unroll
             for (int r = 0; r < kPrepRows; ++r) *reinterpret_cast<uint4*>(a.dot + (prow + r) * a.D + vec * 8) = gv[r];     // zeros on padding rows
         }

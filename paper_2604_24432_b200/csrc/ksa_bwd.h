@@ -27,7 +27,7 @@ struct BwdArgs {
     float* dkt; float* dvt;     // [Hkv][text_rows][D] fp32, elements as acc_at() places them
     float* dks; float* dvs;     // [Hkv][summ_rows][D] fp32, likewise
     int32_t* status;            // device status word of the context (bounded waits report here)
-    int32_t direct;             // tensor-core kernels read q, k, v, dout through chunked views: no packed copies
+    int32_t direct;             // ReadMode
 };
 
 // Place of element d of a row in the accumulators: 128-row tiles (the streams' parts are whole tiles), in a tile four
@@ -39,9 +39,9 @@ __host__ __device__ inline size_t acc_at(size_t row, int d, int D)
 }
 
 // Tensor maps for the tensor-core kernels (128-byte swizzle, boxes of 64 elements x 128 rows): Q and dO per query
-// head, K and V of the text and the summary rows per KV head -- of the packed streams, or (direct mode) chunked
-// 4-D views of the caller's interleaved tensors.
-struct BwdMaps { CUtensorMap qt, dot, kt, vt, ks, vs; };
+// head, K and V of the text and the summary rows per KV head -- of the packed streams, or (read in place) chunked
+// 4-D views of the caller's interleaved tensors; kReadTails: 5-D views, and the packed streams for the last tiles (TextMaps).
+struct BwdMaps { CUtensorMap qt, dot, kt, vt, ks, vs, qt_tail, dot_tail, kt_tail, vt_tail, ks_tail, vs_tail; };
 
 // Packs the text rows of dO, lse (in log2 units) and delta = <dO, O>.
 cudaError_t launch_bwd_prep(const BwdArgs& a, cudaStream_t stream);

@@ -238,25 +238,36 @@ __device__ __forceinline__ void bt_accumulate_half(uint32_t leader, uint32_t tme
 }
 
 // ---- producer helpers (one thread) ----------------------------------------------------------------
-// The two 64-column halves of a 128-row tile.  Packed streams: rows pos .. pos + 127 of a 3-D map.  Direct mode
-// (no packed copies: every sequence a whole number of chunks): chunks pos .. of a 4-D view [D, rows per chunk,
-// chunk, head] of the caller's interleaved tensor, whose box lands in shared memory as the same dense tile.
-template <int D>
-__device__ __forceinline__ void bt_issue_tile(uint32_t dst, uint32_t bar, const CUtensorMap* map, int pos, int head, bool direct)
+// Tile `tile` of a sequence's text (summary) rows, its two 64-column halves, as ReadMode says: rows of a 3-D map of a packed
+// stream, or chunks of a 4-D (5-D) view [D, rows per chunk, (start,) chunk, head] of the caller's interleaved tensor, whose box
+// lands in shared memory as the same dense tile.
+struct BtPlace {
+    int mode, per_text, per_summ;                                         // ReadMode, chunks of a text / a summary tile
+    int chunk0, start, text_off, summ_off, n_text, n_summ;                // of the sequence
+};
+__device__ __forceinline__ BtPlace bt_place(const BwdArgs& a, const SeqInfo& sq)
 {
-    if (direct) {
-        tma_load_4d(dst, map, bar, 0, 0, pos, head);
-        if (D == 128) tma_load_4d(dst + 16384, map, bar, 64, 0, pos, head);
-    } else {
-        tma_load_3d(dst, map, bar, 0, pos, head);
-        if (D == 128) tma_load_3d(dst + 16384, map, bar, 64, pos, head);
+    return BtPlace{a.direct, 128 / a.k, a.m > 0 ? 128 / a.m : 0, sq.chunk0, a.direct == kReadTails ? row_in_chunk(sq, a.k, a.m) : 0,
+                   sq.text_off, sq.summ_off, sq.n_text, sq.n_summ};
+}
+template <int D>
+__device__ __forceinline__ void bt_issue_tile(uint32_t dst, uint32_t bar, const CUtensorMap* map, const CUtensorMap* tail, const BtPlace& p, bool summ, int tile, int head)
+{
+    const int row = (summ ? p.summ_off : p.text_off) + tile * 128, chunk = p.chunk0 + tile * (summ ? p.per_summ : p.per_text);
+#pragma unroll
+    for (int h = 0; h < D / 64; ++h) {
+        const uint32_t to = dst + h * 16384;
+        if (p.mode == kReadInPlace) tma_load_4d(to, map, bar, h * 64, 0, chunk, head);
+        else if (p.mode == kReadPacked) tma_load_3d(to, map, bar, h * 64, row, head);
+        else if ((tile + 1) * 128 <= (summ ? p.n_summ : p.n_text)) tma_load_5d(to, map, bar, h * 64, 0, p.start, chunk, head);
+        else tma_load_3d(to, tail, bar, h * 64, row, head);
     }
 }
 template <int D>
-__device__ __forceinline__ void bt_load_tile(uint32_t dst, uint32_t bar, const CUtensorMap* map, int pos, int head, bool direct)
+__device__ __forceinline__ void bt_load_tile(uint32_t dst, uint32_t bar, const CUtensorMap* map, const CUtensorMap* tail, const BtPlace& p, bool summ, int tile, int head)
 {
     mbar_arrive_expect_tx(bar, (uint32_t)BtMap<D>::kTile);
-    bt_issue_tile<D>(dst, bar, map, pos, head, direct);
+    bt_issue_tile<D>(dst, bar, map, tail, p, summ, tile, head);
 }
 // After an abort: leave no copy in flight.  Bounded waits (the second flag is never set) for the last fill of
 // every stage; filled_a / filled1 / filled2 = A pairs / B1 / B2 tiles whose load was issued; asked = requests for a block that
@@ -336,7 +347,7 @@ __device__ __forceinline__ bool bt_unit_free(const BtSmem<D>& sm, int n, int32_t
 // x / segs of the packed stream (its rows are numbered over all sequences), KV head y.  (Segments first: the units in flight
 // then share their query tiles.  Tiles first, the launch over the summary keys at 32,768 tokens read them from memory again and
 // again and took 4,060 instead of 3,390 us.)
-struct BtDkvUnit { int J, kt, hk, seg0, n_keys, krow0, text_off, chunk0; };
+struct BtDkvUnit { int J, kt, hk, seg0, n_keys, krow0; BtPlace at; };
 __device__ __forceinline__ bool bt_dkv_unit(const BwdArgs& a, const BtBlock& blk, const int summ, const int seg_tiles, const int segs, BtDkvUnit& u)
 {
     const int tile = blk.x / segs;
@@ -345,7 +356,7 @@ __device__ __forceinline__ bool bt_dkv_unit(const BwdArgs& a, const BtBlock& blk
     u.kt = tile - (summ ? sq.summ_off : sq.text_off) / 128;
     u.hk = blk.y;
     u.n_keys = summ ? sq.n_summ : sq.n_text;
-    u.text_off = sq.text_off; u.chunk0 = sq.chunk0;
+    u.at = bt_place(a, sq);
     if (u.kt * 128 >= u.n_keys) return false;
     const int n_qt = (sq.n_text + 127) / 128;
     int qt_lo, qt_hi;                                                     // the query tiles that see the keys (Eq. 3)
@@ -376,11 +387,10 @@ __device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& ma
     if (!bt_layout(sm, bsm_raw, a.status)) return;
 
     // ---- the producer's thread: descriptor and loads of a unit ------------------------------------
-    const bool direct = a.direct != 0;
     BtDkvUnit u{};
     bool started = false;                                                 // unit 0: described, first tile on its way
     auto publish = [&](int n) {
-        bt_st_shared(sm.unit(n, U_TEXT_OFF), (uint32_t)u.text_off); bt_st_shared(sm.unit(n, U_TILE), (uint32_t)u.kt);
+        bt_st_shared(sm.unit(n, U_TEXT_OFF), (uint32_t)u.at.text_off); bt_st_shared(sm.unit(n, U_TILE), (uint32_t)u.kt);
         bt_st_shared(sm.unit(n, U_HEAD), (uint32_t)u.hk); bt_st_shared(sm.unit(n, U_A), (uint32_t)u.seg0);
         bt_st_shared(sm.unit(n, U_B), (uint32_t)u.n_keys); bt_st_shared(sm.unit(n, U_C), (uint32_t)u.krow0);
         bt_st_shared(sm.unit(n, U_J), (uint32_t)u.J);
@@ -388,21 +398,19 @@ __device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& ma
     };
     auto load_a = [&]() {                                                 // K and V tile
         mbar_arrive_expect_tx(sm.bar(BB_AFULL), 2u * BtMap<D>::kTile);
-        const int kpos = direct ? u.chunk0 + u.kt * (128 / (summ ? a.m : a.k)) : u.krow0;
-        bt_issue_tile<D>(sm.a1(), sm.bar(BB_AFULL), summ ? &maps.ks : &maps.kt, kpos, u.hk, direct);
-        bt_issue_tile<D>(sm.a2(), sm.bar(BB_AFULL), summ ? &maps.vs : &maps.vt, kpos, u.hk, direct);
+        bt_issue_tile<D>(sm.a1(), sm.bar(BB_AFULL), summ ? &maps.ks : &maps.kt, summ ? &maps.ks_tail : &maps.kt_tail, u.at, summ != 0, u.kt, u.hk);
+        bt_issue_tile<D>(sm.a2(), sm.bar(BB_AFULL), summ ? &maps.vs : &maps.vt, summ ? &maps.vs_tail : &maps.vt_tail, u.at, summ != 0, u.kt, u.hk);
     };
-    auto load_b = [&](int j, uint32_t dst, uint32_t bar, const CUtensorMap* map) {   // pair (query tile, head of the group) j
-        const int qt = u.seg0 + j / G;
-        bt_load_tile<D>(dst, bar, map, direct ? u.chunk0 + qt * (128 / a.k) : u.text_off + qt * 128, u.hk * G + j % G, direct);
+    auto load_b = [&](int j, uint32_t dst, uint32_t bar, const CUtensorMap* map, const CUtensorMap* tail) {   // pair (query tile, head of the group) j
+        bt_load_tile<D>(dst, bar, map, tail, u.at, false, u.seg0 + j / G, u.hk * G + j % G);
     };
     if (warp == 16 && lane == 0) {
         bt_init_barriers(sm);
         started = bt_dkv_unit(a, BtBlock{(int)blockIdx.x, (int)blockIdx.y, 0}, summ, seg_tiles, segs, u);
         if (started) {
-            load_b(0, sm.b1(0), sm.bar(BB_B1FULL), &maps.qt);
+            load_b(0, sm.b1(0), sm.bar(BB_B1FULL), &maps.qt, &maps.qt_tail);
             load_a();
-            load_b(0, sm.b2(0), sm.bar(BB_B2FULL), &maps.dot);
+            load_b(0, sm.b2(0), sm.bar(BB_B2FULL), &maps.dot, &maps.dot_tail);
             publish(0);
         }
     }
@@ -436,7 +444,7 @@ __device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& ma
                 for (int j = started ? 1 : 0; j < u.J; ++j) {
                     if (j + 1 == u.J) { bt_request_block(sm); pending = true; }          // comes while the stages are waited for
                     if (!bt_stage_free(sm, BB_B1EMPTY, kB1Stages, g1, a.status)) { alive = false; break; }
-                    load_b(j, sm.b1(g1 % kB1Stages), sm.bar(BB_B1FULL + g1 % kB1Stages), &maps.qt);
+                    load_b(j, sm.b1(g1 % kB1Stages), sm.bar(BB_B1FULL + g1 % kB1Stages), &maps.qt, &maps.qt_tail);
                     ++g1;
                     if (j == 0) {                                         // the unit before has formed its last products
                         if (na > 0 && !bt_wait(sm.bar(BB_AEMPTY), (uint32_t)((na - 1) & 1), sm.abort_addr(), a.status, kStatusWaitQEmpty)) { alive = false; break; }
@@ -444,7 +452,7 @@ __device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& ma
                         ++na;
                     }
                     if (!bt_stage_free(sm, BB_B2EMPTY, kB2Stages, g2, a.status)) { alive = false; break; }
-                    load_b(j, sm.b2(g2 & 1), sm.bar(BB_B2FULL + (g2 & 1)), &maps.dot);
+                    load_b(j, sm.b2(g2 & 1), sm.bar(BB_B2FULL + (g2 & 1)), &maps.dot, &maps.dot_tail);
                     ++g2;
                 }
                 started = false;
@@ -709,14 +717,14 @@ __device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& ma
 // =====================================================================================================
 // A unit: one query tile and one query head, over the visible summary tiles, then the visible text tiles (Eq. 3).  Block
 // (x, y): x-th query tile of the packed stream from its end (a sequence's long rows first), head y.
-struct BtDqUnit { int J, n_s, t_lo, qt, h, n_text, text_off, summ_off, chunk0; long long aug_off; };
+struct BtDqUnit { int J, n_s, t_lo, qt, h; BtPlace at; long long aug_off; };
 __device__ __forceinline__ void bt_dq_unit(const BwdArgs& a, const BtBlock& blk, BtDqUnit& u)
 {
     const int row0 = (int)a.text_rows - 128 - blk.x * 128;
     const SeqInfo sq = a.seqs[seq_of_row(a.seqs, a.num_seqs, row0, true)];
     u.qt = (row0 - sq.text_off) / 128;
     u.h = blk.y;
-    u.n_text = sq.n_text; u.text_off = sq.text_off; u.summ_off = sq.summ_off; u.chunk0 = sq.chunk0; u.aug_off = sq.aug_off;
+    u.at = bt_place(a, sq); u.aug_off = sq.aug_off;
     const int i_first = u.qt * 128, i_last = min(sq.n_text, i_first + 128) - 1;
     const int far_first = max(0, i_first / a.k - a.C), far_last = max(0, i_last / a.k - a.C);
     u.n_s = a.m > 0 ? (min(sq.n_summ, far_last * a.m) + 127) / 128 : 0;               // summary tiles seen by the last row
@@ -734,34 +742,30 @@ __device__ __forceinline__ void bt_dq_block(const BwdArgs& a, const BwdMaps& map
     if (!bt_layout(sm, bsm_raw, a.status)) return;
 
     // ---- the producer's thread: descriptor and loads of a unit ------------------------------------
-    const bool direct = a.direct != 0;
     BtDqUnit u{};
     auto publish = [&](int n) {
-        bt_st_shared(sm.unit(n, U_TEXT_OFF), (uint32_t)u.text_off); bt_st_shared(sm.unit(n, U_TILE), (uint32_t)u.qt);
+        bt_st_shared(sm.unit(n, U_TEXT_OFF), (uint32_t)u.at.text_off); bt_st_shared(sm.unit(n, U_TILE), (uint32_t)u.qt);
         bt_st_shared(sm.unit(n, U_HEAD), (uint32_t)u.h); bt_st_shared(sm.unit(n, U_A), (uint32_t)u.n_s);
-        bt_st_shared(sm.unit(n, U_B), (uint32_t)u.t_lo); bt_st_shared(sm.unit(n, U_C), (uint32_t)u.n_text);
+        bt_st_shared(sm.unit(n, U_B), (uint32_t)u.t_lo); bt_st_shared(sm.unit(n, U_C), (uint32_t)u.at.n_text);
         bt_st_shared(sm.unit(n, U_AUG), (uint32_t)u.aug_off); bt_st_shared(sm.unit(n, U_AUG + 1), (uint32_t)(u.aug_off >> 32));
         bt_st_shared(sm.unit(n, U_J), (uint32_t)u.J);
         mbar_arrive(sm.bar(BB_UFULL + (n & 1)));
     };
     auto load_a = [&]() {                                                 // Q and dO tile
         mbar_arrive_expect_tx(sm.bar(BB_AFULL), 2u * BtMap<D>::kTile);
-        const int qpos = direct ? u.chunk0 + u.qt * (128 / a.k) : u.text_off + u.qt * 128;
-        bt_issue_tile<D>(sm.a1(), sm.bar(BB_AFULL), &maps.qt, qpos, u.h, direct);
-        bt_issue_tile<D>(sm.a2(), sm.bar(BB_AFULL), &maps.dot, qpos, u.h, direct);
+        bt_issue_tile<D>(sm.a1(), sm.bar(BB_AFULL), &maps.qt, &maps.qt_tail, u.at, false, u.qt, u.h);
+        bt_issue_tile<D>(sm.a2(), sm.bar(BB_AFULL), &maps.dot, &maps.dot_tail, u.at, false, u.qt, u.h);
     };
-    auto load_b = [&](int j, uint32_t dst, uint32_t bar, const CUtensorMap* map_s, const CUtensorMap* map_t) {
+    auto load_b = [&](int j, uint32_t dst, uint32_t bar, const CUtensorMap* map_s, const CUtensorMap* map_t, const CUtensorMap* tail_s, const CUtensorMap* tail_t) {
         const bool is_summ = j < u.n_s;
-        const int tile = is_summ ? j : u.t_lo + j - u.n_s;
-        bt_load_tile<D>(dst, bar, is_summ ? map_s : map_t,
-                        direct ? u.chunk0 + tile * (128 / (is_summ ? a.m : a.k)) : (is_summ ? u.summ_off : u.text_off) + tile * 128, u.h / G, direct);
+        bt_load_tile<D>(dst, bar, is_summ ? map_s : map_t, is_summ ? tail_s : tail_t, u.at, is_summ, is_summ ? j : u.t_lo + j - u.n_s, u.h / G);
     };
     if (warp == 16 && lane == 0) {
         bt_init_barriers(sm);
         bt_dq_unit(a, BtBlock{(int)blockIdx.x, (int)blockIdx.y, 0}, u);
-        load_b(0, sm.b1(0), sm.bar(BB_B1FULL), &maps.ks, &maps.kt);
+        load_b(0, sm.b1(0), sm.bar(BB_B1FULL), &maps.ks, &maps.kt, &maps.ks_tail, &maps.kt_tail);
         load_a();
-        load_b(0, sm.b2(0), sm.bar(BB_B2FULL), &maps.vs, &maps.vt);
+        load_b(0, sm.b2(0), sm.bar(BB_B2FULL), &maps.vs, &maps.vt, &maps.vs_tail, &maps.vt_tail);
         publish(0);
     }
     bt_ready(sm, warp);
@@ -796,7 +800,7 @@ __device__ __forceinline__ void bt_dq_block(const BwdArgs& a, const BwdMaps& map
                 for (int j = n > 0 ? 0 : 1; j < u.J; ++j) {
                     if (j + 1 == u.J) { bt_request_block(sm); pending = true; }          // comes while the stages are waited for
                     if (!bt_stage_free(sm, BB_B1EMPTY, kB1Stages, g1, a.status)) { alive = false; break; }
-                    load_b(j, sm.b1(g1 % kB1Stages), sm.bar(BB_B1FULL + g1 % kB1Stages), &maps.ks, &maps.kt);
+                    load_b(j, sm.b1(g1 % kB1Stages), sm.bar(BB_B1FULL + g1 % kB1Stages), &maps.ks, &maps.kt, &maps.ks_tail, &maps.kt_tail);
                     ++g1;
                     if (j == 0) {                                         // the unit before has formed its last products
                         if (!bt_wait(sm.bar(BB_AEMPTY), (uint32_t)((na - 1) & 1), sm.abort_addr(), a.status, kStatusWaitQEmpty)) { alive = false; break; }
@@ -804,7 +808,7 @@ __device__ __forceinline__ void bt_dq_block(const BwdArgs& a, const BwdMaps& map
                         ++na;
                     }
                     if (!bt_stage_free(sm, BB_B2EMPTY, kB2Stages, g2, a.status)) { alive = false; break; }
-                    load_b(j, sm.b2(g2 & 1), sm.bar(BB_B2FULL + (g2 & 1)), &maps.vs, &maps.vt);
+                    load_b(j, sm.b2(g2 & 1), sm.bar(BB_B2FULL + (g2 & 1)), &maps.vs, &maps.vt, &maps.vs_tail, &maps.vt_tail);
                     ++g2;
                 }
             }

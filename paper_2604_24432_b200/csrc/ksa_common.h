@@ -38,6 +38,14 @@ struct WorkItem {
 };
 static_assert(sizeof(WorkItem) == 48, "WorkItem layout");
 
+// Where the tensor-core kernels find the 128-row tiles of q, k, v (and dout).
+enum ReadMode : int32_t {
+    kReadPacked = 0,        // in the packed streams
+    kReadInPlace = 1,       // in the caller's tensors: every sequence is a whole number of chunks
+    kReadTails = 2,         // in the caller's tensors, but for a sequence's last text (summary) tile that is not full: that one in
+                            // the packed streams, zero-padded there; the rest of the streams is not written
+};
+
 // Arguments common to the kernels.
 struct KernelArgs {
     const SeqInfo* seqs;
@@ -57,7 +65,7 @@ struct KernelArgs {
     // Row range (pack and summary kernels): r_seq < 0 means every sequence in full; otherwise only
     // sequence r_seq, packed text rows [r_text0, r_text1), summary-stream rows [r_summ0, r_summ1)
     // (pack) and summary query rows [r_summ0, r_summq1) (summary-row kernel).
-    int32_t direct;         // text kernel reads Q/K/V tiles straight from the caller's tensors (no packed streams)
+    int32_t direct;         // ReadMode: where the tensor-core kernels find their tiles
     int32_t r_seq;
     int32_t r_text0, r_text1, r_summ0, r_summ1, r_summq1;
     // user tensors (bf16 as uint16)
@@ -95,6 +103,9 @@ __device__ __forceinline__ bool ksa_in_bounds(bool ok, int32_t* status)
 #else
 __device__ __forceinline__ bool ksa_in_bounds(bool, int32_t*) { return true; }
 #endif
+// Where a tile of the text (summary) stream stands under kReadTails: chunk and row of the sequence's start in the [chunk, k + m]
+// grid of the caller's rows.
+__device__ __forceinline__ int row_in_chunk(const SeqInfo& sq, int k, int m) { return (int)(sq.aug_off - (int64_t)sq.chunk0 * (k + m)); }
 // The sequence that holds row `row` of the packed text (summary) stream: the last one that starts at or before it.
 __device__ __forceinline__ int seq_of_row(const SeqInfo* seqs, int n, int row, bool text)
 {

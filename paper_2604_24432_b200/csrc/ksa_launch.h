@@ -45,7 +45,9 @@ cudaError_t launch_text_ref(const KernelArgs& a, cudaStream_t stream);
 // caller's interleaved tensors as [D, k, chunks, H] (text rows; box {64, k, 128/k, 1}) and
 // [D, m, chunks, H] starting k rows in (summary rows; box {64, m, 128/m, 1}): the box lands in
 // shared memory as the same dense 128-row tile either way.
-struct TextMaps { CUtensorMap qt, kt, vt, ks, vs; };
+// kReadTails: maps of both kinds, those of the caller's tensors as [D, k, start, chunks, H] (box {64, k, 1, 128/k, 1}; `start`
+// picks the row of the [chunk, k + m] grid at which the sequence's chunks start), and those of the packed streams as *_tail.
+struct TextMaps { CUtensorMap qt, kt, vt, ks, vs, qt_tail, kt_tail, vt_tail, ks_tail, vs_tail; };
 cudaError_t launch_text_tc(const KernelArgs& a, const TextMaps& maps, int num_sms, cudaStream_t stream);
 // One-time per-device setup (dynamic shared memory opt-in).
 cudaError_t setup_text_tc();

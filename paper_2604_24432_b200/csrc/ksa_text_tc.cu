@@ -161,6 +161,9 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
                 const bool is_v = warp == kLoadVWarp;
                 const CUtensorMap* map_t = is_v ? &maps.vt : &maps.kt;
                 const CUtensorMap* map_s = is_v ? &maps.vs : &maps.ks;
+                const CUtensorMap* tail_t = is_v ? &maps.vt_tail : &maps.kt_tail;
+                const CUtensorMap* tail_s = is_v ? &maps.vs_tail : &maps.ks_tail;
+                const bool tails = a.direct == kReadTails;
                 prefetch_tensormap(map_t); prefetch_tensormap(map_s);
                 if (!is_v) prefetch_tensormap(&maps.qt);
                 const int stages = is_v ? Cfg::kStagesV : Cfg::kStagesK;
@@ -177,36 +180,35 @@ ksa_text_tc_kernel(const __grid_constant__ KernelArgs a, const __grid_constant__
                     const SeqInfo sq = a.seqs[w.seq];
                     const int hk = w.kv_head, nsplit = w.kv_per_tile;
                     const int T = w.ns_tiles + (w.band_hi - w.band_lo + 1);
+                    const int start = tails ? row_in_chunk(sq, a.k, a.m) : 0;
+                    // Half h of a tile: `tile` of the text (summary) rows of this sequence
+                    auto load = [&](uint32_t dst, const CUtensorMap* map, const CUtensorMap* tail, uint32_t full, int h, bool summ, int tile, int head) {
+                        const int per = kTileN / (summ ? max(a.m, 1) : a.k);                     // chunks of a tile
+                        const int row = (summ ? sq.summ_off : sq.text_off) + tile * kTileN;
+                        if (a.direct == kReadInPlace) tma_load_4d(dst, map, full, h * 64, 0, sq.chunk0 + tile * per, head);
+                        else if (!tails) tma_load_3d(dst, map, full, h * 64, row, head);
+                        else if ((tile + 1) * kTileN <= (summ ? sq.n_summ : sq.n_text)) tma_load_5d(dst, map, full, h * 64, 0, start, sq.chunk0 + tile * per, head);
+                        else tma_load_3d(dst, tail, full, h * 64, row, head);
+                    };
                     auto load_q = [&](int t) {
                         if (!bounded_wait(bar(BAR_QEMPTY + t), ((q_phase >> t) & 1u) ^ 1u, abort_addr, a.status, kStatusWaitQEmpty)) { alive = false; return; }
                         q_phase ^= 1u << t;
                         mbar_arrive_expect_tx(bar(BAR_QFULL + t), (uint32_t)Cfg::kTileBytes);
                         q_armed |= 1u << t;
                         for (int h = 0; h < Cfg::kHalves; ++h)
-                            if (a.direct)
-                                tma_load_4d(sQ + t * Cfg::kTileBytes + h * 16384, &maps.qt, bar(BAR_QFULL + t),
-                                            h * 64, 0, sq.chunk0 + w.q_tile * (kTileM / a.k), w.head0 + t);
-                            else
-                                tma_load_3d(sQ + t * Cfg::kTileBytes + h * 16384, &maps.qt, bar(BAR_QFULL + t),
-                                            h * 64, sq.text_off + w.q_tile * kTileM, w.head0 + t);
+                            load(sQ + t * Cfg::kTileBytes + h * 16384, &maps.qt, &maps.qt_tail, bar(BAR_QFULL + t), h, false, w.q_tile, w.head0 + t);
                     };
                     if (!is_v) load_q(0);
                     for (int j = 0; j < T && alive; ++j) {
                         const bool summ = j < w.ns_tiles;
-                        const CUtensorMap* map = summ ? map_s : map_t;
-                        // direct views: a tile is 128/m chunks of the summary view or 128/k chunks of the text view
-                        const int pos = a.direct ? sq.chunk0 + (summ ? j * (kTileN / max(a.m, 1)) : (w.band_lo + j - w.ns_tiles) * (kTileN / a.k))
-                                                 : (summ ? sq.summ_off + j * kTileN : sq.text_off + (w.band_lo + j - w.ns_tiles) * kTileN);
+                        const int tile = summ ? j : w.band_lo + j - w.ns_tiles;
                         for (int u = 0; u < nsplit; ++u) {
                             if (!bounded_wait(empty0 + 8u * stage, ring_phase ^ 1u, abort_addr, a.status, kStatusWaitKvEmpty)) { alive = false; break; }
                             mbar_arrive_expect_tx(full0 + 8u * stage, (uint32_t)Cfg::kTileBytes);
                             armed_mask |= 1u << stage;
                             armed_parity = (armed_parity & ~(1u << stage)) | (ring_phase << stage);
                             for (int h = 0; h < Cfg::kHalves; ++h)
-                                if (a.direct)
-                                    tma_load_4d(ring + stage * Cfg::kTileBytes + h * 16384, map, full0 + 8u * stage, h * 64, 0, pos, hk + u);
-                                else
-                                    tma_load_3d(ring + stage * Cfg::kTileBytes + h * 16384, map, full0 + 8u * stage, h * 64, pos, hk + u);
+                                load(ring + stage * Cfg::kTileBytes + h * 16384, summ ? map_s : map_t, summ ? tail_s : tail_t, full0 + 8u * stage, h, summ, tile, hk + u);
                             if (++stage == stages) { stage = 0; ring_phase ^= 1u; }
                             if (j == 0 && u == 0 && !is_v && w.n_heads == 2) { load_q(1); if (!alive) break; }
                         }

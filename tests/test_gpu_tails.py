@@ -1,0 +1,78 @@
+"""Ragged batches read in place: full tiles straight from the caller's tensors, each sequence's last tile from the packed
+streams.  Against the packed path (every tile from the streams), bit for bit: the same tiles reach the same kernels."""
+import pytest
+import torch
+
+from paper_2604_24432_b200 import binding as ksa
+from paper_2604_24432_b200 import build as ksa_build
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    ksa_build.build()
+    c = ksa.Context(0)
+    yield c
+    c.close()
+
+
+def _rows(total, H, D, gen, strided):
+    """bf16 rows [total, H, D]; strided: heads with a gap between them, rows with a longer one."""
+    full = torch.randn((total, H + 1, D + 8) if strided else (total, H, D), generator=gen, device="cuda").bfloat16()
+    return full[:, 1:, :D] if strided else full
+
+
+@pytest.mark.parametrize("lens,k,m,C,Hq,Hkv,D", [
+    ([129, 127, 1, 257], 8, 1, 4, 4, 2, 128),            # a last tile of one row, of 127, no full tile
+    ([1027, 5, 130, 643], 8, 1, 16, 8, 2, 64),           # sequences that start at every row of a chunk
+    ([1153, 2175], 8, 1, 16, 4, 4, 128),                 # 144 and 271 summary rows: full tiles and last ones
+    ([4097, 70], 64, 8, 4, 8, 2, 128),                   # 64 chunks of eight summaries: four full tiles, none left over
+    ([300, 1011], 8, 0, 1 << 20, 4, 2, 128),             # no summaries
+    ([513, 255, 771], 1, 1, 100, 4, 2, 64),              # chunks of one token: no length is ragged but for the tile
+    ([400, 999], 128, 2, 1, 6, 2, 128),                  # a chunk fills a tile; head pairs across KV heads
+])
+@pytest.mark.parametrize("strided", [False, True])
+def test_tails_equal_the_packed_path(ctx, lens, k, m, C, Hq, Hkv, D, strided):
+    gen = torch.Generator("cuda").manual_seed(11)
+    packed = ksa.Problem(lens, k, m, C, Hq, Hkv, D, D ** -0.5, ksa.KSA_FLAG_BWD_MMA_SYNC_KERNELS)     # these read the streams only
+    prob = ksa.Problem(lens, k, m, C, Hq, Hkv, D, D ** -0.5)
+    total = ksa.total_aug_len(prob)
+    q, kk, v = (_rows(total, H, D, gen, strided) for H in (Hq, Hkv, Hkv))
+    got = []
+    for p in (packed, prob):
+        out = torch.empty((total, Hq, D), dtype=torch.bfloat16, device="cuda")
+        lse = torch.empty((Hq, total), dtype=torch.float32, device="cuda")
+        ws = torch.full((max(256, ksa.workspace_bytes(p)),), 0xFF, dtype=torch.uint8, device="cuda")   # NaN patterns
+        ctx.clear_device_status()
+        ctx.attn_fwd(p, q, kk, v, out, lse, ws)
+        torch.cuda.synchronize()
+        assert ctx.device_status() == 0
+        got.append((out, lse))
+    assert torch.equal(got[0][0].view(torch.int16), got[1][0].view(torch.int16))
+    assert torch.equal(got[0][1].view(torch.int32), got[1][1].view(torch.int32))
+
+
+def test_a_sequence_does_not_see_its_neighbour(ctx):
+    """NaN and infinities in one sequence of a ragged batch leave the others' outputs and gradients finite."""
+    lens, k, m, C, Hq, Hkv, D = [333, 258, 131], 8, 1, 4, 4, 2, 128
+    gen = torch.Generator("cuda").manual_seed(12)
+    prob = ksa.Problem(lens, k, m, C, Hq, Hkv, D, D ** -0.5)
+    total = ksa.total_aug_len(prob)
+    q, kk, v, dout = (_rows(total, H, D, gen, False) for H in (Hq, Hkv, Hkv, Hq))
+    lo, hi = ksa.aug_len(333, k, m), ksa.aug_len(333, k, m) + ksa.aug_len(258, k, m)
+    for t in (kk, v, dout):
+        t[lo:hi] = float("nan")
+        t[lo:lo + 3] = float("inf")
+    out, dq = torch.empty_like(q), torch.empty_like(q)
+    dk, dv = torch.empty_like(kk), torch.empty_like(v)
+    lse = torch.empty((Hq, total), dtype=torch.float32, device="cuda")
+    ws = torch.full((ksa.workspace_bytes(prob),), 0xFF, dtype=torch.uint8, device="cuda")
+    wsb = torch.full((ksa.bwd_workspace_bytes(prob),), 0xFF, dtype=torch.uint8, device="cuda")
+    ctx.clear_device_status()
+    ctx.attn_fwd(prob, q, kk, v, out, lse, ws)
+    ctx.attn_bwd(prob, q, kk, v, out, lse, dout, dq, dk, dv, wsb)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    for t in (out, dq, dk, dv):
+        assert torch.isfinite(t[:lo].float()).all() and torch.isfinite(t[hi:].float()).all()
