@@ -154,8 +154,9 @@ int ksa_visible_pairs(const ksa_params* p, int64_t* pairs);
  *             4-D tensor maps and nothing is packed
  *   cuda_stream  a cudaStream_t (NULL = legacy default stream)
  * Steps enqueued: pack (de-interleave text Q/K/V and summary K/V into dense streams;
- * skipped in the case above), summary-row attention, text-row attention over the
- * scheduled tiles.  In the no-pack case the padding rows of a partial tile hold rows
+ * skipped in the case above, and reduced to each sequence's last, partial text and summary
+ * tile where only the sequence lengths stand in its way: full tiles are then read in place),
+ * summary-row attention, text-row attention over the scheduled tiles.  In the no-pack case the padding rows of a partial tile hold rows
  * of the following sequence; they are masked, but like any masked row their V values
  * must be finite (a NaN or Inf there would reach the accumulators as 0 * NaN).
  * Errors: KSA_ERR_INVALID_ARG / UNSUPPORTED / WORKSPACE before anything is launched;
