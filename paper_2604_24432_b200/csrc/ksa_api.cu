@@ -161,12 +161,18 @@ bool direct_ok(const ksa_params* p)
 // both views, the kernels read full tiles in place and only each sequence's last text and summary tile is packed, so that no
 // sequence sees rows of its neighbour.  Packing all rows took 478 us of 7.0 ms for 127,475 tokens of 32/8 heads, 12 - 25 % of a
 // prompt of a few thousand tokens and, of a ragged training layer of 7,942 tokens with 16/16 heads, 64 of 550 us.
-static int read_mode(const ksa_params* p)
+static int read_mode(const ksa_params* p, bool backward)
 {
     if (direct_ok(p)) return kReadInPlace;
     const int k = p->chunk_len, m = p->summaries_per_chunk;
     if (p->flags & (KSA_FLAG_REFERENCE_KERNEL | KSA_FLAG_CTA_PAIR_KERNEL | KSA_FLAG_BWD_MMA_SYNC_KERNELS)) return kReadPacked;      // those kernels know the streams only
-    return kTileM % k == 0 && (m == 0 || kTileN % m == 0) ? kReadTails : kReadPacked;
+    if (kTileM % k != 0 || (m > 0 && kTileN % m != 0)) return kReadPacked;
+    // A tensor map's strides are less than 2^40 bytes.  (A head stride may be any number where there is one head.)
+    const int64_t st[8] = {p->q_stride_tok, p->q_stride_head, p->k_stride_tok, p->k_stride_head,
+                           p->v_stride_tok, p->v_stride_head, p->o_stride_tok, p->o_stride_head};      // the last two: dout
+    for (int i = 0; i < (backward ? 8 : 6); ++i)
+        if (st[i] >= (1ll << 39) / (i & 1 ? 1 : k + m)) return kReadPacked;
+    return kReadTails;
 }
 
 void build_layout(const ksa_params* p, HostSchedule& hs)
@@ -896,7 +902,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_fwd(ksa_ctx* ctx,
     for (int i = 0; i < 5; ++i) if (ptrs[i] & 15) return KSA_ERR_INVALID_ARG;
     if ((rc = ensure_schedule(ctx, p, true, 0, (cudaStream_t)cuda_stream)) != KSA_OK) return rc;
     const HostSchedule& hs = ctx->sched;
-    const int mode = read_mode(p);
+    const int mode = read_mode(p, false);
     const WorkspaceLayout wl = workspace_layout(p, hs);
     if (mode != kReadInPlace && (!workspace || workspace_bytes < wl.total || ((uintptr_t)workspace & 255))) return KSA_ERR_WORKSPACE;
 
@@ -1080,7 +1086,7 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_bwd(ksa_ctx* ctx,
     // packed streams of the forward pass (text Q, K, V and summary K, V) -- not needed when the tensor-core kernels
     // can read whole tiles straight from the caller's tensors (the no-pack case of the forward pass)
     const bool direct = direct_ok(p) && !(p->flags & KSA_FLAG_BWD_MMA_SYNC_KERNELS);
-    const int mode = direct ? kReadInPlace : read_mode(p) == kReadTails ? kReadTails : kReadPacked;
+    const int mode = direct ? kReadInPlace : read_mode(p, true) == kReadTails ? kReadTails : kReadPacked;
     KernelArgs fa = make_args(ctx, p, q, k, v, dq /* unused */, const_cast<float*>(lse), workspace, bl.fwd, mode);
     if (!direct && (e = launch_pack(fa, stream)) != cudaSuccess) return cuda_fail(ctx, e);
     BwdArgs a{};

@@ -76,3 +76,37 @@ def test_a_sequence_does_not_see_its_neighbour(ctx):
     assert ctx.device_status() == 0
     for t in (out, dq, dk, dv):
         assert torch.isfinite(t[:lo].float()).all() and torch.isfinite(t[hi:].float()).all()
+
+
+@pytest.mark.parametrize("wide", ["q", "k", "v", "o"])
+def test_a_head_stride_that_no_tensor_map_holds(ctx, wide):
+    """The head stride of a tensor with one head is never used, and may be any number: a ragged batch gives the same with 2^40
+    bytes, more than a tensor map's stride may be."""
+    lens, k, m, C, D = [333, 130, 8], 8, 1, 4, 128
+    Hq = 1 if wide in "qo" else 4
+    total = sum(ksa.aug_len(n, k, m) for n in lens)
+    prob = ksa.Problem(lens, k, m, C, Hq, 1, D, D ** -0.5)
+    gen = torch.Generator("cuda").manual_seed(13)
+    q, kk, v, dout = (_rows(total, H, D, gen, False) for H in (Hq, 1, 1, Hq))
+
+    def view(t, name):
+        return t.as_strided(t.shape, (t.stride(0), 1 << 39, 1)) if name == wide else t
+
+    got = []
+    for shape in (lambda t, name: t, view):
+        out, dq, dk, dv = (shape(torch.full_like(t, 7.0), n) for t, n in ((q, "o"), (q, "q"), (kk, "k"), (v, "v")))
+        lse = torch.empty((Hq, total), dtype=torch.float32, device="cuda")
+        ws = torch.full((ksa.workspace_bytes(prob),), 0xFF, dtype=torch.uint8, device="cuda")
+        wsb = torch.full((ksa.bwd_workspace_bytes(prob),), 0xFF, dtype=torch.uint8, device="cuda")
+        args = shape(q, "q"), shape(kk, "k"), shape(v, "v"), out, lse
+        ctx.clear_device_status()
+        ctx.attn_fwd(prob, *args, ws)
+        ctx.attn_bwd(prob, *args, shape(dout, "o"), dq, dk, dv, wsb)
+        torch.cuda.synchronize()
+        assert ctx.device_status() == 0
+        got.append((out, lse, dq, dk, dv))
+    for a, b in zip(got[0][:3], got[1][:3]):
+        assert torch.equal(a, b)
+    for a, b in zip(got[0][3:], got[1][3:]):                  # fp32 atomics in either order, then bf16: one rounding apart
+        a, b = a.float(), b.float()
+        assert ((a - b).abs() <= 2 ** -7 * b.abs() + 1e-6 * b.abs().max()).all()
