@@ -163,9 +163,11 @@ bool direct_ok(const ksa_params* p)
 // prompt of a few thousand tokens and, of a ragged training layer of 7,942 tokens with 16/16 heads, 64 of 550 us.
 static int read_mode(const ksa_params* p, bool backward)
 {
+    // the mma.sync kernels know the streams only, the cross-check and the CTA-pair kernel no tails
+    if (backward && (p->flags & KSA_FLAG_BWD_MMA_SYNC_KERNELS)) return kReadPacked;
     if (direct_ok(p)) return kReadInPlace;
+    if (p->flags & (KSA_FLAG_REFERENCE_KERNEL | KSA_FLAG_CTA_PAIR_KERNEL)) return kReadPacked;
     const int k = p->chunk_len, m = p->summaries_per_chunk;
-    if (p->flags & (KSA_FLAG_REFERENCE_KERNEL | KSA_FLAG_CTA_PAIR_KERNEL | KSA_FLAG_BWD_MMA_SYNC_KERNELS)) return kReadPacked;      // those kernels know the streams only
     if (kTileM % k != 0 || (m > 0 && kTileN % m != 0)) return kReadPacked;
     // A tensor map's strides are less than 2^40 bytes.  (A head stride may be any number where there is one head.)
     const int64_t st[8] = {p->q_stride_tok, p->q_stride_head, p->k_stride_tok, p->k_stride_head,
@@ -799,7 +801,7 @@ static constexpr bool kPairKernelByDefault = false;
 static bool pair_ok(const KernelArgs& a, uint32_t flags)
 {
     if (flags & (KSA_FLAG_REFERENCE_KERNEL | KSA_FLAG_SINGLE_CTA_KERNEL)) return false;
-    if (a.D != 128 || ((a.Hq / a.Hkv) & 1)) return false;
+    if (a.D != 128 || ((a.Hq / a.Hkv) & 1) || a.direct == kReadTails) return false;
     if (a.direct && (64 % a.k != 0 || (a.m > 0 && 64 % a.m != 0))) return false;
     return kPairKernelByDefault || (flags & KSA_FLAG_CTA_PAIR_KERNEL);
 }
@@ -1033,7 +1035,7 @@ static BwdLayout bwd_layout(const ksa_params* p, const HostSchedule& hs)
 {
     BwdLayout b{};
     // no packed streams and no packed dO where the tensor-core kernels read the caller's tensors in place
-    const bool direct = direct_ok(p) && !(p->flags & KSA_FLAG_BWD_MMA_SYNC_KERNELS);
+    const bool direct = read_mode(p, true) == kReadInPlace;
     if (!direct) b.fwd = workspace_layout(p, hs);
     size_t off = b.fwd.total;
     auto take = [&](size_t bytes) { size_t o = off; off = (size_t)round_up((int64_t)(off + bytes), 1024); return o; };
@@ -1085,8 +1087,8 @@ extern "C" __attribute__((visibility("default"))) int ksa_attn_bwd(ksa_ctx* ctx,
     }
     // packed streams of the forward pass (text Q, K, V and summary K, V) -- not needed when the tensor-core kernels
     // can read whole tiles straight from the caller's tensors (the no-pack case of the forward pass)
-    const bool direct = direct_ok(p) && !(p->flags & KSA_FLAG_BWD_MMA_SYNC_KERNELS);
-    const int mode = direct ? kReadInPlace : read_mode(p, true) == kReadTails ? kReadTails : kReadPacked;
+    const int mode = read_mode(p, true);
+    const bool direct = mode == kReadInPlace;
     KernelArgs fa = make_args(ctx, p, q, k, v, dq /* unused */, const_cast<float*>(lse), workspace, bl.fwd, mode);
     if (!direct && (e = launch_pack(fa, stream)) != cudaSuccess) return cuda_fail(ctx, e);
     BwdArgs a{};

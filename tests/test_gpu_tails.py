@@ -8,6 +8,9 @@ from paper_2604_24432_b200 import build as ksa_build
 
 pytestmark = pytest.mark.gpu
 
+# every tile from the streams, as the CTA-pair kernel wants them, in the same kernels as without flags
+PACKED = ksa.KSA_FLAG_CTA_PAIR_KERNEL | ksa.KSA_FLAG_SINGLE_CTA_KERNEL
+
 
 @pytest.fixture(scope="module")
 def ctx():
@@ -35,7 +38,7 @@ def _rows(total, H, D, gen, strided):
 @pytest.mark.parametrize("strided", [False, True])
 def test_tails_equal_the_packed_path(ctx, lens, k, m, C, Hq, Hkv, D, strided):
     gen = torch.Generator("cuda").manual_seed(11)
-    packed = ksa.Problem(lens, k, m, C, Hq, Hkv, D, D ** -0.5, ksa.KSA_FLAG_BWD_MMA_SYNC_KERNELS)     # these read the streams only
+    packed = ksa.Problem(lens, k, m, C, Hq, Hkv, D, D ** -0.5, PACKED)
     prob = ksa.Problem(lens, k, m, C, Hq, Hkv, D, D ** -0.5)
     total = ksa.total_aug_len(prob)
     q, kk, v = (_rows(total, H, D, gen, strided) for H in (Hq, Hkv, Hkv))
@@ -51,6 +54,21 @@ def test_tails_equal_the_packed_path(ctx, lens, k, m, C, Hq, Hkv, D, strided):
         got.append((out, lse))
     assert torch.equal(got[0][0].view(torch.int16), got[1][0].view(torch.int16))
     assert torch.equal(got[0][1].view(torch.int32), got[1][1].view(torch.int32))
+
+
+def test_the_forward_pass_ignores_the_backward_flag(ctx):
+    """What stands in the workspace behind a ragged call: with full tiles read in place the streams' last tiles, whether the
+    backward pass is to run on mma.sync kernels, which want whole streams, or not."""
+    left = []
+    for flags in (0, ksa.KSA_FLAG_BWD_MMA_SYNC_KERNELS, PACKED):
+        prob = ksa.Problem([1027, 333], 8, 1, 4, 4, 2, 128, 128 ** -0.5, flags)
+        total = ksa.total_aug_len(prob)
+        gen = torch.Generator("cuda").manual_seed(14)
+        q, kk, v = (_rows(total, H, 128, gen, False) for H in (4, 2, 2))
+        lse = torch.empty((4, total), dtype=torch.float32, device="cuda")
+        left.append(torch.full((ksa.workspace_bytes(prob),), 0xFF, dtype=torch.uint8, device="cuda"))
+        ctx.attn_fwd(prob, q, kk, v, torch.empty_like(q), lse, left[-1])
+    assert torch.equal(left[0], left[1]) and not torch.equal(left[0], left[2])
 
 
 def test_a_sequence_does_not_see_its_neighbour(ctx):
