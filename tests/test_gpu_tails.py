@@ -1,5 +1,7 @@
 """Ragged batches read in place: full tiles straight from the caller's tensors, each sequence's last tile from the packed
 streams.  Against the packed path (every tile from the streams), bit for bit: the same tiles reach the same kernels."""
+import random
+
 import pytest
 import torch
 
@@ -128,3 +130,40 @@ def test_a_head_stride_that_no_tensor_map_holds(ctx, wide):
     for a, b in zip(got[0][3:], got[1][3:]):                  # fp32 atomics in either order, then bf16: one rounding apart
         a, b = a.float(), b.float()
         assert ((a - b).abs() <= 2 ** -7 * b.abs() + 1e-6 * b.abs().max()).all()
+
+
+@pytest.mark.parametrize("k,m", [(8, 1), (24, 8)])
+def test_schedules_that_share_memory(ctx, k, m):
+    """One context, another split of the same rows into sequences in every call: the schedules' memory goes round several times,
+    and the kernels that start beside the one in front of them read the table of this call.  Against contexts of one call each."""
+    Hq, Hkv, D, n = 8, 4, 64, 1536
+    rng = random.Random(15)
+    gen = torch.Generator("cuda").manual_seed(15)
+    q, kk, v, dout = (_rows(n + n // k * m, H, D, gen, False) for H in (Hq, Hkv, Hkv, Hq))
+    once = ksa.Context(0)
+    own = ksa.Context(0)
+    for call in range(150):
+        cuts = sorted(rng.sample(range(1, n), rng.randrange(1, 8)))
+        lens = [b - a for a, b in zip([0] + cuts, cuts + [n])]
+        prob = ksa.Problem(lens, k, m, 4, Hq, Hkv, D, D ** -0.5)
+        total = ksa.total_aug_len(prob)
+        args = q[:total], kk[:total], v[:total]
+        ws = torch.empty(max(256, ksa.workspace_bytes(prob)), dtype=torch.uint8, device="cuda")
+        wsb = torch.empty(ksa.bwd_workspace_bytes(prob), dtype=torch.uint8, device="cuda")
+        got = []
+        for c in (own, once):
+            out, dq, dk, dv = (torch.full_like(t, 7.0) for t in (args[0], *args))
+            lse = torch.empty((Hq, total), dtype=torch.float32, device="cuda")
+            c.attn_fwd(prob, *args, out, lse, ws)
+            c.attn_bwd(prob, *args, out, lse, dout[:total], dq, dk, dv, wsb)
+            got.append((out, lse, dq, dk, dv))
+        torch.cuda.synchronize()
+        once.close()
+        once = ksa.Context(0)
+        for a, b in zip(got[0][:3], got[1][:3]):
+            assert torch.equal(a, b), (call, lens)
+        for a, b in zip(got[0][3:], got[1][3:]):              # (as above)
+            a, b = a.float(), b.float()
+            assert ((a - b).abs() <= 2 ** -7 * b.abs() + 1e-6 * b.abs().max()).all(), (call, lens)
+    once.close()
+    own.close()
