@@ -119,15 +119,22 @@ __device__ __forceinline__ bool bt_wait(uint32_t bar, uint32_t parity, uint32_t 
 }
 // A converged warp waits, every branch on a vote of the whole warp: after a wait of each lane, or of one lane, for itself the
 // compiler no longer takes the warp for converged (dK / dV 822 -> 759 thousand cycles; cases of the head comment)
-__device__ __forceinline__ bool bt_wait_converged(uint32_t bar, uint32_t parity, uint32_t abort_addr, int32_t* status, int code)
+// progress: the address of a word that changes while somebody still works towards this barrier; the limit then starts again.
+__device__ __forceinline__ bool bt_wait_converged(uint32_t bar, uint32_t parity, uint32_t abort_addr, int32_t* status, int code,
+                                                  long long limit = 1ll << 31, uint32_t progress = 0)
 {
     if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    const long long t0 = clock64();
+    long long t0 = clock64();
+    uint32_t seen = 0;
     for (uint32_t it = 1;; ++it) {
         if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
         if ((it & 63u) == 0u) {
             if (__any_sync(0xffffffffu, bt_ld_shared(abort_addr) != 0u)) return false;
-            if (__any_sync(0xffffffffu, clock64() - t0 > (1ll << 31))) {
+            if (__any_sync(0xffffffffu, clock64() - t0 > limit)) {
+                if (progress != 0u) {
+                    const uint32_t now = __shfl_sync(0xffffffffu, bt_ld_shared(progress), 0);
+                    if (now != seen) { seen = now; t0 = clock64(); continue; }
+                }
                 atomicCAS(status, 0, code);
                 bt_st_shared(abort_addr, 1u);
                 return false;
@@ -148,6 +155,7 @@ struct BtSmem {
     __device__ __forceinline__ uint32_t bar(int i) const { return base + M::kOffBars + 8u * (uint32_t)i; }
     __device__ __forceinline__ uint32_t tmem_slot() const { return base + M::kOffMisc; }
     __device__ __forceinline__ uint32_t abort_addr() const { return base + M::kOffMisc + 4; }
+    __device__ __forceinline__ uint32_t blocks_taken() const { return base + M::kOffMisc + 12; }       // answered requests
     __device__ __forceinline__ uint32_t next_block() const { return base + M::kOffMisc + 16; }
     __device__ __forceinline__ uint32_t unit(int n, int word) const { return base + M::kOffUnit + (uint32_t)(n & 1) * 64u + 4u * (uint32_t)word; }
 };
@@ -187,6 +195,7 @@ __device__ __forceinline__ void bt_init_barriers(const BtSmem<D>& sm)
     mbar_init(sm.bar(BB_DRAIN), 1);
     bt_st_shared(sm.abort_addr(), 0u);
     bt_st_shared(sm.abort_addr() + 4, 0u);
+    bt_st_shared(sm.blocks_taken(), 0u);
     fence_mbar_init();
 }
 template <int D>
@@ -325,6 +334,19 @@ __device__ __forceinline__ int bt_take_block(const BtSmem<D>& sm, int n, BtBlock
     if (!bt_wait(sm.bar(BB_CLC), (uint32_t)(n & 1), sm.abort_addr(), status, kStatusWaitNextBlock)) return -1;
     return clc_query(sm.next_block(), blk.x, blk.y, blk.z) ? 1 : 0;
 }
+// The other side for dK / dV: descriptor n is there.  The producer may have to pass any number of blocks without work on its way
+// to the next unit (every tile has the segments that a tile of the longest sequence may need): a long sequence among 65,000 short
+// ones has tens of millions of them in a row, at 2 us each on 148 SMs a second's worth, so the limit holds from one to the next.
+#ifdef KSA_DEBUG
+constexpr long long kUnitWaitCycles = 1ll << 17;        // (so that a test of milliseconds passes it)
+#else
+constexpr long long kUnitWaitCycles = 1ll << 31;
+#endif
+template <int D>
+__device__ __forceinline__ bool bt_wait_unit(const BtSmem<D>& sm, int n, int32_t* status)
+{
+    return bt_wait_converged(sm.bar(BB_UFULL + (n & 1)), (uint32_t)((n >> 1) & 1), sm.abort_addr(), status, kStatusWaitUnit, kUnitWaitCycles, sm.blocks_taken());
+}
 // A word of descriptor n for a whole warp, known to the compiler as the same in every lane: loop counts and addresses that come
 // of it stay in uniform registers.
 template <int D>
@@ -433,6 +455,7 @@ __device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& ma
                         const int got = bt_take_block(sm, asked, blk, a.status);
                         if (got < 0) { alive = false; break; }
                         ++asked; pending = false;
+                        bt_st_shared(sm.blocks_taken(), (uint32_t)asked);
                         took_first |= got > 0 && blk.x + blk.y == 0;
                         if (got == 0 || bt_dkv_unit(a, blk, summ, seg_tiles, segs, u)) break;
                         u.J = 0;
@@ -473,7 +496,7 @@ __device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& ma
             int g = 0, s1 = 0;                                            // tiles of the units before; the next tile's B1 stage ...
             uint32_t b1_phase = 0;                                        // ... and the parity of its fill
             for (int n = 0; alive; ++n) {
-                if (!wait(su.bar(BB_UFULL + (n & 1)), (n >> 1) & 1, kStatusWaitUnit)) break;
+                if (!bt_wait_unit(su, n, a.status)) break;
                 const int Ju = bt_unit_word(su, n, U_J);
                 mbar_arrive_warp(leader, su.bar(BB_UEMPTY + (n & 1)));
                 if (Ju == 0) break;
@@ -540,7 +563,7 @@ __device__ __forceinline__ void bt_dkv_block(const BwdArgs& a, const BwdMaps& ma
         int J = 0, kt = 0, hk = 0, qt = 0, text_off = 0, krow0 = 0, key = 0;       // the unit; the next pair's query tile
         bool alive = true;
         auto take_unit = [&](int n) -> bool {
-            if (!bt_wait_converged(sm.bar(BB_UFULL + (n & 1)), (n >> 1) & 1, sm.abort_addr(), a.status, kStatusWaitUnit)) return false;
+            if (!bt_wait_unit(sm, n, a.status)) return false;
             __syncwarp();
             J = bt_unit_word(sm, n, U_J); text_off = bt_unit_word(sm, n, U_TEXT_OFF);
             kt = bt_unit_word(sm, n, U_TILE); hk = bt_unit_word(sm, n, U_HEAD);

@@ -80,3 +80,52 @@ def test_debug_build_edge_shapes():
     r = subprocess.run([sys.executable, "-c", DEBUG_SCRIPT % dict(root=ROOT)], capture_output=True, text=True, env=env, timeout=1500, cwd=ROOT)
     assert r.returncode == 0, (r.stdout[-1500:], r.stderr[-3000:])
     assert "debug build ok" in r.stdout
+
+
+DEBUG_BWD_SCRIPT = r"""
+import sys
+sys.path.insert(0, %(root)r)
+import torch
+from paper_2604_24432_b200 import binding as ksa
+assert ksa.LIB_PATH.endswith("_debug.so")
+ctx = ksa.Context(0)
+k, m, C, Hq, Hkv, D, n_long = 8, 1, 4, 4, 1, 64, 32768
+def backward(before, behind):
+    lens = [9] * before + [n_long] + [9] * behind
+    prob = ksa.Problem(lens, k, m, C, Hq, Hkv, D, 0.125)
+    total, at, rows = ksa.total_aug_len(prob), before * ksa.aug_len(9, k, m), ksa.aug_len(n_long, k, m)
+    t = []
+    for i, H in enumerate((Hq, Hkv, Hkv, Hq)):            # the long sequence's rows are the same in both calls
+        x = torch.randn((rows, H, D), generator=torch.Generator("cuda").manual_seed(i), device="cuda")
+        t.append(torch.ones((total, H, D), dtype=torch.bfloat16, device="cuda"))
+        t[-1][at:at + rows] = x
+    q, kk, v, dout = t
+    out, lse = torch.empty_like(q), torch.empty((Hq, total), dtype=torch.float32, device="cuda")
+    dq, dk, dv = (torch.full_like(x, 7.0) for x in (q, kk, v))
+    ws = torch.empty(max(256, ksa.workspace_bytes(prob)), dtype=torch.uint8, device="cuda")
+    ctx.attn_fwd(prob, q, kk, v, out, lse, ws)
+    ctx.attn_bwd(prob, q, kk, v, out, lse, dout, dq, dk, dv, torch.empty(ksa.bwd_workspace_bytes(prob), dtype=torch.uint8, device="cuda"))
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0, ctx.device_status()
+    for x in (dq, dk, dv):
+        assert torch.isfinite(x.float()).all()
+    return dq[at:at + rows], dk[at:at + rows].float(), dv[at:at + rows].float()
+alone, among = backward(0, 0), backward(3000, 3000)
+assert torch.equal(alone[0], among[0])
+for a, b in zip(alone[1:], among[1:]):                    # fp32 atomics in either order, then bf16: one rounding apart
+    assert ((a - b).abs() <= 2 ** -7 * b.abs() + 1e-6 * b.abs().max()).all()
+print("debug backward ok")
+"""
+
+
+@pytest.mark.gpu
+def test_debug_build_passes_blocks_without_work():
+    """dK / dV of one long sequence among 6,000 short ones: of the 6,032 x 16 blocks of the summary keys' launch those of the short
+    sequences hold no work, some 300 a CTA one after the other on either side.  Units that are waited for meanwhile keep waiting beyond the limit
+    of a wait (2^17 cycles in the debug build), and what comes out is what the long sequence gives alone."""
+    from paper_2604_24432_b200 import build as ksa_build
+    ksa_build.build(variant="debug")
+    env = dict(os.environ, KSA_B200_LIB_VARIANT="debug")
+    r = subprocess.run([sys.executable, "-c", DEBUG_BWD_SCRIPT % dict(root=ROOT)], capture_output=True, text=True, env=env, timeout=600, cwd=ROOT)
+    assert r.returncode == 0, (r.stdout[-1500:], r.stderr[-3000:])
+    assert "debug backward ok" in r.stdout
