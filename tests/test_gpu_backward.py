@@ -44,6 +44,7 @@ def _check(name, got, ref):
     ([600, 9], 8, 1, 0, 4, 2, 128, 0),                # no window beyond the own chunk
     ([900], 8, 1, 1000, 4, 2, 128, 0),                # window longer than the sequence: plain causal attention
     ([5, 130, 64, 1, 257], 8, 1, 4, 8, 1, 128, 0),    # many short sequences, one KV head for 8 query heads
+    ([2300, 300], 8, 1, 1000, 4, 1, 128, 0),          # two segments of query tiles, most second ones empty
     # whole chunks everywhere: the tensor-core kernels read q, k, v, dout in place (no packed copies)
     ([1024, 264, 8], 8, 1, 4, 4, 2, 128, 0),          # sequences that end inside a 128-row tile
     ([1280], 64, 8, 4, 4, 2, 128, 0),
@@ -96,13 +97,26 @@ def test_backward_matches_oracle(ctx, lens, k, m, C, Hq, Hkv, D, flags):
     _check("dv", dv.double().cpu().numpy(), rdv)
 
 
-@pytest.mark.parametrize("lens,k,m,C,Hq,Hkv,D", [
-    ([7, 1, 90, 128, 129, 3, 64, 256, 5] * 6, 8, 1, 4, 8, 4, 64),      # units of one and two tiles, several to a CTA
-    ([3, 1500, 5, 7, 900, 2], 8, 1, 16, 16, 8, 128),                   # sequences without summary rows between others
-    ([2300, 300], 8, 1, 1000, 4, 1, 128),                              # two segments of query tiles, most second ones empty
+def _blocks(lens, k, m, C, Hq, Hkv):
+    """Blocks of the three tensor-core launches: dK / dV of the summary keys and of the text keys, dQ."""
+    tiles = [-(-n // 128) for n in lens]
+    seg = max(16, 64 // (Hq // Hkv))                                   # query tiles of a segment
+    segs = lambda span: -(-span // seg)
+    return (sum(-(-(n // k * m) // 128) for n in lens) * segs(max(tiles)) * Hkv,
+            sum(tiles) * segs(min(max(tiles), (C + 1) * k // 128 + 2)) * Hkv, sum(tiles) * Hq)
+
+
+@pytest.mark.parametrize("lens,k,m,C,Hq,Hkv,D,summ", [
+    ([7, 1, 90, 128, 129, 3, 64, 256, 5] * 8, 8, 1, 4, 8, 4, 64, True),       # units of one and two tiles, several to a CTA
+    ([3, 1500, 5, 7, 900, 2], 8, 1, 16, 16, 8, 128, False),                   # sequences without summary rows between others
+    ([40] * 15 + [2300] + [40] * 15, 8, 1, 1000, 16, 4, 64, True),            # two segments of query tiles, all second ones but the long
+    ([40] * 15 + [2300] + [40] * 15, 8, 1, 4, 16, 4, 128, True),              # sequence's empty; ... of the summary keys
 ])
-def test_backward_many_units_per_cta(ctx, lens, k, m, C, Hq, Hkv, D):
-    """More units of work than SMs: CTAs go on to the blocks that have not started."""
+def test_backward_many_units_per_cta(ctx, lens, k, m, C, Hq, Hkv, D, summ):
+    """More blocks than SMs in the launches of the text keys and of dQ, where `summ` says so in that of the summary keys, too: CTAs
+    go on to blocks that have not started, and past those without work."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert all(n > sms for n in _blocks(lens, k, m, C, Hq, Hkv)[0 if summ else 1:])
     test_backward_matches_oracle(ctx, lens, k, m, C, Hq, Hkv, D, 0)
 
 
