@@ -22,10 +22,28 @@ def ctx():
     c.close()
 
 
-def _rows(total, H, D, gen, strided):
-    """bf16 rows [total, H, D]; strided: heads with a gap between them, rows with a longer one."""
-    full = torch.randn((total, H + 1, D + 8) if strided else (total, H, D), generator=gen, device="cuda").bfloat16()
-    return full[:, 1:, :D] if strided else full
+def _rows(total, H, D, gen, layout="dense", gap=8):
+    """bf16 rows [total, H, D]; "gaps": heads with `gap` elements between them, rows with more; "heads first": [H, total, D] in memory."""
+    if layout == "heads first":
+        return torch.randn((H, total, D), generator=gen, device="cuda").bfloat16().transpose(0, 1)
+    if layout == "gaps":
+        return torch.randn((total, H + 1, D + gap), generator=gen, device="cuda").bfloat16()[:, 1:, :D]
+    return torch.randn((total, H, D), generator=gen, device="cuda").bfloat16()
+
+
+def _like(t):
+    return torch.empty_strided(t.shape, t.stride(), dtype=t.dtype, device=t.device).fill_(7.0)
+
+
+def _assert_same_bits(a, b, what=None):
+    as_int = {torch.bfloat16: torch.int16, torch.float32: torch.int32}[a.dtype]
+    assert torch.equal(a.view(as_int), b.view(as_int)), what
+
+
+def _assert_one_rounding_apart(a, b, what=None):
+    """dk, dv: sums of fp32 atomics in either order, then bf16."""
+    a, b = a.float(), b.float()
+    assert ((a - b).abs() <= 2 ** -7 * b.abs() + 1e-6 * b.abs().max()).all(), what
 
 
 @pytest.mark.parametrize("lens,k,m,C,Hq,Hkv,D", [
@@ -34,28 +52,34 @@ def _rows(total, H, D, gen, strided):
     ([1153, 2175], 8, 1, 16, 4, 4, 128),                 # 144 and 271 summary rows: full tiles and last ones
     ([4097, 70], 64, 8, 4, 8, 2, 128),                   # 64 chunks of eight summaries: four full tiles, none left over
     ([300, 1011], 8, 0, 1 << 20, 4, 2, 128),             # no summaries
-    ([513, 255, 771], 1, 1, 100, 4, 2, 64),              # chunks of one token: no length is ragged but for the tile
+    ([513, 255, 771], 1, 1, 100, 4, 2, 64),              # chunks of one token: never ragged, read in place either way
+    ([513, 255, 771], 2, 2, 50, 4, 2, 64),               # chunks of two
     ([400, 999], 128, 2, 1, 6, 2, 128),                  # a chunk fills a tile; head pairs across KV heads
 ])
-@pytest.mark.parametrize("strided", [False, True])
-def test_tails_equal_the_packed_path(ctx, lens, k, m, C, Hq, Hkv, D, strided):
+@pytest.mark.parametrize("layout", ["dense", "gaps", "heads first"])
+def test_tails_equal_the_packed_path(ctx, lens, k, m, C, Hq, Hkv, D, layout):
     gen = torch.Generator("cuda").manual_seed(11)
     packed = ksa.Problem(lens, k, m, C, Hq, Hkv, D, D ** -0.5, PACKED)
     prob = ksa.Problem(lens, k, m, C, Hq, Hkv, D, D ** -0.5)
     total = ksa.total_aug_len(prob)
-    q, kk, v = (_rows(total, H, D, gen, strided) for H in (Hq, Hkv, Hkv))
+    # (strides of their own for q, k, v and for out and dout)
+    q, kk, v, dout = (_rows(total, H, D, gen, layout, gap) for H, gap in ((Hq, 8), (Hkv, 16), (Hkv, 24), (Hq, 40)))
     got = []
     for p in (packed, prob):
-        out = torch.empty((total, Hq, D), dtype=torch.bfloat16, device="cuda")
+        out, dq, dk, dv = (_like(t) for t in (dout, q, kk, v))
         lse = torch.empty((Hq, total), dtype=torch.float32, device="cuda")
         ws = torch.full((max(256, ksa.workspace_bytes(p)),), 0xFF, dtype=torch.uint8, device="cuda")   # NaN patterns
+        wsb = torch.full((ksa.bwd_workspace_bytes(p),), 0xFF, dtype=torch.uint8, device="cuda")
         ctx.clear_device_status()
         ctx.attn_fwd(p, q, kk, v, out, lse, ws)
+        ctx.attn_bwd(p, q, kk, v, out, lse, dout, dq, dk, dv, wsb)
         torch.cuda.synchronize()
         assert ctx.device_status() == 0
-        got.append((out, lse))
-    assert torch.equal(got[0][0].view(torch.int16), got[1][0].view(torch.int16))
-    assert torch.equal(got[0][1].view(torch.int32), got[1][1].view(torch.int32))
+        got.append((out, lse, dq, dk, dv))
+    for a, b in zip(got[0][:3], got[1][:3]):
+        _assert_same_bits(a, b)
+    for a, b in zip(got[0][3:], got[1][3:]):
+        _assert_one_rounding_apart(a, b)
 
 
 def test_the_forward_pass_ignores_the_backward_flag(ctx):
@@ -66,7 +90,7 @@ def test_the_forward_pass_ignores_the_backward_flag(ctx):
         prob = ksa.Problem([1027, 333], 8, 1, 4, 4, 2, 128, 128 ** -0.5, flags)
         total = ksa.total_aug_len(prob)
         gen = torch.Generator("cuda").manual_seed(14)
-        q, kk, v = (_rows(total, H, 128, gen, False) for H in (4, 2, 2))
+        q, kk, v = (_rows(total, H, 128, gen) for H in (4, 2, 2))
         lse = torch.empty((4, total), dtype=torch.float32, device="cuda")
         left.append(torch.full((ksa.workspace_bytes(prob),), 0xFF, dtype=torch.uint8, device="cuda"))
         ctx.attn_fwd(prob, q, kk, v, torch.empty_like(q), lse, left[-1])
@@ -79,7 +103,7 @@ def test_a_sequence_does_not_see_its_neighbour(ctx):
     gen = torch.Generator("cuda").manual_seed(12)
     prob = ksa.Problem(lens, k, m, C, Hq, Hkv, D, D ** -0.5)
     total = ksa.total_aug_len(prob)
-    q, kk, v, dout = (_rows(total, H, D, gen, False) for H in (Hq, Hkv, Hkv, Hq))
+    q, kk, v, dout = (_rows(total, H, D, gen) for H in (Hq, Hkv, Hkv, Hq))
     lo, hi = ksa.aug_len(333, k, m), ksa.aug_len(333, k, m) + ksa.aug_len(258, k, m)
     for t in (kk, v, dout):
         t[lo:hi] = float("nan")
@@ -107,7 +131,7 @@ def test_a_head_stride_that_no_tensor_map_holds(ctx, wide):
     total = sum(ksa.aug_len(n, k, m) for n in lens)
     prob = ksa.Problem(lens, k, m, C, Hq, 1, D, D ** -0.5)
     gen = torch.Generator("cuda").manual_seed(13)
-    q, kk, v, dout = (_rows(total, H, D, gen, False) for H in (Hq, 1, 1, Hq))
+    q, kk, v, dout = (_rows(total, H, D, gen) for H in (Hq, 1, 1, Hq))
 
     def view(t, name):
         return t.as_strided(t.shape, (t.stride(0), 1 << 39, 1)) if name == wide else t
@@ -126,10 +150,9 @@ def test_a_head_stride_that_no_tensor_map_holds(ctx, wide):
         assert ctx.device_status() == 0
         got.append((out, lse, dq, dk, dv))
     for a, b in zip(got[0][:3], got[1][:3]):
-        assert torch.equal(a, b)
-    for a, b in zip(got[0][3:], got[1][3:]):                  # fp32 atomics in either order, then bf16: one rounding apart
-        a, b = a.float(), b.float()
-        assert ((a - b).abs() <= 2 ** -7 * b.abs() + 1e-6 * b.abs().max()).all()
+        _assert_same_bits(a, b)
+    for a, b in zip(got[0][3:], got[1][3:]):
+        _assert_one_rounding_apart(a, b)
 
 
 @pytest.mark.parametrize("k,m", [(8, 1), (24, 8)])
@@ -139,7 +162,7 @@ def test_schedules_that_share_memory(ctx, k, m):
     Hq, Hkv, D, n = 8, 4, 64, 1536
     rng = random.Random(15)
     gen = torch.Generator("cuda").manual_seed(15)
-    q, kk, v, dout = (_rows(n + n // k * m, H, D, gen, False) for H in (Hq, Hkv, Hkv, Hq))
+    q, kk, v, dout = (_rows(n + n // k * m, H, D, gen) for H in (Hq, Hkv, Hkv, Hq))
     once = ksa.Context(0)
     own = ksa.Context(0)
     for call in range(150):
@@ -161,9 +184,8 @@ def test_schedules_that_share_memory(ctx, k, m):
         once.close()
         once = ksa.Context(0)
         for a, b in zip(got[0][:3], got[1][:3]):
-            assert torch.equal(a, b), (call, lens)
-        for a, b in zip(got[0][3:], got[1][3:]):              # (as above)
-            a, b = a.float(), b.float()
-            assert ((a - b).abs() <= 2 ** -7 * b.abs() + 1e-6 * b.abs().max()).all(), (call, lens)
+            _assert_same_bits(a, b, (call, lens))
+        for a, b in zip(got[0][3:], got[1][3:]):
+            _assert_one_rounding_apart(a, b, (call, lens))
     once.close()
     own.close()
