@@ -886,10 +886,12 @@ static int launch_text(ksa_ctx* ctx, const KernelArgs& a, uint32_t flags, const 
 
 // Where the text rows' kernel is short, the SMs that it leaves idle (small calls) or leaves early (its last round of work
 // items) are worth the summary rows' time.  In front -> behind, in rounds of work items per SM, 32/8 heads of 128: tiles read in
-// place 213 -> 202 us at 7, 547 -> 543 at 14; packed 33.2 -> 30.9 us at 1, 79.6 -> 76.8 at 3, equal to 1 % at 7 - 21; heads of
-// 64 436 -> 419 us at 14, long chunks 448 -> 444 us at 14.  Further out packed calls lose (1,597 -> 1,648 us at 28, 6,905 ->
-// 6,966 at 108), so the line lies in front of those; calls read in place would still gain 1 - 3 % (973 -> 962 us at 21,
-// 9.8 -> 9.5 ms at 83).
+// place 213 -> 202 us at 7, 547 -> 543 at 14; packed whole 33.2 -> 30.9 us at 1, 79.6 -> 76.8 at 3, equal to 1 % at 7 - 21;
+// heads of 64 436 -> 419 us at 14, long chunks 448 -> 444 us at 14.  Further out packed calls lose (1,597 -> 1,648 us at 28,
+// 6,905 -> 6,966 at 108), so the line lies in front of those; whole-chunk calls read in place would still gain 1 - 3 % (973 ->
+// 962 us at 21, 9.8 -> 9.5 ms at 83).  The packed figures are those of ragged batches when all their rows were packed; packed
+// whole are now prepared calls and chunks that do not divide a tile.  Ragged batches with full tiles in place are under the same
+// line; beyond it they were not timed on both sides.
 static constexpr int kBehindTextRounds = 16;
 static bool behind_text_pays(const ksa_ctx* ctx, const KernelArgs& a) { return a.num_work <= kBehindTextRounds * ctx->num_sms; }
 

@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(128) ksa_bwd_dkv_kernel(BwdArgs a, int summ)
 }
 
 // =================================================================================================
-// preparation: text rows of dO into the packed layout (not in direct mode), lse in log2 units, delta = <dO, O>
+// preparation: the text rows of dO that ReadMode wants into the packed layout, lse in log2 units, delta = <dO, O>
 // =================================================================================================
 // A block takes four neighbouring rows of the text stream, all heads: a thread keeps its vector of a head and walks the
 // heads with eight loads in flight (HBM-bound: 2 x 32,768 tokens, 32 heads 308 -> 178 us = 6.8 TB/s; a thread

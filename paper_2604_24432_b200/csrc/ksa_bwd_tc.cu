@@ -45,11 +45,14 @@
 //
 // What bounds them: the row warps and the shared-memory reads of the products (X and Y read both operands from there: 160 KB a
 // tile of dQ and 192 KB of dK / dV beside 64 KB that TMA writes, at 128 bytes a cycle).  Thousand cycles of 148 SMs, a CTA per
-// unit -> CTAs that stay: 2 x 8,192 tokens in 64 + 8 chunks, 32/8 heads: dQ 961 -> 810, dK / dV 454 + 878 -> 388 + 752; 7,942
-// ragged tokens, 16/16 heads: 206 -> 155, 77 + 270 -> 70 + 217.  A training layer 2,107 -> 1,983 us, 585 -> 548 us; 2 x 32,768
-// tokens 14.5 -> 13.9 ms (power cap).  A unit's end costs about 3,500 cycles (last product, epilogue, first loads of the next
-// unit's scalars) where the end of a CTA and the start of the next took some 10,000.  The scalars of the next tile
-// are negated when they are stored and not beside their load, which stalled every tile of dK / dV for it (5 - 7 %).
+// unit -> CTAs that stay: 2 x 8,192 tokens in 64 + 8 chunks, 32/8 heads: dQ 961 -> 774, dK / dV 454 + 878 -> 386 + 751 (tensor pipe
+// 73, 69 and 74 % active at 2 x 32,768); 7,942 ragged tokens, 16/16 heads, packed: 206 -> 155, 77 + 270 -> 70 + 217.  A training
+// layer 2,107 -> 1,983 us, 585 -> 548 us; 2 x 32,768 tokens 14.5 -> 13.9 ms (power cap).  Full tiles read in place take these
+// ragged launches 118 us of dQ where packed ones take 104, 191 of dK / dV where they take 185, and spare 52 us of pack.
+// dK / dV spills 8 bytes (32 of loads) at head_dim 128, 4 (24) at 64; dQ nothing.
+// A unit's end costs about 3,500 cycles (last product, epilogue, first loads of the next unit's scalars) where the end of a CTA
+// and the start of the next took some 10,000.  The scalars of the next tile are negated when they are stored and not beside their
+// load, which stalled every tile of dK / dV for it (5 - 7 %).
 // Tried and taken back: a second issuing warp (dQ 811 -> 841), the Q / K stage checked a tile ahead (759 -> 943).
 #include <cuda_bf16.h>
 
@@ -190,7 +193,7 @@ __device__ __forceinline__ void bt_init_barriers(const BtSmem<D>& sm)
     mbar_init(sm.bar(BB_PB2), 16);
     mbar_init(sm.bar(BB_OFULL), 1);
     mbar_init(sm.bar(BB_AEMPTY), 1);
-    for (int s = 0; s < 2; ++s) { mbar_init(sm.bar(BB_UFULL + s), 1); mbar_init(sm.bar(BB_UEMPTY + s), 17); }   // read by 16 row warps and two issuers
+    for (int s = 0; s < 2; ++s) { mbar_init(sm.bar(BB_UFULL + s), 1); mbar_init(sm.bar(BB_UEMPTY + s), 17); }   // 16 row warps and the issuer
     mbar_init(sm.bar(BB_CLC), 1);
     mbar_init(sm.bar(BB_DRAIN), 1);
     bt_st_shared(sm.abort_addr(), 0u);

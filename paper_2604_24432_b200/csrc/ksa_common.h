@@ -17,7 +17,8 @@ struct SeqInfo {
     int32_t summ_off;   // first row in the packed summary stream (multiple of kTileN)
     int32_t text_pad;   // padded text rows (multiple of kTileM)
     int32_t summ_pad;   // padded summary rows (multiple of kTileN)
-    int32_t chunk0;     // aug_off / (k + m): first chunk of the sequence in the direct views (valid if every length is a multiple of k)
+    int32_t chunk0;     // aug_off / (k + m): where the sequence starts in the [chunk, k + m] grid of the caller's rows, at row
+                        // row_in_chunk() of that chunk (0 in whole-chunk batches)
     int32_t summ_base;  // summary rows of the sequences before this one (unpadded count)
 };
 
@@ -57,7 +58,7 @@ struct KernelArgs {
     uint32_t flags;
     float scale;            // softmax scale
     float scale_log2;       // scale * log2(e)
-    uint64_t k_inverse;     // floor(2^64 / k) + 1, for i / k as a product (0 where k is 1); set by the text kernel's launch
+    uint64_t k_inverse;     // 2^64 / k rounded up, for i / k as a product (0 where k is 1); set by the text kernel's launch
     int64_t total_aug;
     int64_t text_rows;      // padded rows of the packed text stream
     int64_t summ_rows;      // padded rows of the packed summary stream

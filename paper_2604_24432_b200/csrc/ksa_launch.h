@@ -41,7 +41,7 @@ cudaError_t launch_summary_mma(const KernelArgs& a, int max_chunks, unsigned ny,
 cudaError_t launch_text_ref(const KernelArgs& a, cudaStream_t stream);
 
 // Text rows, tcgen05/TMA kernel.  The five tensor maps describe the packed streams
-// as [D, rows, H] with a {64, 128, 1} box and 128-byte swizzle, or (KernelArgs::direct) the
+// as [D, rows, H] with a {64, 128, 1} box and 128-byte swizzle, or (kReadInPlace) the
 // caller's interleaved tensors as [D, k, chunks, H] (text rows; box {64, k, 128/k, 1}) and
 // [D, m, chunks, H] starting k rows in (summary rows; box {64, m, 128/m, 1}): the box lands in
 // shared memory as the same dense 128-row tile either way.
@@ -53,7 +53,7 @@ cudaError_t launch_text_tc(const KernelArgs& a, const TextMaps& maps, int num_sm
 cudaError_t setup_text_tc();
 
 // Text rows on CTA pairs (head_dim 128, work items of two query heads): same tensor maps, except that kt and ks
-// have boxes of 64 key rows ({64, 64, 1}; direct: {64, k, 64 / k, 1} and {64, m, 64 / m, 1}) -- each CTA of a pair
+// have boxes of 64 key rows ({64, 64, 1}; read in place: {64, k, 64 / k, 1} and {64, m, 64 / m, 1}) -- each CTA of a pair
 // loads half of a K tile.  max_pairs = clusters of two CTAs the device runs at once (from setup_text_pair).
 struct PairMaps { CUtensorMap qt, kt, vt, ks, vs; };
 cudaError_t launch_text_pair(const KernelArgs& a, const PairMaps& maps, int max_pairs, cudaStream_t stream);
