@@ -341,7 +341,7 @@ __device__ __forceinline__ int bt_take_block(const BtSmem<D>& sm, int n, BtBlock
 // to the next unit (every tile has the segments that a tile of the longest sequence may need): a long sequence among 65,000 short
 // ones has tens of millions of them in a row, at 2 us each on 148 SMs a second's worth, so the limit holds from one to the next.
 #ifdef KSA_DEBUG
-constexpr long long kUnitWaitCycles = 1ll << 17;        // (so that a test of milliseconds passes it)
+constexpr long long kUnitWaitCycles = 1ll << 19;        // (so that a test of milliseconds passes it)
 #else
 constexpr long long kUnitWaitCycles = 1ll << 31;
 #endif

@@ -121,8 +121,9 @@ print("debug backward ok")
 @pytest.mark.gpu
 def test_debug_build_passes_blocks_without_work():
     """dK / dV of one long sequence among 6,000 short ones: of the 6,032 x 16 blocks of the summary keys' launch those of the short
-    sequences hold no work, some 300 a CTA one after the other on either side.  Units that are waited for meanwhile keep waiting beyond the limit
-    of a wait (2^17 cycles in the debug build), and what comes out is what the long sequence gives alone."""
+    sequences hold no work, some 300 a CTA one after the other on either side.  Units that are waited for meanwhile keep waiting
+    beyond the limit of a wait (2^19 cycles, 0.27 ms, in the debug build; the blocks of either side take 0.7 ms), and what comes
+    out is what the long sequence gives alone."""
     from paper_2604_24432_b200 import build as ksa_build
     ksa_build.build(variant="debug")
     env = dict(os.environ, KSA_B200_LIB_VARIANT="debug")
